@@ -184,7 +184,7 @@ Layout make_layout(const pm_config& c, size_t work_bytes) {
   L.srow = take((N * N + 1) * 4);
   L.mrow = take((N * N + 1) * 4);
   L.tile_cnt = take(16);  // (stayers, movers) of the last re-sort
-  L.row_start = take((N * N + 1) * 4);
+  L.row_start = take((N * N + CROWD_WORDS) * 4);
   L.rho = take(n3 * rsz);
   L.phi = take(n3 * rsz);
   L.q = take(n3 * rsz);
@@ -418,7 +418,8 @@ pm_status sort_particles(pm_sim* s) {
   CU(s, cudaMemsetAsync(hist, 0, hist_bytes(), s->stream));
   {
     PROF(s, PM_STAGE_SORT_HISTOGRAM);
-    CU(s, launch_sort_histogram(s->keys, n, L.passes, L.digit_bits, L.key_bits, hist, s->errword() + 1, s->stream));
+    CU(s, launch_sort_histogram(s->keys, n, L.passes, L.digit_bits, L.key_bits, hist, s->errword() + 1, s->stream,
+                                nullptr, s->at<uint32_t>(L.row_start) + s->mesh.n2 + 1));
   }
   const uint32_t* kin = s->keys;
   const uint32_t* vin = nullptr;
@@ -1663,8 +1664,10 @@ pm_status pm_load(pm_sim* s, const void* host, size_t bytes) {
   CU(s, cudaMemcpyAsync(s->keys, in + CKPT_HEADER + 2 * rb, size_t(s->n()) * 4, cudaMemcpyHostToDevice, s->stream));
   CU(s, cudaMemcpyAsync(s->sort_stats(), stats, sizeof stats, cudaMemcpyHostToDevice, s->stream));
   // sorted records: the deposit reads the row starts of the keys (integer, so the same as the re-sort's)
-  if (h.flags & 1)
+  if (h.flags & 1) {
+    CU(s, cudaMemsetAsync(s->at<uint32_t>(s->L.row_start) + s->mesh.n2 + 1, 0, 4, s->stream));
     CU(s, launch_row_start(s->keys, s->n(), uint32_t(s->cfg.n_mesh), s->at<uint32_t>(s->L.row_start), s->stream));
+  }
   CU(s, cudaStreamSynchronize(s->stream));
   s->have_particles = true;
   s->sorted = (h.flags & 1) != 0;

@@ -106,6 +106,17 @@ constexpr int RS_MAX_BITS = 10;
 // set in a sort key by the drift when the particle's cell changed (keys use at most 30 bits)
 constexpr uint32_t KEY_MOVER = 0x80000000u;
 
+// Mesh rows with more records than this are "crowded": the deposit computes the rows they add to by whole
+// blocks instead of one warp each.  A warp takes 0.4 us per batch of 32 records when few warps are busy,
+// so a tile of nine rows of 256 records is ~30 us, about the length of the whole kernel at 256^3.
+// The word after the row starts, row_start[N^2 + 1], says whether any row is (CROWD_WORDS entries follow
+// the N^2 row starts: the closing one and the flag).
+#ifndef PM_DEP_CROWD
+#define PM_DEP_CROWD 256
+#endif
+constexpr uint32_t DEP_CROWD = PM_DEP_CROWD;
+constexpr size_t CROWD_WORDS = 2;
+
 constexpr int KICK_THREADS = 256;
 constexpr int MESH_THREADS = 256;
 constexpr int RED_GRID = 608;    // 4 blocks per SM on 152 SMs, fixed for deterministic reductions
@@ -123,7 +134,7 @@ cudaError_t launch_init_particles(const double* x, const double* p, int64_t n, M
 // n_dev (may be null): device word that overrides n (the grid is sized for n, which must bound it)
 cudaError_t launch_sort_histogram(const uint32_t* keys, int64_t n, int passes, int digit_bits, int key_bits,
                                   uint32_t* hist, uint32_t* epoch, cudaStream_t s,
-                                  const uint32_t* n_dev = nullptr);
+                                  const uint32_t* n_dev = nullptr, uint32_t* crowd = nullptr);
 template <typename R>
 cudaError_t launch_sort_pass(bool last, const uint32_t* keys_in, const uint32_t* vals_in, int64_t n, int shift,
                              int bits, const uint32_t* digit_total, uint64_t* status, uint32_t* tile_counter,
@@ -156,7 +167,8 @@ cudaError_t launch_xy_r2c(const float* rho, void* spec, const void* tw, int n_me
                           size_t ms = 0);
 cudaError_t launch_xy_c2r(const void* spec, float* phi, const void* tw, int n_mesh, cudaStream_t s, int nm = 1,
                           size_t ms = 0);
-// row starts of sorted keys
+// row starts of sorted keys; the crowded-row flag behind them is set if a row is crowded, and has been
+// cleared before (by the sort's histogram: its `crowd` argument)
 cudaError_t launch_row_start(const uint32_t* keys, int64_t n, uint32_t n_mesh, uint32_t* row_start, cudaStream_t s);
 // (nm, ms: a packed group of nm members, ms bytes apart; coefp/qcp: member
 // 0's coefficient in device memory, read per member)

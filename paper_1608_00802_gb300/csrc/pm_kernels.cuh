@@ -9,6 +9,7 @@
 // None of these kernels use floating-point atomics on the step's data, so a
 // step is bitwise reproducible for a fixed launch configuration.
 #pragma once
+#include <algorithm>
 #include <type_traits>
 #include <cuda_runtime.h>
 #include <math.h>
@@ -307,6 +308,8 @@ __device__ __forceinline__ uint32_t divu32(uint32_t e, DivU32 dv) {
 //    (to the next row); within a phase no two source rows meet.
 // The warp alone writes its rows, in a fixed order of chains, batches and
 // phases, so the result is reproducible.
+// Tiles with crowded source rows are left to the launch's last `helpers`
+// blocks (deposit_crowded).
 constexpr int DEP_WARPS = 8;
 
 // slots of a deposit row: N + 1 rounded up to 16 bytes
@@ -316,11 +319,192 @@ __host__ __device__ inline int deposit_stride_of(int n) {
   return (n + 1 + q - 1) / q * q;
 }
 
+// sums v over each run of lanes with equal keys (a segmented inclusive scan in a fixed tree order; the
+// run's last lane ends with the run's sum); runs: the ballot of the lanes that start a run.  The scan stops
+// after the steps the longest run needs (the skipped steps would add nothing).
+template <typename R, int NV>
+__device__ __forceinline__ void run_sums(R (&v)[NV], uint32_t runs, int lane) {
+  const uint32_t above = runs & ~((2u << lane) - 1u);
+  // length of the run that starts at this lane (0 elsewhere)
+  const int len = ((runs >> lane) & 1u) ? (above ? __ffs(above) - 1 : 32) - lane : 0;
+  const int longest = int(__reduce_max_sync(0xffffffffu, uint32_t(len)));
+  for (int off = 1; off < longest; off <<= 1) {
+    R u[NV];
+#pragma unroll
+    for (int a = 0; a < NV; ++a) u[a] = __shfl_up_sync(0xffffffffu, v[a], off);
+    // lane - off is in this lane's run iff no run starts in (lane - off, lane]
+    const uint32_t span = lane >= off ? ((2u << lane) - 1u) & ~((2u << (lane - off)) - 1u) : 0u;
+    if (lane >= off && !(runs & span)) {
+#pragma unroll
+      for (int a = 0; a < NV; ++a) v[a] += u[a];
+    }
+  }
+}
+
+// ---- crowded tiles.  A tile one of whose source rows holds more than DEP_CROWD records (clustered
+// states: a core of 10^6 particles puts thousands into each of a few hundred rows) is left to helper
+// blocks of the same launch, one destination row at a time, because its warp's chain would be the whole
+// kernel's length: 1496 us for that core on a 128^3 mesh, 87 us with the helpers.  The helpers add the
+// same values in the same order as the tile's warp would, so the split does not show in the result.  What is serial about a sum is only each node's own chain of additions, one per batch its two
+// cells are in, so the block computes the sums of all batches first (a warp per batch, any order) and then
+// every node adds up its own (a thread per node, in the batches' order).
+
+// records per window (the batch sums of a window are kept in shared memory)
+template <typename R>
+constexpr int DEP_WINDOW = sizeof(R) == 4 ? 2048 : 1024;
+// shared memory of a helper block: the window's sums, each cell's first and last record of the window, the row
+template <typename R>
+__host__ __device__ inline size_t deposit_crowd_smem(int n) {
+  return size_t(2 * DEP_WINDOW<R> + deposit_stride_of<R>(n)) * sizeof(R) + size_t(2 * n) * sizeof(uint32_t);
+}
+
+struct DepRow {
+  uint32_t b, e;  // records of a source row
+};
+__device__ __forceinline__ DepRow deposit_row_of(const uint32_t* __restrict__ row_start, uint32_t row, uint32_t np) {
+  DepRow r;
+  r.b = __ldg(row_start + row);
+  r.e = min(__ldg(row_start + row + 1), np);
+  if (r.e < r.b) r.e = r.b;  // (only corrupt starts)
+  return r;
+}
+
+// Adds the records [s0, s1) of one source row (base: its first cell's key; batches of 32 counted from
+// record cs) with the weights of (dy, dz) to the row's nodes acc[0 .. n].
+template <typename R>
+__device__ __forceinline__ void deposit_add_segment(const typename VT<R>::v4* __restrict__ pos, uint32_t s0, uint32_t s1,
+                                                    uint32_t cs, uint32_t base, bool dy, bool dz, int n, R* acc,
+                                                    R* sums, uint32_t* cell_range) {
+  constexpr uint32_t W = DEP_WINDOW<R>;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+  uint32_t* first = cell_range;    // first[c], last[c]: the window's records of cell c (last < first: none)
+  uint32_t* last = cell_range + n;
+  // windows of whole batches
+  for (uint32_t w0 = s0; w0 < s1;) {
+    const uint32_t w1 = min(s1, cs + ((w0 - cs) / 32 + W / 32) * 32);
+    for (int c = threadIdx.x; c < n; c += blockDim.x) first[c] = 1, last[c] = 0;
+    __syncthreads();
+    for (uint32_t k = (w0 - cs) / 32 + warp; cs + 32 * k < w1; k += nw) {
+      const uint32_t p = cs + 32 * k + lane;
+      const bool in = p >= w0 && p < w1;
+      typename VT<R>::v4 rec = {};
+      if (in) rec = ldg(pos + p);
+      const uint32_t x = rec_cell(rec) - base;
+      const bool valid = in && x < uint32_t(n);
+      const uint32_t key = valid ? x : 0x80000000u + uint32_t(lane);
+      const R w = (dy ? rec.z : R(1) - rec.z) * (dz ? rec.w : R(1) - rec.w);
+      R v[2] = {(R(1) - rec.y) * w, rec.y * w};
+      const uint32_t kp = __shfl_up_sync(0xffffffffu, key, 1);
+      const uint32_t runs = __ballot_sync(0xffffffffu, lane == 0 || kp != key);
+      if (runs != 0xffffffffu) run_sums<R, 2>(v, runs, lane);
+      if (valid) {
+        // a run's first lane opens the cell unless the cell's previous run is in this window too
+        if (((runs >> lane) & 1u) && !(p > w0 && lane == 0 && rec_cell(ldg(pos + p - 1)) == rec_cell(rec))) first[x] = p;
+        if (lane == 31 || ((runs >> (lane + 1)) & 1u)) {
+          sums[2 * (p - w0)] = v[0];
+          sums[2 * (p - w0) + 1] = v[1];
+          if (!(p + 1 < w1 && lane == 31 && rec_cell(ldg(pos + p + 1)) == rec_cell(rec))) last[x] = p;
+        }
+      }
+    }
+    __syncthreads();
+    // node X: the runs of cell X - 1 (weight f_x), then those of cell X (1 - f_x), in the batches' order
+    for (int X = threadIdx.x; X <= n; X += blockDim.x) {
+      R a = acc[X];
+#pragma unroll
+      for (int h = 1; h >= 0; --h) {
+        const int c = X - h;
+        if (c < 0 || c >= n) continue;
+        const uint32_t l = last[c];
+        for (uint32_t p = first[c]; p <= l;) {
+          const uint32_t at = min(l, cs + ((p - cs) | 31u));  // the run's last record: the cell's, or the batch's
+          a += sums[2 * (at - w0) + h];
+          p = at + 1;
+        }
+      }
+      acc[X] = a;
+    }
+    __syncthreads();
+    w0 = w1;
+  }
+}
+
+// destination row (z, y) by the whole block, in the order of its tile's warp: the plane behind (dz = 1),
+// then its own (dz = 0); in each, the records of source row A = y - 1 (dy = 1) and B = y (dy = 0), except
+// that a batch holding records of both adds B's before A's (its phases dy = 0, dy = 1)
+template <typename R, int TY>
+__device__ __forceinline__ void deposit_crowded_row(const typename VT<R>::v4* __restrict__ pos,
+                                                    const uint32_t* __restrict__ row_start, uint32_t np, const Mesh& m,
+                                                    R norm, R* __restrict__ rho, unsigned char* smem, uint32_t row) {
+  const int n = m.n;
+  R* sums = reinterpret_cast<R*>(smem);
+  R* acc = sums + 2 * DEP_WINDOW<R>;
+  uint32_t* cell_range = reinterpret_cast<uint32_t*>(acc + deposit_stride_of<R>(n));
+  const int z = int(row / uint32_t(n)), y = int(row - uint32_t(z) * uint32_t(n)), y0 = y - y % TY;
+  for (int i = threadIdx.x; i <= n; i += blockDim.x) acc[i] = R(0);
+  __syncthreads();
+#pragma unroll 1
+  for (int dz = 1; dz >= 0; --dz) {
+    const uint32_t plane = uint32_t(wrap(z - dz, n)) * uint32_t(n);
+    const uint32_t ra = plane + uint32_t(wrap(y - 1, n)), rb = plane + uint32_t(y);
+    const DepRow A = deposit_row_of(row_start, ra, np), B = deposit_row_of(row_start, rb, np);
+    // the chains' first records: the tile's rows y0 - 1 .. y0 + TY - 1, split at the seam below y = 0
+    const uint32_t c0 = __ldg(row_start + plane + uint32_t(wrap(y0 - 1, n))), c1 = __ldg(row_start + plane);
+    const uint32_t ca = y0 == 0 && y > 0 ? c1 : c0, cb = y0 == 0 ? c1 : c0;
+    uint32_t ae = A.e, bs = B.b;  // A's records up to ae and B's from bs lie in no common batch
+    if (ca == cb && A.e > A.b && B.e > B.b && (B.b - cb) % 32 != 0) {
+      const uint32_t k0 = cb + (B.b - cb) / 32 * 32;
+      ae = max(A.b, k0), bs = min(B.e, k0 + 32);
+    }
+    deposit_add_segment<R>(pos, A.b, ae, ca, ra * uint32_t(n), true, dz, n, acc, sums, cell_range);
+    if (bs > B.b) {
+      deposit_add_segment<R>(pos, B.b, bs, cb, rb * uint32_t(n), false, dz, n, acc, sums, cell_range);
+      deposit_add_segment<R>(pos, ae, A.e, ca, ra * uint32_t(n), true, dz, n, acc, sums, cell_range);
+    }
+    deposit_add_segment<R>(pos, bs, B.e, cb, rb * uint32_t(n), false, dz, n, acc, sums, cell_range);
+  }
+  R* out = rho + size_t(row) * n;
+  for (int i = threadIdx.x; i < n; i += blockDim.x) out[i] = (i == 0 ? acc[0] + acc[n] : acc[i]) * norm;
+  __syncthreads();  // the row is cleared for the next
+}
+
+// helper block hb of H: its share of the destination rows (every H-th, so that neighbouring rows, crowded
+// together, go to different blocks), of which it computes those of crowded tiles
+template <typename R, int TY, int TZ>
+__device__ __noinline__ void deposit_crowded(const typename VT<R>::v4* __restrict__ pos,
+                                             const uint32_t* __restrict__ row_start, uint32_t np, const Mesh m, R norm,
+                                             R* __restrict__ rho, unsigned char* smem, uint32_t hb, uint32_t H) {
+  __shared__ uint32_t list[DEP_WARPS * 32];
+  __shared__ uint32_t found;
+  const int n = m.n;
+  for (uint32_t k0 = 0; hb + k0 * H < m.n2; k0 += blockDim.x) {
+    if (threadIdx.x == 0) found = 0;
+    __syncthreads();
+    const uint32_t row = hb + (k0 + threadIdx.x) * H;
+    if (row < m.n2) {
+      const int z = int(row / uint32_t(n)), y = int(row - uint32_t(z) * uint32_t(n));
+      const int y0 = y - y % TY, z0 = z - z % TZ, ty = min(TY, n - y0), tz = min(TZ, n - z0);
+      uint32_t most = 0;
+      for (int sz = 0; sz <= tz; ++sz)
+        for (int ly = 0; ly <= ty; ++ly) {
+          const uint32_t src = uint32_t(wrap(z0 - 1 + sz, n)) * uint32_t(n) + uint32_t(wrap(y0 - 1 + ly, n));
+          const DepRow r = deposit_row_of(row_start, src, np);
+          most = max(most, r.e - r.b);
+        }
+      if (most > DEP_CROWD) list[atomicAdd(&found, 1u)] = row;
+    }
+    __syncthreads();
+    const uint32_t c = found;
+    for (uint32_t i = 0; i < c; ++i) deposit_crowded_row<R, TY>(pos, row_start, np, m, norm, rho, smem, list[i]);
+    __syncthreads();
+  }
+}
+
 template <typename R, int TY, int TZ, bool PACKED>
 __global__ void __launch_bounds__(DEP_WARPS * 32) k_deposit(const typename VT<R>::v4* __restrict__ pos,
                                                             const uint32_t* __restrict__ row_start, uint32_t np,
                                                             Mesh m, DivU32 dvn, R norm, R* __restrict__ rho,
-                                                            size_t ms) {
+                                                            uint32_t helpers, size_t ms) {
   using V4 = typename VT<R>::v4;
   static_assert((TY + 1) * (TZ + 1) <= 32, "one source row per lane");
   if constexpr (PACKED) {  // member blockIdx.y of a packed group
@@ -328,6 +512,11 @@ __global__ void __launch_bounds__(DEP_WARPS * 32) k_deposit(const typename VT<R>
     pos = moff(pos, o), row_start = moff(row_start, o), rho = moff(rho, o);
   }
   extern __shared__ __align__(16) unsigned char dep_smem[];
+  if (blockIdx.x >= gridDim.x - helpers) {
+    if (__ldg(row_start + m.n2 + 1))  // some row is crowded
+      deposit_crowded<R, TY, TZ>(pos, row_start, np, m, norm, rho, dep_smem, blockIdx.x - (gridDim.x - helpers), helpers);
+    return;
+  }
   const int n = m.n, stride = deposit_stride_of<R>(n);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
   const int span_y = nw * TY, tiles_y = (n + span_y - 1) / span_y;
@@ -353,6 +542,7 @@ __global__ void __launch_bounds__(DEP_WARPS * 32) k_deposit(const typename VT<R>
     head = ly_l == 0 || yr != wrap(y0 - 2 + ly_l, n) + 1;
     base = srow * uint32_t(n);
   }
+  if (helpers && __any_sync(0xffffffffu, e > b && e - b > DEP_CROWD)) return;  // a crowded tile: the helpers'
   const uint32_t heads = __ballot_sync(0xffffffffu, head);
   const uint32_t later = heads & ~((2u << lane) - 1u);
   const int last = (later ? __ffs(later) - 1 : nr) - 1;                  // the chain's last row (head lanes)
@@ -408,24 +598,8 @@ __global__ void __launch_bounds__(DEP_WARPS * 32) k_deposit(const typename VT<R>
       }
       const uint32_t kp = __shfl_up_sync(0xffffffffu, key, 1);
       const uint32_t runs = __ballot_sync(0xffffffffu, lane == 0 || kp != key);
-      if (runs != 0xffffffffu) {  // some cell holds several particles of the batch
-        // length of the run that starts at this lane (0 elsewhere), and the longest; the scan stops
-        // after the steps the longest run needs (the skipped steps would add nothing)
-        const uint32_t above = runs & ~((2u << lane) - 1u);
-        const int len = ((runs >> lane) & 1u) ? (above ? __ffs(above) - 1 : 32) - lane : 0;
-        const int longest = int(__reduce_max_sync(0xffffffffu, uint32_t(len)));
-        for (int off = 1; off < longest; off <<= 1) {
-          R u[2][2][2];
-#pragma unroll
-          for (int a = 0; a < 8; ++a) (&u[0][0][0])[a] = __shfl_up_sync(0xffffffffu, (&v[0][0][0])[a], off);
-          // lane - off is in this lane's run iff no run starts in (lane - off, lane]
-          const uint32_t span = lane >= off ? ((2u << lane) - 1u) & ~((2u << (lane - off)) - 1u) : 0u;
-          if (lane >= off && !(runs & span)) {
-#pragma unroll
-            for (int a = 0; a < 8; ++a) (&v[0][0][0])[a] += (&u[0][0][0])[a];
-          }
-        }
-      }
+      if (runs != 0xffffffffu)  // some cell holds several particles of the batch
+        run_sums<R, 8>(reinterpret_cast<R(&)[8]>(v), runs, lane);
       const bool add = valid && (lane == 31 || ((runs >> (lane + 1)) & 1u));
       // planes sz - 1 (dz = 0) and sz (dz = 1); the edge plane slots of the tile have one of the two,
       // and the chain's slot is the same for the whole warp, so the adds branch on it instead of
@@ -1892,6 +2066,9 @@ cudaError_t launch_init_particles(const double* x, const double* p, int64_t n, M
 // PM_DEPOSIT_WARP_BYTES of shared memory per 4-byte accumulator (4.25 KB: 2 x 2 rows of a 256^3
 // fp32 mesh; measured there: 43 us against 53 us for 2 x 4 rows, whose 8.3 KB per warp leave
 // too few resident warps)
+#ifndef PM_DEP_HELPERS
+#define PM_DEP_HELPERS 304
+#endif
 #ifndef PM_DEPOSIT_WARP_BYTES
 #define PM_DEPOSIT_WARP_BYTES 4352
 #endif
@@ -1910,16 +2087,25 @@ template <typename R, int TY, int TZ>
 cudaError_t launch_deposit_tile(const void* pos, const uint32_t* row_start, int64_t n, Mesh m, double norm, R* rho,
                                 cudaStream_t s, int warps, int nm, size_t ms) {
   using V4 = typename VT<R>::v4;
-  const size_t smem = size_t(warps) * TY * TZ * deposit_stride_of<R>(m.n) * sizeof(R);
+  // helper blocks for crowded tiles (none with so few particles): at most PM_DEP_HELPERS of 8 warps in all,
+  // and no fewer than 16 rows each
+  unsigned helpers = 0;
+  size_t smem = size_t(warps) * TY * TZ * deposit_stride_of<R>(m.n) * sizeof(R);
+  if (n > int64_t(DEP_CROWD)) {
+    const unsigned most = unsigned(PM_DEP_HELPERS * DEP_WARPS / (warps * nm)), rows = m.n2 / 16 + 1;
+    helpers = most < rows ? most : rows;
+    if (helpers < 8) helpers = 8;
+    smem = std::max(smem, deposit_crowd_smem<R>(m.n));
+  }
   const unsigned tiles_y = unsigned((m.n + warps * TY - 1) / (warps * TY));
   const unsigned blocks = tiles_y * unsigned((m.n + TZ - 1) / TZ);
   const DivU32 dv = divu32_make(uint32_t(m.n));
   if (nm > 1)
-    k_deposit<R, TY, TZ, true><<<dim3(blocks, unsigned(nm)), warps * 32, smem, s>>>(
-        (const V4*)pos, row_start, uint32_t(n), m, dv, R(norm), rho, ms);
+    k_deposit<R, TY, TZ, true><<<dim3(blocks + helpers, unsigned(nm)), warps * 32, smem, s>>>(
+        (const V4*)pos, row_start, uint32_t(n), m, dv, R(norm), rho, helpers, ms);
   else
-    k_deposit<R, TY, TZ, false><<<blocks, warps * 32, smem, s>>>((const V4*)pos, row_start, uint32_t(n), m, dv,
-                                                                 R(norm), rho, 0);
+    k_deposit<R, TY, TZ, false><<<blocks + helpers, warps * 32, smem, s>>>((const V4*)pos, row_start, uint32_t(n), m, dv,
+                                                                           R(norm), rho, helpers, 0);
   return cudaGetLastError();
 }
 
@@ -1929,7 +2115,7 @@ cudaError_t launch_deposit(const void* pos, const uint32_t* row_start, int64_t n
   if (warps < 1 || warps > DEP_WARPS) warps = DEP_WARPS;
   int ty = 1, tz = 1;
   const int shape = deposit_shape<R>(m.n, ty, tz);
-  if (size_t(warps) * ty * tz * deposit_stride_of<R>(m.n) * sizeof(R) > 48 * 1024) {
+  if (size_t(warps) * ty * tz * deposit_stride_of<R>(m.n) * sizeof(R) > 40 * 1024) {
     // once per device, for every tile shape, so that no attribute call falls inside a stream capture
     static bool done[64];
     int dev = 0;

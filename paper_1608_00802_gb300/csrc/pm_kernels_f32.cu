@@ -17,12 +17,13 @@ cudaError_t launch_step_inc(uint32_t* step, cudaStream_t s, int nm, size_t ms) {
 }
 
 cudaError_t launch_sort_histogram(const uint32_t* keys, int64_t n, int passes, int digit_bits, int key_bits,
-                                  uint32_t* hist, uint32_t* epoch, cudaStream_t s, const uint32_t* n_dev) {
+                                  uint32_t* hist, uint32_t* epoch, cudaStream_t s, const uint32_t* n_dev,
+                                  uint32_t* crowd) {
   int64_t blocks = (n + RS_THREADS * 16 - 1) / (RS_THREADS * 16);
   if (blocks > 2 * 152) blocks = 2 * 152;
   if (blocks < 1) blocks = 1;
   k_sort_histogram<<<unsigned(blocks), RS_THREADS, 0, s>>>(keys, n, passes, digit_bits, key_bits, hist, epoch,
-                                                            n_dev);
+                                                            n_dev, crowd);
   return cudaGetLastError();
 }
 

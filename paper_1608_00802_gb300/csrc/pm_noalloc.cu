@@ -42,7 +42,7 @@ constexpr size_t kVals1 = kVals0 + align256(kMaxPart * 4);
 constexpr size_t kHist = kVals1 + align256(kMaxPart * 4);  // 3 histograms + 4 tile counters
 constexpr size_t kStatus = kHist + align256((3 * kRadixMax + 4) * 4);
 constexpr size_t kRows = kStatus + align256(size_t(kMaxTiles) * kRadixMax * 8);
-constexpr size_t kErr = kRows + align256((size_t(kMaxMesh) * kMaxMesh + 1) * 4);
+constexpr size_t kErr = kRows + align256((size_t(kMaxMesh) * kMaxMesh + CROWD_WORDS) * 4);
 constexpr size_t kTotal = kErr + 256;
 static_assert(kTotal <= PM_NOALLOC_SCRATCH_BYTES, "scratch layout exceeds PM_NOALLOC_SCRATCH_BYTES");
 
@@ -140,7 +140,8 @@ pm_status pm_deposit_noalloc(const double* x_dev, int64_t n_part, int32_t n_mesh
   NA_CU(cudaMemsetAsync(err, 0, 8, s));  // error word and sort epoch word
   // positions to cell + offset as pm_set_particles converts them (1/dx with dx = box/N), at rest
   NA_CU(launch_init_particles<float>(x_dev, nullptr, n, m, 1.0 / (box / n_mesh), pos[0], mom[0], keys[0], err, s));
-  NA_CU(launch_sort_histogram(keys[0], n, passes, digit_bits, bits, hist, err + 1, s));
+  uint32_t* rows = reinterpret_cast<uint32_t*>(base + kRows);
+  NA_CU(launch_sort_histogram(keys[0], n, passes, digit_bits, bits, hist, err + 1, s, nullptr, rows + m.n2 + 1));
   const uint32_t* kin = keys[0];
   const uint32_t* vin = nullptr;
   int tmp = 0;
@@ -162,7 +163,6 @@ pm_status pm_deposit_noalloc(const double* x_dev, int64_t n_part, int32_t n_mesh
       sorted_keys = kout;
     }
   }
-  uint32_t* rows = reinterpret_cast<uint32_t*>(base + kRows);
   NA_CU(launch_row_start(sorted_keys, n, uint32_t(n_mesh), rows, s));
   NA_CU(launch_deposit<float>(pos[1], rows, n, m, double(m.n3) / double(n), rho_dev, s));
   if (err_dev) {

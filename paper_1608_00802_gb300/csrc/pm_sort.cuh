@@ -81,10 +81,14 @@ static __global__ void __launch_bounds__(RS_THREADS) k_sort_histogram(const uint
                                                                       int passes, int digit_bits, int key_bits,
                                                                       uint32_t* __restrict__ hist,
                                                                       uint32_t* __restrict__ epoch,
-                                                                      const uint32_t* __restrict__ n_dev) {
+                                                                      const uint32_t* __restrict__ n_dev,
+                                                                      uint32_t* __restrict__ crowd) {
   __shared__ uint32_t sh[3 * (1 << RS_MAX_BITS)];
   if (n_dev) n = *n_dev;  // element count known on the device only
-  if (blockIdx.x == 0 && threadIdx.x == 0) *epoch = (*epoch + uint32_t(passes)) % 65530u + 1u;
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    *epoch = (*epoch + uint32_t(passes)) % 65530u + 1u;
+    if (crowd) *crowd = 0;  // the row starts' flag, set by k_row_start after the passes
+  }
   const int radix = 1 << digit_bits;
   for (int i = threadIdx.x; i < passes * radix; i += blockDim.x) sh[i] = 0;
   __syncthreads();
@@ -313,6 +317,9 @@ static __global__ void k_row_start(const uint32_t* __restrict__ keys, int64_t n,
   const int64_t prev = i == 0 ? -1 : min(int64_t(__ldg(keys + i - 1) / n_mesh), int64_t(nrows));
   const int64_t cur = i == n ? int64_t(nrows) : min(int64_t(__ldg(keys + i) / n_mesh), int64_t(nrows));
   for (int64_t r = prev + 1; r <= cur; ++r) row_start[r] = uint32_t(i);
+  // row of slot i holds slot i - DEP_CROWD too: more than DEP_CROWD records (every such slot stores the same)
+  if (i < n && i >= int64_t(DEP_CROWD) && cur < int64_t(nrows) && int64_t(__ldg(keys + i - DEP_CROWD) / n_mesh) == cur)
+    row_start[nrows + 1] = 1u;
 }
 
 // Fixed-order fp64 reduction of per-block partials: out[v] = sum_b part[v*nblocks + b].
@@ -516,12 +523,14 @@ static __global__ void __launch_bounds__(RS_THREADS) k_mover_partition(
 // mrow, with the closing entries at r = N^2.
 
 static __global__ void __launch_bounds__(RT_THREADS) k_row_totals(const uint32_t* __restrict__ rcnt, uint32_t nrows,
-                                                                  uint32_t* __restrict__ btot, size_t ms) {
+                                                                  uint32_t* __restrict__ btot,
+                                                                  uint32_t* __restrict__ row_start, size_t ms) {
   __shared__ uint32_t sh[2][32];
   if (ms) {
     const size_t o = size_t(blockIdx.y) * ms;
-    rcnt = moff(rcnt, o), btot = moff(btot, o);
+    rcnt = moff(rcnt, o), btot = moff(btot, o), row_start = moff(row_start, o);
   }
+  if (blockIdx.x == 0 && threadIdx.x == 0) row_start[nrows + 1] = 0;  // the crowded flag, set by k_row_scan
   const uint32_t r0 = blockIdx.x * RT_TILE;
   uint32_t a = 0, b = 0;
 #pragma unroll
@@ -624,6 +633,7 @@ static __global__ void __launch_bounds__(RT_THREADS) k_row_scan(const uint32_t* 
       srow[r] = xa;
       mrow[r] = xb;
       row_start[r] = xa + xb;
+      if (ca[k] + cb[k] > DEP_CROWD) row_start[nrows + 1] = 1u;  // (every such row stores the same)
     }
     xa += ca[k];
     xb += cb[k];
@@ -739,7 +749,7 @@ inline cudaError_t launch_resort_place(int part, const uint32_t* keys, int64_t n
                                                                        N, m.log2n, stats, own, o);
   } else if (part == 1) {
     const unsigned nb = (nrows + RT_TILE - 1) / RT_TILE;
-    k_row_totals<<<dim3(nb, unsigned(nm)), RT_THREADS, 0, s>>>(rcnt, nrows, btot, o);
+    k_row_totals<<<dim3(nb, unsigned(nm)), RT_THREADS, 0, s>>>(rcnt, nrows, btot, row_start, o);
     k_row_scan<<<dim3(nb, unsigned(nm)), RT_THREADS, 0, s>>>(rcnt, nrows, btot, srow, mrow, row_start, o);
     // the bucket scatter runs over the device's mover count: a grid of resident blocks shared by the members
     int64_t cap = int64_t(16) * sms / nm;
