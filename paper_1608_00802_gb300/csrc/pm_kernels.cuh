@@ -345,9 +345,10 @@ __device__ __forceinline__ void run_sums(R (&v)[NV], uint32_t runs, int lane) {
 // states: a core of 10^6 particles puts thousands into each of a few hundred rows) is left to helper
 // blocks of the same launch, one destination row at a time, because its warp's chain would be the whole
 // kernel's length: 1496 us for that core on a 128^3 mesh, 87 us with the helpers.  The helpers add the
-// same values in the same order as the tile's warp would, so the split does not show in the result.  What is serial about a sum is only each node's own chain of additions, one per batch its two
-// cells are in, so the block computes the sums of all batches first (a warp per batch, any order) and then
-// every node adds up its own (a thread per node, in the batches' order).
+// same values in the same order as the tile's warp would, so the split does not show in the result.  What
+// is serial about a sum is only each node's own chain of additions, one per batch its two cells are in, so
+// the block computes the sums of all batches first (a warp per batch, any order) and then every node adds
+// up its own (a thread per node, in the batches' order).
 
 // records per window (the batch sums of a window are kept in shared memory)
 template <typename R>
