@@ -1442,7 +1442,7 @@ pm_status pm_power_spectrum(pm_sim* s, int32_t nbins, double* k, double* P, int6
     CF(s, cufftExecR2C(s->plan_fwd, s->at<cufftReal>(L.rho), (cufftComplex*)(s->arena + L.spec)));
   }
   double* part = s->part();
-  CU(s, DISPATCH(s, launch_power, s->arena + L.spec, s->mesh, nbins, part, s->stream));
+  CU(s, DISPATCH(s, launch_power, s->arena + L.spec, s->mesh, nbins, s->staging(), part, s->stream));
   double* red = s->red();
   CU(s, launch_reduce(part, RED_GRID, 3 * nbins, red, s->stream));
   double* h = new double[3 * nbins];

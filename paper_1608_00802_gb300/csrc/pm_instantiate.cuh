@@ -25,7 +25,7 @@
   template cudaError_t launch_kick<R>(void*, void*, uint32_t*, uint32_t*, int64_t, const R*, const R*, Mesh,      \
                                       KickParams, const KickParams*, const uint32_t*,                              \
                                       double*, double*, uint32_t*, int, cudaStream_t, int, size_t);                \
-  template cudaError_t launch_power<R>(const void*, Mesh, int, double*, cudaStream_t);                            \
+  template cudaError_t launch_power<R>(const void*, Mesh, int, double*, double*, cudaStream_t);                   \
   template cudaError_t launch_get_particles<R>(const void*, const void*, int64_t, Mesh, double, double*, double*, \
                                                cudaStream_t);                                                     \
   template cudaError_t launch_get_order<R>(const void*, const void*, int64_t, uint32_t*, uint32_t*, cudaStream_t); \

@@ -217,8 +217,9 @@ cudaError_t launch_kick(void* pos, void* mom, uint32_t* keys, uint32_t* tcount, 
                         Mesh m, KickParams kp,
                         const KickParams* kp_tab, const uint32_t* step, double* part, double* acc, uint32_t* err,
                         int threads, cudaStream_t s, int nm = 1, size_t ms = 0);
+// iw: scratch of n_mesh/2 + 1 doubles
 template <typename R>
-cudaError_t launch_power(const void* spec, Mesh m, int nbins, double* part, cudaStream_t s);
+cudaError_t launch_power(const void* spec, Mesh m, int nbins, double* iw, double* part, cudaStream_t s);
 cudaError_t launch_reduce(const double* part, int nblocks, int nvals, double* out, cudaStream_t s);
 // out[v] = max_b part[v*nblocks + b]
 cudaError_t launch_reduce_max(const double* part, int nblocks, int nvals, double* out, cudaStream_t s);
