@@ -486,7 +486,8 @@ pm_status stencil_stage(pm_sim* s, bool diag = false) {
   s->krho_valid = diag || s->fp64() || s->cfg.lap != PM_LAP_COMPACT;  // the generic kernel always sums
   PROF(s, PM_STAGE_STENCIL);
   CU(s, launch_stencil<R>(s->at<R>(density_field(s)), s->mesh, sp, s->at<R>(s->direct ? L.rho : L.q), kr_part(s),
-                          s->at<uint32_t>(L.st_list), s->at<uint32_t>(L.st_count), s->errword(), s->stream));
+                          s->at<uint32_t>(L.st_list), s->at<uint32_t>(L.st_count), s->errword(), s->arena + L.spec,
+                          s->stream));  // (the spectrum is free here: both potentials are back from it)
   return PM_OK;
 }
 
@@ -1951,8 +1952,8 @@ pm_status packed_step(pm_batch::Class& C, const std::vector<pm_sim*>& sims, cuda
   }
   if (s->cfg.quantum)
     PCU(launch_stencil<float>(s->at<float>(L.rho), s->mesh, stencil_params(s, false), s->at<float>(L.q), kr_part(s),
-                              s->at<uint32_t>(L.st_list), s->at<uint32_t>(L.st_count), s->errword(), st,
-                              s->coefs() + 1, nm, ms));
+                              s->at<uint32_t>(L.st_list), s->at<uint32_t>(L.st_count), s->errword(),
+                              nullptr, st, s->coefs() + 1, nm, ms));
   PCU(launch_step_inc(s->errword() + 2, st, nm, ms));
   for (int i : C.members) {
     pm_sim* m = sims[i];

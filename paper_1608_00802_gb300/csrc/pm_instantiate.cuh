@@ -21,7 +21,7 @@
   template cudaError_t launch_green_spline<R>(void*, void*, const void*, Mesh, double, double*, cudaStream_t, int); \
   template cudaError_t launch_smooth_spec<R>(void*, const void*, Mesh, cudaStream_t);                             \
   template cudaError_t launch_stencil<R>(const R*, Mesh, StencilParams, R*, double*, uint32_t*, uint32_t*,       \
-                                          uint32_t*, cudaStream_t, const double*, int, size_t);                   \
+                                          uint32_t*, void*, cudaStream_t, const double*, int, size_t);            \
   template cudaError_t launch_kick<R>(void*, void*, uint32_t*, uint32_t*, int64_t, const R*, const R*, Mesh,      \
                                       KickParams, const KickParams*, const uint32_t*,                              \
                                       double*, double*, uint32_t*, int, cudaStream_t, int, size_t);                \

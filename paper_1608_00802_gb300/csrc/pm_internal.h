@@ -195,10 +195,11 @@ template <typename R>
 cudaError_t launch_smooth_direct(const R* in, R* out, Mesh m, const double* g, int maxr2, cudaStream_t s);
 template <typename R>
 cudaError_t launch_smooth_spec(void* spec, const void* what, Mesh m, cudaStream_t s);
+// (scratch: N^3 values, written by the fp64 stencil; may be null in fp32)
 template <typename R>
 cudaError_t launch_stencil(const R* rho, Mesh m, StencilParams sp, R* q, double* part, uint32_t* list,
-                           uint32_t* list_count, uint32_t* err, cudaStream_t s, const double* qcp = nullptr,
-                           int nm = 1, size_t ms = 0);
+                           uint32_t* list_count, uint32_t* err, void* scratch, cudaStream_t s,
+                           const double* qcp = nullptr, int nm = 1, size_t ms = 0);
 // fp32 stencil tiling (defined with the kernels): list length of the
 // register-column kernel, blocks (= K_rho partials) of a shape and the most
 // over every valid shape, shape validity and the default shape

@@ -1161,14 +1161,28 @@ __device__ __forceinline__ bool q_needs_ext(float s0, float sxp, float sxm, floa
   return mag > __fmul_rn(ST_KAPPA, fabsf(lap));
 }
 
+// The generic stencil (fp64, and fp32 with the wide Laplacian).  In fp64 it is bound by the fp64 pipe, where a
+// square root costs as much as the rest of a node's arithmetic, so the square roots are taken once per node
+// by k_sqrt_floor into a scratch field (sq) that the stencil then reads, instead of seven (thirteen with the
+// wide Laplacian) per node: 49 -> 24 us (both kernels) on a 64^3 mesh.  fp32 takes them where they are needed (sq null), because
+// the near-empty nodes read the densities anyway.
 template <typename R>
-__global__ void __launch_bounds__(MESH_THREADS) k_stencil(const R* __restrict__ rho, Mesh m, StencilParams sp,
-                                                          R* __restrict__ q, double* part) {
+__global__ void __launch_bounds__(MESH_THREADS) k_sqrt_floor(const R* __restrict__ rho, uint32_t n3, R fl,
+                                                             R* __restrict__ sq) {
+  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n3; i += gridDim.x * blockDim.x) sq[i] = sfloor(rho[i], fl);
+}
+
+template <typename R>
+__global__ void __launch_bounds__(MESH_THREADS) k_stencil(const R* __restrict__ rho, const R* __restrict__ sq, Mesh m,
+                                                          StencilParams sp, R* __restrict__ q, double* part) {
+  constexpr bool ROOTS = sizeof(R) == 8;  // the square roots come from sq
   const int n = m.n;
   R ksum = R(0);
   const R fl = R(sp.rho_floor);
   const R qc = R(sp.qcoef);
   const float slim = sp.rho_fp64 > 0 ? float(sqrt(sp.rho_fp64)) : 0.0f;  // fp32 only
+  const R* src = ROOTS ? sq : rho;
+  auto root = [&](R v) { return ROOTS ? v : sfloor(v, fl); };
   for (uint32_t node = blockIdx.x * blockDim.x + threadIdx.x; node < m.n3; node += gridDim.x * blockDim.x) {
     int x, y, z;
     split_cell(node, m, x, y, z);
@@ -1177,14 +1191,14 @@ __global__ void __launch_bounds__(MESH_THREADS) k_stencil(const R* __restrict__ 
     const uint32_t xp = wrap(x + st, n), xm = wrap(x - st, n);
     const uint32_t yp = uint32_t(wrap(y + st, n)) * n, ym = uint32_t(wrap(y - st, n)) * n;
     const uint32_t zp = uint32_t(wrap(z + st, n)) * m.n2, zm = uint32_t(wrap(z - st, n)) * m.n2;
-    const R r0 = __ldg(rho + node);
-    const R rxp = __ldg(rho + zn + yn + xp), rxm = __ldg(rho + zn + yn + xm);
-    const R ryp = __ldg(rho + zn + yp + x), rym = __ldg(rho + zn + ym + x);
-    const R rzp = __ldg(rho + zp + yn + x), rzm = __ldg(rho + zm + yn + x);
-    R s0 = sfloor(r0, fl);
-    R sxp = sfloor(rxp, fl), sxm = sfloor(rxm, fl);
-    R syp = sfloor(ryp, fl), sym = sfloor(rym, fl);
-    R szp = sfloor(rzp, fl), szm = sfloor(rzm, fl);
+    const R r0 = __ldg(src + node);
+    const R rxp = __ldg(src + zn + yn + xp), rxm = __ldg(src + zn + yn + xm);
+    const R ryp = __ldg(src + zn + yp + x), rym = __ldg(src + zn + ym + x);
+    const R rzp = __ldg(src + zp + yn + x), rzm = __ldg(src + zm + yn + x);
+    R s0 = root(r0);
+    R sxp = root(rxp), sxm = root(rxm);
+    R syp = root(ryp), sym = root(rym);
+    R szp = root(rzp), szm = root(rzm);
     R lap = ((sxp - s0) + (sxm - s0)) + ((syp - s0) + (sym - s0)) + ((szp - s0) + (szm - s0));
     R qv = qc * lap / s0;
     if (sizeof(R) == 4 && q_needs_ext(float(s0), float(sxp), float(sxm), float(syp), float(sym), float(szp),
@@ -1197,12 +1211,12 @@ __global__ void __launch_bounds__(MESH_THREADS) k_stencil(const R* __restrict__ 
       ksum += a * a + b * b + c * c;
     } else {
       // printed form of Eq. (diskpoten): central differences over +-dx
-      const R cxp = sfloor(__ldg(rho + zn + yn + wrap(x + 1, n)), fl);
-      const R cxm = sfloor(__ldg(rho + zn + yn + wrap(x - 1, n)), fl);
-      const R cyp = sfloor(__ldg(rho + zn + uint32_t(wrap(y + 1, n)) * n + x), fl);
-      const R cym = sfloor(__ldg(rho + zn + uint32_t(wrap(y - 1, n)) * n + x), fl);
-      const R czp = sfloor(__ldg(rho + uint32_t(wrap(z + 1, n)) * m.n2 + yn + x), fl);
-      const R czm = sfloor(__ldg(rho + uint32_t(wrap(z - 1, n)) * m.n2 + yn + x), fl);
+      const R cxp = root(__ldg(src + zn + yn + wrap(x + 1, n)));
+      const R cxm = root(__ldg(src + zn + yn + wrap(x - 1, n)));
+      const R cyp = root(__ldg(src + zn + uint32_t(wrap(y + 1, n)) * n + x));
+      const R cym = root(__ldg(src + zn + uint32_t(wrap(y - 1, n)) * n + x));
+      const R czp = root(__ldg(src + uint32_t(wrap(z + 1, n)) * m.n2 + yn + x));
+      const R czm = root(__ldg(src + uint32_t(wrap(z - 1, n)) * m.n2 + yn + x));
       R a = cxp - cxm, b = cyp - cym, c = czp - czm;
       ksum += R(0.25) * (a * a + b * b + c * c);
     }
@@ -1977,7 +1991,7 @@ __global__ void __launch_bounds__(KICK_THREADS, (FM == KICK_FM_HYBRID_Q && !PACK
 // correction.  A warp takes one quadrant row (|m_y|, |m_z|): along x the shell index does not fall, so
 // equal shells are runs of lanes, summed by a segmented scan, and the run's last lane adds to the warp's
 // own bins (no atomics; the sums are reproducible).  150^3: 365 us with a square root, three sinpi and three
-// shared fp64 atomics (compare-and-swap loops) per mode, about 35 us so.
+// shared fp64 atomics (compare-and-swap loops) per mode, 38 us so.
 
 // 1 / sinc^4(m / N), m = 0 .. N/2: the inverse cloud-in-cell window of |delta_k|^2 along one axis
 static __global__ void k_power_window(double* iw, int n) {
@@ -2297,8 +2311,8 @@ inline int stencil_blocks(int n) {
 
 template <typename R>
 cudaError_t launch_stencil(const R* rho, Mesh m, StencilParams sp, R* q, double* part, uint32_t* list,
-                           uint32_t* list_count, uint32_t* err, cudaStream_t s, const double* qcp, int nm,
-                           size_t ms) {
+                           uint32_t* list_count, uint32_t* err, void* scratch, cudaStream_t s, const double* qcp,
+                           int nm, size_t ms) {
   // a packed group steps its members in one launch of the one-shot tiles only
   if (nm > 1 && !stencil_tile_path(m.n, sp, sizeof(R) == 4)) return cudaErrorInvalidValue;
   if (sizeof(R) == 4 && sp.step == 1) {
@@ -2349,7 +2363,10 @@ cudaError_t launch_stencil(const R* rho, Mesh m, StencilParams sp, R* q, double*
     k_stencil_tiled<<<g, b, 0, s>>>((const float*)rho, m, float(sp.rho_floor), float(sp.qcoef), slim, zlen, (float*)q,
                                     list, list_count, part, sp.diag);
   } else {
-    k_stencil<R><<<MESH_GRID, MESH_THREADS, 0, s>>>(rho, m, sp, q, part);
+    if (sizeof(R) == 8)
+      k_sqrt_floor<R><<<std::min(mesh_grid(m.n3), unsigned(MESH_GRID)), MESH_THREADS, 0, s>>>(rho, m.n3, R(sp.rho_floor),
+                                                                                             (R*)scratch);
+    k_stencil<R><<<MESH_GRID, MESH_THREADS, 0, s>>>(rho, (const R*)scratch, m, sp, q, part);
   }
   return cudaGetLastError();
 }
