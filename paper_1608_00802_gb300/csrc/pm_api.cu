@@ -89,7 +89,7 @@ size_t align_up(size_t v) { return (v + 255) & ~size_t(255); }
 
 struct Layout {
   size_t pos[2], mom[2], keys[4], vals[3], tcount, rcnt, btot, srow, mrow, tile_cnt, row_start, rho, phi, q, spec, what,
-      spec2, work, staging, hist, status, st_list, st_count, part, part_aux, red, err, ktab, green, total;
+      spec2, work, staging, hist, status, st_list, st_count, part, part_aux, red, err, ktab, green, sin2, total;
   int key_bits, passes, digit_bits, ntiles;
 };
 
@@ -215,6 +215,7 @@ Layout make_layout(const pm_config& c, size_t work_bytes) {
   L.ktab = take(size_t(std::max(PM_RUN_GRAPH_MAX_STEPS, PM_BATCH_MAX_STEPS)) * sizeof(KickParams));
   // the z transform's twiddles and the Green's sin^2 table (fp32 cloud-in-cell, power-of-two meshes)
   L.green = take(c.precision == PM_FP32 && !spline && spec_z_supported(int(N)) ? N * 12 : 0);
+  L.sin2 = take(N * rsz);  // sin^2(pi j / N) for the flat Green passes
   L.total = off;
   return L;
 }
@@ -674,12 +675,12 @@ pm_status mesh_from_density(pm_sim* s) {
   {
     PROF(s, PM_STAGE_GREEN);
     if (spline(s))
-      CU(s, launch_green_spline<R>(s->arena + L.spec, nullptr, s->arena + L.what, s->mesh, green_coef(s), wg_part(s),
-                                   s->stream, 0));
+      CU(s, launch_green_spline<R>(s->arena + L.spec, nullptr, s->arena + L.what, s->mesh, s->arena + L.sin2,
+                                   green_coef(s), wg_part(s), s->stream, 0));
     else
-      CU(s, launch_green<R>(s->arena + L.spec, s->mesh, green_coef(s), wg_part(s), s->stream));
+      CU(s, launch_green<R>(s->arena + L.spec, s->mesh, s->arena + L.sin2, green_coef(s), wg_part(s), s->stream));
   }
-  s->wg_count = MESH_GRID;
+  s->wg_count = int(green_blocks(s->cfg.n_mesh));
   PMST(fft_c2r<R>(s, s->arena + L.spec, s->arena + L.phi));
   PMST(quantum_stage<R>(s));
   s->fields_valid = true;
@@ -697,9 +698,9 @@ pm_status spline_fields(pm_sim* s) {
   {
     PROF(s, PM_STAGE_GREEN);
     CU(s, launch_green_spline<R>(s->arena + L.spec, s->direct ? nullptr : s->arena + L.spec2, s->arena + L.what,
-                                 s->mesh, green_coef(s), wg_part(s), s->stream, 1));
+                                 s->mesh, s->arena + L.sin2, green_coef(s), wg_part(s), s->stream, 1));
   }
-  s->wg_count = MESH_GRID;
+  s->wg_count = int(green_blocks(s->cfg.n_mesh));
   if (s->direct)
     PMST(smooth_field<R>(s, L.rho, L.spec2));
   else
@@ -1079,6 +1080,13 @@ pm_status pm_create(const pm_config* c, void* dev_arena, size_t bytes, void* str
       delete s;
       return fail(nullptr, PM_ERR_CUDA, "coefficient upload failed");
     }
+  }
+  if (DISPATCH(s, launch_sin2_table, s->arena + L.sin2, N, s->stream) != cudaSuccess ||
+      cudaStreamSynchronize(s->stream) != cudaSuccess) {
+    cufftDestroy(s->plan_fwd);
+    cufftDestroy(s->plan_inv);
+    delete s;
+    return fail(nullptr, PM_ERR_CUDA, "sin^2 table failed");
   }
   if (c->precision == PM_FP32) kick_stream_prepare();
   // fp32 cloud-in-cell on power-of-two meshes from 128^3: the Green multiplication inside the z
@@ -1947,7 +1955,8 @@ pm_status packed_step(pm_batch::Class& C, const std::vector<pm_sim*>& sims, cuda
     CF(s, cufftSetStream(C.fwd, st));
     CF(s, cufftSetStream(C.inv, st));
     CF(s, cufftExecR2C(C.fwd, s->at<cufftReal>(L.rho), (cufftComplex*)(s->arena + L.spec)));
-    PCU(launch_green<float>(s->arena + L.spec, s->mesh, green_coef(s), wg_part(s), st, s->coefs(), nm, ms));
+    PCU(launch_green<float>(s->arena + L.spec, s->mesh, s->arena + L.sin2, green_coef(s), wg_part(s), st, s->coefs(),
+                            nm, ms));
     CF(s, cufftExecC2R(C.inv, (cufftComplex*)(s->arena + L.spec), s->at<cufftReal>(L.phi)));
   }
   if (s->cfg.quantum)
@@ -1962,7 +1971,7 @@ pm_status packed_step(pm_batch::Class& C, const std::vector<pm_sim*>& sims, cuda
     m->sorted = true;
     m->fields_valid = true;
     m->krho_valid = false;
-    m->wg_count = fused ? spec_z_tiles(N) : MESH_GRID;
+    m->wg_count = fused ? spec_z_tiles(N) : int(green_blocks(N));
   }
   return PM_OK;
 }

@@ -15,10 +15,13 @@
                                         uint32_t*, uint32_t*, uint32_t*, uint32_t*, uint32_t*, uint32_t*, uint32_t*, \
                                         uint32_t*, uint32_t*, Mesh, unsigned long long*, uint32_t*, const void*,     \
                                         const void*, void*, void*, int, cudaStream_t, int, size_t);               \
-  template cudaError_t launch_green<R>(void*, Mesh, double, double*, cudaStream_t, const double*, int, size_t);   \
+  template cudaError_t launch_green<R>(void*, Mesh, const void*, double, double*, cudaStream_t, const double*, int, \
+                                       size_t);                                                                  \
+  template cudaError_t launch_sin2_table<R>(void*, int, cudaStream_t);                                            \
   template cudaError_t launch_spline_weights<R>(void*, Mesh, double, cudaStream_t);                               \
   template cudaError_t launch_spline_symbol<R>(const void*, void*, Mesh, cudaStream_t);                           \
-  template cudaError_t launch_green_spline<R>(void*, void*, const void*, Mesh, double, double*, cudaStream_t, int); \
+  template cudaError_t launch_green_spline<R>(void*, void*, const void*, Mesh, const void*, double, double*,       \
+                                              cudaStream_t, int);                                                \
   template cudaError_t launch_smooth_spec<R>(void*, const void*, Mesh, cudaStream_t);                             \
   template cudaError_t launch_stencil<R>(const R*, Mesh, StencilParams, R*, double*, uint32_t*, uint32_t*,       \
                                           uint32_t*, void*, cudaStream_t, const double*, int, size_t);            \

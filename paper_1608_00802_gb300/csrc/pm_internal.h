@@ -176,8 +176,16 @@ template <typename R>
 cudaError_t launch_deposit(const void* pos, const uint32_t* row_start, int64_t n, Mesh m, double norm, R* rho,
                            cudaStream_t s, int warps = 8, int nm = 1, size_t ms = 0);
 template <typename R>
-cudaError_t launch_green(void* spec, Mesh m, double coef, double* part, cudaStream_t s,
+cudaError_t launch_green(void* spec, Mesh m, const void* s2, double coef, double* part, cudaStream_t s,
                          const double* coefp = nullptr, int nm = 1, size_t ms = 0);
+// blocks (= W_g partials) of the flat Green passes: one element per thread up to MESH_GRID blocks
+inline unsigned green_blocks(int n) {
+  const int64_t need = (int64_t(n) * n * (n / 2 + 1) + MESH_THREADS - 1) / MESH_THREADS;
+  return unsigned(need < MESH_GRID ? need : MESH_GRID);
+}
+// sin^2(pi j / N) for j < N in the working precision, read by the Green passes
+template <typename R>
+cudaError_t launch_sin2_table(void* s2, int n, cudaStream_t s);
 // cubic spline kernel: node weights, their normalised real symbol, the Green
 // multiplication with the symbol (spec2 null: spec already holds rho_W^) and
 // the smoothing of a transformed field
@@ -186,8 +194,8 @@ cudaError_t launch_spline_weights(void* w, Mesh m, double hc, cudaStream_t s);
 template <typename R>
 cudaError_t launch_spline_symbol(const void* spec, void* what, Mesh m, cudaStream_t s);
 template <typename R>
-cudaError_t launch_green_spline(void* spec, void* spec2, const void* what, Mesh m, double coef, double* part,
-                                cudaStream_t s, int smooth_in);
+cudaError_t launch_green_spline(void* spec, void* spec2, const void* what, Mesh m, const void* s2, double coef,
+                                double* part, cudaStream_t s, int smooth_in);
 // the spline smoothing in real space for supports within three cells (fp32):
 // g[s*4 + i] = normalised node weight at squared distance i^2 + s (s <= 18);
 // maxr2: the largest squared distance with a nonzero weight
