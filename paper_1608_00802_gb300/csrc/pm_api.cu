@@ -412,6 +412,15 @@ pm_status sort_particles(pm_sim* s) {
   if (s->keys_marked) return resort_movers<R>(s);
   const Layout& L = s->L;
   const int64_t n = s->n();
+  if (n <= SORT_SMALL_MAX) {  // one kernel, the keys in place
+    const int nxt = s->cur ^ 1;
+    PROF(s, PM_STAGE_SORT_PASS);
+    CU(s, launch_sort_small<R>(s->keys, n, L.key_bits, s->keys, s->pos(), s->mom(), s->arena + L.pos[nxt],
+                               s->arena + L.mom[nxt], s->at<uint32_t>(L.row_start), s->mesh, nullptr, s->stream));
+    s->cur = nxt;
+    s->sorted = true;
+    return PM_OK;
+  }
   uint32_t* hist = s->at<uint32_t>(L.hist);
   uint32_t* counters = hist + 3 * (1 << RS_MAX_BITS);
   uint64_t* status = s->at<uint64_t>(L.status);

@@ -142,6 +142,13 @@ cudaError_t launch_sort_pass(bool last, const uint32_t* keys_in, const uint32_t*
                              const void* pos_in, const void* mom_in, void* pos_out, void* mom_out, uint32_t* err,
                              cudaStream_t s, const uint32_t* n_dev = nullptr, int nm = 1, size_t ms = 0,
                              int spin_limit = 0);  // polls of a look-back wait before it gives up (0: default)
+// the full sort of up to SORT_SMALL_MAX particles in one kernel (records gathered, row starts and the
+// crowded-row flag written; keys_out may be keys_in); mom_in null: no momenta; clear (nullable): a word set to 0
+constexpr int SORT_SMALL_MAX = 65536;
+template <typename R>
+cudaError_t launch_sort_small(const uint32_t* keys_in, int64_t n, int key_bits, uint32_t* keys_out, const void* pos_in,
+                              const void* mom_in, void* pos_out, void* mom_out, uint32_t* row_start, Mesh m,
+                              uint32_t* clear, cudaStream_t s);
 // incremental re-sort after a drift (keys carry KEY_MOVER; tcount holds the
 // drift's mover counts per tile and per group of tiles): stable partition
 // into stayers (sk, sv) and movers (mk, mv) with per-row counts (rcnt: 3 N^2

@@ -297,9 +297,8 @@ __global__ void k_init_particles(const double* __restrict__ x, const double* __r
   }
   uint32_t cell = (uint32_t(c[2]) * uint32_t(m.n) + uint32_t(c[1])) * uint32_t(m.n) + uint32_t(c[0]);
   pos[i] = make_pos(cell, f[0], f[1], f[2]);
-  // p null: particles at rest (the allocation-free deposit needs no momenta)
-  mom[i] = p ? make_mom(R(p[3 * i]), R(p[3 * i + 1]), R(p[3 * i + 2]), uint32_t(i))
-             : make_mom(R(0), R(0), R(0), uint32_t(i));
+  // p null: positions only (the allocation-free deposit needs no momenta)
+  if (p) mom[i] = make_mom(R(p[3 * i]), R(p[3 * i + 1]), R(p[3 * i + 2]), uint32_t(i));
   keys[i] = cell;
 }
 

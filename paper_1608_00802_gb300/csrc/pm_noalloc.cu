@@ -24,24 +24,15 @@ namespace {
 
 constexpr int64_t kMaxPart = PM_NOALLOC_MAX_PARTICLES;
 constexpr int kMaxMesh = PM_NOALLOC_MAX_MESH;
-constexpr int kMaxTiles = int((kMaxPart + RS_TILE - 1) / RS_TILE);
-constexpr size_t kRadixMax = size_t(1) << RS_MAX_BITS;
+static_assert(kMaxPart <= SORT_SMALL_MAX, "the deposit sorts with the one-kernel sort");
 
 constexpr size_t align256(size_t v) { return (v + 255) & ~size_t(255); }
 
 // offsets inside the static scratch array
 constexpr size_t kPos0 = 0;
 constexpr size_t kPos1 = kPos0 + align256(kMaxPart * 16);
-constexpr size_t kMom0 = kPos1 + align256(kMaxPart * 16);
-constexpr size_t kMom1 = kMom0 + align256(kMaxPart * 16);
-constexpr size_t kKeys0 = kMom1 + align256(kMaxPart * 16);
-constexpr size_t kKeys1 = kKeys0 + align256(kMaxPart * 4);
-constexpr size_t kKeys2 = kKeys1 + align256(kMaxPart * 4);
-constexpr size_t kVals0 = kKeys2 + align256(kMaxPart * 4);
-constexpr size_t kVals1 = kVals0 + align256(kMaxPart * 4);
-constexpr size_t kHist = kVals1 + align256(kMaxPart * 4);  // 3 histograms + 4 tile counters
-constexpr size_t kStatus = kHist + align256((3 * kRadixMax + 4) * 4);
-constexpr size_t kRows = kStatus + align256(size_t(kMaxTiles) * kRadixMax * 8);
+constexpr size_t kKeys = kPos1 + align256(kMaxPart * 16);
+constexpr size_t kRows = kKeys + align256(kMaxPart * 4);
 constexpr size_t kErr = kRows + align256((size_t(kMaxMesh) * kMaxMesh + CROWD_WORDS) * 4);
 constexpr size_t kTotal = kErr + 256;
 static_assert(kTotal <= PM_NOALLOC_SCRATCH_BYTES, "scratch layout exceeds PM_NOALLOC_SCRATCH_BYTES");
@@ -57,7 +48,11 @@ bool g_ready[64];
 thread_local char g_msg[256];
 
 // the call's error bits to the caller's word (device or mapped host memory)
-__global__ void k_copy_error(const uint32_t* err, uint32_t* out) { *out = *err; }
+// hands the call's error bits over and clears them for the next call
+__global__ void k_copy_error(uint32_t* err, uint32_t* out) {
+  *out = *err;
+  *err = 0;
+}
 
 // the message goes where pm_last_error(NULL) reads it
 pm_status nfail(pm_status st, const char* msg) {
@@ -112,19 +107,10 @@ pm_status pm_deposit_noalloc(const double* x_dev, int64_t n_part, int32_t n_mesh
   m.n3 = m.n2 * uint32_t(n_mesh);
   int bits = 0;
   while ((uint32_t(1) << bits) < m.n3) ++bits;
-  int passes = (bits + RS_MAX_BITS - 1) / RS_MAX_BITS;
-  if (passes < 1) passes = 1;
-  const int digit_bits = (bits + passes - 1) / passes;
-  const int ntiles = int((n + RS_TILE - 1) / RS_TILE);
-  uint32_t* hist = reinterpret_cast<uint32_t*>(base + kHist);
-  uint32_t* counters = hist + 3 * kRadixMax;
-  uint64_t* status = reinterpret_cast<uint64_t*>(base + kStatus);
   uint32_t* err = reinterpret_cast<uint32_t*>(base + kErr);
-  uint32_t* keys[3] = {reinterpret_cast<uint32_t*>(base + kKeys0), reinterpret_cast<uint32_t*>(base + kKeys1),
-                       reinterpret_cast<uint32_t*>(base + kKeys2)};
-  uint32_t* vals[2] = {reinterpret_cast<uint32_t*>(base + kVals0), reinterpret_cast<uint32_t*>(base + kVals1)};
+  uint32_t* keys = reinterpret_cast<uint32_t*>(base + kKeys);
+  uint32_t* rows = reinterpret_cast<uint32_t*>(base + kRows);
   void* pos[2] = {base + kPos0, base + kPos1};
-  void* mom[2] = {base + kMom0, base + kMom1};
 
 #define NA_CU(expr)                                                                             \
   do {                                                                                          \
@@ -134,36 +120,13 @@ pm_status pm_deposit_noalloc(const double* x_dev, int64_t n_part, int32_t n_mesh
       return nfail(PM_ERR_CUDA, g_msg);                                                         \
     }                                                                                           \
   } while (0)
-  // the array keeps the previous call's contents: clear what must start at zero
-  NA_CU(cudaMemsetAsync(hist, 0, (3 * kRadixMax + 4) * 4, s));
-  NA_CU(cudaMemsetAsync(status, 0, size_t(ntiles) * (size_t(1) << digit_bits) * 8, s));
-  NA_CU(cudaMemsetAsync(err, 0, 8, s));  // error word and sort epoch word
-  // positions to cell + offset as pm_set_particles converts them (1/dx with dx = box/N), at rest
-  NA_CU(launch_init_particles<float>(x_dev, nullptr, n, m, 1.0 / (box / n_mesh), pos[0], mom[0], keys[0], err, s));
-  uint32_t* rows = reinterpret_cast<uint32_t*>(base + kRows);
-  NA_CU(launch_sort_histogram(keys[0], n, passes, digit_bits, bits, hist, err + 1, s, nullptr, rows + m.n2 + 1));
-  const uint32_t* kin = keys[0];
-  const uint32_t* vin = nullptr;
-  int tmp = 0;
-  uint32_t* sorted_keys = keys[0];
-  for (int p = 0; p < passes; ++p) {
-    const int shift = p * digit_bits;
-    const int pb = (shift + digit_bits <= bits) ? digit_bits : (bits - shift);
-    const bool last = p == passes - 1;
-    if (!last) {
-      NA_CU(launch_sort_pass<float>(false, kin, vin, n, shift, pb, hist + p * kRadixMax, status, counters + p, err + 1,
-                                    p, ntiles, keys[1 + tmp], vals[tmp], nullptr, nullptr, nullptr, nullptr, err, s));
-      kin = keys[1 + tmp];
-      vin = vals[tmp];
-      tmp ^= 1;
-    } else {
-      uint32_t* kout = (kin == keys[0]) ? keys[1 + tmp] : keys[0];
-      NA_CU(launch_sort_pass<float>(true, kin, vin, n, shift, pb, hist + p * kRadixMax, status, counters + p, err + 1,
-                                    p, ntiles, kout, nullptr, pos[0], mom[0], pos[1], mom[1], err, s));
-      sorted_keys = kout;
-    }
-  }
-  NA_CU(launch_row_start(sorted_keys, n, uint32_t(n_mesh), rows, s));
+  // the array keeps the previous call's contents; every buffer is written before it is read, except the error
+  // word, which starts at zero and is zero again after each call: cleared as it is handed over, or, with
+  // nobody to hand it to, by the sort
+  // positions to cell + offset as pm_set_particles converts them (1/dx with dx = box/N)
+  NA_CU(launch_init_particles<float>(x_dev, nullptr, n, m, 1.0 / (box / n_mesh), pos[0], nullptr, keys, err, s));
+  NA_CU(launch_sort_small<float>(keys, n, bits, keys, pos[0], nullptr, pos[1], nullptr, rows, m,
+                                 err_dev ? nullptr : err, s));
   NA_CU(launch_deposit<float>(pos[1], rows, n, m, double(m.n3) / double(n), rho_dev, s));
   if (err_dev) {
     k_copy_error<<<1, 1, 0, s>>>(err, err_dev);

@@ -22,6 +22,7 @@
 // Equal keys keep their previous order, so the order after a step is the
 // stable sort of the new cells with ties broken by the previous order.
 #pragma once
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -727,6 +728,230 @@ __global__ void __launch_bounds__(PF_THREADS) k_place(
     pos_out[out] = pr;
     mom_out[out] = mr;
   }
+}
+
+// ---------------------------------------------------------------- the sort of few particles in one kernel
+// Up to SS_MAX_PARTICLES particles the full sort is a chain of short kernels (clears, histogram, a look-back
+// pass per digit, row starts): 5-10 launches of 2-15 us, each with a few tiles in flight.  Here one cluster
+// of up to eight CTAs sorts in its shared memory instead: CTA c holds the keys of places
+// [c chunk, (c+1) chunk) and their slots (16 bits), and every pass ranks its chunk by a digit (warp match
+// and per-warp counters, in order), exchanges the CTAs' digit totals through distributed shared memory,
+// stages the chunk in digit order and sends each run of equal digits, contiguous at its destination, to the
+// CTAs that hold those places.  The last pass is followed by the gather of the records, the row starts and
+// the crowded-row flag.  Same order as the general sort (stable, so it is the only one there is).
+// 65536 particles on 128^3: SS_FIG.
+constexpr int SS_MAX_PARTICLES = SORT_SMALL_MAX, SS_THREADS = 1024, SS_WARPS = 32, SS_CHUNK = SS_MAX_PARTICLES / 8;
+constexpr int SS_BITS = 10, SS_ITEMS = SS_CHUNK / SS_THREADS;
+
+struct SortSmallShared {
+  uint32_t keys[2][SS_CHUNK];
+  uint16_t vals[2][SS_CHUNK];
+  uint16_t cnt[SS_WARPS << SS_BITS];
+  uint32_t tot[1 << SS_BITS];     // records of each digit in this CTA (read by its peers)
+  uint32_t dstart[1 << SS_BITS];  // where the digit starts in the staged chunk
+  uint32_t gbase[1 << SS_BITS];   // where this CTA's records of the digit go
+  uint2 scratch[SS_WARPS];
+};
+
+// exclusive scans of two values per thread over the block
+__device__ __forceinline__ uint2 block_excl_scan2(uint2 v, uint2* scratch) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  uint2 inc = v;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t x = __shfl_up_sync(0xffffffffu, inc.x, o), y = __shfl_up_sync(0xffffffffu, inc.y, o);
+    if (lane >= o) inc.x += x, inc.y += y;
+  }
+  if (lane == 31) scratch[warp] = inc;
+  __syncthreads();
+  uint2 w = lane < SS_WARPS && lane < warp ? scratch[lane] : make_uint2(0, 0);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    w.x += __shfl_xor_sync(0xffffffffu, w.x, o);
+    w.y += __shfl_xor_sync(0xffffffffu, w.y, o);
+  }
+  return make_uint2(w.x + inc.x - v.x, w.y + inc.y - v.y);
+}
+
+// rows a .. b of the table start at slot v; a warp fills the long gaps (meshes far larger than the particles) together
+__device__ __forceinline__ void fill_rows(uint32_t* __restrict__ row_start, int a, int b, uint32_t v) {
+  const int lane = threadIdx.x & 31;
+  const bool wide = b - a >= 8;
+  if (!wide)
+    for (int r = a; r <= b; ++r) row_start[r] = v;
+  for (uint32_t todo = __ballot_sync(0xffffffffu, wide); todo; todo &= todo - 1) {
+    const int l = __ffs(todo) - 1;
+    const int aa = __shfl_sync(0xffffffffu, a, l), bb = __shfl_sync(0xffffffffu, b, l);
+    const uint32_t vv = __shfl_sync(0xffffffffu, v, l);
+    for (int r = aa + lane; r <= bb; r += 32) row_start[r] = vv;
+  }
+}
+
+// keys may be sorted in place (keys_out = keys_in); mom_in null: no momenta; clear (nullable): a word set to 0
+template <typename V4>
+__global__ void __launch_bounds__(SS_THREADS, 1) k_sort_small(const uint32_t* keys_in, uint32_t n, int chunk_shift,
+                                                              int passes, int digit_bits, int key_bits, uint32_t* keys_out,
+                                                              const V4* __restrict__ pos_in, const V4* __restrict__ mom_in,
+                                                              V4* __restrict__ pos_out, V4* __restrict__ mom_out,
+                                                              uint32_t* __restrict__ row_start, uint32_t n_mesh,
+                                                              int log2n, uint32_t* clear) {
+  namespace cg = cooperative_groups;
+  extern __shared__ __align__(16) unsigned char ss_smem[];
+  SortSmallShared& S = *reinterpret_cast<SortSmallShared*>(ss_smem);
+  cg::cluster_group cl = cg::this_cluster();
+  const uint32_t rank = cl.block_rank(), ncta = cl.num_blocks();
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const uint32_t chunk = 1u << chunk_shift, base = rank << chunk_shift;
+  const uint32_t cnt_here = base < n ? min(chunk, n - base) : 0u;
+  const uint32_t nrows = n_mesh * n_mesh;
+  const uint32_t lt = lanemask_lt();
+  const int items = int((chunk + SS_THREADS - 1) / SS_THREADS);  // rounds of a warp (its slots are contiguous)
+  for (uint32_t i = tid; i < cnt_here; i += SS_THREADS) {
+    S.keys[0][i] = keys_in[base + i];
+    S.vals[0][i] = uint16_t(base + i);
+  }
+  if (rank == 0 && tid == 0) {
+    row_start[nrows + 1] = 0;  // the crowded-row flag
+    if (clear) *clear = 0;
+  }
+  int cur = 0;
+  for (int p = 0; p < passes; ++p) {
+    const int shift = p * digit_bits, bits = min(digit_bits, key_bits - shift), radix = 1 << bits;
+    const uint32_t mask = uint32_t(radix - 1);
+    for (int d = tid; d < (SS_WARPS * radix) / 2; d += SS_THREADS) reinterpret_cast<uint32_t*>(S.cnt)[d] = 0;
+    __syncthreads();
+    uint32_t key[SS_ITEMS], rk[SS_ITEMS];
+    uint16_t val[SS_ITEMS];
+    uint16_t* mine = S.cnt + warp * radix;
+#pragma unroll
+    for (int r = 0; r < SS_ITEMS; ++r) {
+      if (r >= items) break;
+      const uint32_t li = uint32_t(warp * items + r) * 32u + lane;
+      const bool valid = li < cnt_here;
+      key[r] = valid ? S.keys[cur][li] : 0u;
+      val[r] = valid ? S.vals[cur][li] : uint16_t(0);
+      const uint32_t d = valid ? (key[r] >> shift) & mask : 0xffffffffu;
+      const uint32_t peers = __match_any_sync(0xffffffffu, d);
+      const uint32_t before = valid ? mine[d] : 0u, within = __popc(peers & lt);
+      __syncwarp();
+      if (valid && within == 0) mine[d] = uint16_t(before + __popc(peers));
+      __syncwarp();
+      rk[r] = before + within;
+    }
+    __syncthreads();
+    // per digit (one thread each): the earlier warps' records, the CTA's total
+    if (tid < radix) {
+      uint32_t run = 0;
+#pragma unroll 8
+      for (int w = 0; w < SS_WARPS; ++w) {
+        const uint32_t t = S.cnt[w * radix + tid];
+        S.cnt[w * radix + tid] = uint16_t(run);
+        run += t;
+      }
+      S.tot[tid] = run;
+    }
+    cl.sync();
+    uint2 v = make_uint2(0, 0);
+    uint32_t below = 0;
+    if (tid < radix) {
+      for (uint32_t c = 0; c < ncta; ++c) {
+        const uint32_t t = cl.map_shared_rank(S.tot, c)[tid];
+        v.x += t;
+        if (c < rank) below += t;
+      }
+      v.y = S.tot[tid];
+    }
+    const uint2 ex = block_excl_scan2(v, S.scratch);
+    if (tid < radix) {
+      S.gbase[tid] = ex.x + below;
+      S.dstart[tid] = ex.y;
+    }
+    __syncthreads();
+    // the chunk in digit order (every key of it is in registers)
+#pragma unroll
+    for (int r = 0; r < SS_ITEMS; ++r) {
+      if (r >= items) break;
+      const uint32_t li = uint32_t(warp * items + r) * 32u + lane;
+      if (li < cnt_here) {
+        const uint32_t d = (key[r] >> shift) & mask, at = S.dstart[d] + mine[d] + rk[r];
+        S.keys[cur][at] = key[r];
+        S.vals[cur][at] = val[r];
+      }
+    }
+    __syncthreads();
+    for (uint32_t li = tid; li < cnt_here; li += SS_THREADS) {
+      const uint32_t k = S.keys[cur][li], d = (k >> shift) & mask, to = S.gbase[d] + li - S.dstart[d];
+      SortSmallShared* peer = cl.map_shared_rank(&S, to >> chunk_shift);
+      peer->keys[cur ^ 1][to & (chunk - 1)] = k;
+      peer->vals[cur ^ 1][to & (chunk - 1)] = S.vals[cur][li];
+    }
+    cl.sync();
+    cur ^= 1;
+  }
+  // records, row starts and the flag, 32 consecutive places per warp and round (whole warps: fill_rows votes)
+  for (uint32_t w0 = warp * 32u; w0 < cnt_here; w0 += SS_THREADS) {
+    const uint32_t li = w0 + lane, i = base + li;
+    const bool valid = li < cnt_here;
+    int a = 0, b = -1, a2 = 0, b2 = -1;
+    if (valid) {
+      const uint32_t k = S.keys[cur][li], v = S.vals[cur][li];
+      keys_out[i] = k;
+      pos_out[i] = pos_in[v];
+      if (mom_in) mom_out[i] = mom_in[v];
+      const int row = int(min(key_row(k, n_mesh, log2n), nrows - 1));
+      if (i > 0) {
+        const uint32_t j = i - 1;
+        a = int(min(key_row(cl.map_shared_rank(&S, j >> chunk_shift)->keys[cur][j & (chunk - 1)], n_mesh, log2n), nrows - 1)) + 1;
+      }
+      b = row;
+      if (i == n - 1) a2 = row + 1, b2 = int(nrows);
+      if (i >= DEP_CROWD) {
+        const uint32_t j = i - DEP_CROWD;
+        if (key_row(cl.map_shared_rank(&S, j >> chunk_shift)->keys[cur][j & (chunk - 1)], n_mesh, log2n) == uint32_t(row))
+          row_start[nrows + 1] = 1u;
+      }
+    }
+    fill_rows(row_start, a, b, i);
+    fill_rows(row_start, a2, b2, n);
+  }
+  cl.sync();  // no CTA leaves while a peer reads its keys
+}
+
+template <typename R>
+cudaError_t launch_sort_small(const uint32_t* keys_in, int64_t n, int key_bits, uint32_t* keys_out, const void* pos_in,
+                              const void* mom_in, void* pos_out, void* mom_out, uint32_t* row_start, Mesh m,
+                              uint32_t* clear, cudaStream_t s) {
+  using V4 = typename VT<R>::v4;
+  if (n < 1 || n > SS_MAX_PARTICLES) return cudaErrorInvalidValue;
+  static bool done[64];  // the shared-memory opt-in, once per device
+  int dev = 0;
+  cudaGetDevice(&dev);
+  if (dev < 0 || dev >= 64 || !done[dev]) {
+    const cudaError_t e = cudaFuncSetAttribute(k_sort_small<V4>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                               int(sizeof(SortSmallShared)));
+    if (e != cudaSuccess) return e;
+    if (dev >= 0 && dev < 64) done[dev] = true;
+  }
+  // chunks of 1024 .. 8192 slots, a power of two, for up to eight CTAs
+  int shift = 10;
+  while ((int64_t(8) << shift) < n) ++shift;
+  unsigned ctas = 1;
+  while ((int64_t(ctas) << shift) < n) ctas *= 2;
+  const int passes = (key_bits + SS_BITS - 1) / SS_BITS, digit_bits = (key_bits + passes - 1) / passes;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(ctas);
+  cfg.blockDim = dim3(SS_THREADS);
+  cfg.dynamicSmemBytes = sizeof(SortSmallShared);
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = ctas;
+  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, k_sort_small<V4>, keys_in, uint32_t(n), shift, passes, digit_bits, key_bits, keys_out,
+                            (const V4*)pos_in, (const V4*)mom_in, (V4*)pos_out, (V4*)mom_out, row_start, uint32_t(m.n),
+                            m.log2n, clear);
 }
 
 // the three parts of the re-sort: the partition, the rows (scan and
