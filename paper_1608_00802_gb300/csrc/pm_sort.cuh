@@ -36,6 +36,19 @@ __device__ __forceinline__ uint32_t lanemask_lt() {
   return m;
 }
 
+// lanes whose digit of `bits` bits equals this lane's (all lanes take part): one vote per bit
+__device__ __forceinline__ uint32_t digit_peers(uint32_t d, int bits) {
+  uint32_t peers = 0xffffffffu;
+#pragma unroll
+  for (int b = 0; b < RS_MAX_BITS; ++b) {
+    if (b >= bits) break;
+    const bool on = (d >> b) & 1u;
+    const uint32_t v = __ballot_sync(0xffffffffu, on);
+    peers &= on ? v : ~v;
+  }
+  return peers;
+}
+
 constexpr uint64_t RS_FLAG_AGG = 1ull << 32;
 constexpr int RS_PASS_BLOCKS = 1216;  // blocks of one radix pass (8 per SM on 152 SMs)
 constexpr uint64_t RS_FLAG_PREFIX = 2ull << 32;
@@ -191,8 +204,8 @@ __global__ void __launch_bounds__(RS_THREADS) k_sort_pass(
     for (int r = 0; r < RS_ITEMS; ++r) {
       const int li = warp * (RS_ITEMS * 32) + r * 32 + lane;
       const bool valid = li < tile_n;
-      const uint32_t d = valid ? (key[r] >> shift) & mask : 0xffffffffu;
-      const uint32_t peers = __match_any_sync(0xffffffffu, d);
+      const uint32_t d = (key[r] >> shift) & mask;
+      const uint32_t peers = digit_peers(d, bits) & __ballot_sync(0xffffffffu, valid);
       const uint32_t before = valid ? my_cnt[d] : 0u;
       __syncwarp();
       const uint32_t within = __popc(peers & lt);
@@ -830,8 +843,8 @@ __global__ void __launch_bounds__(SS_THREADS, 1) k_sort_small(const uint32_t* ke
       const bool valid = li < cnt_here;
       key[r] = valid ? S.keys[cur][li] : 0u;
       val[r] = valid ? S.vals[cur][li] : uint16_t(0);
-      const uint32_t d = valid ? (key[r] >> shift) & mask : 0xffffffffu;
-      const uint32_t peers = __match_any_sync(0xffffffffu, d);
+      const uint32_t d = (key[r] >> shift) & mask;
+      const uint32_t peers = digit_peers(d, bits) & __ballot_sync(0xffffffffu, valid);
       const uint32_t before = valid ? mine[d] : 0u, within = __popc(peers & lt);
       __syncwarp();
       if (valid && within == 0) mine[d] = uint16_t(before + __popc(peers));
@@ -842,11 +855,16 @@ __global__ void __launch_bounds__(SS_THREADS, 1) k_sort_small(const uint32_t* ke
     // per digit (one thread each): the earlier warps' records, the CTA's total
     if (tid < radix) {
       uint32_t run = 0;
-#pragma unroll 8
-      for (int w = 0; w < SS_WARPS; ++w) {
-        const uint32_t t = S.cnt[w * radix + tid];
-        S.cnt[w * radix + tid] = uint16_t(run);
-        run += t;
+#pragma unroll
+      for (int w0 = 0; w0 < SS_WARPS; w0 += 16) {
+        uint16_t t[16];  // (read before any is overwritten, so that the loads overlap)
+#pragma unroll
+        for (int w = 0; w < 16; ++w) t[w] = S.cnt[(w0 + w) * radix + tid];
+#pragma unroll
+        for (int w = 0; w < 16; ++w) {
+          S.cnt[(w0 + w) * radix + tid] = uint16_t(run);
+          run += t[w];
+        }
       }
       S.tot[tid] = run;
     }
@@ -899,17 +917,14 @@ __global__ void __launch_bounds__(SS_THREADS, 1) k_sort_small(const uint32_t* ke
       pos_out[i] = pos_in[v];
       if (mom_in) mom_out[i] = mom_in[v];
       const int row = int(min(key_row(k, n_mesh, log2n), nrows - 1));
-      if (i > 0) {
-        const uint32_t j = i - 1;
-        a = int(min(key_row(cl.map_shared_rank(&S, j >> chunk_shift)->keys[cur][j & (chunk - 1)], n_mesh, log2n), nrows - 1)) + 1;
-      }
+      // the key of place j <= i: this CTA's, or a peer's
+      auto key_at = [&](uint32_t j) {
+        return j >= base ? S.keys[cur][j - base] : cl.map_shared_rank(&S, j >> chunk_shift)->keys[cur][j & (chunk - 1)];
+      };
+      if (i > 0) a = int(min(key_row(key_at(i - 1), n_mesh, log2n), nrows - 1)) + 1;
       b = row;
       if (i == n - 1) a2 = row + 1, b2 = int(nrows);
-      if (i >= DEP_CROWD) {
-        const uint32_t j = i - DEP_CROWD;
-        if (key_row(cl.map_shared_rank(&S, j >> chunk_shift)->keys[cur][j & (chunk - 1)], n_mesh, log2n) == uint32_t(row))
-          row_start[nrows + 1] = 1u;
-      }
+      if (i >= DEP_CROWD && key_row(key_at(i - DEP_CROWD), n_mesh, log2n) == uint32_t(row)) row_start[nrows + 1] = 1u;
     }
     fill_rows(row_start, a, b, i);
     fill_rows(row_start, a2, b2, n);
