@@ -23,6 +23,7 @@
 // stable sort of the new cells with ties broken by the previous order.
 #pragma once
 #include <cooperative_groups.h>
+#include <type_traits>
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -746,19 +747,22 @@ __global__ void __launch_bounds__(PF_THREADS) k_place(
 // ---------------------------------------------------------------- the sort of few particles in one kernel
 // Up to SS_MAX_PARTICLES particles the full sort is a chain of short kernels (clears, histogram, a look-back
 // pass per digit, row starts): 5-10 launches of 2-15 us, each with a few tiles in flight.  Here one cluster
-// of up to eight CTAs sorts in its shared memory instead: CTA c holds the keys of places
-// [c chunk, (c+1) chunk) and their slots (16 bits), and every pass ranks its chunk by a digit (warp match
-// and per-warp counters, in order), exchanges the CTAs' digit totals through distributed shared memory,
-// stages the chunk in digit order and sends each run of equal digits, contiguous at its destination, to the
-// CTAs that hold those places.  The last pass is followed by the gather of the records, the row starts and
-// the crowded-row flag.  Same order as the general sort (stable, so it is the only one there is).
-// 65536 particles on 128^3: SS_FIG.
-constexpr int SS_MAX_PARTICLES = SORT_SMALL_MAX, SS_THREADS = 1024, SS_WARPS = 32, SS_CHUNK = SS_MAX_PARTICLES / 8;
-constexpr int SS_BITS = 10, SS_ITEMS = SS_CHUNK / SS_THREADS;
+// of up to sixteen CTAs sorts in its shared memory instead: CTA c holds the records {key, slot} of places
+// [c chunk, (c+1) chunk), and every pass ranks its chunk by a digit (votes and per-warp counters, in
+// order), exchanges the CTAs' digit totals through distributed shared memory, stages the chunk in digit
+// order and sends each run of equal digits, contiguous at its destination, to the CTAs that hold those
+// places.  The last pass is followed by the gather of the particles' records, the row starts and the
+// crowded-row flag.  Same order as the general sort (stable, so it is the only one there is).  Bound by the
+// latency of its phases (ranking, staging, sending, two cluster barriers a pass) on few SMs, so the CTAs are
+// many and small and every loop over a thread's records issues all its loads first.  32768 particles on
+// 64^3: five launches of 38 us in all -> 17 us (27 us with eight CTAs and one load at a time); the whole
+// deposit call of 65536 on 128^3: 84 -> 46 us.
+constexpr int SS_MAX_PARTICLES = SORT_SMALL_MAX, SS_THREADS = 1024, SS_WARPS = 32, SS_BITS = 10;
 
+// ITEMS: records per thread; a CTA's chunk is ITEMS * SS_THREADS places
+template <int ITEMS>
 struct SortSmallShared {
-  uint32_t keys[2][SS_CHUNK];
-  uint16_t vals[2][SS_CHUNK];
+  uint64_t rec[2][ITEMS * SS_THREADS];  // key << 32 | slot
   uint16_t cnt[SS_WARPS << SS_BITS];
   uint32_t tot[1 << SS_BITS];     // records of each digit in this CTA (read by its peers)
   uint32_t dstart[1 << SS_BITS];  // where the digit starts in the staged chunk
@@ -777,7 +781,7 @@ __device__ __forceinline__ uint2 block_excl_scan2(uint2 v, uint2* scratch) {
   }
   if (lane == 31) scratch[warp] = inc;
   __syncthreads();
-  uint2 w = lane < SS_WARPS && lane < warp ? scratch[lane] : make_uint2(0, 0);
+  uint2 w = lane < warp ? scratch[lane] : make_uint2(0, 0);
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
     w.x += __shfl_xor_sync(0xffffffffu, w.x, o);
@@ -800,28 +804,50 @@ __device__ __forceinline__ void fill_rows(uint32_t* __restrict__ row_start, int 
   }
 }
 
+// a thread's records in[slot of each of its places] to out, all loads in flight (fp32; the 32-byte fp64 records
+// four at a time)
+template <typename V4, int ITEMS>
+__device__ __forceinline__ void gather_records(const V4* __restrict__ in, V4* __restrict__ out, const uint64_t* rec,
+                                               uint32_t base, uint32_t cnt) {
+  constexpr int G = sizeof(V4) == 16 || ITEMS < 8 ? ITEMS : 4;
+  for (int r0 = 0; r0 < ITEMS; r0 += G) {
+    V4 v[G];
+#pragma unroll
+    for (int r = 0; r < G; ++r) {
+      const uint32_t li = uint32_t(r0 + r) * SS_THREADS + threadIdx.x;
+      if (li < cnt) v[r] = in[uint32_t(rec[li])];
+    }
+#pragma unroll
+    for (int r = 0; r < G; ++r) {
+      const uint32_t li = uint32_t(r0 + r) * SS_THREADS + threadIdx.x;
+      if (li < cnt) out[base + li] = v[r];
+    }
+  }
+}
+
 // keys may be sorted in place (keys_out = keys_in); mom_in null: no momenta; clear (nullable): a word set to 0
-template <typename V4>
-__global__ void __launch_bounds__(SS_THREADS, 1) k_sort_small(const uint32_t* keys_in, uint32_t n, int chunk_shift,
-                                                              int passes, int digit_bits, int key_bits, uint32_t* keys_out,
+template <typename V4, int ITEMS>
+__global__ void __launch_bounds__(SS_THREADS, 1) k_sort_small(const uint32_t* keys_in, uint32_t n, int passes, int digit_bits,
+                                                              int key_bits, uint32_t* keys_out,
                                                               const V4* __restrict__ pos_in, const V4* __restrict__ mom_in,
                                                               V4* __restrict__ pos_out, V4* __restrict__ mom_out,
                                                               uint32_t* __restrict__ row_start, uint32_t n_mesh,
                                                               int log2n, uint32_t* clear) {
+  constexpr uint32_t chunk = ITEMS * SS_THREADS;
   namespace cg = cooperative_groups;
   extern __shared__ __align__(16) unsigned char ss_smem[];
-  SortSmallShared& S = *reinterpret_cast<SortSmallShared*>(ss_smem);
+  SortSmallShared<ITEMS>& S = *reinterpret_cast<SortSmallShared<ITEMS>*>(ss_smem);
   cg::cluster_group cl = cg::this_cluster();
   const uint32_t rank = cl.block_rank(), ncta = cl.num_blocks();
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const uint32_t chunk = 1u << chunk_shift, base = rank << chunk_shift;
+  const uint32_t base = rank * chunk;
   const uint32_t cnt_here = base < n ? min(chunk, n - base) : 0u;
   const uint32_t nrows = n_mesh * n_mesh;
   const uint32_t lt = lanemask_lt();
-  const int items = int((chunk + SS_THREADS - 1) / SS_THREADS);  // rounds of a warp (its slots are contiguous)
-  for (uint32_t i = tid; i < cnt_here; i += SS_THREADS) {
-    S.keys[0][i] = keys_in[base + i];
-    S.vals[0][i] = uint16_t(base + i);
+#pragma unroll
+  for (int r = 0; r < ITEMS; ++r) {
+    const uint32_t i = uint32_t(r) * SS_THREADS + tid;
+    if (i < cnt_here) S.rec[0][i] = (uint64_t(keys_in[base + i]) << 32) | (base + i);
   }
   if (rank == 0 && tid == 0) {
     row_start[nrows + 1] = 0;  // the crowded-row flag
@@ -833,17 +859,16 @@ __global__ void __launch_bounds__(SS_THREADS, 1) k_sort_small(const uint32_t* ke
     const uint32_t mask = uint32_t(radix - 1);
     for (int d = tid; d < (SS_WARPS * radix) / 2; d += SS_THREADS) reinterpret_cast<uint32_t*>(S.cnt)[d] = 0;
     __syncthreads();
-    uint32_t key[SS_ITEMS], rk[SS_ITEMS];
-    uint16_t val[SS_ITEMS];
+    uint64_t rec[ITEMS];
+    uint32_t rk[ITEMS];
     uint16_t* mine = S.cnt + warp * radix;
+    const uint32_t l0 = uint32_t(warp * ITEMS) * 32u + lane;  // a warp's places are contiguous
 #pragma unroll
-    for (int r = 0; r < SS_ITEMS; ++r) {
-      if (r >= items) break;
-      const uint32_t li = uint32_t(warp * items + r) * 32u + lane;
-      const bool valid = li < cnt_here;
-      key[r] = valid ? S.keys[cur][li] : 0u;
-      val[r] = valid ? S.vals[cur][li] : uint16_t(0);
-      const uint32_t d = (key[r] >> shift) & mask;
+    for (int r = 0; r < ITEMS; ++r) rec[r] = l0 + r * 32u < cnt_here ? S.rec[cur][l0 + r * 32u] : 0ull;
+#pragma unroll
+    for (int r = 0; r < ITEMS; ++r) {
+      const bool valid = l0 + r * 32u < cnt_here;
+      const uint32_t d = (uint32_t(rec[r] >> 32) >> shift) & mask;
       const uint32_t peers = digit_peers(d, bits) & __ballot_sync(0xffffffffu, valid);
       const uint32_t before = valid ? mine[d] : 0u, within = __popc(peers & lt);
       __syncwarp();
@@ -872,6 +897,7 @@ __global__ void __launch_bounds__(SS_THREADS, 1) k_sort_small(const uint32_t* ke
     uint2 v = make_uint2(0, 0);
     uint32_t below = 0;
     if (tid < radix) {
+#pragma unroll 8
       for (uint32_t c = 0; c < ncta; ++c) {
         const uint32_t t = cl.map_shared_rank(S.tot, c)[tid];
         v.x += t;
@@ -885,41 +911,49 @@ __global__ void __launch_bounds__(SS_THREADS, 1) k_sort_small(const uint32_t* ke
       S.dstart[tid] = ex.y;
     }
     __syncthreads();
-    // the chunk in digit order (every key of it is in registers)
+    // the chunk in digit order (every record of it is in registers)
 #pragma unroll
-    for (int r = 0; r < SS_ITEMS; ++r) {
-      if (r >= items) break;
-      const uint32_t li = uint32_t(warp * items + r) * 32u + lane;
+    for (int r = 0; r < ITEMS; ++r) {
+      const uint32_t d = (uint32_t(rec[r] >> 32) >> shift) & mask;
+      rk[r] += S.dstart[d] + mine[d];
+    }
+#pragma unroll
+    for (int r = 0; r < ITEMS; ++r)
+      if (l0 + r * 32u < cnt_here) S.rec[cur][rk[r]] = rec[r];
+    __syncthreads();
+    // and on to the places' CTAs
+#pragma unroll
+    for (int r = 0; r < ITEMS; ++r) {
+      const uint32_t li = uint32_t(r) * SS_THREADS + tid;
       if (li < cnt_here) {
-        const uint32_t d = (key[r] >> shift) & mask, at = S.dstart[d] + mine[d] + rk[r];
-        S.keys[cur][at] = key[r];
-        S.vals[cur][at] = val[r];
+        rec[r] = S.rec[cur][li];
+        const uint32_t d = (uint32_t(rec[r] >> 32) >> shift) & mask;
+        rk[r] = S.gbase[d] + li - S.dstart[d];
       }
     }
-    __syncthreads();
-    for (uint32_t li = tid; li < cnt_here; li += SS_THREADS) {
-      const uint32_t k = S.keys[cur][li], d = (k >> shift) & mask, to = S.gbase[d] + li - S.dstart[d];
-      SortSmallShared* peer = cl.map_shared_rank(&S, to >> chunk_shift);
-      peer->keys[cur ^ 1][to & (chunk - 1)] = k;
-      peer->vals[cur ^ 1][to & (chunk - 1)] = S.vals[cur][li];
+#pragma unroll
+    for (int r = 0; r < ITEMS; ++r) {
+      const uint32_t li = uint32_t(r) * SS_THREADS + tid;
+      if (li < cnt_here)
+        cl.map_shared_rank(&S, rk[r] / chunk)->rec[cur ^ 1][rk[r] & (chunk - 1)] = rec[r];
     }
     cl.sync();
     cur ^= 1;
   }
-  // records, row starts and the flag, 32 consecutive places per warp and round (whole warps: fill_rows votes)
+  gather_records<V4, ITEMS>(pos_in, pos_out, S.rec[cur], base, cnt_here);
+  if (mom_in) gather_records<V4, ITEMS>(mom_in, mom_out, S.rec[cur], base, cnt_here);
+  // keys, row starts and the flag, 32 consecutive places per warp and round (whole warps: fill_rows votes)
   for (uint32_t w0 = warp * 32u; w0 < cnt_here; w0 += SS_THREADS) {
     const uint32_t li = w0 + lane, i = base + li;
-    const bool valid = li < cnt_here;
     int a = 0, b = -1, a2 = 0, b2 = -1;
-    if (valid) {
-      const uint32_t k = S.keys[cur][li], v = S.vals[cur][li];
+    if (li < cnt_here) {
+      const uint32_t k = uint32_t(S.rec[cur][li] >> 32);
       keys_out[i] = k;
-      pos_out[i] = pos_in[v];
-      if (mom_in) mom_out[i] = mom_in[v];
       const int row = int(min(key_row(k, n_mesh, log2n), nrows - 1));
       // the key of place j <= i: this CTA's, or a peer's
       auto key_at = [&](uint32_t j) {
-        return j >= base ? S.keys[cur][j - base] : cl.map_shared_rank(&S, j >> chunk_shift)->keys[cur][j & (chunk - 1)];
+        return uint32_t((j >= base ? S.rec[cur][j - base]
+                                   : cl.map_shared_rank(&S, j / chunk)->rec[cur][j & (chunk - 1)]) >> 32);
       };
       if (i > 0) a = int(min(key_row(key_at(i - 1), n_mesh, log2n), nrows - 1)) + 1;
       b = row;
@@ -932,41 +966,75 @@ __global__ void __launch_bounds__(SS_THREADS, 1) k_sort_small(const uint32_t* ke
   cl.sync();  // no CTA leaves while a peer reads its keys
 }
 
+template <typename V4, int ITEMS>
+cudaError_t launch_sort_small_items(const uint32_t* keys_in, uint32_t n, int key_bits, uint32_t* keys_out, const V4* pos_in,
+                                    const V4* mom_in, V4* pos_out, V4* mom_out, uint32_t* row_start, Mesh m,
+                                    uint32_t* clear, cudaStream_t s, int* ctas_max) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.blockDim = dim3(SS_THREADS);
+  cfg.dynamicSmemBytes = sizeof(SortSmallShared<ITEMS>);
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  if (ctas_max) {  // preparation: the shared-memory opt-in, and whether clusters beyond the portable eight fit
+    const cudaError_t e = cudaFuncSetAttribute(k_sort_small<V4, ITEMS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                               int(sizeof(SortSmallShared<ITEMS>)));
+    if (e != cudaSuccess) return e;
+    int clusters = 0;
+    cfg.gridDim = dim3(16);
+    at[0].val.clusterDim.x = 16;
+    if (cudaFuncSetAttribute(k_sort_small<V4, ITEMS>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
+        cudaOccupancyMaxActiveClusters(&clusters, k_sort_small<V4, ITEMS>, &cfg) != cudaSuccess || clusters < 1) {
+      cudaGetLastError();
+      *ctas_max = 8;
+    }
+    return cudaSuccess;
+  }
+  unsigned ctas = 1;
+  while (ctas * ITEMS * SS_THREADS < n) ctas *= 2;
+  const int passes = (key_bits + SS_BITS - 1) / SS_BITS, digit_bits = (key_bits + passes - 1) / passes;
+  cfg.gridDim = dim3(ctas);
+  at[0].val.clusterDim.x = ctas;
+  return cudaLaunchKernelEx(&cfg, k_sort_small<V4, ITEMS>, keys_in, n, passes, digit_bits, key_bits, keys_out, pos_in,
+                            mom_in, pos_out, mom_out, row_start, uint32_t(m.n), m.log2n, clear);
+}
+
 template <typename R>
 cudaError_t launch_sort_small(const uint32_t* keys_in, int64_t n, int key_bits, uint32_t* keys_out, const void* pos_in,
                               const void* mom_in, void* pos_out, void* mom_out, uint32_t* row_start, Mesh m,
                               uint32_t* clear, cudaStream_t s) {
   using V4 = typename VT<R>::v4;
   if (n < 1 || n > SS_MAX_PARTICLES) return cudaErrorInvalidValue;
-  static bool done[64];  // the shared-memory opt-in, once per device
-  int dev = 0;
+  auto run = [&](auto items, int* prepare) {
+    return launch_sort_small_items<V4, decltype(items)::value>(keys_in, uint32_t(n), key_bits, keys_out, (const V4*)pos_in,
+                                                               (const V4*)mom_in, (V4*)pos_out, (V4*)mom_out, row_start,
+                                                               m, clear, s, prepare);
+  };
+  using I1 = std::integral_constant<int, 1>;
+  using I2 = std::integral_constant<int, 2>;
+  using I4 = std::integral_constant<int, 4>;
+  using I8 = std::integral_constant<int, 8>;
+  static int most[64];  // CTAs of a cluster on each device (0: not prepared)
+  int dev = 0, ctas = 16;
   cudaGetDevice(&dev);
-  if (dev < 0 || dev >= 64 || !done[dev]) {
-    const cudaError_t e = cudaFuncSetAttribute(k_sort_small<V4>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                               int(sizeof(SortSmallShared)));
+  if (dev < 0 || dev >= 64 || most[dev] == 0) {
+    cudaError_t e = run(I1(), &ctas);
+    if (e == cudaSuccess) e = run(I2(), &ctas);
+    if (e == cudaSuccess) e = run(I4(), &ctas);
+    if (e == cudaSuccess) e = run(I8(), &ctas);
     if (e != cudaSuccess) return e;
-    if (dev >= 0 && dev < 64) done[dev] = true;
+    if (dev >= 0 && dev < 64) most[dev] = ctas;
+  } else {
+    ctas = most[dev];
   }
-  // chunks of 1024 .. 8192 slots, a power of two, for up to eight CTAs
-  int shift = 10;
-  while ((int64_t(8) << shift) < n) ++shift;
-  unsigned ctas = 1;
-  while ((int64_t(ctas) << shift) < n) ctas *= 2;
-  const int passes = (key_bits + SS_BITS - 1) / SS_BITS, digit_bits = (key_bits + passes - 1) / passes;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(ctas);
-  cfg.blockDim = dim3(SS_THREADS);
-  cfg.dynamicSmemBytes = sizeof(SortSmallShared);
-  cfg.stream = s;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = ctas;
-  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, k_sort_small<V4>, keys_in, uint32_t(n), shift, passes, digit_bits, key_bits, keys_out,
-                            (const V4*)pos_in, (const V4*)mom_in, (V4*)pos_out, (V4*)mom_out, row_start, uint32_t(m.n),
-                            m.log2n, clear);
+  // the smallest chunks whose cluster holds all particles
+  if (n <= int64_t(ctas) * SS_THREADS) return run(I1(), nullptr);
+  if (n <= int64_t(ctas) * SS_THREADS * 2) return run(I2(), nullptr);
+  if (n <= int64_t(ctas) * SS_THREADS * 4) return run(I4(), nullptr);
+  return run(I8(), nullptr);
 }
 
 // the three parts of the re-sort: the partition, the rows (scan and
