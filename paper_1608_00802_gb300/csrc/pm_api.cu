@@ -385,12 +385,11 @@ int kr_blocks(const pm_sim* s) {
 // buckets, the placement of each particle with its records into the other
 // buffer; see pm_sort.cuh).  Same order as the full sort; also writes the row
 // starts.
+// step (nullable): the device step counter of captured steps, advanced on the way.
 template <typename R>
-pm_status resort_movers(pm_sim* s) {
+pm_status resort_movers(pm_sim* s, uint32_t* step) {
   const Layout& L = s->L;
-  const int N = s->cfg.n_mesh;
   const int nxt = s->cur ^ 1;
-  CU(s, cudaMemsetAsync(s->at<uint32_t>(L.rcnt), 0, size_t(3) * N * N * 4, s->stream));
   const int stages[3] = {PM_STAGE_SORT_PARTITION, PM_STAGE_SORT_PASS, PM_STAGE_SORT_MERGE};
   for (int part = 0; part < 3; ++part) {
     PROF(s, stages[part]);
@@ -398,8 +397,8 @@ pm_status resort_movers(pm_sim* s) {
                            s->at<uint32_t>(L.vals[0]), s->keys_tmp[1], s->at<uint32_t>(L.vals[1]),
                            s->at<uint32_t>(L.keys[3]), s->at<uint32_t>(L.vals[2]), s->at<uint32_t>(L.tile_cnt),
                            s->at<uint32_t>(L.rcnt), s->at<uint32_t>(L.btot), s->at<uint32_t>(L.srow),
-                           s->at<uint32_t>(L.mrow), s->at<uint32_t>(L.row_start), s->mesh, s->sort_stats(), s->keys,
-                           s->pos(), s->mom(), s->arena + L.pos[nxt], s->arena + L.mom[nxt], s->sms, s->stream));
+                           s->at<uint32_t>(L.mrow), s->at<uint32_t>(L.row_start), s->mesh, s->sort_stats(), step,
+                           s->keys, s->pos(), s->mom(), s->arena + L.pos[nxt], s->arena + L.mom[nxt], s->sms, s->stream));
   }
   s->cur = nxt;
   s->keys_marked = false;
@@ -408,8 +407,8 @@ pm_status resort_movers(pm_sim* s) {
 }
 
 template <typename R>
-pm_status sort_particles(pm_sim* s) {
-  if (s->keys_marked) return resort_movers<R>(s);
+pm_status sort_particles(pm_sim* s, uint32_t* step = nullptr) {
+  if (s->keys_marked) return resort_movers<R>(s, step);
   const Layout& L = s->L;
   const int64_t n = s->n();
   if (n <= SORT_SMALL_MAX) {  // one kernel, the keys in place
@@ -777,10 +776,7 @@ pm_status kick(pm_sim* s, const KickParams& kp, double* acc, const KickParams* k
     pm_status st = sort_particles<R>(s);
     if (st != PM_OK) return st;
   }
-  // a drift counts its movers per tile (for the re-sort's partition)
-  if (drift)
-    CU(s, cudaMemsetAsync(s->at<uint32_t>(L.tcount), 0, size_t(mover_count_words(s->n())) * 4, s->stream));
-  {
+  {  // (a drift counts its movers per tile for the re-sort's partition: zero since the last placement)
     PROF(s, PM_STAGE_KICK);
     CU(s, launch_kick<R>(s->pos(), s->mom(), s->keys, s->at<uint32_t>(L.tcount), s->n(), s->at<R>(L.phi),
                          s->at<R>(L.q), s->mesh, kp, kp_tab, step, s->part(), acc, s->errword(),
@@ -861,10 +857,10 @@ pm_status table_step(pm_sim* s, const KickParams* tab, uint32_t* step) {
   kp.drift = 1.0;  // host-side marker only: the positions move, the weights come from the table
   pm_status st = DISPATCH(s, kick, s, kp, nullptr, tab, step);
   if (st != PM_OK) return st;
-  st = ensure_fields(s);
+  // the re-sort advances the step counter
+  st = s->fp64() ? sort_particles<double>(s, step) : sort_particles<float>(s, step);
   if (st != PM_OK) return st;
-  CU(s, launch_step_inc(step, s->stream));
-  return PM_OK;
+  return ensure_fields(s);
 }
 
 void to_public(const Tuning& t, pm_tuning* o) {
@@ -1072,6 +1068,8 @@ pm_status pm_create(const pm_config* c, void* dev_arena, size_t bytes, void* str
     }
   }
   if (cudaMemsetAsync(s->errword(), 0, 256, s->stream) != cudaSuccess ||
+      cudaMemsetAsync(s->arena + L.tcount, 0, size_t(mover_count_words(c->n_part)) * 4, s->stream) != cudaSuccess ||
+      cudaMemsetAsync(s->arena + L.rcnt, 0, size_t(3) * N * N * 4, s->stream) != cudaSuccess ||
       cudaMemsetAsync(s->arena + L.status, 0, (size_t(1) << L.digit_bits) * size_t(L.ntiles) * 8, s->stream) !=
           cudaSuccess ||
       cudaStreamSynchronize(s->stream) != cudaSuccess) {
@@ -1162,8 +1160,10 @@ pm_status pm_set_particles(pm_sim* s, const double* x, const double* p) {
   CU(s, DISPATCH(s, launch_init_particles, dx, dp, s->n(), s->mesh, 1.0 / s->dx, s->pos(), s->mom(), s->keys,
                  s->errword(), s->stream));
   s->have_particles = true;
+  if (s->keys_marked)  // a drift whose re-sort did not run (an error between them): its counts are dropped
+    CU(s, cudaMemsetAsync(s->at<uint32_t>(s->L.tcount), 0, size_t(mover_count_words(s->n())) * 4, s->stream));
   s->sorted = s->fields_valid = s->keys_marked = false;
-  pm_status st = DISPATCH(s, sort_particles, s);
+  pm_status st = DISPATCH(s, sort_particles, s, nullptr);
   if (st != PM_OK) return st;
   return device_errors(s);
 }
@@ -1683,6 +1683,7 @@ pm_status pm_load(pm_sim* s, const void* host, size_t bytes) {
   CU(s, cudaMemcpyAsync(s->mom(), in + CKPT_HEADER + rb, rb, cudaMemcpyHostToDevice, s->stream));
   CU(s, cudaMemcpyAsync(s->keys, in + CKPT_HEADER + 2 * rb, size_t(s->n()) * 4, cudaMemcpyHostToDevice, s->stream));
   CU(s, cudaMemcpyAsync(s->sort_stats(), stats, sizeof stats, cudaMemcpyHostToDevice, s->stream));
+  CU(s, cudaMemsetAsync(s->at<uint32_t>(s->L.tcount), 0, size_t(mover_count_words(s->n())) * 4, s->stream));
   // sorted records: the deposit reads the row starts of the keys (integer, so the same as the re-sort's)
   if (h.flags & 1) {
     CU(s, cudaMemsetAsync(s->at<uint32_t>(s->L.row_start) + s->mesh.n2 + 1, 0, 4, s->stream));
@@ -1916,20 +1917,18 @@ pm_status packed_step(pm_batch::Class& C, const std::vector<pm_sim*>& sims, cuda
   // kick + drift with the weights of the members' step counters
   KickParams kp = base_kick(s);
   kp.drift = 1.0;  // host-side marker only: the positions move, the weights come from the tables
-  PCU(cudaMemset2DAsync(s->at<uint32_t>(L.tcount), ms, 0, size_t(mover_count_words(n)) * 4, size_t(nm), st));
   PCU(launch_kick<float>(s->pos(), s->mom(), s->keys, s->at<uint32_t>(L.tcount), n, s->at<float>(L.phi),
                          s->at<float>(L.q), s->mesh, kp, s->at<KickParams>(L.ktab), s->errword() + 2, s->part(),
                          nullptr, s->errword(), s->tune.kick_threads, st, nm, ms));
   // re-sort into the other record buffer (the movers' count on the device of every member)
   const int N = s->cfg.n_mesh;
-  PCU(cudaMemset2DAsync(s->at<uint32_t>(L.rcnt), ms, 0, size_t(3) * N * N * 4, size_t(nm), st));
   for (int part = 0; part < 3; ++part)
     PCU(launch_resort<float>(part, s->keys, n, s->at<uint32_t>(L.tcount), s->keys_tmp[0], s->at<uint32_t>(L.vals[0]),
                              s->keys_tmp[1], s->at<uint32_t>(L.vals[1]), s->at<uint32_t>(L.keys[3]),
                              s->at<uint32_t>(L.vals[2]), s->at<uint32_t>(L.tile_cnt), s->at<uint32_t>(L.rcnt),
                              s->at<uint32_t>(L.btot), s->at<uint32_t>(L.srow), s->at<uint32_t>(L.mrow),
-                             s->at<uint32_t>(L.row_start), s->mesh, s->sort_stats(), s->keys, s->pos(), s->mom(),
-                             s->arena + L.pos[nxt], s->arena + L.mom[nxt], s->sms, st, nm, ms));
+                             s->at<uint32_t>(L.row_start), s->mesh, s->sort_stats(), s->errword() + 2, s->keys, s->pos(),
+                             s->mom(), s->arena + L.pos[nxt], s->arena + L.mom[nxt], s->sms, st, nm, ms));
   // deposit, potential, quantum pressure
   PCU(launch_deposit<float>(s->arena + L.pos[nxt], s->at<uint32_t>(L.row_start), n, s->mesh, s->norm,
                             s->at<float>(L.rho), st, s->tune.dep_warps, nm, ms));
@@ -1972,7 +1971,6 @@ pm_status packed_step(pm_batch::Class& C, const std::vector<pm_sim*>& sims, cuda
     PCU(launch_stencil<float>(s->at<float>(L.rho), s->mesh, stencil_params(s, false), s->at<float>(L.q), kr_part(s),
                               s->at<uint32_t>(L.st_list), s->at<uint32_t>(L.st_count), s->errword(),
                               nullptr, st, s->coefs() + 1, nm, ms));
-  PCU(launch_step_inc(s->errword() + 2, st, nm, ms));
   for (int i : C.members) {
     pm_sim* m = sims[i];
     m->cur = nxt;

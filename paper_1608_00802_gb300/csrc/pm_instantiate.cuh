@@ -13,9 +13,9 @@
                                             void*, void*, uint32_t*, Mesh, uint32_t*, cudaStream_t);              \
   template cudaError_t launch_deposit<R>(const void*, const uint32_t*, int64_t, Mesh, double, R*, cudaStream_t,    \
                                          int, int, size_t);                                                       \
-  template cudaError_t launch_resort<R>(int, const uint32_t*, int64_t, const uint32_t*, uint32_t*, uint32_t*, uint32_t*, \
+  template cudaError_t launch_resort<R>(int, const uint32_t*, int64_t, uint32_t*, uint32_t*, uint32_t*, uint32_t*, \
                                         uint32_t*, uint32_t*, uint32_t*, uint32_t*, uint32_t*, uint32_t*, uint32_t*, \
-                                        uint32_t*, uint32_t*, Mesh, unsigned long long*, uint32_t*, const void*,     \
+                                        uint32_t*, uint32_t*, Mesh, unsigned long long*, uint32_t*, uint32_t*, const void*, \
                                         const void*, void*, void*, int, cudaStream_t, int, size_t);               \
   template cudaError_t launch_green<R>(void*, Mesh, const void*, double, double*, cudaStream_t, const double*, int, \
                                        size_t);                                                                  \

@@ -156,17 +156,18 @@ cudaError_t launch_sort_small(const uint32_t* keys_in, int64_t n, int key_bits, 
 // counts (btot: 2 ceil(N^2 / 4096) words; srow, mrow, row_start: N^2 + 1
 // words), the movers in per-row buckets (bk, bv) and the placement of every
 // particle: sorted keys to keys_out, records from (pos_in, mom_in) to
-// (pos_out, mom_out) in sorted order.  stats (nullable): re-sorts and movers.
+// (pos_out, mom_out) in sorted order.  stats (nullable): re-sorts and movers; step (nullable): the device step
+// counter, advanced by the row scan.  tcount and rcnt are zero again afterwards.
 // part 0: the partition; 1: the rows (scan, buckets, movers' placement); 2:
 // the stayers' placement (launched in this order).
 template <typename R>
-cudaError_t launch_resort(int part, const uint32_t* keys, int64_t n, const uint32_t* tcount, uint32_t* sk, uint32_t* sv,
+cudaError_t launch_resort(int part, const uint32_t* keys, int64_t n, uint32_t* tcount, uint32_t* sk, uint32_t* sv,
                           uint32_t* mk, uint32_t* mv, uint32_t* bk, uint32_t* bv, uint32_t* counts, uint32_t* rcnt,
                           uint32_t* btot, uint32_t* srow, uint32_t* mrow, uint32_t* row_start, Mesh m,
-                          unsigned long long* stats, uint32_t* keys_out, const void* pos_in, const void* mom_in,
-                          void* pos_out, void* mom_out, int sms, cudaStream_t s, int nm = 1, size_t ms = 0);
+                          unsigned long long* stats, uint32_t* step, uint32_t* keys_out, const void* pos_in,
+                          const void* mom_in, void* pos_out, void* mom_out, int sms, cudaStream_t s, int nm = 1,
+                          size_t ms = 0);
 inline size_t row_scan_tiles(int n_mesh) { return (size_t(n_mesh) * n_mesh + 1023) / 1024; }  // tiles of 1024 rows
-cudaError_t launch_step_inc(uint32_t* step, cudaStream_t s, int nm = 1, size_t ms = 0);
 // the x-y transforms of the z-planes of a 256^3 fp32 mesh, one kernel per direction (unnormalised,
 // the layouts of the batched 2D R2C / C2R); tw: exp(-2 pi i t / 256), t < 256
 bool xy_fft_supported(int n_mesh);
@@ -227,7 +228,7 @@ Tuning default_tuning(int n);
 // call outside any stream capture, before the first kick)
 void kick_stream_prepare();
 // updates the records in place; with a drift also the keys and the mover
-// counts tcount (cleared before)
+// counts tcount (zero before)
 template <typename R>
 cudaError_t launch_kick(void* pos, void* mom, uint32_t* keys, uint32_t* tcount, int64_t n, const R* phi, const R* q,
                         Mesh m, KickParams kp,

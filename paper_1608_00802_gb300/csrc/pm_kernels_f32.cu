@@ -5,17 +5,6 @@
 
 namespace pm {
 
-// the device step counters of nm members (ms bytes apart)
-static __global__ void k_step_inc(uint32_t* step, int nm, size_t ms) {
-  const int m = blockIdx.x * blockDim.x + threadIdx.x;
-  if (m < nm) *moff(step, size_t(m) * ms) += 1u;
-}
-
-cudaError_t launch_step_inc(uint32_t* step, cudaStream_t s, int nm, size_t ms) {
-  k_step_inc<<<unsigned((nm + 255) / 256), 256, 0, s>>>(step, nm, ms);
-  return cudaGetLastError();
-}
-
 cudaError_t launch_sort_histogram(const uint32_t* keys, int64_t n, int passes, int digit_bits, int key_bits,
                                   uint32_t* hist, uint32_t* epoch, cudaStream_t s, const uint32_t* n_dev,
                                   uint32_t* crowd) {

@@ -436,20 +436,21 @@ static __global__ void __launch_bounds__(TS_THREADS) k_tile_scan(uint32_t* tcoun
 // earlier tiles come from the tile scan.  It writes its stayers to (s_keys, s_vals) and its
 // movers, flag cleared, to (m_keys, m_vals) (values: previous slots), adds
 // its stayers and movers to the per-row counts rcnt[0][row] and rcnt[1][row]
-// (cleared before; one atomic per run of equal rows in a warp for the
+// (zero before; one atomic per run of equal rows in a warp for the
 // stayers), and the last tile stores counts[0] = stayers, counts[1] = movers
 // and adds one re-sort and the movers to stats (nullable).
 static __global__ void __launch_bounds__(RS_THREADS) k_mover_partition(
     const uint32_t* __restrict__ keys, int64_t n, const uint32_t* __restrict__ tcount,
     uint32_t* __restrict__ s_keys, uint32_t* __restrict__ s_vals, uint32_t* __restrict__ m_keys,
     uint32_t* __restrict__ m_vals, uint32_t* __restrict__ counts, uint32_t* __restrict__ rcnt,
-    uint32_t n_mesh, int log2n, unsigned long long* __restrict__ stats, int own_scan, size_t ms) {
+    uint32_t* __restrict__ row_start, uint32_t n_mesh, int log2n, unsigned long long* __restrict__ stats, int own_scan,
+    size_t ms) {
   __shared__ uint32_t wm[RS_WARPS];
   if (ms) {  // member blockIdx.y of a packed group
     const size_t o = size_t(blockIdx.y) * ms;
     keys = moff(keys, o), tcount = moff(tcount, o), s_keys = moff(s_keys, o), s_vals = moff(s_vals, o);
     m_keys = moff(m_keys, o), m_vals = moff(m_vals, o), counts = moff(counts, o), rcnt = moff(rcnt, o);
-    stats = moff(stats, o);
+    stats = moff(stats, o), row_start = moff(row_start, o);
   }
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const uint32_t nrows = n_mesh * n_mesh;
@@ -503,6 +504,7 @@ static __global__ void __launch_bounds__(RS_THREADS) k_mover_partition(
   if (tile == ntiles - 1 && threadIdx.x == 0) {
     counts[0] = uint32_t(n) - (excl + total);
     counts[1] = excl + total;
+    row_start[nrows + 1] = 0;  // the crowded-row flag, set by k_row_scan
     if (stats) {  // re-sorts and moved particles so far (a diagnostic)
       stats[0] += 1ull;
       stats[1] += (unsigned long long)(excl + total);
@@ -535,17 +537,20 @@ static __global__ void __launch_bounds__(RS_THREADS) k_mover_partition(
 // in tiles of RT_TILE rows: k_row_totals sums each tile, k_row_scan adds the
 // earlier tiles' totals and scans its own, writing srow (stayers before row
 // r), mrow (movers before row r) and the new row starts row_start = srow +
-// mrow, with the closing entries at r = N^2.
+// mrow, with the closing entries at r = N^2.  With few tiles (up to
+// RT_DIRECT_TILES: meshes up to 128^2 rows) k_row_scan sums the earlier tiles'
+// rows itself (btot null), which costs less than a launch; at 256^2 rows that
+// took 25 us against 17 for the two kernels and the buckets.  step (nullable): the device step counter, which
+// a captured step advances here.
+constexpr uint32_t RT_DIRECT_TILES = 16;
 
 static __global__ void __launch_bounds__(RT_THREADS) k_row_totals(const uint32_t* __restrict__ rcnt, uint32_t nrows,
-                                                                  uint32_t* __restrict__ btot,
-                                                                  uint32_t* __restrict__ row_start, size_t ms) {
+                                                                  uint32_t* __restrict__ btot, size_t ms) {
   __shared__ uint32_t sh[2][32];
   if (ms) {
     const size_t o = size_t(blockIdx.y) * ms;
-    rcnt = moff(rcnt, o), btot = moff(btot, o), row_start = moff(row_start, o);
+    rcnt = moff(rcnt, o), btot = moff(btot, o);
   }
-  if (blockIdx.x == 0 && threadIdx.x == 0) row_start[nrows + 1] = 0;  // the crowded flag, set by k_row_scan
   const uint32_t r0 = blockIdx.x * RT_TILE;
   uint32_t a = 0, b = 0;
 #pragma unroll
@@ -577,21 +582,33 @@ static __global__ void __launch_bounds__(RT_THREADS) k_row_totals(const uint32_t
 static __global__ void __launch_bounds__(RT_THREADS) k_row_scan(const uint32_t* __restrict__ rcnt, uint32_t nrows,
                                                                 const uint32_t* __restrict__ btot,
                                                                 uint32_t* __restrict__ srow, uint32_t* __restrict__ mrow,
-                                                                uint32_t* __restrict__ row_start, size_t ms) {
+                                                                uint32_t* __restrict__ row_start,
+                                                                uint32_t* __restrict__ step, size_t ms) {
   __shared__ uint32_t sh[2][32];
   __shared__ uint32_t base[2];
   if (ms) {
     const size_t o = size_t(blockIdx.y) * ms;
     rcnt = moff(rcnt, o), btot = moff(btot, o), srow = moff(srow, o), mrow = moff(mrow, o);
-    row_start = moff(row_start, o);
+    row_start = moff(row_start, o), step = moff(step, o);
   }
+  if (step && blockIdx.x == 0 && threadIdx.x == 0) *step += 1u;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const uint32_t nb = gridDim.x;
   // totals of the earlier tiles
   uint32_t pa = 0, pb = 0;
-  for (uint32_t t = threadIdx.x; t < blockIdx.x; t += RT_THREADS) {
-    pa += __ldg(btot + t);
-    pb += __ldg(btot + nb + t);
+  if (btot) {
+    for (uint32_t t = threadIdx.x; t < blockIdx.x; t += RT_THREADS) {
+      pa += __ldg(btot + t);
+      pb += __ldg(btot + nb + t);
+    }
+  } else {  // (whole tiles before this one: multiples of four rows)
+    const uint4 *ra = reinterpret_cast<const uint4*>(rcnt), *rb = reinterpret_cast<const uint4*>(rcnt + nrows);
+#pragma unroll 4
+    for (uint32_t t = threadIdx.x; t < blockIdx.x * (RT_TILE / 4); t += RT_THREADS) {
+      const uint4 a = __ldg(ra + t), b = __ldg(rb + t);
+      pa += a.x + a.y + a.z + a.w;
+      pb += b.x + b.y + b.z + b.w;
+    }
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
@@ -701,13 +718,18 @@ __global__ void __launch_bounds__(PF_THREADS) k_place(
     const uint32_t* __restrict__ bv, const uint32_t* __restrict__ srow, const uint32_t* __restrict__ mrow,
     const uint32_t* __restrict__ row_start, const uint32_t* __restrict__ counts, uint32_t n, uint32_t n_mesh,
     int log2n, uint32_t* __restrict__ keys_out, const V4* __restrict__ pos_in, const V4* __restrict__ mom_in,
-    V4* __restrict__ pos_out, V4* __restrict__ mom_out, size_t ms) {
+    V4* __restrict__ pos_out, V4* __restrict__ mom_out, uint32_t* __restrict__ rcnt, uint32_t* __restrict__ tcount,
+    uint32_t ntiles, size_t ms) {
   if constexpr (PACKED) {
     const size_t o = size_t(blockIdx.y) * ms;
     sk = moff(sk, o), sv = moff(sv, o), bk = moff(bk, o), bv = moff(bv, o), srow = moff(srow, o);
     mrow = moff(mrow, o), row_start = moff(row_start, o), counts = moff(counts, o), keys_out = moff(keys_out, o);
     pos_in = moff(pos_in, o), mom_in = moff(mom_in, o), pos_out = moff(pos_out, o), mom_out = moff(mom_out, o);
+    rcnt = moff(rcnt, o), tcount = moff(tcount, o);
   }
+  // nothing reads the counts any more: zero for the next drift and re-sort
+  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < 3 * n_mesh * n_mesh; i += gridDim.x * blockDim.x) rcnt[i] = 0;
+  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < ntiles; i += gridDim.x * blockDim.x) tcount[i] = 0;
   const uint32_t ns = counts[0], nrows = n_mesh * n_mesh;
   for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
     const bool stayer = i < ns;
@@ -1040,25 +1062,27 @@ cudaError_t launch_sort_small(const uint32_t* keys_in, int64_t n, int key_bits, 
 // the three parts of the re-sort: the partition, the rows (scan and
 // buckets) and the placement
 template <typename V4>
-inline cudaError_t launch_resort_place(int part, const uint32_t* keys, int64_t n, const uint32_t* tcount, uint32_t* sk,
+inline cudaError_t launch_resort_place(int part, const uint32_t* keys, int64_t n, uint32_t* tcount, uint32_t* sk,
                                        uint32_t* sv, uint32_t* mk, uint32_t* mv, uint32_t* bk, uint32_t* bv,
                                        uint32_t* counts, uint32_t* rcnt, uint32_t* btot, uint32_t* srow, uint32_t* mrow,
-                                       uint32_t* row_start, Mesh m, unsigned long long* stats, uint32_t* keys_out,
-                                       const V4* pos_in, const V4* mom_in, V4* pos_out, V4* mom_out, int sms,
+                                       uint32_t* row_start, Mesh m, unsigned long long* stats, uint32_t* step,
+                                       uint32_t* keys_out, const V4* pos_in, const V4* mom_in, V4* pos_out, V4* mom_out, int sms,
                                        cudaStream_t s, int nm, size_t ms) {
   const size_t o = nm > 1 ? ms : 0;
   const uint32_t N = uint32_t(m.n), nrows = N * N;
+  const unsigned ntiles = unsigned((n + RS_TILE - 1) / RS_TILE);
   if (part == 0) {
-    const unsigned ntiles = unsigned((n + RS_TILE - 1) / RS_TILE);
     // up to PART_OWN_SCAN_TILES tiles each block sums the counts of the tiles before it
     const int own = ntiles <= PART_OWN_SCAN_TILES;
-    if (!own) k_tile_scan<<<dim3(1, unsigned(nm)), TS_THREADS, 0, s>>>(const_cast<uint32_t*>(tcount), ntiles, o);
+    if (!own) k_tile_scan<<<dim3(1, unsigned(nm)), TS_THREADS, 0, s>>>(tcount, ntiles, o);
     k_mover_partition<<<dim3(ntiles, unsigned(nm)), RS_THREADS, 0, s>>>(keys, n, tcount, sk, sv, mk, mv, counts, rcnt,
-                                                                       N, m.log2n, stats, own, o);
+                                                                       row_start, N, m.log2n, stats, own, o);
   } else if (part == 1) {
     const unsigned nb = (nrows + RT_TILE - 1) / RT_TILE;
-    k_row_totals<<<dim3(nb, unsigned(nm)), RT_THREADS, 0, s>>>(rcnt, nrows, btot, row_start, o);
-    k_row_scan<<<dim3(nb, unsigned(nm)), RT_THREADS, 0, s>>>(rcnt, nrows, btot, srow, mrow, row_start, o);
+    const bool direct = nb <= RT_DIRECT_TILES;
+    if (!direct) k_row_totals<<<dim3(nb, unsigned(nm)), RT_THREADS, 0, s>>>(rcnt, nrows, btot, o);
+    k_row_scan<<<dim3(nb, unsigned(nm)), RT_THREADS, 0, s>>>(rcnt, nrows, direct ? nullptr : btot, srow, mrow, row_start,
+                                                            step, o);
     // the bucket scatter runs over the device's mover count: a grid of resident blocks shared by the members
     int64_t cap = int64_t(16) * sms / nm;
     if (cap < 1) cap = 1;
@@ -1074,23 +1098,25 @@ inline cudaError_t launch_resort_place(int part, const uint32_t* keys, int64_t n
     const dim3 grid(unsigned(need < cap ? need : cap), unsigned(nm));
     if (nm > 1)
       k_place<V4, true><<<grid, PF_THREADS, 0, s>>>(sk, sv, bk, bv, srow, mrow, row_start, counts, uint32_t(n), N,
-                                                    m.log2n, keys_out, pos_in, mom_in, pos_out, mom_out, o);
+                                                    m.log2n, keys_out, pos_in, mom_in, pos_out, mom_out, rcnt, tcount,
+                                                    ntiles, o);
     else
       k_place<V4, false><<<grid, PF_THREADS, 0, s>>>(sk, sv, bk, bv, srow, mrow, row_start, counts, uint32_t(n), N,
-                                                     m.log2n, keys_out, pos_in, mom_in, pos_out, mom_out, 0);
+                                                     m.log2n, keys_out, pos_in, mom_in, pos_out, mom_out, rcnt, tcount,
+                                                     ntiles, 0);
   }
   return cudaGetLastError();
 }
 
 template <typename R>
-cudaError_t launch_resort(int part, const uint32_t* keys, int64_t n, const uint32_t* tcount, uint32_t* sk,
+cudaError_t launch_resort(int part, const uint32_t* keys, int64_t n, uint32_t* tcount, uint32_t* sk,
                           uint32_t* sv, uint32_t* mk, uint32_t* mv, uint32_t* bk, uint32_t* bv, uint32_t* counts,
                           uint32_t* rcnt, uint32_t* btot, uint32_t* srow, uint32_t* mrow, uint32_t* row_start, Mesh m,
-                          unsigned long long* stats, uint32_t* keys_out, const void* pos_in, const void* mom_in,
-                          void* pos_out, void* mom_out, int sms, cudaStream_t s, int nm, size_t ms) {
+                          unsigned long long* stats, uint32_t* step, uint32_t* keys_out, const void* pos_in,
+                          const void* mom_in, void* pos_out, void* mom_out, int sms, cudaStream_t s, int nm, size_t ms) {
   using V4 = typename VT<R>::v4;
   return launch_resort_place<V4>(part, keys, n, tcount, sk, sv, mk, mv, bk, bv, counts, rcnt, btot, srow, mrow,
-                                 row_start, m, stats, keys_out, (const V4*)pos_in, (const V4*)mom_in, (V4*)pos_out,
+                                 row_start, m, stats, step, keys_out, (const V4*)pos_in, (const V4*)mom_in, (V4*)pos_out,
                                  (V4*)mom_out, sms, s, nm, ms);
 }
 
