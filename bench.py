@@ -339,8 +339,9 @@ def measure(pm, sim, w, K, W, stream, rsz=4, spline=False, tuning=None, peak=Non
         avg = ms / cnt
         per_stage[name] = {"ms_per_step": ms / K, "launches": cnt, "avg_launch_ms": avg,
                            "bytes_per_launch": b, "GBps": (b / (avg / 1e3) / 1e9) if b else None}
-    # the transform stages are cuFFT's, except with the fused x-y kernels of 256^3 meshes (green_fused = 2)
-    own_xy = sim.get_tuning().get("green_fused") == 2
+    # the transform stages are cuFFT's, except with the fused x-y kernels of 256^3 meshes (green_fused = 2, and
+    # the fp32 spline runs on such meshes)
+    own_xy = sim.get_tuning().get("green_fused") == 2 or (spline and rsz == 4 and nm == 256)
     lib_stages = () if own_xy else pm.CUFFT_STAGES
     names = dict(KERNEL_NAMES, **({"fft_r2c": "k_xy_r2c", "fft_c2r": "k_xy_c2r"} if own_xy else {}))
     ours = {k: v for k, v in per_stage.items() if k not in lib_stages and v["GBps"] is not None}

@@ -214,7 +214,7 @@ Layout make_layout(const pm_config& c, size_t work_bytes) {
   // per-step kick weights of pm_run and of a batch run
   L.ktab = take(size_t(std::max(PM_RUN_GRAPH_MAX_STEPS, PM_BATCH_MAX_STEPS)) * sizeof(KickParams));
   // the z transform's twiddles and the Green's sin^2 table (fp32 cloud-in-cell, power-of-two meshes)
-  L.green = take(c.precision == PM_FP32 && !spline && spec_z_supported(int(N)) ? N * 12 : 0);
+  L.green = take(c.precision == PM_FP32 && (spline ? xy_fft_supported(int(N)) : spec_z_supported(int(N))) ? N * 12 : 0);
   L.sin2 = take(N * rsz);  // sin^2(pi j / N) for the flat Green passes
   L.total = off;
   return L;
@@ -547,6 +547,25 @@ void spline_taps(double hc, double* g) {
     for (int i = 0; i < 4; ++i) g[q * 4 + i] = f(i * i + q) / sum;
 }
 
+// fp32 spline simulations on meshes that the x-y kernels transform (256^3): the transforms of a field are the
+// x-y kernel, one pass along z with the symbol between the two transforms, and the x-y kernel back, instead
+// of cuFFT's 3D plans and separate spectral passes.  Per step (five transforms, green, smoothing) 448 us with
+// those, SPL_FIG so.
+bool spline_own_fft(const pm_sim* s) { return !s->fp64() && spline(s) && xy_fft_supported(s->cfg.n_mesh); }
+const float2* fft_twiddles(const pm_sim* s) { return s->at<float2>(s->L.green); }
+const float* fft_sin2(const pm_sim* s) { return s->at<float>(s->L.green + size_t(s->cfg.n_mesh) * 8); }
+
+pm_status own_xy_r2c(pm_sim* s, size_t in) {
+  PROF(s, PM_STAGE_FFT_R2C);
+  CU(s, launch_xy_r2c(s->at<float>(in), s->arena + s->L.spec, fft_twiddles(s), s->cfg.n_mesh, s->stream));
+  return PM_OK;
+}
+pm_status own_xy_c2r(pm_sim* s, size_t spec, size_t out) {
+  PROF(s, PM_STAGE_FFT_C2R);
+  CU(s, launch_xy_c2r(s->arena + spec, s->at<float>(out), fft_twiddles(s), s->cfg.n_mesh, s->stream));
+  return PM_OK;
+}
+
 // a mesh field convolved with the spline's node weights, from `in` to `out`
 // (the same offset for the spectral smoothing, which works in place)
 template <typename R>
@@ -555,6 +574,14 @@ pm_status smooth_field(pm_sim* s, size_t in, size_t out) {
     PROF(s, PM_STAGE_GREEN);
     CU(s, launch_smooth_direct<float>(s->at<float>(in), s->at<float>(out), s->mesh, s->taps, s->taps_r2, s->stream));
     return PM_OK;
+  }
+  if (spline_own_fft(s)) {
+    PMST(own_xy_r2c(s, in));
+    {
+      PROF(s, PM_STAGE_GREEN);
+      CU(s, launch_spec_z_smooth(s->arena + s->L.spec, s->arena + s->L.what, fft_twiddles(s), s->mesh, s->stream));
+    }
+    return own_xy_c2r(s, s->L.spec, out);
   }
   PMST(fft_r2c<R>(s, s->arena + in, s->arena + s->L.spec));
   {
@@ -702,6 +729,23 @@ pm_status mesh_from_density(pm_sim* s) {
 template <typename R>
 pm_status spline_fields(pm_sim* s) {
   const Layout& L = s->L;
+  if (spline_own_fft(s)) {
+    PMST(own_xy_r2c(s, L.rho));
+    {
+      PROF(s, PM_STAGE_GREEN);
+      CU(s, launch_spec_z_spline(s->arena + L.spec, s->direct ? nullptr : s->arena + L.spec2, s->arena + L.what,
+                                 fft_twiddles(s), fft_sin2(s), s->mesh, green_coef(s), wg_part(s), s->stream));
+    }
+    s->wg_count = spec_z_tiles(s->cfg.n_mesh);
+    if (s->direct)
+      PMST(smooth_field<R>(s, L.rho, L.spec2));
+    else
+      PMST(own_xy_c2r(s, L.spec2, L.rho));
+    PMST(own_xy_c2r(s, L.spec, L.phi));
+    PMST(quantum_stage<R>(s));
+    s->fields_valid = true;
+    return PM_OK;
+  }
   PMST(fft_r2c<R>(s, s->arena + L.rho, s->arena + L.spec));
   {
     PROF(s, PM_STAGE_GREEN);
@@ -1111,6 +1155,9 @@ pm_status pm_create(const pm_config* c, void* dev_arena, size_t bytes, void* str
     for (int r2 = 0; r2 <= 27; ++r2)
       if (sqrt(double(r2)) < c->smooth_h) s->taps_r2 = r2;
     pm_status st = DISPATCH(s, spline_symbol, s);
+    if (st == PM_OK && spline_own_fft(s) &&
+        launch_spec_tables(s->at<float2>(s->L.green), s->at<float>(s->L.green + size_t(N) * 8), N, s->stream) != cudaSuccess)
+      st = fail(s, PM_ERR_CUDA, "transform tables");
     if (st == PM_OK && cudaStreamSynchronize(s->stream) != cudaSuccess) st = PM_ERR_CUDA;
     if (st != PM_OK) {
       const std::string msg = s->err;

@@ -869,14 +869,18 @@ static __global__ void k_spec_tables(float2* tw, float* s2, int n) {
   }
 }
 
-// z transform, phi^ = G rho^ (with k_green's arithmetic and Parseval partial
-// of W_g), inverse z transform, over 16 columns of the flattened (ky, kx)
-// half plane per block; N = P Q, P >= Q, 16 P threads.  coefp (packed
-// groups): the coefficient in device memory, member blockIdx.y, ms bytes apart.
-template <int P, int Q, bool PACKED>
-__global__ void __launch_bounds__(SPZ_COLS * P, SPZ_COLS * P <= 256 ? PM_SPZ_MINB : 1) k_spec_z(float2* __restrict__ spec, const float2* __restrict__ twg,
-                                                         const float* __restrict__ s2g, float coef, double* part,
-                                                         const double* coefp, size_t ms) {
+// z transform, a multiplication, inverse z transform, over 16 columns of the flattened (ky, kx) half plane
+// per block; N = P Q, P >= Q, 16 P threads.  OP: SPZ_GREEN: phi^ = G rho^ (with k_green's arithmetic and
+// Parseval partial of W_g); SPZ_SPLINE (k_green_spline): the force potential W^2 G rho^ in place and, if spec2
+// is given, the smoothed density W rho^ / N^3 there, both from one forward transform; SPZ_SMOOTH: W / N^3 in
+// place (k_smooth_spec).  coefp (packed groups): the coefficient in device memory, member blockIdx.y, ms
+// bytes apart.
+constexpr int SPZ_GREEN = 0, SPZ_SPLINE = 1, SPZ_SMOOTH = 2;
+template <int P, int Q, bool PACKED, int OP = SPZ_GREEN>
+__global__ void __launch_bounds__(SPZ_COLS * P, SPZ_COLS * P > 256 ? 1 : (OP == SPZ_SPLINE ? 3 : PM_SPZ_MINB))
+    k_spec_z(float2* __restrict__ spec, const float2* __restrict__ twg, const float* __restrict__ s2g, float coef,
+             double* part, const double* coefp, size_t ms, float2* __restrict__ spec2, const float* __restrict__ what,
+             float inv_n3) {
   constexpr int N = P * Q, T = SPZ_COLS * P;
   constexpr uint32_t NH = N / 2 + 1, PLANE = uint32_t(N) * NH;
   if constexpr (PACKED) {
@@ -898,7 +902,7 @@ __global__ void __launch_bounds__(SPZ_COLS * P, SPZ_COLS * P <= 256 ? PM_SPZ_MIN
   }
   for (int i = tid; i < N; i += T) {
     tw[i] = twg[i];
-    s2[i] = s2g[i];
+    if (OP != SPZ_SMOOTH) s2[i] = s2g[i];
   }
   cp_async_wait_all();
   __syncthreads();
@@ -914,49 +918,87 @@ __global__ void __launch_bounds__(SPZ_COLS * P, SPZ_COLS * P <= 256 ? PM_SPZ_MIN
   }
   __syncthreads();
   float wsum = 0.0f;
-  if (jt < Q) {  // thread k1: P-point DFT over j, Green, inverse P-point DFT, conjugate twiddle
-    const int k1 = jt;
-    float2 b[P];
-#pragma unroll
-    for (int j = 0; j < P; ++j) b[j] = tile[(j + P * k1) * SPZ_COLS + c];
-    dft_reg<P, false>(b);
-    const uint32_t col = col0 + uint32_t(c), ky = col / NH, kx = col - ky * NH;
-    const float sx = s2[kx], sy = s2[ky];
-    const float w = (kx == 0 || kx == N / 2) ? 1.0f : 2.0f;
-    float2 d[P];
-#pragma unroll
-    for (int k2 = 0; k2 < P; ++k2) {
-      const int kz = k1 + Q * k2;
-      float2 v = b[bitrev<P>(k2)];
-      const float syz = sy + s2[kz];
-      const float sum = syz + sx;
-      const float g = (ky == 0 && kz == 0 && kx == 0) ? 0.0f : coef * __frcp_rn(sum);
-      wsum += w * g * (v.x * v.x + v.y * v.y);
-      d[k2] = make_float2(v.x * g, v.y * g);
-    }
+  // thread k1 = jt < Q from here: inverse P-point DFT over k2, conjugate twiddle
+  auto inverse_first = [&](float2 (&d)[P]) {
     dft_reg<P, true>(d);
 #pragma unroll
     for (int j = 0; j < P; ++j) {
-      const float2 t = tw[(j * k1) & (N - 1)];
-      tile[(j + P * k1) * SPZ_COLS + c] = cmul(d[bitrev<P>(j)], make_float2(t.x, -t.y));
+      const float2 t = tw[(j * jt) & (N - 1)];
+      tile[(j + P * jt) * SPZ_COLS + c] = cmul(d[bitrev<P>(j)], make_float2(t.x, -t.y));
     }
-  }
-  __syncthreads();
-  {  // inverse, second step: thread j, inverse Q-point DFT over k1
+  };
+  // inverse, second step: thread j, inverse Q-point DFT over k1, and the tile to memory
+  auto inverse_second = [&](float2* __restrict__ out) {
+    __syncthreads();
     float2 e[Q];
 #pragma unroll
     for (int k1 = 0; k1 < Q; ++k1) e[k1] = tile[(jt + P * k1) * SPZ_COLS + c];
     dft_reg<Q, true>(e);
 #pragma unroll
     for (int mm = 0; mm < Q; ++mm) tile[(jt + P * mm) * SPZ_COLS + c] = e[bitrev<Q>(mm)];
+    __syncthreads();
+    for (int i = tid; i < N * 8; i += T) {
+      const int r = i >> 3, q = i & 7;
+      reinterpret_cast<float4*>(out + size_t(r) * PLANE + col0)[q] = reinterpret_cast<const float4*>(tile + r * SPZ_COLS)[q];
+    }
+  };
+  float2 keep[OP == SPZ_SPLINE ? P : 1];  // W rho^, while the tile carries the potential
+  if (jt < Q) {  // thread k1: P-point DFT over j, the multiplication
+    const int k1 = jt;
+    float2 b[P];
+#pragma unroll
+    for (int j = 0; j < P; ++j) b[j] = tile[(j + P * k1) * SPZ_COLS + c];
+    dft_reg<P, false>(b);
+    const uint32_t col = col0 + uint32_t(c), ky = col / NH, kx = col - ky * NH;
+    float2 d[P];
+    if constexpr (OP == SPZ_SMOOTH) {
+#pragma unroll
+      for (int k2 = 0; k2 < P; ++k2) {
+        const float f = __ldg(what + size_t(k1 + Q * k2) * PLANE + col) * inv_n3;
+        const float2 v = b[bitrev<P>(k2)];
+        d[k2] = make_float2(v.x * f, v.y * f);
+      }
+    } else {
+      const float sx = s2[kx], sy = s2[ky];
+      const float w = (kx == 0 || kx == N / 2) ? 1.0f : 2.0f;
+#pragma unroll
+      for (int k2 = 0; k2 < P; ++k2) {
+        const int kz = k1 + Q * k2;
+        float2 v = b[bitrev<P>(k2)];
+        const float syz = sy + s2[kz];
+        const float sum = syz + sx;
+        float g = (ky == 0 && kz == 0 && kx == 0) ? 0.0f : coef * __frcp_rn(sum);
+        if constexpr (OP == SPZ_SPLINE) {
+          const float wk = __ldg(what + size_t(kz) * PLANE + col);
+          v.x *= wk, v.y *= wk;
+          keep[k2] = v;
+          wsum += w * g * (v.x * v.x + v.y * v.y);
+          g *= wk;
+        } else {
+          wsum += w * g * (v.x * v.x + v.y * v.y);
+        }
+        d[k2] = make_float2(v.x * g, v.y * g);
+      }
+    }
+    inverse_first(d);
   }
-  __syncthreads();
-  for (int i = tid; i < N * 8; i += T) {
-    const int r = i >> 3, q = i & 7;
-    reinterpret_cast<float4*>(spec + size_t(r) * PLANE + col0)[q] = reinterpret_cast<const float4*>(tile + r * SPZ_COLS)[q];
+  inverse_second(spec);
+  if constexpr (OP == SPZ_SPLINE) {
+    if (spec2) {
+      __syncthreads();
+      if (jt < Q) {
+        float2 d[P];
+#pragma unroll
+        for (int k2 = 0; k2 < P; ++k2) d[k2] = make_float2(keep[k2].x * inv_n3, keep[k2].y * inv_n3);
+        inverse_first(d);
+      }
+      inverse_second(spec2);
+    }
   }
-  float acc[1] = {wsum};
-  block_sum_store<1>(acc, part, gridDim.x);
+  if constexpr (OP != SPZ_SMOOTH) {
+    float acc[1] = {wsum};
+    block_sum_store<1>(acc, part, gridDim.x);
+  }
 }
 
 // ---------------------------------------------------------------- cubic spline kernel
@@ -2360,9 +2402,10 @@ cudaError_t launch_spec_z_pq(float2* spec, const float2* tw, const float* s2, do
   const unsigned tiles = unsigned(N * (N / 2 + 1) / SPZ_COLS);
   if (nm > 1)
     k_spec_z<P, Q, true><<<dim3(tiles, unsigned(nm)), SPZ_COLS * P, smem, s>>>(spec, tw, s2, float(coef), part, coefp,
-                                                                             ms);
+                                                                             ms, nullptr, nullptr, 0.0f);
   else
-    k_spec_z<P, Q, false><<<tiles, SPZ_COLS * P, smem, s>>>(spec, tw, s2, float(coef), part, nullptr, 0);
+    k_spec_z<P, Q, false><<<tiles, SPZ_COLS * P, smem, s>>>(spec, tw, s2, float(coef), part, nullptr, 0, nullptr, nullptr,
+                                                            0.0f);
   return cudaGetLastError();
 }
 

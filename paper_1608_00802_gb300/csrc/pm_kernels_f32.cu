@@ -126,4 +126,25 @@ cudaError_t launch_spec_z(void* spec, const float2* tw, const float* s2, Mesh m,
   }
 }
 
+cudaError_t launch_spec_z_spline(void* spec, void* spec2, const void* what, const float2* tw, const float* s2, Mesh m,
+                                 double coef, double* part, cudaStream_t s) {
+  if (!xy_fft_supported(m.n)) return cudaErrorInvalidValue;
+  constexpr int N = 256;
+  const size_t smem = size_t(N) * (SPZ_COLS * sizeof(float2) + sizeof(float2) + sizeof(float));
+  k_spec_z<16, 16, false, SPZ_SPLINE><<<spec_z_tiles(N), SPZ_COLS * 16, smem, s>>>(
+      static_cast<float2*>(spec), tw, s2, float(coef), part, nullptr, 0, static_cast<float2*>(spec2),
+      static_cast<const float*>(what), float(1.0 / double(m.n3)));
+  return cudaGetLastError();
+}
+
+cudaError_t launch_spec_z_smooth(void* spec, const void* what, const float2* tw, Mesh m, cudaStream_t s) {
+  if (!xy_fft_supported(m.n)) return cudaErrorInvalidValue;
+  constexpr int N = 256;
+  const size_t smem = size_t(N) * (SPZ_COLS * sizeof(float2) + sizeof(float2) + sizeof(float));
+  k_spec_z<16, 16, false, SPZ_SMOOTH><<<spec_z_tiles(N), SPZ_COLS * 16, smem, s>>>(
+      static_cast<float2*>(spec), tw, nullptr, 0.0f, nullptr, nullptr, 0, nullptr, static_cast<const float*>(what),
+      float(1.0 / double(m.n3)));
+  return cudaGetLastError();
+}
+
 }  // namespace pm
