@@ -367,9 +367,9 @@ def measure(pm, sim, w, K, W, stream, rsz=4, spline=False, tuning=None, peak=Non
                      "note": ("no library kernels on the path (the transforms are the fused x-y kernels)" if own_xy
                               else "cuFFT time taken from the profiled pass; peak as in roofline")}
     # our kernels per timed region: the profiled pass launches the same kernels one by one (the "sort_pass"
-    # record covers the row scan, the bucket scatter and, beyond 16 tiles of 1024 rows, the row totals; the
+    # record covers the row scan, the bucket scatter and, beyond 8 tiles of 1024 rows, the row totals; the
     # partition adds a tile scan beyond 2048 tiles of 2048 particles; the fp64 stencil is two kernels)
-    per_record = {"sort_pass": 2 + int(nm * nm > 16 * 1024), "sort_partition": 1 + int((n + 2047) // 2048 > 2048),
+    per_record = {"sort_pass": 2 + int(nm * nm > 8 * 1024), "sort_partition": 1 + int((n + 2047) // 2048 > 2048),
                   "stencil": 1 + int(rsz == 8)}
     launches = sum(v["launches"] * per_record.get(k, 1) for k, v in per_stage.items() if k not in lib_stages)
     return {"value": n * K / (t_ms / 1e3), "t_ms": t_ms, "ms_per_step": t_step, "stages": per_stage,

@@ -579,7 +579,8 @@ pm_status smooth_field(pm_sim* s, size_t in, size_t out) {
     PMST(own_xy_r2c(s, in));
     {
       PROF(s, PM_STAGE_GREEN);
-      CU(s, launch_spec_z_smooth(s->arena + s->L.spec, s->arena + s->L.what, fft_twiddles(s), s->mesh, s->stream));
+      CU(s, launch_spec_z_smooth(s->arena + s->L.spec, s->arena + s->L.spec, s->arena + s->L.what, fft_twiddles(s),
+                                 s->mesh, s->stream));
     }
     return own_xy_c2r(s, s->L.spec, out);
   }
@@ -733,8 +734,11 @@ pm_status spline_fields(pm_sim* s) {
     PMST(own_xy_r2c(s, L.rho));
     {
       PROF(s, PM_STAGE_GREEN);
-      CU(s, launch_spec_z_spline(s->arena + L.spec, s->direct ? nullptr : s->arena + L.spec2, s->arena + L.what,
-                                 fft_twiddles(s), fft_sin2(s), s->mesh, green_coef(s), wg_part(s), s->stream));
+      if (!s->direct)
+        CU(s, launch_spec_z_smooth(s->arena + L.spec, s->arena + L.spec2, s->arena + L.what, fft_twiddles(s), s->mesh,
+                                   s->stream));
+      CU(s, launch_spec_z_spline(s->arena + L.spec, s->arena + L.what, fft_twiddles(s), fft_sin2(s), s->mesh,
+                                 green_coef(s), wg_part(s), s->stream));
     }
     s->wg_count = spec_z_tiles(s->cfg.n_mesh);
     if (s->direct)
@@ -1085,7 +1089,7 @@ pm_status pm_create(const pm_config* c, void* dev_arena, size_t bytes, void* str
   s->keys_tmp[0] = s->at<uint32_t>(L.keys[1]);
   s->keys_tmp[1] = s->at<uint32_t>(L.keys[2]);
   s->have_particles = s->sorted = s->fields_valid = false;
-  s->tune = default_tuning(N);
+  s->tune = default_tuning(N, c->n_part);
   {
     int dev = 0, sm = 0;
     if (cudaGetDevice(&dev) == cudaSuccess &&

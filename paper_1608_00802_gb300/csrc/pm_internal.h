@@ -90,11 +90,11 @@ cudaError_t launch_spec_tables(float2* tw, float* s2, int n, cudaStream_t s);
 cudaError_t launch_spec_z(void* spec, const float2* tw, const float* s2, Mesh m, double coef, double* part,
                           cudaStream_t s, const double* coefp = nullptr, int nm = 1, size_t ms = 0);
 
-// the same for the spline kernel on meshes whose planes the x-y kernels transform: W^2 G in place and (spec2
-// given) W / N^3 there; or W / N^3 in place.  what: the symbol W over the half spectrum
-cudaError_t launch_spec_z_spline(void* spec, void* spec2, const void* what, const float2* tw, const float* s2, Mesh m,
-                                 double coef, double* part, cudaStream_t s);
-cudaError_t launch_spec_z_smooth(void* spec, const void* what, const float2* tw, Mesh m, cudaStream_t s);
+// the same for the spline kernel on meshes whose planes the x-y kernels transform: W^2 G in place; or W / N^3
+// from spec to out (which may be spec).  what: the symbol W over the half spectrum
+cudaError_t launch_spec_z_spline(void* spec, const void* what, const float2* tw, const float* s2, Mesh m, double coef,
+                                 double* part, cudaStream_t s);
+cudaError_t launch_spec_z_smooth(void* spec, void* out, const void* what, const float2* tw, Mesh m, cudaStream_t s);
 
 // error bits of the device error word
 enum : uint32_t { ERR_NONFINITE = 1u, ERR_TIMEOUT = 2u };
@@ -229,7 +229,7 @@ size_t stencil_list_entries(int n);
 int stencil_launch_blocks(int n, int ty, int zlen);
 int stencil_max_blocks(int n);
 bool stencil_shape_ok(int n, int ty, int zlen, int stages);
-Tuning default_tuning(int n);
+Tuning default_tuning(int n, int64_t n_part);
 // sizes the fp32 streaming kick's grid for this device (an occupancy query;
 // call outside any stream capture, before the first kick)
 void kick_stream_prepare();

@@ -505,8 +505,8 @@ __device__ __forceinline__ void deposit_crowded_row(const typename VT<R>::v4* __
   __syncthreads();  // the row is cleared for the next
 }
 
-// helper block hb of H: its share of the destination rows (every H-th, so that neighbouring rows, crowded
-// together, go to different blocks), of which it computes those of crowded tiles
+// helper block hb of H, when the row starts' flag says that a row is crowded: its share of the destination
+// rows (every H-th), of which it computes those of crowded tiles
 template <typename R, int TY, int TZ>
 __device__ __noinline__ void deposit_crowded(const typename VT<R>::v4* __restrict__ pos,
                                              const uint32_t* __restrict__ row_start, uint32_t np, const Mesh m, R norm,
@@ -871,15 +871,16 @@ static __global__ void k_spec_tables(float2* tw, float* s2, int n) {
 
 // z transform, a multiplication, inverse z transform, over 16 columns of the flattened (ky, kx) half plane
 // per block; N = P Q, P >= Q, 16 P threads.  OP: SPZ_GREEN: phi^ = G rho^ (with k_green's arithmetic and
-// Parseval partial of W_g); SPZ_SPLINE (k_green_spline): the force potential W^2 G rho^ in place and, if spec2
-// is given, the smoothed density W rho^ / N^3 there, both from one forward transform; SPZ_SMOOTH: W / N^3 in
-// place (k_smooth_spec).  coefp (packed groups): the coefficient in device memory, member blockIdx.y, ms
-// bytes apart.
+// Parseval partial of W_g); SPZ_SPLINE: the force potential W^2 G rho^ (k_green_spline); SPZ_SMOOTH: W / N^3
+// (k_smooth_spec), to `out` if given.  Otherwise in place.  The spline step needs both from one spectrum:
+// two launches, 72 us, against 92 us for one that kept the transform in registers for a second inverse (80
+// registers, three blocks per SM).  coefp (packed groups): the coefficient in device memory, member
+// blockIdx.y, ms bytes apart.
 constexpr int SPZ_GREEN = 0, SPZ_SPLINE = 1, SPZ_SMOOTH = 2;
 template <int P, int Q, bool PACKED, int OP = SPZ_GREEN>
-__global__ void __launch_bounds__(SPZ_COLS * P, SPZ_COLS * P > 256 ? 1 : (OP == SPZ_SPLINE ? 3 : PM_SPZ_MINB))
-    k_spec_z(float2* __restrict__ spec, const float2* __restrict__ twg, const float* __restrict__ s2g, float coef,
-             double* part, const double* coefp, size_t ms, float2* __restrict__ spec2, const float* __restrict__ what,
+__global__ void __launch_bounds__(SPZ_COLS * P, SPZ_COLS * P > 256 ? 1 : PM_SPZ_MINB)
+    k_spec_z(float2* spec, const float2* __restrict__ twg, const float* __restrict__ s2g, float coef, double* part,
+             const double* coefp, size_t ms, float2* out, const float* __restrict__ what,
              float inv_n3) {
   constexpr int N = P * Q, T = SPZ_COLS * P;
   constexpr uint32_t NH = N / 2 + 1, PLANE = uint32_t(N) * NH;
@@ -892,6 +893,7 @@ __global__ void __launch_bounds__(SPZ_COLS * P, SPZ_COLS * P > 256 ? 1 : (OP == 
   float2* tile = reinterpret_cast<float2*>(spz_smem);  // [z][16 columns]
   float2* tw = tile + N * SPZ_COLS;
   float* s2 = reinterpret_cast<float*>(tw + N);
+  float* wt = s2 + N;  // the symbol's tile [z][16 columns] (not SPZ_GREEN)
   const int tid = threadIdx.x;
   const uint32_t col0 = blockIdx.x * SPZ_COLS;
   // the tile by asynchronous 16-byte copies: every copy of a thread in flight at once
@@ -899,6 +901,13 @@ __global__ void __launch_bounds__(SPZ_COLS * P, SPZ_COLS * P > 256 ? 1 : (OP == 
     const int r = i >> 3, q = i & 7;
     cp_async16(reinterpret_cast<float4*>(tile + r * SPZ_COLS) + q,
                reinterpret_cast<const float4*>(spec + size_t(r) * PLANE + col0) + q);
+  }
+  if constexpr (OP != SPZ_GREEN) {
+    for (int i = tid; i < N * 4; i += T) {
+      const int r = i >> 2, q = i & 3;
+      cp_async16(reinterpret_cast<float4*>(wt + r * SPZ_COLS) + q,
+                 reinterpret_cast<const float4*>(what + size_t(r) * PLANE + col0) + q);
+    }
   }
   for (int i = tid; i < N; i += T) {
     tw[i] = twg[i];
@@ -918,31 +927,6 @@ __global__ void __launch_bounds__(SPZ_COLS * P, SPZ_COLS * P > 256 ? 1 : (OP == 
   }
   __syncthreads();
   float wsum = 0.0f;
-  // thread k1 = jt < Q from here: inverse P-point DFT over k2, conjugate twiddle
-  auto inverse_first = [&](float2 (&d)[P]) {
-    dft_reg<P, true>(d);
-#pragma unroll
-    for (int j = 0; j < P; ++j) {
-      const float2 t = tw[(j * jt) & (N - 1)];
-      tile[(j + P * jt) * SPZ_COLS + c] = cmul(d[bitrev<P>(j)], make_float2(t.x, -t.y));
-    }
-  };
-  // inverse, second step: thread j, inverse Q-point DFT over k1, and the tile to memory
-  auto inverse_second = [&](float2* __restrict__ out) {
-    __syncthreads();
-    float2 e[Q];
-#pragma unroll
-    for (int k1 = 0; k1 < Q; ++k1) e[k1] = tile[(jt + P * k1) * SPZ_COLS + c];
-    dft_reg<Q, true>(e);
-#pragma unroll
-    for (int mm = 0; mm < Q; ++mm) tile[(jt + P * mm) * SPZ_COLS + c] = e[bitrev<Q>(mm)];
-    __syncthreads();
-    for (int i = tid; i < N * 8; i += T) {
-      const int r = i >> 3, q = i & 7;
-      reinterpret_cast<float4*>(out + size_t(r) * PLANE + col0)[q] = reinterpret_cast<const float4*>(tile + r * SPZ_COLS)[q];
-    }
-  };
-  float2 keep[OP == SPZ_SPLINE ? P : 1];  // W rho^, while the tile carries the potential
   if (jt < Q) {  // thread k1: P-point DFT over j, the multiplication
     const int k1 = jt;
     float2 b[P];
@@ -954,7 +938,7 @@ __global__ void __launch_bounds__(SPZ_COLS * P, SPZ_COLS * P > 256 ? 1 : (OP == 
     if constexpr (OP == SPZ_SMOOTH) {
 #pragma unroll
       for (int k2 = 0; k2 < P; ++k2) {
-        const float f = __ldg(what + size_t(k1 + Q * k2) * PLANE + col) * inv_n3;
+        const float f = wt[(k1 + Q * k2) * SPZ_COLS + c] * inv_n3;
         const float2 v = b[bitrev<P>(k2)];
         d[k2] = make_float2(v.x * f, v.y * f);
       }
@@ -969,9 +953,8 @@ __global__ void __launch_bounds__(SPZ_COLS * P, SPZ_COLS * P > 256 ? 1 : (OP == 
         const float sum = syz + sx;
         float g = (ky == 0 && kz == 0 && kx == 0) ? 0.0f : coef * __frcp_rn(sum);
         if constexpr (OP == SPZ_SPLINE) {
-          const float wk = __ldg(what + size_t(kz) * PLANE + col);
+          const float wk = wt[kz * SPZ_COLS + c];
           v.x *= wk, v.y *= wk;
-          keep[k2] = v;
           wsum += w * g * (v.x * v.x + v.y * v.y);
           g *= wk;
         } else {
@@ -980,20 +963,28 @@ __global__ void __launch_bounds__(SPZ_COLS * P, SPZ_COLS * P > 256 ? 1 : (OP == 
         d[k2] = make_float2(v.x * g, v.y * g);
       }
     }
-    inverse_first(d);
-  }
-  inverse_second(spec);
-  if constexpr (OP == SPZ_SPLINE) {
-    if (spec2) {
-      __syncthreads();
-      if (jt < Q) {
-        float2 d[P];
+    // inverse P-point DFT over k2, conjugate twiddle
+    dft_reg<P, true>(d);
 #pragma unroll
-        for (int k2 = 0; k2 < P; ++k2) d[k2] = make_float2(keep[k2].x * inv_n3, keep[k2].y * inv_n3);
-        inverse_first(d);
-      }
-      inverse_second(spec2);
+    for (int j = 0; j < P; ++j) {
+      const float2 t = tw[(j * k1) & (N - 1)];
+      tile[(j + P * k1) * SPZ_COLS + c] = cmul(d[bitrev<P>(j)], make_float2(t.x, -t.y));
     }
+  }
+  __syncthreads();
+  {  // inverse, second step: thread j, inverse Q-point DFT over k1
+    float2 e[Q];
+#pragma unroll
+    for (int k1 = 0; k1 < Q; ++k1) e[k1] = tile[(jt + P * k1) * SPZ_COLS + c];
+    dft_reg<Q, true>(e);
+#pragma unroll
+    for (int mm = 0; mm < Q; ++mm) tile[(jt + P * mm) * SPZ_COLS + c] = e[bitrev<Q>(mm)];
+  }
+  __syncthreads();
+  float2* dst = OP == SPZ_SMOOTH && out ? out : spec;
+  for (int i = tid; i < N * 8; i += T) {
+    const int r = i >> 3, q = i & 7;
+    reinterpret_cast<float4*>(dst + size_t(r) * PLANE + col0)[q] = reinterpret_cast<const float4*>(tile + r * SPZ_COLS)[q];
   }
   if constexpr (OP != SPZ_SMOOTH) {
     float acc[1] = {wsum};
@@ -2243,7 +2234,7 @@ cudaError_t launch_init_particles(const double* x, const double* p, int64_t n, M
 // fp32 mesh; measured there: 43 us against 53 us for 2 x 4 rows, whose 8.3 KB per warp leave
 // too few resident warps)
 #ifndef PM_DEP_HELPERS
-#define PM_DEP_HELPERS 304
+#define PM_DEP_HELPERS 608
 #endif
 #ifndef PM_DEPOSIT_WARP_BYTES
 #define PM_DEPOSIT_WARP_BYTES 4352
@@ -2264,13 +2255,16 @@ cudaError_t launch_deposit_tile(const void* pos, const uint32_t* row_start, int6
                                 cudaStream_t s, int warps, int nm, size_t ms) {
   using V4 = typename VT<R>::v4;
   // helper blocks for crowded tiles (none with so few particles): at most PM_DEP_HELPERS of 8 warps in all,
-  // and no fewer than 16 rows each
+  // and no fewer than 16 rows each.  A helper takes every helpers-th row, and rows crowd together, so their
+  // number is q N + 0.382 N: a block's rows then lie far apart in y from plane to plane (a core of 10^6
+  // particles on 128^3: the longest share is one row's, 1.0 .. 1.1 of it over meshes of 64 .. 160; with
+  // 2 N + 1 blocks it is 7 of them, 800 us instead of 87)
   unsigned helpers = 0;
   size_t smem = size_t(warps) * TY * TZ * deposit_stride_of<R>(m.n) * sizeof(R);
   if (n > int64_t(DEP_CROWD)) {
-    const unsigned most = unsigned(PM_DEP_HELPERS * DEP_WARPS / (warps * nm)), rows = m.n2 / 16 + 1;
-    helpers = most < rows ? most : rows;
-    if (helpers < 8) helpers = 8;
+    const unsigned most = std::max(8u, std::min(unsigned(PM_DEP_HELPERS * DEP_WARPS / (warps * nm)), m.n2 / 16 + 1));
+    const unsigned N = unsigned(m.n), part = unsigned(0.382 * m.n);
+    helpers = most >= N + part ? (most - part) / N * N + part : most;
     smem = std::max(smem, deposit_crowd_smem<R>(m.n));
   }
   const unsigned tiles_y = unsigned((m.n + warps * TY - 1) / (warps * TY));

@@ -46,10 +46,17 @@ bool stencil_shape_ok(int n, int ty, int zlen, int stages) {
   return stages == 0 ? stencil_tile_shape_ok(n, ty, zlen) : stencil_bulk_shape_ok(n, ty, zlen, stages);
 }
 
-Tuning default_tuning(int n) {
+Tuning default_tuning(int n, int64_t n_part) {
   Tuning t;
-  t.kick_threads = KICK_THREADS;
+  // few particles: twice the blocks of half the threads while 256 would leave SMs idle
+  t.kick_threads = n_part < int64_t(KICK_THREADS) * 2 * 152 ? 128 : KICK_THREADS;
+  // small meshes: fewer warps per deposit block while the tiles would leave SMs idle (512 tiles of 2 x 4 rows on
+  // 64^3: 64 blocks of 8 warps 7.0 us, fp64 17.9; 256 of 2 warps 6.8 and 14.1 us)
+  int ty = 1, tz = 1;
+  deposit_shape<float>(n, ty, tz);
+  const int tiles = ((n + ty - 1) / ty) * ((n + tz - 1) / tz);
   t.dep_warps = 8;
+  while (t.dep_warps > 2 && tiles / t.dep_warps < 152) t.dep_warps /= 2;
   t.green_fused = 0;
   // one-shot tiles of 4 rows x 4 planes where they fit (the multiple-of-4 meshes up to 1024)
   if (stencil_tile_shape_ok(n, 4, 4)) {
@@ -126,24 +133,45 @@ cudaError_t launch_spec_z(void* spec, const float2* tw, const float* s2, Mesh m,
   }
 }
 
-cudaError_t launch_spec_z_spline(void* spec, void* spec2, const void* what, const float2* tw, const float* s2, Mesh m,
-                                 double coef, double* part, cudaStream_t s) {
+// shared memory of the z kernel with the symbol's tile, and its opt-in, once per device
+static size_t spec_z_symbol_smem(int n) {
+  return size_t(n) * (SPZ_COLS * (sizeof(float2) + sizeof(float)) + sizeof(float2) + sizeof(float));
+}
+static cudaError_t spec_z_symbol_prepare() {
+  static bool done[64];
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess || (dev >= 0 && dev < 64 && done[dev])) return e;
+  const int most = int(spec_z_symbol_smem(256));
+  e = cudaFuncSetAttribute(k_spec_z<16, 16, false, SPZ_SPLINE>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(k_spec_z<16, 16, false, SPZ_SMOOTH>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+  if (e == cudaSuccess && dev >= 0 && dev < 64) done[dev] = true;
+  return e;
+}
+
+cudaError_t launch_spec_z_spline(void* spec, const void* what, const float2* tw, const float* s2, Mesh m, double coef,
+                                 double* part, cudaStream_t s) {
   if (!xy_fft_supported(m.n)) return cudaErrorInvalidValue;
   constexpr int N = 256;
-  const size_t smem = size_t(N) * (SPZ_COLS * sizeof(float2) + sizeof(float2) + sizeof(float));
+  const size_t smem = spec_z_symbol_smem(N);
+  cudaError_t e = spec_z_symbol_prepare();
+  if (e != cudaSuccess) return e;
   k_spec_z<16, 16, false, SPZ_SPLINE><<<spec_z_tiles(N), SPZ_COLS * 16, smem, s>>>(
-      static_cast<float2*>(spec), tw, s2, float(coef), part, nullptr, 0, static_cast<float2*>(spec2),
-      static_cast<const float*>(what), float(1.0 / double(m.n3)));
+      static_cast<float2*>(spec), tw, s2, float(coef), part, nullptr, 0, nullptr, static_cast<const float*>(what),
+      0.0f);
   return cudaGetLastError();
 }
 
-cudaError_t launch_spec_z_smooth(void* spec, const void* what, const float2* tw, Mesh m, cudaStream_t s) {
+cudaError_t launch_spec_z_smooth(void* spec, void* out, const void* what, const float2* tw, Mesh m, cudaStream_t s) {
   if (!xy_fft_supported(m.n)) return cudaErrorInvalidValue;
   constexpr int N = 256;
-  const size_t smem = size_t(N) * (SPZ_COLS * sizeof(float2) + sizeof(float2) + sizeof(float));
+  const size_t smem = spec_z_symbol_smem(N);
+  cudaError_t e = spec_z_symbol_prepare();
+  if (e != cudaSuccess) return e;
   k_spec_z<16, 16, false, SPZ_SMOOTH><<<spec_z_tiles(N), SPZ_COLS * 16, smem, s>>>(
-      static_cast<float2*>(spec), tw, nullptr, 0.0f, nullptr, nullptr, 0, nullptr, static_cast<const float*>(what),
-      float(1.0 / double(m.n3)));
+      static_cast<float2*>(spec), tw, nullptr, 0.0f, nullptr, nullptr, 0, static_cast<float2*>(out),
+      static_cast<const float*>(what), float(1.0 / double(m.n3)));
   return cudaGetLastError();
 }
 

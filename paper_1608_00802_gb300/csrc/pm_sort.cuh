@@ -538,11 +538,11 @@ static __global__ void __launch_bounds__(RS_THREADS) k_mover_partition(
 // earlier tiles' totals and scans its own, writing srow (stayers before row
 // r), mrow (movers before row r) and the new row starts row_start = srow +
 // mrow, with the closing entries at r = N^2.  With few tiles (up to
-// RT_DIRECT_TILES: meshes up to 128^2 rows) k_row_scan sums the earlier tiles'
-// rows itself (btot null), which costs less than a launch; at 256^2 rows that
-// took 25 us against 17 for the two kernels and the buckets.  step (nullable): the device step counter, which
-// a captured step advances here.
-constexpr uint32_t RT_DIRECT_TILES = 16;
+// RT_DIRECT_TILES: meshes up to 90^2 rows) k_row_scan sums the earlier tiles'
+// rows itself (btot null), which costs less than a launch: 3.7 us for 4 tiles
+// (64^2 rows) against 2.5 + 1.4 and the gap, but 7.7 us for 16 (128^2).  step
+// (nullable): the device step counter, which a captured step advances here.
+constexpr uint32_t RT_DIRECT_TILES = 8;
 
 static __global__ void __launch_bounds__(RT_THREADS) k_row_totals(const uint32_t* __restrict__ rcnt, uint32_t nrows,
                                                                   uint32_t* __restrict__ btot, size_t ms) {
