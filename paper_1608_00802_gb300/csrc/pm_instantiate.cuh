@@ -7,8 +7,8 @@
                                                 uint32_t*, uint32_t*, cudaStream_t);                              \
   template cudaError_t launch_sort_pass<R>(bool, const uint32_t*, const uint32_t*, int64_t, int, int,             \
                                            const uint32_t*, uint64_t*, uint32_t*, const uint32_t*, int, int,       \
-                                           uint32_t*, uint32_t*, const void*, const void*, void*, void*,           \
-                                           uint32_t*, cudaStream_t, const uint32_t*, int, size_t, int);           \
+                                           uint32_t*, uint32_t*, const void*, const void*, const double*, void*,   \
+                                           void*, uint32_t*, cudaStream_t, const uint32_t*, int, size_t, int);           \
   template cudaError_t launch_sort_small<R>(const uint32_t*, int64_t, int, uint32_t*, const void*, const void*,   \
                                             void*, void*, uint32_t*, Mesh, uint32_t*, cudaStream_t);              \
   template cudaError_t launch_deposit<R>(const void*, const uint32_t*, int64_t, Mesh, double, R*, cudaStream_t,    \

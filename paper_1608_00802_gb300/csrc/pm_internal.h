@@ -145,8 +145,8 @@ template <typename R>
 cudaError_t launch_sort_pass(bool last, const uint32_t* keys_in, const uint32_t* vals_in, int64_t n, int shift,
                              int bits, const uint32_t* digit_total, uint64_t* status, uint32_t* tile_counter,
                              const uint32_t* epoch, int pass, int ntiles, uint32_t* keys_out, uint32_t* vals_out,
-                             const void* pos_in, const void* mom_in, void* pos_out, void* mom_out, uint32_t* err,
-                             cudaStream_t s, const uint32_t* n_dev = nullptr, int nm = 1, size_t ms = 0,
+                             const void* pos_in, const void* mom_in, const double* p_in, void* pos_out, void* mom_out,
+                             uint32_t* err, cudaStream_t s, const uint32_t* n_dev = nullptr, int nm = 1, size_t ms = 0,
                              int spin_limit = 0);  // polls of a look-back wait before it gives up (0: default)
 // the full sort of up to SORT_SMALL_MAX particles in one kernel (records gathered, row starts and the
 // crowded-row flag written; keys_out may be keys_in); mom_in null: no momenta; clear (nullable): a word set to 0

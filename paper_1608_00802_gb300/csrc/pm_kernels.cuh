@@ -297,7 +297,7 @@ __global__ void k_init_particles(const double* __restrict__ x, const double* __r
   }
   uint32_t cell = (uint32_t(c[2]) * uint32_t(m.n) + uint32_t(c[1])) * uint32_t(m.n) + uint32_t(c[0]);
   pos[i] = make_pos(cell, f[0], f[1], f[2]);
-  // p null: positions only (the allocation-free deposit needs no momenta)
+  // p null: positions only (the allocation-free deposit needs no momenta; a large load reads them later)
   if (p) mom[i] = make_mom(R(p[3 * i]), R(p[3 * i + 1]), R(p[3 * i + 2]), uint32_t(i));
   keys[i] = cell;
 }

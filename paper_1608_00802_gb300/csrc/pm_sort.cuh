@@ -132,14 +132,25 @@ static __global__ void __launch_bounds__(RS_THREADS) k_sort_histogram(const uint
     if (sh[i]) atomicAdd(hist + (i / radix) * (1 << RS_MAX_BITS) + (i % radix), sh[i]);
 }
 
+// the momentum record of input particle i from the caller's momenta p (the input index is the id)
+template <typename V4>
+__device__ __forceinline__ V4 loaded_momentum(const double* __restrict__ p, uint32_t i) {
+  const size_t j = 3 * size_t(i);
+  if constexpr (sizeof(V4) == 16)
+    return make_mom(float(__ldg(p + j)), float(__ldg(p + j + 1)), float(__ldg(p + j + 2)), i);
+  else
+    return make_mom(__ldg(p + j), __ldg(p + j + 1), __ldg(p + j + 2), i);
+}
+
+// p_in (last pass; nullable): the momenta come from the caller's array instead of mom_in
 template <bool LAST, typename V4>
 __global__ void __launch_bounds__(RS_THREADS) k_sort_pass(
     const uint32_t* __restrict__ keys_in, const uint32_t* __restrict__ vals_in, int64_t n, int shift, int bits,
     const uint32_t* __restrict__ digit_total, uint64_t* status, uint32_t* tile_counter,
     const uint32_t* __restrict__ epoch_base, int pass,
     uint32_t* __restrict__ keys_out, uint32_t* __restrict__ vals_out, const V4* __restrict__ pos_in,
-    const V4* __restrict__ mom_in, V4* __restrict__ pos_out, V4* __restrict__ mom_out, uint32_t* err,
-    const uint32_t* __restrict__ n_dev, size_t ms, int spin_limit) {
+    const V4* __restrict__ mom_in, const double* __restrict__ p_in, V4* __restrict__ pos_out, V4* __restrict__ mom_out,
+    uint32_t* err, const uint32_t* __restrict__ n_dev, size_t ms, int spin_limit) {
   extern __shared__ uint32_t smem[];
   if (ms) {  // member blockIdx.y of a packed group (the passes over its movers)
     const size_t o = size_t(blockIdx.y) * ms;
@@ -311,7 +322,7 @@ __global__ void __launch_bounds__(RS_THREADS) k_sort_pass(
       if (LAST) {
         const uint32_t src = s_vals[li];
         pos_out[dest] = pos_in[src];
-        mom_out[dest] = mom_in[src];
+        mom_out[dest] = p_in ? loaded_momentum<V4>(p_in, src) : mom_in[src];
       } else {
         vals_out[dest] = s_vals[li];
       }
@@ -1124,8 +1135,8 @@ template <typename R>
 cudaError_t launch_sort_pass(bool last, const uint32_t* keys_in, const uint32_t* vals_in, int64_t n, int shift,
                              int bits, const uint32_t* digit_total, uint64_t* status, uint32_t* tile_counter,
                              const uint32_t* epoch, int pass, int ntiles, uint32_t* keys_out, uint32_t* vals_out,
-                             const void* pos_in, const void* mom_in, void* pos_out, void* mom_out, uint32_t* err,
-                             cudaStream_t s, const uint32_t* n_dev, int nm, size_t ms, int spin_limit) {
+                             const void* pos_in, const void* mom_in, const double* p_in, void* pos_out, void* mom_out,
+                             uint32_t* err, cudaStream_t s, const uint32_t* n_dev, int nm, size_t ms, int spin_limit) {
   if (spin_limit < 1) spin_limit = RS_SPIN_LIMIT;
   using V4 = typename VT<R>::v4;
   if (nm > 1 && (last || !n_dev)) return cudaErrorInvalidValue;  // packed groups: mover passes only
@@ -1150,12 +1161,13 @@ cudaError_t launch_sort_pass(bool last, const uint32_t* keys_in, const uint32_t*
   if (last) {
     k_sort_pass<true, V4><<<grid, RS_THREADS, smem, s>>>(keys_in, vals_in, n, shift, bits, digit_total, status,
                                                          tile_counter, epoch, pass, keys_out, vals_out,
-                                                         (const V4*)pos_in, (const V4*)mom_in, (V4*)pos_out,
+                                                         (const V4*)pos_in, (const V4*)mom_in, p_in, (V4*)pos_out,
                                                          (V4*)mom_out, err, n_dev, o, spin_limit);
   } else {
     k_sort_pass<false, V4><<<grid, RS_THREADS, smem, s>>>(keys_in, vals_in, n, shift, bits, digit_total, status,
                                                           tile_counter, epoch, pass, keys_out, vals_out, nullptr,
-                                                          nullptr, nullptr, nullptr, err, n_dev, o, spin_limit);
+                                                          nullptr, nullptr, nullptr, nullptr, err, n_dev, o,
+                                                          spin_limit);
   }
   return cudaGetLastError();
 }
