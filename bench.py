@@ -341,9 +341,13 @@ def measure(pm, sim, w, K, W, stream, rsz=4, spline=False, tuning=None, peak=Non
                            "bytes_per_launch": b, "GBps": (b / (avg / 1e3) / 1e9) if b else None}
     # the transform stages are cuFFT's, except with the fused x-y kernels of 256^3 meshes (green_fused = 2, and
     # the fp32 spline runs on such meshes)
+    # and, pass by pass, of 384^3 and (green_fused = 1) 512^3 meshes
     own_xy = sim.get_tuning().get("green_fused") == 2 or (spline and rsz == 4 and nm == 256)
-    lib_stages = () if own_xy else pm.CUFFT_STAGES
-    names = dict(KERNEL_NAMES, **({"fft_r2c": "k_xy_r2c", "fft_c2r": "k_xy_c2r"} if own_xy else {}))
+    own_passes = rsz == 4 and not spline and (nm == 384 or (nm == 512 and sim.get_tuning().get("green_fused") == 1))
+    lib_stages = () if own_xy or own_passes else pm.CUFFT_STAGES
+    names = dict(KERNEL_NAMES, **({"fft_r2c": "k_xy_r2c", "fft_c2r": "k_xy_c2r"} if own_xy else
+                                  {"fft_r2c": "k_x_r2c+k_y_forward", "green": "k_z_green",
+                                   "fft_c2r": "k_y_inverse+k_x_c2r"} if own_passes else {}))
     ours = {k: v for k, v in per_stage.items() if k not in lib_stages and v["GBps"] is not None}
     dom = max(ours, key=lambda k: ours[k]["ms_per_step"])
     d = per_stage[dom]
@@ -364,13 +368,13 @@ def measure(pm, sim, w, K, W, stream, rsz=4, spline=False, tuning=None, peak=Non
                      "frac": step_bytes / (t_step / 1e3) / 1e9 / peak,
                      "frac_excl_cufft": ((step_bytes - step_bytes_fft) / (max(t_step - fft_ms, 1e-9) / 1e3) / 1e9
                                          / peak),
-                     "note": ("no library kernels on the path (the transforms are the fused x-y kernels)" if own_xy
+                     "note": ("no library kernels on the path (the transforms are its own kernels)" if own_xy or own_passes
                               else "cuFFT time taken from the profiled pass; peak as in roofline")}
     # our kernels per timed region: the profiled pass launches the same kernels one by one (the "sort_pass"
     # record covers the row scan, the bucket scatter and, beyond 8 tiles of 1024 rows, the row totals; the
     # partition adds a tile scan beyond 2048 tiles of 2048 particles; the fp64 stencil is two kernels)
     per_record = {"sort_pass": 2 + int(nm * nm > 8 * 1024), "sort_partition": 1 + int((n + 2047) // 2048 > 2048),
-                  "stencil": 1 + int(rsz == 8)}
+                  "stencil": 1 + int(rsz == 8), "fft_r2c": 1 + int(own_passes), "fft_c2r": 1 + int(own_passes)}
     launches = sum(v["launches"] * per_record.get(k, 1) for k, v in per_stage.items() if k not in lib_stages)
     return {"value": n * K / (t_ms / 1e3), "t_ms": t_ms, "ms_per_step": t_step, "stages": per_stage,
             "roofline": roofline, "step_roofline": step_roofline, "launches": launches,

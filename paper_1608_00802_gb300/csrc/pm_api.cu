@@ -208,13 +208,15 @@ Layout make_layout(const pm_config& c, size_t work_bytes) {
   L.st_count = take(size_t(stencil_max_blocks(int(N))) * 4);
   size_t aux = std::max<size_t>(MESH_GRID, size_t(stencil_max_blocks(int(N))));
   if (spec_z_supported(int(N))) aux = std::max<size_t>(aux, size_t(spec_z_tiles(int(N))));
+  if (pass_fft_supported(int(N))) aux = std::max<size_t>(aux, size_t(pass_fft_tiles(int(N))));
   L.part_aux = take(2 * aux * 8);
   L.red = take(3 * PK_MAX_BINS * 8 + 64);
   L.err = take(256);
   // per-step kick weights of pm_run and of a batch run
   L.ktab = take(size_t(std::max(PM_RUN_GRAPH_MAX_STEPS, PM_BATCH_MAX_STEPS)) * sizeof(KickParams));
   // the z transform's twiddles and the Green's sin^2 table (fp32 cloud-in-cell, power-of-two meshes)
-  L.green = take(c.precision == PM_FP32 && (spline ? xy_fft_supported(int(N)) : spec_z_supported(int(N))) ? N * 12 : 0);
+  L.green = take(c.precision == PM_FP32 && (spline ? xy_fft_supported(int(N)) : (spec_z_supported(int(N)) || pass_fft_supported(int(N))))
+                     ? N * 12 : 0);
   L.sin2 = take(N * rsz);  // sin^2(pi j / N) for the flat Green passes
   L.total = off;
   return L;
@@ -374,6 +376,7 @@ size_t aux_len(const pm_sim* s) {
   const int N = s->cfg.n_mesh;
   size_t aux = std::max<size_t>(MESH_GRID, size_t(stencil_max_blocks(N)));
   if (spec_z_supported(N)) aux = std::max<size_t>(aux, size_t(spec_z_tiles(N)));
+  if (pass_fft_supported(N)) aux = std::max<size_t>(aux, size_t(pass_fft_tiles(N)));
   return aux;
 }
 double* kr_part(pm_sim* s) { return wg_part(s) + aux_len(s); }
@@ -602,6 +605,13 @@ double green_coef(const pm_sim* s) {
   return -1.5 * s->cfg.omega_m * s->dx * s->dx / (4.0 * N * N * N);
 }
 
+// fp32 cloud-in-cell on 384^3 and 512^3: the transforms pass by pass.  On 512^3 they are the plane transforms of
+// green_fused = 1 (0: cuFFT's 3D transforms); 384^3, no power of two, has no such choice and always takes them
+bool pass_fft(const pm_sim* s) {
+  return !s->fp64() && s->cfg.kernel == PM_KERNEL_CIC && pass_fft_supported(s->cfg.n_mesh) &&
+         (!spec_z_supported(s->cfg.n_mesh) || s->tune.green_fused == 1);
+}
+
 // the Green multiplication inside the z transform, between batched 2D transforms
 bool green_fused(const pm_sim* s) { return s->tune.green_fused && s->have_plan2; }
 
@@ -686,6 +696,18 @@ pm_status krho_stage(pm_sim* s) {
 template <typename R>
 pm_status mesh_from_density(pm_sim* s) {
   const Layout& L = s->L;
+  if (pass_fft(s)) {
+    const int N = s->cfg.n_mesh, stages[3] = {PM_STAGE_FFT_R2C, PM_STAGE_GREEN, PM_STAGE_FFT_C2R};
+    for (int k = 0; k < 3; ++k) {
+      PROF(s, stages[k]);
+      CU(s, launch_pass_fft(k, s->at<float>(L.rho), s->at<float>(L.phi), s->arena + L.spec, s->at<float2>(L.green),
+                            s->at<float>(L.green + size_t(N) * 8), N, green_coef(s), wg_part(s), s->stream));
+    }
+    s->wg_count = pass_fft_tiles(N);
+    PMST(quantum_stage<R>(s));
+    s->fields_valid = true;
+    return PM_OK;
+  }
   if (green_fused(s)) {  // 2D transforms of the planes; z transforms and Green in one pass between them
     const int N = s->cfg.n_mesh;
     {
@@ -1156,6 +1178,14 @@ pm_status pm_create(const pm_config* c, void* dev_arena, size_t bytes, void* str
   if (c->precision == PM_FP32 && c->kernel == PM_KERNEL_CIC && spec_z_supported(N) && N >= GREEN_FUSE_MIN_MESH) {
     std::string ignored;
     if (spec_plan_setup(s, &ignored) == CUFFT_SUCCESS) s->tune.green_fused = xy_fft_supported(N) ? 2 : 1;
+  }
+  if (c->precision == PM_FP32 && c->kernel == PM_KERNEL_CIC && pass_fft_supported(N) && !spec_z_supported(N) &&
+      (launch_spec_tables(s->at<float2>(L.green), s->at<float>(L.green + size_t(N) * 8), N, s->stream) != cudaSuccess ||
+       cudaStreamSynchronize(s->stream) != cudaSuccess)) {
+    cufftDestroy(s->plan_fwd);
+    cufftDestroy(s->plan_inv);
+    delete s;
+    return fail(nullptr, PM_ERR_CUDA, "transform tables failed");
   }
   if (s->cfg.kernel == PM_KERNEL_SPLINE) {
     s->direct = c->smooth_real != 0;
@@ -1981,7 +2011,7 @@ bool same_state(const pm_batch::Class& C, const std::vector<pm_sim*>& sims) {
         s->tune.green_fused != a->tune.green_fused)
       return false;
   }
-  if (!green_fused(a) && !C.fwd) return false;  // the class's batched 3D transforms were not planned
+  if (!green_fused(a) && !pass_fft(a) && !C.fwd) return false;  // the class's batched 3D transforms were not planned
   const StencilParams sp = stencil_params(a, false);
   return !a->cfg.quantum || (a->tune.st_ty > 0 && a->tune.st_stages == 0 && stencil_shape_ok(a->cfg.n_mesh, sp.ty, sp.zlen, 0));
 }
@@ -2021,8 +2051,17 @@ pm_status packed_step(pm_batch::Class& C, const std::vector<pm_sim*>& sims, cuda
   // deposit, potential, quantum pressure
   PCU(launch_deposit<float>(s->arena + L.pos[nxt], s->at<uint32_t>(L.row_start), n, s->mesh, s->norm,
                             s->at<float>(L.rho), st, s->tune.dep_warps, nm, ms));
-  const bool fused = green_fused(s);
+  const bool passes = pass_fft(s);  // each member's own transforms, pass by pass (the same as alone)
+  const bool fused = green_fused(s) && !passes;
   const bool own_xy = fused && s->tune.green_fused == 2;
+  if (passes) {
+    for (int i : C.members) {
+      pm_sim* m = sims[i];
+      for (int k = 0; k < 3; ++k)
+        PCU(launch_pass_fft(k, m->at<float>(L.rho), m->at<float>(L.phi), m->arena + L.spec, m->at<float2>(L.green),
+                            m->at<float>(L.green + size_t(N) * 8), N, green_coef(m), wg_part(m), st));
+    }
+  }
   if (own_xy)  // the x-y transforms of every member's planes in one launch
     PCU(launch_xy_r2c(s->at<float>(L.rho), s->arena + L.spec, s->at<float2>(L.green), N, st, nm, ms));
   if (fused && !own_xy) {  // each member's own 2D transforms (the same as alone)
@@ -2048,7 +2087,7 @@ pm_status packed_step(pm_batch::Class& C, const std::vector<pm_sim*>& sims, cuda
       CF(s, r);
     }
   }
-  if (!fused) {
+  if (!fused && !passes) {
     CF(s, cufftSetStream(C.fwd, st));
     CF(s, cufftSetStream(C.inv, st));
     CF(s, cufftExecR2C(C.fwd, s->at<cufftReal>(L.rho), (cufftComplex*)(s->arena + L.spec)));
@@ -2067,7 +2106,7 @@ pm_status packed_step(pm_batch::Class& C, const std::vector<pm_sim*>& sims, cuda
     m->sorted = true;
     m->fields_valid = true;
     m->krho_valid = false;
-    m->wg_count = fused ? spec_z_tiles(N) : int(green_blocks(N));
+    m->wg_count = passes ? pass_fft_tiles(N) : (fused ? spec_z_tiles(N) : int(green_blocks(N)));
   }
   return PM_OK;
 }
@@ -2140,7 +2179,7 @@ pm_status pm_batch_create(const pm_config* cfgs, int32_t n, void* dev_arena, siz
       b->classes.push_back(C);
       return cleanup(PM_ERR_CUDA, "class stream creation failed");
     }
-    if (C.packed && !green_fused(b->sims[C.members[0]])) {  // fused members transform with their own 2D plans
+    if (C.packed && !green_fused(b->sims[C.members[0]]) && !pass_fft(b->sims[C.members[0]])) {  // fused members transform with their own 2D plans
       size_t w = 0;
       const pm_config& c = cfgs[C.members[0]];
       if (class_plans(c, int(C.members.size()), C.stride, &C.fwd, &C.inv, &w) != CUFFT_SUCCESS || w > BC.work ||

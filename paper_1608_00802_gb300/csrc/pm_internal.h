@@ -174,6 +174,13 @@ cudaError_t launch_resort(int part, const uint32_t* keys, int64_t n, uint32_t* t
                           const void* mom_in, void* pos_out, void* mom_out, int sms, cudaStream_t s, int nm = 1,
                           size_t ms = 0);
 inline size_t row_scan_tiles(int n_mesh) { return (size_t(n_mesh) * n_mesh + 1023) / 1024; }  // tiles of 1024 rows
+// phi~ from the density on 384^3 and 512^3 fp32 meshes, transform by transform: stage 0 the x and y transforms
+// (through phi, as scratch), 1 the z transforms with the Green multiplication (one W_g partial per tile), 2 the
+// inverse y and x transforms.  tw, s2: the tables of launch_spec_tables
+bool pass_fft_supported(int n);
+int pass_fft_tiles(int n);
+cudaError_t launch_pass_fft(int stage, const float* rho, float* phi, void* spec, const float2* tw, const float* s2, int n,
+                            double coef, double* part, cudaStream_t s);
 // the x-y transforms of the z-planes of a 256^3 fp32 mesh, one kernel per direction (unnormalised,
 // the layouts of the batched 2D R2C / C2R); tw: exp(-2 pi i t / 256), t < 256
 bool xy_fft_supported(int n_mesh);

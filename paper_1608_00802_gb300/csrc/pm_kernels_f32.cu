@@ -101,7 +101,7 @@ bool spec_z_supported(int n) { return n >= 16 && n <= 512 && (n & (n - 1)) == 0;
 int spec_z_tiles(int n) { return n * (n / 2 + 1) / SPZ_COLS; }
 
 cudaError_t launch_spec_tables(float2* tw, float* s2, int n, cudaStream_t s) {
-  if (!spec_z_supported(n)) return cudaErrorInvalidValue;
+  if (!spec_z_supported(n) && !pass_fft_supported(n)) return cudaErrorInvalidValue;
   // the 512-point blocks take 70 KB of shared memory (set once, outside any stream capture)
   static bool done[64];
   int dev = 0;

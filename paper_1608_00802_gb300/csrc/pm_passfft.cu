@@ -1,0 +1,370 @@
+// The mesh transforms of 384^3 and 512^3 fp32 meshes as five passes over memory (cloud-in-cell; other sizes
+// have the x-y kernels or cuFFT):
+//   x  forward : each row of N reals -> N/2 complex, X[0] + i X[N/2] packed first  (rho -> tmp)
+//   y  forward : 8 columns of a z-plane per block, the packed column split          (tmp -> spectrum)
+//   z          : 8 columns of the half spectrum per block, Green multiplication, W_g partial, back (in place)
+//   y  inverse : the columns packed again                                           (spectrum -> tmp)
+//   x  inverse : each row back to N reals                                           (tmp, in place)
+// tmp is the potential's mesh: N/2 complex values are a row of it.  A plane of these meshes (0.6 and 1 MB)
+// does not fit the cluster that the 256^2 x-y kernels use, and cuFFT's passes are far from the copy rate: on a
+// 384^3 mesh 906 us for its 3D pair plus 81 for the Green pass (a pass over memory takes 68 us), on 512^3
+// 996 us for its 2D pair plus 504 for the four-step z kernel at one block of 128 registers per SM (160 us a
+// pass).  So each pass here does as little as it can per value and leaves room for many threads: the five
+// passes take 570 us on 384^3 and 1270 us on 512^3.  The potential's error against float64 (particle
+// density, of the largest |phi|): 384^3 4.2e-6 -> 6.1e-7 (the Green table folds its index), 512^3 4.7e-7 ->
+// 4.1e-7.
+//
+// Rows: 16 threads a row (two rows a warp: the exchanges need no block barrier), H = N/2 = 16 Q points in two
+// steps, n = j + 16 m and k = k1 + Q k2: thread j a Q-point DFT over m (Q = 12, 16) and the twiddle, thread
+// k1 < Q a 16-point DFT over j.  Columns: N = 8 * 8 * C points in three steps (C = 6, 8), n = j + 8 C m,
+// j = j' + C m', k = k1 + 8 (k2 + 8 k3): thread j an 8-point DFT over m and W_N^{j k1}, thread (k1, j') an
+// 8-point DFT over m' and W_{8C}^{j' k2}, thread (k1, k2) a C-point DFT over j'; eight values and ~40
+// registers a thread.  Slots of the exchange tile are padded by one in C, so that the third step's stride of
+// C slots does not meet one bank group.  Inverses run the same steps backwards with conjugate twiddles.
+#include "pm_kernels.cuh"
+
+namespace pm {
+namespace {
+
+// exp(-+2 pi i t / 12) times a (forward: minus), t < 8 known at compile time after unrolling
+template <bool INV>
+__device__ __forceinline__ float2 twiddle12(float2 a, int t) {
+  constexpr float s60 = 0.866025388f;  // sin(pi / 3)
+  constexpr float c[7] = {1.0f, s60, 0.5f, 0.0f, -0.5f, -s60, -1.0f}, s[7] = {0.0f, 0.5f, s60, 1.0f, s60, 0.5f, 0.0f};
+  if (t == 0) return a;
+  if (t == 3) return INV ? make_float2(-a.y, a.x) : make_float2(a.y, -a.x);
+  return cmul(a, make_float2(c[t], INV ? s[t] : -s[t]));
+}
+
+// M-point DFT in registers: dft_reg for powers of two, one radix-3 step before it for M = 3 L; natural order
+// in, X[k] at a[dft_at<M>(k)]
+template <int M>
+__host__ __device__ constexpr int dft_at(int k) {
+  return M % 3 ? bitrev<M>(k) : (M / 3) * (k % 3) + bitrev<M / 3>(k / 3);
+}
+template <int M, bool INV>
+__device__ __forceinline__ void dft_any(float2 (&a)[M]) {
+  if constexpr (M % 3) {
+    dft_reg<M, INV>(a);
+  } else {
+    constexpr int L = M / 3;
+    constexpr float s60 = INV ? 0.866025388f : -0.866025388f;
+#pragma unroll
+    for (int j = 0; j < L; ++j) {
+      const float2 u = a[j], v = a[j + L], w = a[j + 2 * L];
+      const float2 p = make_float2(v.x + w.x, v.y + w.y), d = make_float2(v.x - w.x, v.y - w.y);
+      const float2 h = make_float2(fmaf(-0.5f, p.x, u.x), fmaf(-0.5f, p.y, u.y));
+      a[j] = make_float2(u.x + p.x, u.y + p.y);
+      a[j + L] = twiddle12<INV>(make_float2(fmaf(-s60, d.y, h.x), fmaf(s60, d.x, h.y)), j * (4 / L));
+      a[j + 2 * L] = twiddle12<INV>(make_float2(fmaf(s60, d.y, h.x), fmaf(-s60, d.x, h.y)), 2 * j * (4 / L));
+    }
+#pragma unroll
+    for (int r = 0; r < 3; ++r) {
+      float2 b[L];
+#pragma unroll
+      for (int j = 0; j < L; ++j) b[j] = a[L * r + j];
+      dft_reg<L, INV>(b);
+#pragma unroll
+      for (int j = 0; j < L; ++j) a[L * r + j] = b[j];
+    }
+  }
+}
+
+__device__ __forceinline__ float2 conj2(float2 a) { return make_float2(a.x, -a.y); }
+
+// ---------------------------------------------------------------- rows
+constexpr int PX_ROWS = 16, PX_THREADS = PX_ROWS * 16;
+template <int N>
+struct RowShape {
+  static constexpr int H = N / 2, Q = H / 16, ROW = H + H / 16 + 1;  // padded row of complex values
+};
+__device__ __forceinline__ int px_pad(int n) { return n + (n >> 4); }
+
+template <int N>
+__global__ void __launch_bounds__(PX_THREADS, 4) k_x_r2c(const float* __restrict__ in, float2* __restrict__ out,
+                                                         const float2* __restrict__ tw) {
+  constexpr int H = RowShape<N>::H, Q = RowShape<N>::Q, ROW = RowShape<N>::ROW;
+  __shared__ float2 S[PX_ROWS * ROW];
+  const int j = threadIdx.x & 15;
+  const uint32_t row = blockIdx.x * PX_ROWS + (threadIdx.x >> 4);  // (N^2 rows: a multiple of PX_ROWS)
+  const float2* src = reinterpret_cast<const float2*>(in) + size_t(row) * H;
+  float2* s = S + (threadIdx.x >> 4) * ROW;
+  {
+    float2 a[Q];
+#pragma unroll
+    for (int m = 0; m < Q; ++m) a[m] = __ldcs(src + j + 16 * m);
+    dft_any<Q, false>(a);
+#pragma unroll
+    for (int k1 = 0; k1 < Q; ++k1) s[px_pad(j + 16 * k1)] = cmul(a[dft_at<Q>(k1)], __ldg(tw + 2 * j * k1));
+  }
+  __syncwarp();
+  float2 b[16];
+  if (j < Q) {
+#pragma unroll
+    for (int i = 0; i < 16; ++i) b[i] = s[px_pad(i + 16 * j)];
+    dft_reg<16, false>(b);
+  }
+  __syncwarp();
+  if (j < Q) {
+#pragma unroll
+    for (int k2 = 0; k2 < 16; ++k2) s[px_pad(j + Q * k2)] = b[bitrev<16>(k2)];
+  }
+  __syncwarp();
+  // X[k] = E + W^k O from Z[k] and Z[H - k]; X[0] and X[H], both real, packed
+  float2* dst = out + size_t(row) * H;
+#pragma unroll
+  for (int i = 0; i < Q; ++i) {
+    const int k = j + 16 * i;
+    const float2 z = s[px_pad(k)], zp = s[px_pad(k ? H - k : 0)];
+    const float ex = 0.5f * (z.x + zp.x), ey = 0.5f * (z.y - zp.y), ox = 0.5f * (z.y + zp.y), oy = -0.5f * (z.x - zp.x);
+    const float2 wo = cmul(make_float2(ox, oy), __ldg(tw + k));
+    dst[k] = k ? make_float2(ex + wo.x, ey + wo.y) : make_float2(ex + ox, ex - ox);
+  }
+}
+
+// in place: a row's values are read before any of them is written (__syncwarp between them)
+template <int N>
+__global__ void __launch_bounds__(PX_THREADS, 4) k_x_c2r(float2* mesh, const float2* __restrict__ tw) {
+  constexpr int H = RowShape<N>::H, Q = RowShape<N>::Q, ROW = RowShape<N>::ROW;
+  __shared__ float2 S[PX_ROWS * ROW];
+  const int j = threadIdx.x & 15;
+  const uint32_t row = blockIdx.x * PX_ROWS + (threadIdx.x >> 4);
+  float2* io = mesh + size_t(row) * H;
+  float2* s = S + (threadIdx.x >> 4) * ROW;
+  float2 x[Q];
+#pragma unroll
+  for (int m = 0; m < Q; ++m) x[m] = __ldcs(io + j + 16 * m);
+#pragma unroll
+  for (int m = 0; m < Q; ++m) s[px_pad(j + 16 * m)] = x[m];
+  __syncwarp();
+  // Z[k] = (X[k] + X*[H-k]) + i W^-k (X[k] - X*[H-k]); k = 0 from the packed value
+#pragma unroll
+  for (int m = 0; m < Q; ++m) {
+    const int k = j + 16 * m;
+    const float2 xp = s[px_pad(k ? H - k : 0)];
+    const float2 d = cmul(make_float2(x[m].x - xp.x, x[m].y + xp.y), conj2(__ldg(tw + k)));
+    x[m] = k ? make_float2(x[m].x + xp.x - d.y, x[m].y - xp.y + d.x) : make_float2(x[m].x + x[m].y, x[m].x - x[m].y);
+  }
+  dft_any<Q, true>(x);
+  __syncwarp();
+#pragma unroll
+  for (int k1 = 0; k1 < Q; ++k1) s[px_pad(j + 16 * k1)] = cmul(x[dft_at<Q>(k1)], conj2(__ldg(tw + 2 * j * k1)));
+  __syncwarp();
+  if (j < Q) {
+    float2 b[16];
+#pragma unroll
+    for (int i = 0; i < 16; ++i) b[i] = s[px_pad(i + 16 * j)];
+    dft_reg<16, true>(b);
+#pragma unroll
+    for (int k2 = 0; k2 < 16; ++k2) io[j + Q * k2] = b[bitrev<16>(k2)];  // (x[2n], x[2n + 1]), n = k1 + Q k2
+  }
+}
+
+// ---------------------------------------------------------------- columns
+constexpr int PC_COLS = 8;
+template <int N>
+struct ColShape {
+  static constexpr int C = N / 64, BC = 8 * C, THREADS = PC_COLS * BC, MINB = 1536 / THREADS;
+  static constexpr int SLOTS = N + N / C;  // padded by one slot in C
+  static constexpr size_t smem() { return size_t(SLOTS) * PC_COLS * sizeof(float2); }
+};
+template <int N>
+__device__ __forceinline__ int pc_slot(int s) {
+  return (s + s / ColShape<N>::C) * PC_COLS;
+}
+
+// the first two steps of a column's transform from its values a[m] = x[j + BC m] (thread (c, j)): the tile
+// T holds the values of the third step
+template <int N>
+__device__ __forceinline__ void cols_forward(float2 (&a)[8], float2* T, const float2* __restrict__ tw, int c, int j) {
+  constexpr int C = ColShape<N>::C, BC = ColShape<N>::BC;
+  dft_reg<8, false>(a);
+#pragma unroll
+  for (int k1 = 0; k1 < 8; ++k1) T[pc_slot<N>(k1 * BC + j) + c] = cmul(a[bitrev<8>(k1)], __ldg(tw + j * k1));
+  __syncthreads();
+  const int k1 = j / C, jp = j - k1 * C;
+#pragma unroll
+  for (int m = 0; m < 8; ++m) a[m] = T[pc_slot<N>(k1 * BC + jp + C * m) + c];
+  dft_reg<8, false>(a);
+#pragma unroll
+  for (int k2 = 0; k2 < 8; ++k2) T[pc_slot<N>(k1 * BC + k2 * C + jp) + c] = cmul(a[bitrev<8>(k2)], __ldg(tw + 8 * jp * k2));
+  __syncthreads();
+}
+// the last two steps of the inverse, from the tile that the first one filled: a[dft_at(m)] = x[j + BC m]
+template <int N>
+__device__ __forceinline__ void cols_inverse(float2 (&a)[8], float2* T, const float2* __restrict__ tw, int c, int j) {
+  constexpr int C = ColShape<N>::C, BC = ColShape<N>::BC;
+  __syncthreads();
+  const int k1 = j / C, jp = j - k1 * C;
+#pragma unroll
+  for (int k2 = 0; k2 < 8; ++k2) a[k2] = T[pc_slot<N>(k1 * BC + k2 * C + jp) + c];
+  dft_reg<8, true>(a);
+#pragma unroll
+  for (int m = 0; m < 8; ++m)
+    T[pc_slot<N>(k1 * BC + jp + C * m) + c] = cmul(a[bitrev<8>(m)], conj2(__ldg(tw + (jp + C * m) * k1)));
+  __syncthreads();
+#pragma unroll
+  for (int i = 0; i < 8; ++i) a[i] = T[pc_slot<N>(i * BC + j) + c];
+  dft_reg<8, true>(a);
+}
+
+// y forward: tmp [z][y][H] -> spec [z][ky][H + 1]
+template <int N>
+__global__ void __launch_bounds__(ColShape<N>::THREADS, ColShape<N>::MINB) k_y_forward(const float2* __restrict__ in,
+                                                                                       float2* __restrict__ spec,
+                                                                                       const float2* __restrict__ tw) {
+  constexpr int H = N / 2, NH = H + 1, C = ColShape<N>::C, BC = ColShape<N>::BC;
+  extern __shared__ __align__(16) unsigned char pc_smem[];
+  float2* T = reinterpret_cast<float2*>(pc_smem);
+  const int c = threadIdx.x & 7, j = threadIdx.x >> 3;
+  const int z = blockIdx.x / (H / PC_COLS), col0 = int(blockIdx.x % (H / PC_COLS)) * PC_COLS;
+  const float2* src = in + size_t(z) * N * H + col0 + c;
+  float2 a[8];
+#pragma unroll
+  for (int m = 0; m < 8; ++m) a[m] = __ldcs(src + (j + BC * m) * H);
+  cols_forward<N>(a, T, tw, c, j);
+  float2* dst = spec + size_t(z) * N * NH + col0 + c;
+  const bool packed = col0 == 0;  // this block's first column is A + i B, the columns 0 and N/2
+  for (int t = j; t < 64; t += BC) {
+    const int k1 = t >> 3, k2 = t & 7;
+    float2 b[C];
+#pragma unroll
+    for (int i = 0; i < C; ++i) b[i] = T[pc_slot<N>(k1 * BC + k2 * C + i) + c];
+    dft_any<C, false>(b);
+#pragma unroll
+    for (int k3 = 0; k3 < C; ++k3) {
+      const int ky = k1 + 8 * (k2 + 8 * k3);
+      const float2 v = b[dft_at<C>(k3)];
+      if (!packed || c) dst[ky * NH] = v;
+      // (the slots this thread has read are its own: the packed column waits there for its mirror)
+      if (packed && c == 0) T[pc_slot<N>(k1 * BC + k2 * C + k3)] = v;
+    }
+  }
+  if (packed) {
+    __syncthreads();
+    for (int ky = threadIdx.x; ky < N; ky += ColShape<N>::THREADS) {
+      auto at = [&](int k) { return T[pc_slot<N>((k & 7) * BC + ((k >> 3) & 7) * C + (k >> 6))]; };
+      const float2 y = at(ky), ym = at(ky ? N - ky : 0);
+      float2* o = spec + (size_t(z) * N + ky) * NH;
+      o[0] = make_float2(0.5f * (y.x + ym.x), 0.5f * (y.y - ym.y));
+      o[H] = make_float2(0.5f * (y.y + ym.y), -0.5f * (y.x - ym.x));
+    }
+  }
+}
+
+// y inverse: spec [z][ky][H + 1] -> tmp [z][y][H]
+template <int N>
+__global__ void __launch_bounds__(ColShape<N>::THREADS, ColShape<N>::MINB) k_y_inverse(const float2* __restrict__ spec,
+                                                                                       float2* __restrict__ out,
+                                                                                       const float2* __restrict__ tw) {
+  constexpr int H = N / 2, NH = H + 1, C = ColShape<N>::C, BC = ColShape<N>::BC;
+  extern __shared__ __align__(16) unsigned char pc_smem[];
+  float2* T = reinterpret_cast<float2*>(pc_smem);
+  const int c = threadIdx.x & 7, j = threadIdx.x >> 3;
+  const int z = blockIdx.x / (H / PC_COLS), col0 = int(blockIdx.x % (H / PC_COLS)) * PC_COLS;
+  const float2* src = spec + size_t(z) * N * NH + col0 + c;
+  const bool packed = col0 + c == 0;
+  for (int t = j; t < 64; t += BC) {
+    const int k1 = t >> 3, k2 = t & 7;
+    float2 b[C];
+#pragma unroll
+    for (int k3 = 0; k3 < C; ++k3) {
+      const int ky = k1 + 8 * (k2 + 8 * k3);
+      b[k3] = __ldcs(src + ky * NH);
+      if (packed) {  // A + i B
+        const float2 h = __ldcs(src + ky * NH + H);
+        b[k3] = make_float2(b[k3].x - h.y, b[k3].y + h.x);
+      }
+    }
+    dft_any<C, true>(b);
+#pragma unroll
+    for (int i = 0; i < C; ++i)
+      T[pc_slot<N>(k1 * BC + k2 * C + i) + c] = cmul(b[dft_at<C>(i)], conj2(__ldg(tw + 8 * i * k2)));
+  }
+  float2 a[8];
+  cols_inverse<N>(a, T, tw, c, j);
+  float2* dst = out + size_t(z) * N * H + col0 + c;
+#pragma unroll
+  for (int m = 0; m < 8; ++m) dst[(j + BC * m) * H] = a[bitrev<8>(m)];
+}
+
+// z: the flattened (ky, kx) half plane, PC_COLS columns per block
+template <int N>
+__global__ void __launch_bounds__(ColShape<N>::THREADS, ColShape<N>::MINB) k_z_green(float2* spec,
+                                                                                     const float2* __restrict__ tw,
+                                                                                     const float* __restrict__ s2, float coef,
+                                                                                     double* part) {
+  constexpr int H = N / 2, NH = H + 1, C = ColShape<N>::C, BC = ColShape<N>::BC;
+  constexpr size_t PLANE = size_t(N) * NH;
+  extern __shared__ __align__(16) unsigned char pc_smem[];
+  float2* T = reinterpret_cast<float2*>(pc_smem);
+  const int c = threadIdx.x & 7, j = threadIdx.x >> 3;
+  const uint32_t col = blockIdx.x * PC_COLS + c, ky = col / NH, kx = col - ky * NH;
+  float2* io = spec + col;
+  float2 a[8];
+#pragma unroll
+  for (int m = 0; m < 8; ++m) a[m] = __ldcs(io + (j + BC * m) * PLANE);
+  const float sxy = __ldg(s2 + ky), sx = __ldg(s2 + kx), w = (kx == 0 || kx == H) ? 1.0f : 2.0f;
+  cols_forward<N>(a, T, tw, c, j);
+  float wsum = 0.0f;
+  for (int t = j; t < 64; t += BC) {
+    const int k1 = t >> 3, k2 = t & 7;
+    float2 b[C], d[C];
+#pragma unroll
+    for (int i = 0; i < C; ++i) b[i] = T[pc_slot<N>(k1 * BC + k2 * C + i) + c];
+    dft_any<C, false>(b);
+#pragma unroll
+    for (int k3 = 0; k3 < C; ++k3) {
+      const int kz = k1 + 8 * (k2 + 8 * k3);
+      const float2 v = b[dft_at<C>(k3)];
+      const float syz = sxy + __ldg(s2 + kz);
+      const float sum = syz + sx;
+      const float g = (ky == 0 && kz == 0 && kx == 0) ? 0.0f : coef * __frcp_rn(sum);
+      wsum += w * g * (v.x * v.x + v.y * v.y);
+      d[k3] = make_float2(v.x * g, v.y * g);
+    }
+    dft_any<C, true>(d);
+#pragma unroll
+    for (int i = 0; i < C; ++i)
+      T[pc_slot<N>(k1 * BC + k2 * C + i) + c] = cmul(d[dft_at<C>(i)], conj2(__ldg(tw + 8 * i * k2)));
+  }
+  cols_inverse<N>(a, T, tw, c, j);
+#pragma unroll
+  for (int m = 0; m < 8; ++m) io[(j + BC * m) * PLANE] = a[bitrev<8>(m)];
+  float acc[1] = {wsum};
+  block_sum_store<1>(acc, part, gridDim.x);
+}
+
+template <int N>
+cudaError_t pass_potential(const float* rho, float* phi, float2* spec, const float2* tw, const float* s2, float coef,
+                           double* part, cudaStream_t s, int stage) {
+  using S = ColShape<N>;
+  constexpr unsigned rows = unsigned(N) * N / PX_ROWS, planes = unsigned(N) * (N / 2 / PC_COLS);
+  float2* tmp = reinterpret_cast<float2*>(phi);
+  if (stage == 0) {
+    k_x_r2c<N><<<rows, PX_THREADS, 0, s>>>(rho, tmp, tw);
+    k_y_forward<N><<<planes, S::THREADS, S::smem(), s>>>(tmp, spec, tw);
+  } else if (stage == 1) {
+    k_z_green<N><<<unsigned(pass_fft_tiles(N)), S::THREADS, S::smem(), s>>>(spec, tw, s2, coef, part);
+  } else {
+    k_y_inverse<N><<<planes, S::THREADS, S::smem(), s>>>(spec, tmp, tw);
+    k_x_c2r<N><<<rows, PX_THREADS, 0, s>>>(tmp, tw);
+  }
+  return cudaGetLastError();
+}
+
+}  // namespace
+
+bool pass_fft_supported(int n) { return n == 384 || n == 512; }
+int pass_fft_tiles(int n) { return n * (n / 2 + 1) / PC_COLS; }
+
+cudaError_t launch_pass_fft(int stage, const float* rho, float* phi, void* spec, const float2* tw, const float* s2, int n,
+                            double coef, double* part, cudaStream_t s) {
+  switch (n) {
+    case 384: return pass_potential<384>(rho, phi, static_cast<float2*>(spec), tw, s2, float(coef), part, s, stage);
+    case 512: return pass_potential<512>(rho, phi, static_cast<float2*>(spec), tw, s2, float(coef), part, s, stage);
+    default: return cudaErrorInvalidValue;
+  }
+}
+
+}  // namespace pm
