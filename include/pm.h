@@ -218,14 +218,14 @@ typedef struct {
   int32_t kick_threads;    /* threads (particles) per interpolate+kick+drift block: 128 or 256 */
   int32_t deposit_warps;   /* warps per deposit block (each warp owns a tile of up to 2 x 4 mesh rows): 1..8 */
   int32_t green_fused;     /* PM_FP32 cloud-in-cell on a power-of-two mesh of 16..512 only: 1 transforms the
-                              planes of constant z with batched 2D transforms and does the z transforms, the
-                              Green multiplication and the inverse z transforms in one kernel between them
-                              (the spectrum crosses device memory once instead of three times; the default
-                              where it applies); 2 (256^3 meshes only, their default) does the same with
-                              the x and y transforms of each plane in one kernel per direction (a cluster of
-                              CTAs per plane) instead of the batched 2D cuFFT plans; 0 uses the 3D
-                              transforms and a separate Green pass.  The potential agrees to fp32 rounding
-                              in every mode */
+                              planes of constant z (kernels of this library on 64^3, 128^3 and 512^3 meshes, batched
+                              2D cuFFT elsewhere) and does the z transforms, the Green multiplication and the
+                              inverse z transforms in one kernel between them (the spectrum crosses device memory
+                              once instead of three times; the default from 128^3); 2 (256^3 meshes only, their
+                              default) does the same with the x and y transforms of each plane in one kernel per
+                              direction (a cluster of CTAs per plane); 0 uses the 3D transforms and a separate
+                              Green pass, except on 64^3 meshes, which take the plane kernels all the same (and so
+                              do 384^3 ones their own).  The potential agrees to fp32 rounding in every mode */
 } pm_tuning;
 
 /* Current shapes. */

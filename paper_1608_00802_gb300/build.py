@@ -1,7 +1,7 @@
 """Builds libpm.so (the C-ABI library) in-tree for sm_103a with nvcc.
 
 The translation units compile in parallel (host API, fp32 kernels, fp64
-kernels, the allocation-free deposit, the fused x-y transforms, the pass-by-pass transforms) and link
+kernels, the allocation-free deposit, the fused x-y transforms, the transforms of other mesh sizes) and link
 against cuFFT.  Usage: ``python -m paper_1608_00802_gb300.build``.
 """
 from __future__ import annotations
@@ -17,7 +17,8 @@ CSRC = os.path.join(HERE, "csrc")
 ROOT = os.path.dirname(HERE)
 BUILD = os.path.join(ROOT, "_build")
 LIB = os.path.join(HERE, "libpm.so")
-SOURCES = ["pm_api.cu", "pm_kernels_f32.cu", "pm_kernels_f64.cu", "pm_noalloc.cu", "pm_xyfft.cu", "pm_passfft.cu"]
+SOURCES = ["pm_api.cu", "pm_kernels_f32.cu", "pm_kernels_f64.cu", "pm_noalloc.cu", "pm_xyfft.cu", "pm_passfft.cu",
+           "pm_planefft.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 

@@ -612,6 +612,14 @@ bool pass_fft(const pm_sim* s) {
          (!spec_z_supported(s->cfg.n_mesh) || s->tune.green_fused == 1);
 }
 
+// fp32 cloud-in-cell on 64^3 and 128^3: the x-y transforms of a plane in one CTA.  On 128^3 they are the plane
+// transforms of green_fused = 1 (0: cuFFT's 3D transforms); on 64^3 (green_fused 0 or 1) there is nothing else
+bool plane_fft(const pm_sim* s) {
+  const int N = s->cfg.n_mesh;
+  return !s->fp64() && s->cfg.kernel == PM_KERNEL_CIC && plane_fft_supported(N) &&
+         (N < GREEN_FUSE_MIN_MESH || s->tune.green_fused == 1);
+}
+
 // the Green multiplication inside the z transform, between batched 2D transforms
 bool green_fused(const pm_sim* s) { return s->tune.green_fused && s->have_plan2; }
 
@@ -708,11 +716,13 @@ pm_status mesh_from_density(pm_sim* s) {
     s->fields_valid = true;
     return PM_OK;
   }
-  if (green_fused(s)) {  // 2D transforms of the planes; z transforms and Green in one pass between them
+  if (plane_fft(s) || green_fused(s)) {  // 2D transforms of the planes; z transforms and Green in one pass between them
     const int N = s->cfg.n_mesh;
     {
       PROF(s, PM_STAGE_FFT_R2C);
-      if (s->tune.green_fused == 2)
+      if (plane_fft(s))
+        CU(s, launch_plane_fft(false, s->at<float>(L.rho), s->arena + L.spec, s->at<float2>(L.green), N, s->stream));
+      else if (s->tune.green_fused == 2)
         CU(s, launch_xy_r2c(s->at<float>(L.rho), s->arena + L.spec, s->at<float2>(L.green), N, s->stream));
       else
         CF(s, cufftExecR2C(s->plan2_fwd, s->at<cufftReal>(L.rho), (cufftComplex*)(s->arena + L.spec)));
@@ -725,7 +735,9 @@ pm_status mesh_from_density(pm_sim* s) {
     s->wg_count = spec_z_tiles(N);
     {
       PROF(s, PM_STAGE_FFT_C2R);
-      if (s->tune.green_fused == 2)
+      if (plane_fft(s))
+        CU(s, launch_plane_fft(true, s->at<float>(L.phi), s->arena + L.spec, s->at<float2>(L.green), N, s->stream));
+      else if (s->tune.green_fused == 2)
         CU(s, launch_xy_c2r(s->arena + L.spec, s->at<float>(L.phi), s->at<float2>(L.green), N, s->stream));
       else
         CF(s, cufftExecC2R(s->plan2_inv, (cufftComplex*)(s->arena + L.spec), s->at<cufftReal>(L.phi)));
@@ -1179,7 +1191,7 @@ pm_status pm_create(const pm_config* c, void* dev_arena, size_t bytes, void* str
     std::string ignored;
     if (spec_plan_setup(s, &ignored) == CUFFT_SUCCESS) s->tune.green_fused = xy_fft_supported(N) ? 2 : 1;
   }
-  if (c->precision == PM_FP32 && c->kernel == PM_KERNEL_CIC && pass_fft_supported(N) && !spec_z_supported(N) &&
+  if (c->precision == PM_FP32 && c->kernel == PM_KERNEL_CIC && ((pass_fft_supported(N) && !spec_z_supported(N)) || (plane_fft_supported(N) && N < GREEN_FUSE_MIN_MESH)) &&
       (launch_spec_tables(s->at<float2>(L.green), s->at<float>(L.green + size_t(N) * 8), N, s->stream) != cudaSuccess ||
        cudaStreamSynchronize(s->stream) != cudaSuccess)) {
     cufftDestroy(s->plan_fwd);
@@ -2011,7 +2023,7 @@ bool same_state(const pm_batch::Class& C, const std::vector<pm_sim*>& sims) {
         s->tune.green_fused != a->tune.green_fused)
       return false;
   }
-  if (!green_fused(a) && !pass_fft(a) && !C.fwd) return false;  // the class's batched 3D transforms were not planned
+  if (!green_fused(a) && !pass_fft(a) && !plane_fft(a) && !C.fwd) return false;  // the class's batched 3D transforms were not planned
   const StencilParams sp = stencil_params(a, false);
   return !a->cfg.quantum || (a->tune.st_ty > 0 && a->tune.st_stages == 0 && stencil_shape_ok(a->cfg.n_mesh, sp.ty, sp.zlen, 0));
 }
@@ -2052,7 +2064,8 @@ pm_status packed_step(pm_batch::Class& C, const std::vector<pm_sim*>& sims, cuda
   PCU(launch_deposit<float>(s->arena + L.pos[nxt], s->at<uint32_t>(L.row_start), n, s->mesh, s->norm,
                             s->at<float>(L.rho), st, s->tune.dep_warps, nm, ms));
   const bool passes = pass_fft(s);  // each member's own transforms, pass by pass (the same as alone)
-  const bool fused = green_fused(s) && !passes;
+  const bool planes = plane_fft(s);
+  const bool fused = (green_fused(s) || planes) && !passes;
   const bool own_xy = fused && s->tune.green_fused == 2;
   if (passes) {
     for (int i : C.members) {
@@ -2064,7 +2077,9 @@ pm_status packed_step(pm_batch::Class& C, const std::vector<pm_sim*>& sims, cuda
   }
   if (own_xy)  // the x-y transforms of every member's planes in one launch
     PCU(launch_xy_r2c(s->at<float>(L.rho), s->arena + L.spec, s->at<float2>(L.green), N, st, nm, ms));
-  if (fused && !own_xy) {  // each member's own 2D transforms (the same as alone)
+  if (planes)  // the x-y transforms of every member's planes in one launch
+    PCU(launch_plane_fft(false, s->at<float>(L.rho), s->arena + L.spec, s->at<float2>(L.green), N, st, nm, ms));
+  if (fused && !own_xy && !planes) {  // each member's own 2D transforms (the same as alone)
     for (int i : C.members) {
       pm_sim* m = sims[i];
       CF(s, cufftSetStream(m->plan2_fwd, st));
@@ -2078,7 +2093,9 @@ pm_status packed_step(pm_batch::Class& C, const std::vector<pm_sim*>& sims, cuda
                       green_coef(s), wg_part(s), st, s->coefs(), nm, ms));
   }
   if (own_xy) PCU(launch_xy_c2r(s->arena + L.spec, s->at<float>(L.phi), s->at<float2>(L.green), N, st, nm, ms));
-  if (fused && !own_xy) {
+  if (planes)
+    PCU(launch_plane_fft(true, s->at<float>(L.phi), s->arena + L.spec, s->at<float2>(L.green), N, st, nm, ms));
+  if (fused && !own_xy && !planes) {
     for (int i : C.members) {
       pm_sim* m = sims[i];
       CF(s, cufftSetStream(m->plan2_inv, st));
@@ -2179,7 +2196,8 @@ pm_status pm_batch_create(const pm_config* cfgs, int32_t n, void* dev_arena, siz
       b->classes.push_back(C);
       return cleanup(PM_ERR_CUDA, "class stream creation failed");
     }
-    if (C.packed && !green_fused(b->sims[C.members[0]]) && !pass_fft(b->sims[C.members[0]])) {  // fused members transform with their own 2D plans
+    if (C.packed && !green_fused(b->sims[C.members[0]]) && !pass_fft(b->sims[C.members[0]]) &&
+        !plane_fft(b->sims[C.members[0]])) {  // fused members transform with their own 2D plans
       size_t w = 0;
       const pm_config& c = cfgs[C.members[0]];
       if (class_plans(c, int(C.members.size()), C.stride, &C.fwd, &C.inv, &w) != CUFFT_SUCCESS || w > BC.work ||

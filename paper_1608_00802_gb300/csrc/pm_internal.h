@@ -174,6 +174,11 @@ cudaError_t launch_resort(int part, const uint32_t* keys, int64_t n, uint32_t* t
                           const void* mom_in, void* pos_out, void* mom_out, int sms, cudaStream_t s, int nm = 1,
                           size_t ms = 0);
 inline size_t row_scan_tiles(int n_mesh) { return (size_t(n_mesh) * n_mesh + 1023) / 1024; }  // tiles of 1024 rows
+// the x-y transforms of the z-planes of 64^3 and 128^3 fp32 meshes, one CTA per plane (unnormalised, the layouts of
+// the batched 2D R2C / C2R)
+bool plane_fft_supported(int n);
+cudaError_t launch_plane_fft(bool inverse, float* mesh, void* spec, const float2* tw, int n, cudaStream_t s, int nm = 1,
+                             size_t ms = 0);
 // phi~ from the density on 384^3 and 512^3 fp32 meshes, transform by transform: stage 0 the x and y transforms
 // (through phi, as scratch), 1 the z transforms with the Green multiplication (one W_g partial per tile), 2 the
 // inverse y and x transforms.  tw, s2: the tables of launch_spec_tables

@@ -1,4 +1,5 @@
-"""The pass-by-pass transforms of 384^3 and 512^3 meshes: a particle density's potential
+"""The transforms of 64^3 and 128^3 meshes (a CTA per plane) and of 384^3 and 512^3 meshes
+(pass by pass): a particle density's potential
 against the same Poisson solve in float64, plane waves on the packed columns and at the edges of
 the column tiles in closed form, the gravitational energy (one partial per tile), and
 packed batch members against single runs."""
@@ -26,7 +27,7 @@ def _sim(pm, n_mesh, box=2.0, **kw):
     return sim
 
 
-@pytest.mark.parametrize("n_mesh", [384, 512])
+@pytest.mark.parametrize("n_mesh", [64, 128, 384, 512])
 def test_potential_of_particles_against_float64(pm, n_mesh):
     """Every mode at once: the density of random particles, as the other transforms are tested on."""
     import torch
@@ -44,12 +45,12 @@ def test_potential_of_particles_against_float64(pm, n_mesh):
     sim.close()
 
 
-@pytest.mark.parametrize("n_mesh", [384, 512])
+@pytest.mark.parametrize("n_mesh", [64, 128, 384, 512])
 def test_plane_waves(pm, n_mesh):
     N, box, dx = n_mesh, 2.0, 2.0 / n_mesh
     h = N // 2
     waves = [((0, 5, 9), 0.3), ((h, 0, 7), 0.2), ((h, 3, 0), 0.15), ((0, h, 1), 0.1), ((1, N - 2, N - 3), 0.1),
-             ((7, 64, 5), 0.05), ((8, 17, 100), 0.05), ((h - 1, 200, h), 0.05), ((h - 8, N - 1, 63), 0.03)]
+             ((7, h - 3, 5), 0.05), ((8, 17, h + 4), 0.05), ((h - 1, h + 8, h), 0.05), ((h - 8, N - 1, 33), 0.03)]
     c = [np.exp(2j * np.pi * np.arange(N) * k / N) for k in range(N)]
     rho, ref = np.ones((N, N, N)), np.zeros((N, N, N))
     for (kx, ky, kz), amp in waves:
@@ -62,10 +63,11 @@ def test_plane_waves(pm, n_mesh):
     sim.close()
 
 
-def test_energy_of_the_tiles(pm):
+@pytest.mark.parametrize("n_mesh", [64, 128, 384])
+def test_energy_of_the_tiles(pm, n_mesh):
     """W_g from the z pass's partials against the sum over the mesh."""
     rng = np.random.default_rng(2)
-    N, n = 384, 100000
+    N, n = n_mesh, 100000
     x = rng.random((n, 3)) * 2.0
     sim = pm.Sim(pm.make_config(n, N, 2.0, quantum=False))
     sim.set_particles(x, np.zeros((n, 3)))
@@ -76,9 +78,10 @@ def test_energy_of_the_tiles(pm):
     sim.close()
 
 
-def test_batch_members_equal_single_runs(pm):
+@pytest.mark.parametrize("n_mesh", [64, 128, 384])
+def test_batch_members_equal_single_runs(pm, n_mesh):
     rng = np.random.default_rng(4)
-    n, N = 70000, 384
+    n, N = 70000, n_mesh
     parts = [(rng.random((n, 3)) * box, 1e-3 * rng.standard_normal((n, 3))) for box in (2.0, 3.0)]
     cfgs = [pm.make_config(n, N, box, quantum=False, force_mode=pm.FORCE_HYBRID) for box in (2.0, 3.0)]
     batch = pm.Batch(cfgs)
