@@ -1128,7 +1128,7 @@ pm_status pm_create(const pm_config* c, void* dev_arena, size_t bytes, void* str
   s->keys_tmp[0] = s->at<uint32_t>(L.keys[1]);
   s->keys_tmp[1] = s->at<uint32_t>(L.keys[2]);
   s->have_particles = s->sorted = s->fields_valid = false;
-  s->tune = default_tuning(N, c->n_part);
+  s->tune = default_tuning(N, c->n_part, c->precision == PM_FP64);
   {
     int dev = 0, sm = 0;
     if (cudaGetDevice(&dev) == cudaSuccess &&

@@ -241,7 +241,7 @@ size_t stencil_list_entries(int n);
 int stencil_launch_blocks(int n, int ty, int zlen);
 int stencil_max_blocks(int n);
 bool stencil_shape_ok(int n, int ty, int zlen, int stages);
-Tuning default_tuning(int n, int64_t n_part);
+Tuning default_tuning(int n, int64_t n_part, bool fp64);
 // sizes the fp32 streaming kick's grid for this device (an occupancy query;
 // call outside any stream capture, before the first kick)
 void kick_stream_prepare();

@@ -2230,7 +2230,7 @@ cudaError_t launch_init_particles(const double* x, const double* p, int64_t n, M
   return cudaGetLastError();
 }
 
-// deposit tile of TY x TZ rows per warp: the largest of 2 x 4, 2 x 2, 1 x 2, 1 x 1 whose rows fit
+// deposit tile of TY x TZ rows per warp: by size the largest of 2 x 4, 2 x 2, 1 x 2, 1 x 1 whose rows fit
 // PM_DEPOSIT_WARP_BYTES of shared memory per 4-byte accumulator (4.25 KB: 2 x 2 rows of a 256^3
 // fp32 mesh; measured there: 43 us against 53 us for 2 x 4 rows, whose 8.3 KB per warp leave
 // too few resident warps)
@@ -2240,13 +2240,22 @@ cudaError_t launch_init_particles(const double* x, const double* p, int64_t n, M
 #ifndef PM_DEPOSIT_WARP_BYTES
 #define PM_DEPOSIT_WARP_BYTES 4352
 #endif
+// Small meshes take fewer planes per tile while the tiles are fewer than PM_DEPOSIT_MIN_TILES warps (16 per SM):
+// a warp's time is its chain of batches, one or two per plane, so 64^3 goes from 512 tiles of five source
+// planes (6.9 us) to 2048 of two (4.2 us; 4096 particles on 32^3 7.2 -> 3.9 us).  Not in fp64, whose pipe pays
+// for every record read again (14.1 -> 14.7 us).  The planes of a tile do not enter its result: a row's batches
+// are cut by its chain, which only the rows in y decide, and added plane by plane.
+#ifndef PM_DEPOSIT_MIN_TILES
+#define PM_DEPOSIT_MIN_TILES 2432
+#endif
 template <typename R>
 inline int deposit_shape(int n, int& ty, int& tz) {
-  static const int shapes[4][2] = {{2, 4}, {2, 2}, {1, 2}, {1, 1}};
+  static const int shapes[5][2] = {{2, 4}, {2, 2}, {2, 1}, {1, 2}, {1, 1}};
   const size_t row = size_t(deposit_stride_of<R>(n)) * sizeof(R);
   const size_t most = size_t(PM_DEPOSIT_WARP_BYTES) * sizeof(R) / 4;
   int s = 0;
-  while (s < 3 && size_t(shapes[s][0] * shapes[s][1]) * row > most) ++s;
+  while (s < 4 && (size_t(shapes[s][0] * shapes[s][1]) * row > most || s == 2)) ++s;
+  while (sizeof(R) == 4 && s < 2 && ((n + 1) / 2) * ((n + shapes[s][1] - 1) / shapes[s][1]) < PM_DEPOSIT_MIN_TILES) ++s;
   ty = shapes[s][0], tz = shapes[s][1];
   return s;
 }
@@ -2294,7 +2303,8 @@ cudaError_t launch_deposit(const void* pos, const uint32_t* row_start, int64_t n
     if (dev < 0 || dev >= 64 || !done[dev]) {
       const int most = int(DEP_WARPS * PM_DEPOSIT_WARP_BYTES * sizeof(R) / 4);
       cudaError_t e = cudaSuccess;
-      void* fns[8] = {(void*)k_deposit<R, 2, 4, false>, (void*)k_deposit<R, 2, 4, true>,
+      void* fns[10] = {(void*)k_deposit<R, 2, 1, false>, (void*)k_deposit<R, 2, 1, true>,
+                       (void*)k_deposit<R, 2, 4, false>, (void*)k_deposit<R, 2, 4, true>,
                       (void*)k_deposit<R, 2, 2, false>, (void*)k_deposit<R, 2, 2, true>,
                       (void*)k_deposit<R, 1, 2, false>, (void*)k_deposit<R, 1, 2, true>,
                       (void*)k_deposit<R, 1, 1, false>, (void*)k_deposit<R, 1, 1, true>};
@@ -2307,7 +2317,8 @@ cudaError_t launch_deposit(const void* pos, const uint32_t* row_start, int64_t n
   switch (shape) {
     case 0: return launch_deposit_tile<R, 2, 4>(pos, row_start, n, m, norm, rho, s, warps, nm, ms);
     case 1: return launch_deposit_tile<R, 2, 2>(pos, row_start, n, m, norm, rho, s, warps, nm, ms);
-    case 2: return launch_deposit_tile<R, 1, 2>(pos, row_start, n, m, norm, rho, s, warps, nm, ms);
+    case 2: return launch_deposit_tile<R, 2, 1>(pos, row_start, n, m, norm, rho, s, warps, nm, ms);
+    case 3: return launch_deposit_tile<R, 1, 2>(pos, row_start, n, m, norm, rho, s, warps, nm, ms);
     default: return launch_deposit_tile<R, 1, 1>(pos, row_start, n, m, norm, rho, s, warps, nm, ms);
   }
 }

@@ -46,14 +46,14 @@ bool stencil_shape_ok(int n, int ty, int zlen, int stages) {
   return stages == 0 ? stencil_tile_shape_ok(n, ty, zlen) : stencil_bulk_shape_ok(n, ty, zlen, stages);
 }
 
-Tuning default_tuning(int n, int64_t n_part) {
+Tuning default_tuning(int n, int64_t n_part, bool fp64) {
   Tuning t;
   // few particles: twice the blocks of half the threads while 256 would leave SMs idle
   t.kick_threads = n_part < int64_t(KICK_THREADS) * 2 * 152 ? 128 : KICK_THREADS;
-  // small meshes: fewer warps per deposit block while the tiles would leave SMs idle (512 tiles of 2 x 4 rows on
-  // 64^3: 64 blocks of 8 warps 7.0 us, fp64 17.9; 256 of 2 warps 6.8 and 14.1 us)
+  // small meshes: fewer warps per deposit block while the tiles would leave SMs idle (the 512 tiles of 2 x 4 rows
+  // of a 64^3 fp64 mesh: 17.9 us in 64 blocks of 8 warps, 14.1 in 256 of 2)
   int ty = 1, tz = 1;
-  deposit_shape<float>(n, ty, tz);
+  fp64 ? deposit_shape<double>(n, ty, tz) : deposit_shape<float>(n, ty, tz);
   const int tiles = ((n + ty - 1) / ty) * ((n + tz - 1) / tz);
   t.dep_warps = 8;
   while (t.dep_warps > 2 && tiles / t.dep_warps < 152) t.dep_warps /= 2;

@@ -128,7 +128,7 @@ pm_status pm_deposit_noalloc(const double* x_dev, int64_t n_part, int32_t n_mesh
   NA_CU(launch_sort_small<float>(keys, n, bits, keys, pos[0], nullptr, pos[1], nullptr, rows, m,
                                  err_dev ? nullptr : err, s));
   NA_CU(launch_deposit<float>(pos[1], rows, n, m, double(m.n3) / double(n), rho_dev, s,
-                              default_tuning(n_mesh, n).dep_warps));
+                              default_tuning(n_mesh, n, false).dep_warps));
   if (err_dev) {
     k_copy_error<<<1, 1, 0, s>>>(err, err_dev);
     NA_CU(cudaGetLastError());
