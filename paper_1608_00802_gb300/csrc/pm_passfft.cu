@@ -2,7 +2,7 @@
 // have the x-y kernels or cuFFT):
 //   x  forward : each row of N reals -> N/2 complex, X[0] + i X[N/2] packed first  (rho -> tmp)
 //   y  forward : 8 columns of a z-plane per block, the packed column split          (tmp -> spectrum)
-//   z          : 8 columns of the half spectrum per block, Green multiplication, W_g partial, back (in place)
+//   z          : 16 columns of the half spectrum per block, Green multiplication, W_g partial, back (in place)
 //   y  inverse : the columns packed again                                           (spectrum -> tmp)
 //   x  inverse : each row back to N reals                                           (tmp, in place)
 // tmp is the potential's mesh: N/2 complex values are a row of it.  A plane of these meshes (0.6 and 1 MB)
@@ -10,7 +10,7 @@
 // 384^3 mesh 906 us for its 3D pair plus 81 for the Green pass (a pass over memory takes 68 us), on 512^3
 // 996 us for its 2D pair plus 504 for the four-step z kernel at one block of 128 registers per SM (160 us a
 // pass).  So each pass here does as little as it can per value and leaves room for many threads: the five
-// passes take 570 us on 384^3 and 1270 us on 512^3.  The potential's error against float64 (particle
+// passes take 530 us on 384^3 and 1200 us on 512^3.  The potential's error against float64 (particle
 // density, of the largest |phi|): 384^3 4.2e-6 -> 6.1e-7 (the Green table folds its index), 512^3 4.7e-7 ->
 // 4.1e-7.
 //
@@ -20,7 +20,9 @@
 // j = j' + C m', k = k1 + 8 (k2 + 8 k3): thread j an 8-point DFT over m and W_N^{j k1}, thread (k1, j') an
 // 8-point DFT over m' and W_{8C}^{j' k2}, thread (k1, k2) a C-point DFT over j'; eight values and ~40
 // registers a thread.  Slots of the exchange tile are padded by one in C, so that the third step's stride of
-// C slots does not meet one bank group.  Inverses run the same steps backwards with conjugate twiddles.
+// C slots does not meet one bank group (the z kernel's slots are whole bank rows).  Inverses run the same steps backwards with conjugate twiddles.
+#include <atomic>
+
 #include "pm_kernels.cuh"
 
 namespace pm {
@@ -288,51 +290,245 @@ __global__ void __launch_bounds__(ColShape<N>::THREADS, ColShape<N>::MINB) k_y_i
   for (int m = 0; m < 8; ++m) dst[(j + BC * m) * H] = a[bitrev<8>(m)];
 }
 
-// z: the flattened (ky, kx) half plane, PC_COLS columns per block
+// ---------------------------------------------------------------- z
+// z: 16 columns of the flattened (ky, kx) half plane per block, in place: phi^ = G rho^ with k_green's arithmetic
+// and Parseval partial of W_g.  A thread carries two adjacent columns through every step as pairs (re0, re1),
+// (im0, im1) in 64-bit registers: the packed fp32 instructions (add, sub, mul, fma .f32x2) do both columns at
+// once, a pair of values is one 16-byte access of memory or shared memory, and twiddles and addresses serve two.
+// With one column a thread and 8 columns a block the kernel was bound by its instructions and by 64-byte
+// segments: 400 -> 327 us on 512^3, 168 -> 136 on 384^3 (two passes over memory take 160 and 68).  Pairs in blocks
+// of 8 columns take 369 and 158; the y passes do not gain by pairs, because a spectrum row starts on 8 bytes
+// only (inverse 235 -> 295 on 512^3, forward 235 -> 239), nor does the z kernel of 256^3 (33 -> 37).
+using u64 = unsigned long long;
+__device__ __forceinline__ u64 pk2(float a, float b) {
+  u64 d;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(a), "f"(b));
+  return d;
+}
+__device__ __forceinline__ float2 un2(u64 a) {
+  float2 d;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(d.x), "=f"(d.y) : "l"(a));
+  return d;
+}
+__device__ __forceinline__ u64 add2(u64 a, u64 b) {
+  u64 d;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+__device__ __forceinline__ u64 sub2(u64 a, u64 b) {
+  u64 d;
+  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+__device__ __forceinline__ u64 mul2(u64 a, u64 b) {
+  u64 d;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+__device__ __forceinline__ u64 fma2(u64 a, u64 b, u64 c) {
+  u64 d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
+}
+struct C2 {  // two complex values of adjacent columns
+  u64 re, im;
+};
+__device__ __forceinline__ C2 c2_of(float4 v) { return {pk2(v.x, v.z), pk2(v.y, v.w)}; }
+__device__ __forceinline__ float4 c2_float4(C2 v) {
+  const float2 r = un2(v.re), i = un2(v.im);
+  return make_float4(r.x, i.x, r.y, i.y);
+}
+__device__ __forceinline__ C2 c2_ld(const ulonglong2* p) {
+  const ulonglong2 v = *p;
+  return {v.x, v.y};
+}
+__device__ __forceinline__ void c2_st(ulonglong2* p, C2 v) { *p = make_ulonglong2(v.re, v.im); }
+// times w = (wx, wx), (wy, wy), or its conjugate
+template <bool CONJ>
+__device__ __forceinline__ C2 c2_mul(C2 a, ulonglong2 w) {
+  if (CONJ) return {fma2(a.im, w.y, mul2(a.re, w.x)), sub2(mul2(a.im, w.x), mul2(a.re, w.y))};
+  return {sub2(mul2(a.re, w.x), mul2(a.im, w.y)), fma2(a.re, w.y, mul2(a.im, w.x))};
+}
+// times exp(-+2 pi i t / 8) (forward: minus) of u - v
+template <bool INV>
+__device__ __forceinline__ C2 c2_diff8(C2 u, C2 v, int t) {
+  if (t == 0) return {sub2(u.re, v.re), sub2(u.im, v.im)};
+  if (t == 2) return INV ? C2{sub2(v.im, u.im), sub2(u.re, v.re)} : C2{sub2(u.im, v.im), sub2(v.re, u.re)};
+  const C2 d = {sub2(u.re, v.re), sub2(u.im, v.im)};
+  const u64 h = pk2(0.707106769f, 0.707106769f), mh = pk2(-0.707106769f, -0.707106769f);
+  if (t == 1)
+    return INV ? C2{mul2(sub2(d.re, d.im), h), mul2(add2(d.re, d.im), h)}
+               : C2{mul2(add2(d.re, d.im), h), mul2(sub2(d.im, d.re), h)};
+  return INV ? C2{mul2(add2(d.re, d.im), mh), mul2(sub2(d.re, d.im), h)}
+             : C2{mul2(sub2(d.im, d.re), h), mul2(add2(d.re, d.im), mh)};
+}
+// DFT of M = 2, 4, 8 points (as dft_reg: natural order in, bit-reversed out)
+template <int M, bool INV>
+__device__ __forceinline__ void c2_dft_pow2(C2* a) {
+#pragma unroll
+  for (int len = M; len >= 2; len >>= 1) {
+    const int half = len >> 1;
+#pragma unroll
+    for (int b = 0; b < M; b += len) {
+#pragma unroll
+      for (int j = 0; j < half; ++j) {
+        const C2 u = a[b + j], v = a[b + j + half];
+        a[b + j] = {add2(u.re, v.re), add2(u.im, v.im)};
+        a[b + j + half] = c2_diff8<INV>(u, v, j * (8 / len));
+      }
+    }
+  }
+}
+// M = 4, 6, 8; X[k] at a[dft_at<M>(k)]
+template <int M, bool INV>
+__device__ __forceinline__ void c2_dft(C2 (&a)[M]) {
+  if constexpr (M == 6) {  // radix 3, twiddles exp(-+2 pi i j r / 6), then three 2-point DFTs
+    const float sg = INV ? 1.0f : -1.0f;
+    const u64 s60 = pk2(sg * 0.866025388f, sg * 0.866025388f), ms60 = pk2(-sg * 0.866025388f, -sg * 0.866025388f);
+    const u64 hf = pk2(0.5f, 0.5f), mhf = pk2(-0.5f, -0.5f);
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+      const C2 u = a[j], v = a[j + 2], w = a[j + 4];
+      const C2 p = {add2(v.re, w.re), add2(v.im, w.im)}, d = {sub2(v.re, w.re), sub2(v.im, w.im)};
+      const C2 h = {fma2(mhf, p.re, u.re), fma2(mhf, p.im, u.im)};
+      a[j] = {add2(u.re, p.re), add2(u.im, p.im)};
+      C2 r1 = {fma2(ms60, d.im, h.re), fma2(s60, d.re, h.im)}, r2 = {fma2(s60, d.im, h.re), fma2(ms60, d.re, h.im)};
+      if (j) {  // times (1/2, -+sin 60), (-1/2, -+sin 60)
+        r1 = {fma2(ms60, r1.im, mul2(hf, r1.re)), fma2(s60, r1.re, mul2(hf, r1.im))};
+        r2 = {fma2(ms60, r2.im, mul2(mhf, r2.re)), fma2(s60, r2.re, mul2(mhf, r2.im))};
+      }
+      a[j + 2] = r1;
+      a[j + 4] = r2;
+    }
+    c2_dft_pow2<2, INV>(a);
+    c2_dft_pow2<2, INV>(a + 2);
+    c2_dft_pow2<2, INV>(a + 4);
+  } else {
+    c2_dft_pow2<M, INV>(a);
+  }
+}
+
+constexpr int ZC_COLS = 16, ZC_PAIRS = ZC_COLS / 2;
 template <int N>
-__global__ void __launch_bounds__(ColShape<N>::THREADS, ColShape<N>::MINB) k_z_green(float2* spec,
-                                                                                     const float2* __restrict__ tw,
-                                                                                     const float* __restrict__ s2, float coef,
-                                                                                     double* part) {
-  constexpr int H = N / 2, NH = H + 1, C = ColShape<N>::C, BC = ColShape<N>::BC;
+struct ZShape {
+  static constexpr int C = N / 64, BC = 8 * C, THREADS = ZC_PAIRS * BC, MINB = 1024 / THREADS + (N == 384);
+  // the exchange tile [slot][pair] (a quarter warp's 16-byte accesses are one slot: no padding), the twiddles as
+  // (wx, wx, wy, wy), the Green table
+  static constexpr size_t smem() { return size_t(N) * (ZC_PAIRS * 16 + 16 + 4); }
+};
+
+__device__ __forceinline__ void load_twiddles(ulonglong2* w, const float2* __restrict__ tw, int n) {
+  for (int i = threadIdx.x; i < n; i += blockDim.x) {
+    const float2 t = __ldg(tw + i);
+    w[i] = make_ulonglong2(pk2(t.x, t.x), pk2(t.y, t.y));
+  }
+}
+
+// the first two steps of the columns' transforms from their values a[m] = x[j + BC m] (thread (c, j)): the tile
+// T holds the values of the third step
+template <int N>
+__device__ __forceinline__ void zc_forward(C2 (&a)[8], ulonglong2* T, const ulonglong2* w, int c, int j) {
+  constexpr int C = ZShape<N>::C, BC = ZShape<N>::BC;
+  c2_dft_pow2<8, false>(a);
+  c2_st(T + j * ZC_PAIRS + c, a[0]);
+#pragma unroll
+  for (int k1 = 1; k1 < 8; ++k1) c2_st(T + (k1 * BC + j) * ZC_PAIRS + c, c2_mul<false>(a[bitrev<8>(k1)], w[j * k1]));
+  __syncthreads();
+  const int k1 = j / C, jp = j - k1 * C;
+  ulonglong2* t = T + (k1 * BC + jp) * ZC_PAIRS + c;
+#pragma unroll
+  for (int m = 0; m < 8; ++m) a[m] = c2_ld(t + C * m * ZC_PAIRS);
+  c2_dft_pow2<8, false>(a);
+  c2_st(t, a[0]);
+#pragma unroll
+  for (int k2 = 1; k2 < 8; ++k2) c2_st(t + k2 * C * ZC_PAIRS, c2_mul<false>(a[bitrev<8>(k2)], w[8 * jp * k2]));
+  __syncthreads();
+}
+// the last two steps of the inverse, from the tile that the first one filled: a[bitrev(m)] = x[j + BC m]
+template <int N>
+__device__ __forceinline__ void zc_inverse(C2 (&a)[8], ulonglong2* T, const ulonglong2* w, int c, int j) {
+  constexpr int C = ZShape<N>::C, BC = ZShape<N>::BC;
+  __syncthreads();
+  const int k1 = j / C, jp = j - k1 * C;
+  ulonglong2* t = T + (k1 * BC + jp) * ZC_PAIRS + c;
+#pragma unroll
+  for (int k2 = 0; k2 < 8; ++k2) a[k2] = c2_ld(t + k2 * C * ZC_PAIRS);
+  c2_dft_pow2<8, true>(a);
+#pragma unroll
+  for (int m = 0; m < 8; ++m) c2_st(t + C * m * ZC_PAIRS, c2_mul<true>(a[bitrev<8>(m)], w[(jp + C * m) * k1]));
+  __syncthreads();
+#pragma unroll
+  for (int i = 0; i < 8; ++i) a[i] = c2_ld(T + (i * BC + j) * ZC_PAIRS + c);
+  c2_dft_pow2<8, true>(a);
+}
+
+template <int N>
+__global__ void __launch_bounds__(ZShape<N>::THREADS, ZShape<N>::MINB) k_z_green(float2* spec, const float2* __restrict__ tw,
+                                                                                 const float* __restrict__ s2g, float coef,
+                                                                                 double* part) {
+  constexpr int H = N / 2, NH = H + 1, C = ZShape<N>::C, BC = ZShape<N>::BC;
   constexpr size_t PLANE = size_t(N) * NH;
   extern __shared__ __align__(16) unsigned char pc_smem[];
-  float2* T = reinterpret_cast<float2*>(pc_smem);
+  ulonglong2 *T = reinterpret_cast<ulonglong2*>(pc_smem), *W = T + N * ZC_PAIRS;
+  float* s2 = reinterpret_cast<float*>(W + N);
   const int c = threadIdx.x & 7, j = threadIdx.x >> 3;
-  const uint32_t col = blockIdx.x * PC_COLS + c, ky = col / NH, kx = col - ky * NH;
-  float2* io = spec + col;
-  float2 a[8];
+  const uint32_t col = blockIdx.x * ZC_COLS + 2 * c;
+  C2 a[8];
+  {
+    const float4* src = reinterpret_cast<const float4*>(spec + col);
 #pragma unroll
-  for (int m = 0; m < 8; ++m) a[m] = __ldcs(io + (j + BC * m) * PLANE);
-  const float sxy = __ldg(s2 + ky), sx = __ldg(s2 + kx), w = (kx == 0 || kx == H) ? 1.0f : 2.0f;
-  cols_forward<N>(a, T, tw, c, j);
-  float wsum = 0.0f;
+    for (int m = 0; m < 8; ++m) a[m] = c2_of(__ldcs(src + (j + BC * m) * (PLANE / 2)));
+  }
+  load_twiddles(W, tw, N);
+  for (int i = threadIdx.x; i < N; i += ZShape<N>::THREADS) s2[i] = __ldg(s2g + i);
+  __syncthreads();
+  zc_forward<N>(a, T, W, c, j);
+  // (ky, kx) of the two columns
+  const uint32_t ky0 = col / NH, kx0 = col - ky0 * NH, kx1 = kx0 + 1 == NH ? 0 : kx0 + 1, ky1 = kx1 ? ky0 : ky0 + 1;
+  const float sx0 = s2[kx0], sx1 = s2[kx1], sy0 = s2[ky0], sy1 = s2[ky1];
+  const u64 w2 = pk2((kx0 == 0 || kx0 == H) ? 1.0f : 2.0f, (kx1 == 0 || kx1 == H) ? 1.0f : 2.0f);
+  u64 wsum = pk2(0.0f, 0.0f);
   for (int t = j; t < 64; t += BC) {
     const int k1 = t >> 3, k2 = t & 7;
-    float2 b[C], d[C];
+    ulonglong2* s = T + (k1 * BC + k2 * C) * ZC_PAIRS + c;
+    C2 b[C], d[C];
 #pragma unroll
-    for (int i = 0; i < C; ++i) b[i] = T[pc_slot<N>(k1 * BC + k2 * C + i) + c];
-    dft_any<C, false>(b);
+    for (int i = 0; i < C; ++i) b[i] = c2_ld(s + i * ZC_PAIRS);
+    c2_dft<C, false>(b);
 #pragma unroll
     for (int k3 = 0; k3 < C; ++k3) {
       const int kz = k1 + 8 * (k2 + 8 * k3);
-      const float2 v = b[dft_at<C>(k3)];
-      const float syz = sxy + __ldg(s2 + kz);
-      const float sum = syz + sx;
-      const float g = (ky == 0 && kz == 0 && kx == 0) ? 0.0f : coef * __frcp_rn(sum);
-      wsum += w * g * (v.x * v.x + v.y * v.y);
-      d[k3] = make_float2(v.x * g, v.y * g);
+      const C2 v = b[dft_at<C>(k3)];
+      const float sz = s2[kz];
+      const float syz0 = sy0 + sz, syz1 = sy1 + sz;
+      const float sum0 = syz0 + sx0, sum1 = syz1 + sx1;
+      const u64 g = pk2((col == 0 && kz == 0) ? 0.0f : coef * __frcp_rn(sum0), coef * __frcp_rn(sum1));
+      wsum = fma2(mul2(w2, g), fma2(v.re, v.re, mul2(v.im, v.im)), wsum);
+      d[k3] = {mul2(v.re, g), mul2(v.im, g)};
     }
-    dft_any<C, true>(d);
+    c2_dft<C, true>(d);
 #pragma unroll
-    for (int i = 0; i < C; ++i)
-      T[pc_slot<N>(k1 * BC + k2 * C + i) + c] = cmul(d[dft_at<C>(i)], conj2(__ldg(tw + 8 * i * k2)));
+    for (int i = 0; i < C; ++i) c2_st(s + i * ZC_PAIRS, c2_mul<true>(d[dft_at<C>(i)], W[8 * i * k2]));
   }
-  cols_inverse<N>(a, T, tw, c, j);
+  zc_inverse<N>(a, T, W, c, j);
+  float4* dst = reinterpret_cast<float4*>(spec + col);
 #pragma unroll
-  for (int m = 0; m < 8; ++m) io[(j + BC * m) * PLANE] = a[bitrev<8>(m)];
-  float acc[1] = {wsum};
+  for (int m = 0; m < 8; ++m) dst[(j + BC * m) * (PLANE / 2)] = c2_float4(a[bitrev<8>(m)]);
+  const float2 ws = un2(wsum);
+  float acc[1] = {ws.x + ws.y};
   block_sum_store<1>(acc, part, gridDim.x);
+}
+
+// the z kernel's shared memory needs the opt-in, once per device
+template <int N>
+cudaError_t z_prepare() {
+  static std::atomic<bool> done[64];
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess || (dev >= 0 && dev < 64 && done[dev])) return e;
+  e = cudaFuncSetAttribute(k_z_green<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(ZShape<N>::smem()));
+  if (e == cudaSuccess && dev >= 0 && dev < 64) done[dev] = true;
+  return e;
 }
 
 template <int N>
@@ -345,7 +541,10 @@ cudaError_t pass_potential(const float* rho, float* phi, float2* spec, const flo
     k_x_r2c<N><<<rows, PX_THREADS, 0, s>>>(rho, tmp, tw);
     k_y_forward<N><<<planes, S::THREADS, S::smem(), s>>>(tmp, spec, tw);
   } else if (stage == 1) {
-    k_z_green<N><<<unsigned(pass_fft_tiles(N)), S::THREADS, S::smem(), s>>>(spec, tw, s2, coef, part);
+    using Z = ZShape<N>;
+    const cudaError_t e = z_prepare<N>();
+    if (e != cudaSuccess) return e;
+    k_z_green<N><<<unsigned(pass_fft_tiles(N)), Z::THREADS, Z::smem(), s>>>(spec, tw, s2, coef, part);
   } else {
     k_y_inverse<N><<<planes, S::THREADS, S::smem(), s>>>(spec, tmp, tw);
     k_x_c2r<N><<<rows, PX_THREADS, 0, s>>>(tmp, tw);
@@ -356,7 +555,7 @@ cudaError_t pass_potential(const float* rho, float* phi, float2* spec, const flo
 }  // namespace
 
 bool pass_fft_supported(int n) { return n == 384 || n == 512; }
-int pass_fft_tiles(int n) { return n * (n / 2 + 1) / PC_COLS; }
+int pass_fft_tiles(int n) { return n * (n / 2 + 1) / ZC_COLS; }
 
 cudaError_t launch_pass_fft(int stage, const float* rho, float* phi, void* spec, const float2* tw, const float* s2, int n,
                             double coef, double* part, cudaStream_t s) {
