@@ -362,7 +362,7 @@ const char* pm_batch_last_error(const pm_batch* b);
  * pinned host memory) receives, in stream order after the deposit, the
  * call's device error bits: 0 = ok, bit 0 (1) = a non-finite position was
  * placed at 0, bit 1 (2) = a bounded wait of the sort gave up and rho_dev is
- * invalid.  The host return value cannot report these without a
+ * invalid (reserved: the one-kernel sort of these sizes has no such wait).  The host return value cannot report these without a
  * synchronisation, which this entry point does not make.  It calls no
  * cudaMalloc, cudaFree or allocating library routine: all temporaries live
  * in one file-scope static device array of PM_NOALLOC_SCRATCH_BYTES, which

@@ -272,10 +272,11 @@ struct pm_sim {
   int sms = 152;              // multiprocessors of the device
   bool krho_valid = false;    // the K_rho partials belong to the current Q~
   cufftHandle plan_fwd, plan_inv;
-  // fp32 cloud-in-cell, power-of-two mesh: batched 2D transforms of the z planes, between which
-  // one kernel does the z transforms and the Green multiplication
+  // fp32 cloud-in-cell, power-of-two mesh without own plane or pass transforms: batched 2D transforms of the
+  // z planes, between which one kernel does the z transforms and the Green multiplication
   cufftHandle plan2_fwd = 0, plan2_inv = 0;
   bool have_plan2 = false;
+  bool spec_ready = false;    // the z kernel's tables are made, and the 2D plans where the size needs them
   int wg_count = MESH_GRID;  // W_g partials the last force evaluation wrote
   bool have_particles, sorted, fields_valid;
   std::string err;
@@ -621,13 +622,22 @@ bool plane_fft(const pm_sim* s) {
 }
 
 // the Green multiplication inside the z transform, between batched 2D transforms
-bool green_fused(const pm_sim* s) { return s->tune.green_fused && s->have_plan2; }
+bool green_fused(const pm_sim* s) { return s->tune.green_fused && s->spec_ready; }
+
+// the counts of a drift whose re-sort did not run, or not to its end (an error between them)
+pm_status drop_mover_counts(pm_sim* s) {
+  const size_t N = size_t(s->cfg.n_mesh);
+  CU(s, cudaMemsetAsync(s->at<uint32_t>(s->L.tcount), 0, size_t(mover_count_words(s->n())) * 4, s->stream));
+  CU(s, cudaMemsetAsync(s->at<uint32_t>(s->L.rcnt), 0, size_t(3) * N * N * 4, s->stream));
+  return PM_OK;
+}
 
 // The batched 2D transforms of the N z planes (forward: the real density to
 // the (ky, kx) half planes; inverse: back to the real potential), sharing the
-// work area of the 3D plans, and the z kernel's tables.  Sync.
+// work area of the 3D plans, and the z kernel's tables.  64^3, 128^3 and 512^3
+// have own plane transforms and need the tables only.  Sync.
 cufftResult spec_plan_setup(pm_sim* s, std::string* why) {
-  if (s->have_plan2) return CUFFT_SUCCESS;
+  if (s->spec_ready) return CUFFT_SUCCESS;
   const int N = s->cfg.n_mesh;
   if (s->fp64() || spline(s) || !spec_z_supported(N)) {
     *why = "not an fp32 cloud-in-cell simulation on a power-of-two mesh of 16..512";
@@ -639,6 +649,10 @@ cufftResult spec_plan_setup(pm_sim* s, std::string* why) {
   if (ce != cudaSuccess) {
     *why = std::string("tables: ") + cudaGetErrorString(ce);
     return CUFFT_SETUP_FAILED;
+  }
+  if (plane_fft_supported(N) || pass_fft_supported(N)) {
+    s->spec_ready = true;
+    return CUFFT_SUCCESS;
   }
   cufftHandle h[2] = {0, 0};
   const char* step = "cufftCreate";
@@ -672,7 +686,7 @@ cufftResult spec_plan_setup(pm_sim* s, std::string* why) {
   }
   s->plan2_fwd = h[0];
   s->plan2_inv = h[1];
-  s->have_plan2 = true;
+  s->have_plan2 = s->spec_ready = true;
   return CUFFT_SUCCESS;
 }
 
@@ -1191,7 +1205,8 @@ pm_status pm_create(const pm_config* c, void* dev_arena, size_t bytes, void* str
     std::string ignored;
     if (spec_plan_setup(s, &ignored) == CUFFT_SUCCESS) s->tune.green_fused = xy_fft_supported(N) ? 2 : 1;
   }
-  if (c->precision == PM_FP32 && c->kernel == PM_KERNEL_CIC && ((pass_fft_supported(N) && !spec_z_supported(N)) || (plane_fft_supported(N) && N < GREEN_FUSE_MIN_MESH)) &&
+  if (c->precision == PM_FP32 && c->kernel == PM_KERNEL_CIC &&
+      ((pass_fft_supported(N) && !spec_z_supported(N)) || (plane_fft_supported(N) && N < GREEN_FUSE_MIN_MESH)) &&
       (launch_spec_tables(s->at<float2>(L.green), s->at<float>(L.green + size_t(N) * 8), N, s->stream) != cudaSuccess ||
        cudaStreamSynchronize(s->stream) != cudaSuccess)) {
     cufftDestroy(s->plan_fwd);
@@ -1282,8 +1297,7 @@ static pm_status load_particles(pm_sim* s, const double* x, const double* p) {
     CU(s, cudaEventRecord(s->ev_p, s->side));
   }
   s->have_particles = true;
-  if (s->keys_marked)  // a drift whose re-sort did not run (an error between them): its counts are dropped
-    CU(s, cudaMemsetAsync(s->at<uint32_t>(s->L.tcount), 0, size_t(mover_count_words(s->n())) * 4, s->stream));
+  if (s->keys_marked) PMST(drop_mover_counts(s));
   s->sorted = s->fields_valid = s->keys_marked = false;
   return DISPATCH(s, sort_particles, s, nullptr, split ? dp : nullptr);
 }
@@ -1814,7 +1828,7 @@ pm_status pm_load(pm_sim* s, const void* host, size_t bytes) {
   CU(s, cudaMemcpyAsync(s->mom(), in + CKPT_HEADER + rb, rb, cudaMemcpyHostToDevice, s->stream));
   CU(s, cudaMemcpyAsync(s->keys, in + CKPT_HEADER + 2 * rb, size_t(s->n()) * 4, cudaMemcpyHostToDevice, s->stream));
   CU(s, cudaMemcpyAsync(s->sort_stats(), stats, sizeof stats, cudaMemcpyHostToDevice, s->stream));
-  CU(s, cudaMemsetAsync(s->at<uint32_t>(s->L.tcount), 0, size_t(mover_count_words(s->n())) * 4, s->stream));
+  PMST(drop_mover_counts(s));
   // sorted records: the deposit reads the row starts of the keys (integer, so the same as the re-sort's)
   if (h.flags & 1) {
     CU(s, cudaMemsetAsync(s->at<uint32_t>(s->L.row_start) + s->mesh.n2 + 1, 0, 4, s->stream));

@@ -4,8 +4,7 @@
 // latency-critical serving loop or a real-time thread cannot afford, and a
 // process that has already handed its whole device-memory budget to fixed
 // arenas has nothing left to allocate from.  This entry point therefore keeps
-// every temporary (particle records, sort keys and values, digit histograms,
-// look-back status words, row starts) in one file-scope static device array
+// every temporary (particle records, sort keys, row starts) in one file-scope static device array
 // of PM_NOALLOC_SCRATCH_BYTES, which every GPU that loads the library holds
 // until the process exits.  It calls no allocating routine, its own or a
 // library's.
@@ -47,8 +46,8 @@ bool g_ready[64];
 
 thread_local char g_msg[256];
 
-// the call's error bits to the caller's word (device or mapped host memory)
-// hands the call's error bits over and clears them for the next call
+// hands the call's error bits to the caller's word (device or mapped host
+// memory) and clears them for the next call
 __global__ void k_copy_error(uint32_t* err, uint32_t* out) {
   *out = *err;
   *err = 0;

@@ -6,7 +6,7 @@
 //                      passes (warp-aggregated shared atomics on integers).
 //   k_sort_pass      : one kernel per pass.  Each block takes the next tile
 //                      (RS_TILE keys, tile ids from an atomic counter), ranks
-//                      its keys stably (warp match + per-warp counters, tile
+//                      its keys stably (warp votes + per-warp counters, tile
 //                      order = warp, round, lane), publishes its per-digit
 //                      counts, and finds the global start of each digit for its
 //                      tile by decoupled look-back over the status words of
