@@ -288,6 +288,9 @@ struct pm_sim {
   // pm_run replays captured steps on its own stream, joined to `stream` by events
   cudaStream_t cap = nullptr;
   cudaEvent_t ev_in = nullptr, ev_out = nullptr;
+  // the captured steps' second branch (the stencil beside the transforms)
+  cudaStream_t branch = nullptr;
+  cudaEvent_t ev_rho = nullptr, ev_q = nullptr;
   // pm_set_particles copies the momenta on a stream of its own while the positions are sorted
   cudaStream_t side = nullptr;
   cudaEvent_t ev_x = nullptr, ev_p = nullptr;
@@ -502,10 +505,11 @@ pm_status stencil_stage(pm_sim* s, bool diag = false) {
   const Layout& L = s->L;
   const StencilParams sp = stencil_params(s, diag);
   s->krho_valid = diag || s->fp64() || s->cfg.lap != PM_LAP_COMPACT;  // the generic kernel always sums
+  // (scratch, fp64 only: the spectrum, free once both potentials are back from it)
   PROF(s, PM_STAGE_STENCIL);
   CU(s, launch_stencil<R>(s->at<R>(density_field(s)), s->mesh, sp, s->at<R>(s->direct ? L.rho : L.q), kr_part(s),
-                          s->at<uint32_t>(L.st_list), s->at<uint32_t>(L.st_count), s->errword(), s->arena + L.spec,
-                          s->stream));  // (the spectrum is free here: both potentials are back from it)
+                          s->at<uint32_t>(L.st_list), s->at<uint32_t>(L.st_count), s->errword(),
+                          s->arena + L.spec, s->stream));
   return PM_OK;
 }
 
@@ -712,12 +716,43 @@ pm_status krho_stage(pm_sim* s) {
   return quantum_stage<R>(s, true);
 }
 
+// In the captured steps of small fp32 meshes the cloud-in-cell stencil, which needs the density only, runs as a
+// second branch beside the transforms and so leaves the chain of launches.  Measured per step without -> with
+// (us): 16^3 30.3 -> 28.2, 32^3 38.0 -> 35.0, 64^3 31.7 -> 29.7, 96^3 61.7 -> 60.8, 128^3 64.5 -> 64.2,
+// 160^3 135.0 -> 135.0, 192^3 193.0 -> 190.9, 256^3 321.2 -> 322.6 (and no gain on 384^3 and 512^3): larger meshes
+// fill the chip with either.  fp64 has one queue for both, its own pipe: 64^3 172 -> 189.
+// Both ends are event waits, so the uncaptured odd step on the same stream takes it too.
+constexpr int FORK_MAX_MESH = 192;
+bool forks(const pm_sim* s) {
+  return !s->fp64() && s->cfg.n_mesh <= FORK_MAX_MESH && s->cfg.quantum && !spline(s) && s->cap &&
+         s->stream == s->cap && !s->prof_on;
+}
+template <typename R>
+pm_status fork_quantum(pm_sim* s) {
+  if (!forks(s)) return PM_OK;
+  CU(s, cudaEventRecord(s->ev_rho, s->stream));
+  CU(s, cudaStreamWaitEvent(s->branch, s->ev_rho, 0));
+  s->stream = s->branch;
+  const pm_status st = quantum_stage<R>(s);
+  s->stream = s->cap;
+  CU(s, cudaEventRecord(s->ev_q, s->branch));
+  return st;
+}
+// Q~ here, or the branch's end
+template <typename R>
+pm_status join_quantum(pm_sim* s) {
+  if (!forks(s)) return quantum_stage<R>(s);
+  CU(s, cudaStreamWaitEvent(s->stream, s->ev_q, 0));
+  return PM_OK;
+}
+
 // phi~ and Q~ from the density (cloud-in-cell kernel: the deposit; spline
 // kernel: the already smoothed density, whose force potential is smoothed
 // once more)
 template <typename R>
 pm_status mesh_from_density(pm_sim* s) {
   const Layout& L = s->L;
+  PMST(fork_quantum<R>(s));
   if (pass_fft(s)) {
     const int N = s->cfg.n_mesh, stages[3] = {PM_STAGE_FFT_R2C, PM_STAGE_GREEN, PM_STAGE_FFT_C2R};
     for (int k = 0; k < 3; ++k) {
@@ -726,7 +761,7 @@ pm_status mesh_from_density(pm_sim* s) {
                             s->at<float>(L.green + size_t(N) * 8), N, green_coef(s), wg_part(s), s->stream));
     }
     s->wg_count = pass_fft_tiles(N);
-    PMST(quantum_stage<R>(s));
+    PMST(join_quantum<R>(s));
     s->fields_valid = true;
     return PM_OK;
   }
@@ -756,7 +791,7 @@ pm_status mesh_from_density(pm_sim* s) {
       else
         CF(s, cufftExecC2R(s->plan2_inv, (cufftComplex*)(s->arena + L.spec), s->at<cufftReal>(L.phi)));
     }
-    PMST(quantum_stage<R>(s));
+    PMST(join_quantum<R>(s));
     s->fields_valid = true;
     return PM_OK;
   }
@@ -771,7 +806,7 @@ pm_status mesh_from_density(pm_sim* s) {
   }
   s->wg_count = int(green_blocks(s->cfg.n_mesh));
   PMST(fft_c2r<R>(s, s->arena + L.spec, s->arena + L.phi));
-  PMST(quantum_stage<R>(s));
+  PMST(join_quantum<R>(s));
   s->fields_valid = true;
   return PM_OK;
 }
@@ -1247,6 +1282,10 @@ pm_status pm_destroy(pm_sim* s) {
     cudaEventDestroy(s->ev_out);
     cudaEventDestroy(s->ev_tab);
     cudaFreeHost(s->tab_host);
+    cudaStreamSynchronize(s->branch);
+    cudaStreamDestroy(s->branch);
+    cudaEventDestroy(s->ev_rho);
+    cudaEventDestroy(s->ev_q);
   }
   if (s->side) {
     cudaStreamSynchronize(s->side);
@@ -1460,6 +1499,9 @@ pm_status pm_run(pm_sim* s, int32_t nsteps, double a_start, double a_end) {
       CU(s, cudaEventCreateWithFlags(&s->ev_in, cudaEventDisableTiming));
       CU(s, cudaEventCreateWithFlags(&s->ev_out, cudaEventDisableTiming));
       CU(s, cudaEventCreateWithFlags(&s->ev_tab, cudaEventDisableTiming));
+      CU(s, cudaStreamCreateWithFlags(&s->branch, cudaStreamNonBlocking));
+      CU(s, cudaEventCreateWithFlags(&s->ev_rho, cudaEventDisableTiming));
+      CU(s, cudaEventCreateWithFlags(&s->ev_q, cudaEventDisableTiming));
       CU(s, cudaMallocHost(&s->tab_host, size_t(PM_RUN_GRAPH_MAX_STEPS) * sizeof(KickParams)));
     }
     if (s->tab_pending) CU(s, cudaEventSynchronize(s->ev_tab));  // the previous upload has left the buffer
