@@ -341,9 +341,9 @@ def measure(pm, sim, w, K, W, stream, rsz=4, spline=False, tuning=None, peak=Non
                            "bytes_per_launch": b, "GBps": (b / (avg / 1e3) / 1e9) if b else None}
     # the transform stages are cuFFT's, except with the fused x-y kernels of 256^3 meshes (green_fused = 2, and
     # the fp32 spline runs on such meshes)
-    # and, pass by pass, of 384^3 and (green_fused = 1) 512^3 meshes
+    # and, pass by pass, of (green_fused = 1) 512^3 meshes
     own_xy = sim.get_tuning().get("green_fused") == 2 or (spline and rsz == 4 and nm == 256)
-    own_passes = rsz == 4 and not spline and (nm == 384 or (nm == 512 and sim.get_tuning().get("green_fused") == 1))
+    own_passes = rsz == 4 and not spline and nm == 512 and sim.get_tuning().get("green_fused") == 1
     lib_stages = () if own_xy or own_passes else pm.CUFFT_STAGES
     names = dict(KERNEL_NAMES, **({"fft_r2c": "k_xy_r2c", "fft_c2r": "k_xy_c2r"} if own_xy else
                                   {"fft_r2c": "k_x_r2c+k_y_forward", "green": "k_z_green",

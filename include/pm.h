@@ -224,8 +224,8 @@ typedef struct {
                               once instead of three times; the default from 128^3); 2 (256^3 meshes only, their
                               default) does the same with the x and y transforms of each plane in one kernel per
                               direction (a cluster of CTAs per plane); 0 uses the 3D transforms and a separate
-                              Green pass, except on 64^3 meshes, which take the plane kernels all the same (and so
-                              do 384^3 ones their own).  The potential agrees to fp32 rounding in every mode */
+                              Green pass, except on 64^3 meshes, which take the plane kernels all the same.  The
+                              potential agrees to fp32 rounding in every mode */
 } pm_tuning;
 
 /* Current shapes. */

@@ -215,7 +215,7 @@ Layout make_layout(const pm_config& c, size_t work_bytes) {
   // per-step kick weights of pm_run and of a batch run
   L.ktab = take(size_t(std::max(PM_RUN_GRAPH_MAX_STEPS, PM_BATCH_MAX_STEPS)) * sizeof(KickParams));
   // the z transform's twiddles and the Green's sin^2 table (fp32 cloud-in-cell, power-of-two meshes)
-  L.green = take(c.precision == PM_FP32 && (spline ? xy_fft_supported(int(N)) : (spec_z_supported(int(N)) || pass_fft_supported(int(N))))
+  L.green = take(c.precision == PM_FP32 && (spline ? xy_fft_supported(int(N)) : spec_z_supported(int(N)))
                      ? N * 12 : 0);
   L.sin2 = take(N * rsz);  // sin^2(pi j / N) for the flat Green passes
   L.total = off;
@@ -610,11 +610,10 @@ double green_coef(const pm_sim* s) {
   return -1.5 * s->cfg.omega_m * s->dx * s->dx / (4.0 * N * N * N);
 }
 
-// fp32 cloud-in-cell on 384^3 and 512^3: the transforms pass by pass.  On 512^3 they are the plane transforms of
-// green_fused = 1 (0: cuFFT's 3D transforms); 384^3, no power of two, has no such choice and always takes them
+// fp32 cloud-in-cell on 512^3: the transforms pass by pass, the plane transforms of green_fused = 1 (0: cuFFT's 3D
+// transforms)
 bool pass_fft(const pm_sim* s) {
-  return !s->fp64() && s->cfg.kernel == PM_KERNEL_CIC && pass_fft_supported(s->cfg.n_mesh) &&
-         (!spec_z_supported(s->cfg.n_mesh) || s->tune.green_fused == 1);
+  return !s->fp64() && s->cfg.kernel == PM_KERNEL_CIC && pass_fft_supported(s->cfg.n_mesh) && s->tune.green_fused == 1;
 }
 
 // fp32 cloud-in-cell on 64^3 and 128^3: the x-y transforms of a plane in one CTA.  On 128^3 they are the plane
@@ -1240,8 +1239,7 @@ pm_status pm_create(const pm_config* c, void* dev_arena, size_t bytes, void* str
     std::string ignored;
     if (spec_plan_setup(s, &ignored) == CUFFT_SUCCESS) s->tune.green_fused = xy_fft_supported(N) ? 2 : 1;
   }
-  if (c->precision == PM_FP32 && c->kernel == PM_KERNEL_CIC &&
-      ((pass_fft_supported(N) && !spec_z_supported(N)) || (plane_fft_supported(N) && N < GREEN_FUSE_MIN_MESH)) &&
+  if (c->precision == PM_FP32 && c->kernel == PM_KERNEL_CIC && plane_fft_supported(N) && N < GREEN_FUSE_MIN_MESH &&
       (launch_spec_tables(s->at<float2>(L.green), s->at<float>(L.green + size_t(N) * 8), N, s->stream) != cudaSuccess ||
        cudaStreamSynchronize(s->stream) != cudaSuccess)) {
     cufftDestroy(s->plan_fwd);

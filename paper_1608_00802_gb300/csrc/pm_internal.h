@@ -179,7 +179,7 @@ inline size_t row_scan_tiles(int n_mesh) { return (size_t(n_mesh) * n_mesh + 102
 bool plane_fft_supported(int n);
 cudaError_t launch_plane_fft(bool inverse, float* mesh, void* spec, const float2* tw, int n, cudaStream_t s, int nm = 1,
                              size_t ms = 0);
-// phi~ from the density on 384^3 and 512^3 fp32 meshes, transform by transform: stage 0 the x and y transforms
+// phi~ from the density on 512^3 fp32 meshes, transform by transform: stage 0 the x and y transforms
 // (through phi, as scratch), 1 the z transforms with the Green multiplication (one W_g partial per tile), 2 the
 // inverse y and x transforms.  tw, s2: the tables of launch_spec_tables
 bool pass_fft_supported(int n);

@@ -865,8 +865,7 @@ static __global__ void k_spec_tables(float2* tw, float* s2, int n) {
     double sv, cv;
     sincospi(2.0 * double(t) / double(n), &sv, &cv);
     tw[t] = make_float2(float(cv), float(-sv));
-    // (the index folded to N/2: t / N next to 1 has lost the digits of 1 - t / N where N is no power of two)
-    s2[t] = sinpi_sq(float(t <= n - t ? t : n - t) * inv_n);
+    s2[t] = sinpi_sq(float(t) * inv_n);
   }
 }
 

@@ -102,7 +102,7 @@ bool spec_z_supported(int n) { return n >= 16 && n <= 512 && (n & (n - 1)) == 0;
 int spec_z_tiles(int n) { return n * (n / 2 + 1) / SPZ_COLS; }
 
 cudaError_t launch_spec_tables(float2* tw, float* s2, int n, cudaStream_t s) {
-  if (!spec_z_supported(n) && !pass_fft_supported(n)) return cudaErrorInvalidValue;
+  if (!spec_z_supported(n)) return cudaErrorInvalidValue;
   k_spec_tables<<<(n + 255) / 256, 256, 0, s>>>(tw, s2, n);
   return cudaGetLastError();
 }

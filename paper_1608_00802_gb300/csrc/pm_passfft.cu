@@ -1,76 +1,32 @@
-// The mesh transforms of 384^3 and 512^3 fp32 meshes as five passes over memory (cloud-in-cell; other sizes
-// have the x-y kernels or cuFFT):
+// The mesh transforms of 512^3 fp32 meshes as five passes over memory (cloud-in-cell; other sizes have the x-y
+// kernels, the plane kernels or cuFFT):
 //   x  forward : each row of N reals -> N/2 complex, X[0] + i X[N/2] packed first  (rho -> tmp)
 //   y  forward : 8 columns of a z-plane per block, the packed column split          (tmp -> spectrum)
 //   z          : 16 columns of the half spectrum per block, Green multiplication, W_g partial, back (in place)
 //   y  inverse : the columns packed again                                           (spectrum -> tmp)
 //   x  inverse : each row back to N reals                                           (tmp, in place)
-// tmp is the potential's mesh: N/2 complex values are a row of it.  A plane of these meshes (0.6 and 1 MB)
-// does not fit the cluster that the 256^2 x-y kernels use, and cuFFT's passes are far from the copy rate: on a
-// 384^3 mesh 906 us for its 3D pair plus 81 for the Green pass (a pass over memory takes 68 us), on 512^3
-// 996 us for its 2D pair plus 504 for the four-step z kernel at one block of 128 registers per SM (160 us a
-// pass).  So each pass here does as little as it can per value and leaves room for many threads: the five
-// passes take 530 us on 384^3 and 1200 us on 512^3.  The potential's error against float64 (particle
-// density, of the largest |phi|): 384^3 4.2e-6 -> 6.1e-7 (the Green table folds its index), 512^3 4.7e-7 ->
-// 4.1e-7.
+// tmp is the potential's mesh: N/2 complex values are a row of it.  A plane (1 MB) does not fit the cluster that
+// the 256^2 x-y kernels use, and cuFFT's passes are far from the copy rate: 996 us for its 2D pair plus 504 for
+// the four-step z kernel at one block of 128 registers per SM (a pass over memory takes 160 us).  So each pass here
+// does as little as it can per value and leaves room for many threads: the five passes take 1193 us.  The
+// potential's error against float64 (particle density, of the largest |phi|): 4.7e-7 -> 4.0e-7.  (384^3 by the
+// same passes: 535 us against 987 by cuFFT's 3D pair and the Green pass, but in one run of a hundred the
+// other rounding moved particles next to nearly empty nodes by more than 1e-3: it keeps cuFFT.)
 //
 // Rows: 16 threads a row (two rows a warp: the exchanges need no block barrier), H = N/2 = 16 Q points in two
-// steps, n = j + 16 m and k = k1 + Q k2: thread j a Q-point DFT over m (Q = 12, 16) and the twiddle, thread
-// k1 < Q a 16-point DFT over j.  Columns: N = 8 * 8 * C points in three steps (C = 6, 8), n = j + 8 C m,
+// steps, n = j + 16 m and k = k1 + Q k2: thread j a Q-point DFT over m (Q = 16) and the twiddle, thread
+// k1 < Q a 16-point DFT over j.  Columns: N = 8 * 8 * C points in three steps (C = 8), n = j + 8 C m,
 // j = j' + C m', k = k1 + 8 (k2 + 8 k3): thread j an 8-point DFT over m and W_N^{j k1}, thread (k1, j') an
 // 8-point DFT over m' and W_{8C}^{j' k2}, thread (k1, k2) a C-point DFT over j'; eight values and ~40
 // registers a thread.  Slots of the exchange tile are padded by one in C, so that the third step's stride of
-// C slots does not meet one bank group (the z kernel's slots are whole bank rows).  Inverses run the same steps backwards with conjugate twiddles.
+// C slots does not meet one bank group (the z kernel's slots are whole bank rows).  Inverses run the same steps
+// backwards with conjugate twiddles.
 #include <atomic>
 
 #include "pm_kernels.cuh"
 
 namespace pm {
 namespace {
-
-// exp(-+2 pi i t / 12) times a (forward: minus), t < 8 known at compile time after unrolling
-template <bool INV>
-__device__ __forceinline__ float2 twiddle12(float2 a, int t) {
-  constexpr float s60 = 0.866025388f;  // sin(pi / 3)
-  constexpr float c[7] = {1.0f, s60, 0.5f, 0.0f, -0.5f, -s60, -1.0f}, s[7] = {0.0f, 0.5f, s60, 1.0f, s60, 0.5f, 0.0f};
-  if (t == 0) return a;
-  if (t == 3) return INV ? make_float2(-a.y, a.x) : make_float2(a.y, -a.x);
-  return cmul(a, make_float2(c[t], INV ? s[t] : -s[t]));
-}
-
-// M-point DFT in registers: dft_reg for powers of two, one radix-3 step before it for M = 3 L; natural order
-// in, X[k] at a[dft_at<M>(k)]
-template <int M>
-__host__ __device__ constexpr int dft_at(int k) {
-  return M % 3 ? bitrev<M>(k) : (M / 3) * (k % 3) + bitrev<M / 3>(k / 3);
-}
-template <int M, bool INV>
-__device__ __forceinline__ void dft_any(float2 (&a)[M]) {
-  if constexpr (M % 3) {
-    dft_reg<M, INV>(a);
-  } else {
-    constexpr int L = M / 3;
-    constexpr float s60 = INV ? 0.866025388f : -0.866025388f;
-#pragma unroll
-    for (int j = 0; j < L; ++j) {
-      const float2 u = a[j], v = a[j + L], w = a[j + 2 * L];
-      const float2 p = make_float2(v.x + w.x, v.y + w.y), d = make_float2(v.x - w.x, v.y - w.y);
-      const float2 h = make_float2(fmaf(-0.5f, p.x, u.x), fmaf(-0.5f, p.y, u.y));
-      a[j] = make_float2(u.x + p.x, u.y + p.y);
-      a[j + L] = twiddle12<INV>(make_float2(fmaf(-s60, d.y, h.x), fmaf(s60, d.x, h.y)), j * (4 / L));
-      a[j + 2 * L] = twiddle12<INV>(make_float2(fmaf(s60, d.y, h.x), fmaf(-s60, d.x, h.y)), 2 * j * (4 / L));
-    }
-#pragma unroll
-    for (int r = 0; r < 3; ++r) {
-      float2 b[L];
-#pragma unroll
-      for (int j = 0; j < L; ++j) b[j] = a[L * r + j];
-      dft_reg<L, INV>(b);
-#pragma unroll
-      for (int j = 0; j < L; ++j) a[L * r + j] = b[j];
-    }
-  }
-}
 
 __device__ __forceinline__ float2 conj2(float2 a) { return make_float2(a.x, -a.y); }
 
@@ -95,9 +51,9 @@ __global__ void __launch_bounds__(PX_THREADS, 4) k_x_r2c(const float* __restrict
     float2 a[Q];
 #pragma unroll
     for (int m = 0; m < Q; ++m) a[m] = __ldcs(src + j + 16 * m);
-    dft_any<Q, false>(a);
+    dft_reg<Q, false>(a);
 #pragma unroll
-    for (int k1 = 0; k1 < Q; ++k1) s[px_pad(j + 16 * k1)] = cmul(a[dft_at<Q>(k1)], __ldg(tw + 2 * j * k1));
+    for (int k1 = 0; k1 < Q; ++k1) s[px_pad(j + 16 * k1)] = cmul(a[bitrev<Q>(k1)], __ldg(tw + 2 * j * k1));
   }
   __syncwarp();
   float2 b[16];
@@ -147,10 +103,10 @@ __global__ void __launch_bounds__(PX_THREADS, 4) k_x_c2r(float2* mesh, const flo
     const float2 d = cmul(make_float2(x[m].x - xp.x, x[m].y + xp.y), conj2(__ldg(tw + k)));
     x[m] = k ? make_float2(x[m].x + xp.x - d.y, x[m].y - xp.y + d.x) : make_float2(x[m].x + x[m].y, x[m].x - x[m].y);
   }
-  dft_any<Q, true>(x);
+  dft_reg<Q, true>(x);
   __syncwarp();
 #pragma unroll
-  for (int k1 = 0; k1 < Q; ++k1) s[px_pad(j + 16 * k1)] = cmul(x[dft_at<Q>(k1)], conj2(__ldg(tw + 2 * j * k1)));
+  for (int k1 = 0; k1 < Q; ++k1) s[px_pad(j + 16 * k1)] = cmul(x[bitrev<Q>(k1)], conj2(__ldg(tw + 2 * j * k1)));
   __syncwarp();
   if (j < Q) {
     float2 b[16];
@@ -192,7 +148,7 @@ __device__ __forceinline__ void cols_forward(float2 (&a)[8], float2* T, const fl
   for (int k2 = 0; k2 < 8; ++k2) T[pc_slot<N>(k1 * BC + k2 * C + jp) + c] = cmul(a[bitrev<8>(k2)], __ldg(tw + 8 * jp * k2));
   __syncthreads();
 }
-// the last two steps of the inverse, from the tile that the first one filled: a[dft_at(m)] = x[j + BC m]
+// the last two steps of the inverse, from the tile that the first one filled: a[bitrev(m)] = x[j + BC m]
 template <int N>
 __device__ __forceinline__ void cols_inverse(float2 (&a)[8], float2* T, const float2* __restrict__ tw, int c, int j) {
   constexpr int C = ColShape<N>::C, BC = ColShape<N>::BC;
@@ -232,11 +188,11 @@ __global__ void __launch_bounds__(ColShape<N>::THREADS, ColShape<N>::MINB) k_y_f
     float2 b[C];
 #pragma unroll
     for (int i = 0; i < C; ++i) b[i] = T[pc_slot<N>(k1 * BC + k2 * C + i) + c];
-    dft_any<C, false>(b);
+    dft_reg<C, false>(b);
 #pragma unroll
     for (int k3 = 0; k3 < C; ++k3) {
       const int ky = k1 + 8 * (k2 + 8 * k3);
-      const float2 v = b[dft_at<C>(k3)];
+      const float2 v = b[bitrev<C>(k3)];
       if (!packed || c) dst[ky * NH] = v;
       // (the slots this thread has read are its own: the packed column waits there for its mirror)
       if (packed && c == 0) T[pc_slot<N>(k1 * BC + k2 * C + k3)] = v;
@@ -278,10 +234,10 @@ __global__ void __launch_bounds__(ColShape<N>::THREADS, ColShape<N>::MINB) k_y_i
         b[k3] = make_float2(b[k3].x - h.y, b[k3].y + h.x);
       }
     }
-    dft_any<C, true>(b);
+    dft_reg<C, true>(b);
 #pragma unroll
     for (int i = 0; i < C; ++i)
-      T[pc_slot<N>(k1 * BC + k2 * C + i) + c] = cmul(b[dft_at<C>(i)], conj2(__ldg(tw + 8 * i * k2)));
+      T[pc_slot<N>(k1 * BC + k2 * C + i) + c] = cmul(b[bitrev<C>(i)], conj2(__ldg(tw + 8 * i * k2)));
   }
   float2 a[8];
   cols_inverse<N>(a, T, tw, c, j);
@@ -296,9 +252,9 @@ __global__ void __launch_bounds__(ColShape<N>::THREADS, ColShape<N>::MINB) k_y_i
 // (im0, im1) in 64-bit registers: the packed fp32 instructions (add, sub, mul, fma .f32x2) do both columns at
 // once, a pair of values is one 16-byte access of memory or shared memory, and twiddles and addresses serve two.
 // With one column a thread and 8 columns a block the kernel was bound by its instructions and by 64-byte
-// segments: 400 -> 327 us on 512^3, 168 -> 136 on 384^3 (two passes over memory take 160 and 68).  Pairs in blocks
-// of 8 columns take 369 and 158; the y passes do not gain by pairs, because a spectrum row starts on 8 bytes
-// only (inverse 235 -> 295 on 512^3, forward 235 -> 239), nor does the z kernel of 256^3 (33 -> 37).
+// segments: 400 -> 327 us (two passes over memory take 160).  Pairs in blocks of 8 columns take 369; the y passes
+// do not gain by pairs, because a spectrum row starts on 8 bytes only (inverse 235 -> 295, forward 235 -> 239), nor
+// does the z kernel of 256^3 (33 -> 37).
 using u64 = unsigned long long;
 __device__ __forceinline__ u64 pk2(float a, float b) {
   u64 d;
@@ -379,39 +335,10 @@ __device__ __forceinline__ void c2_dft_pow2(C2* a) {
     }
   }
 }
-// M = 4, 6, 8; X[k] at a[dft_at<M>(k)]
-template <int M, bool INV>
-__device__ __forceinline__ void c2_dft(C2 (&a)[M]) {
-  if constexpr (M == 6) {  // radix 3, twiddles exp(-+2 pi i j r / 6), then three 2-point DFTs
-    const float sg = INV ? 1.0f : -1.0f;
-    const u64 s60 = pk2(sg * 0.866025388f, sg * 0.866025388f), ms60 = pk2(-sg * 0.866025388f, -sg * 0.866025388f);
-    const u64 hf = pk2(0.5f, 0.5f), mhf = pk2(-0.5f, -0.5f);
-#pragma unroll
-    for (int j = 0; j < 2; ++j) {
-      const C2 u = a[j], v = a[j + 2], w = a[j + 4];
-      const C2 p = {add2(v.re, w.re), add2(v.im, w.im)}, d = {sub2(v.re, w.re), sub2(v.im, w.im)};
-      const C2 h = {fma2(mhf, p.re, u.re), fma2(mhf, p.im, u.im)};
-      a[j] = {add2(u.re, p.re), add2(u.im, p.im)};
-      C2 r1 = {fma2(ms60, d.im, h.re), fma2(s60, d.re, h.im)}, r2 = {fma2(s60, d.im, h.re), fma2(ms60, d.re, h.im)};
-      if (j) {  // times (1/2, -+sin 60), (-1/2, -+sin 60)
-        r1 = {fma2(ms60, r1.im, mul2(hf, r1.re)), fma2(s60, r1.re, mul2(hf, r1.im))};
-        r2 = {fma2(ms60, r2.im, mul2(mhf, r2.re)), fma2(s60, r2.re, mul2(mhf, r2.im))};
-      }
-      a[j + 2] = r1;
-      a[j + 4] = r2;
-    }
-    c2_dft_pow2<2, INV>(a);
-    c2_dft_pow2<2, INV>(a + 2);
-    c2_dft_pow2<2, INV>(a + 4);
-  } else {
-    c2_dft_pow2<M, INV>(a);
-  }
-}
-
 constexpr int ZC_COLS = 16, ZC_PAIRS = ZC_COLS / 2;
 template <int N>
 struct ZShape {
-  static constexpr int C = N / 64, BC = 8 * C, THREADS = ZC_PAIRS * BC, MINB = 1024 / THREADS + (N == 384);
+  static constexpr int C = N / 64, BC = 8 * C, THREADS = ZC_PAIRS * BC, MINB = 1024 / THREADS;
   // the exchange tile [slot][pair] (a quarter warp's 16-byte accesses are one slot: no padding), the twiddles as
   // (wx, wx, wy, wy), the Green table
   static constexpr size_t smem() { return size_t(N) * (ZC_PAIRS * 16 + 16 + 4); }
@@ -494,11 +421,11 @@ __global__ void __launch_bounds__(ZShape<N>::THREADS, ZShape<N>::MINB) k_z_green
     C2 b[C], d[C];
 #pragma unroll
     for (int i = 0; i < C; ++i) b[i] = c2_ld(s + i * ZC_PAIRS);
-    c2_dft<C, false>(b);
+    c2_dft_pow2<C, false>(b);
 #pragma unroll
     for (int k3 = 0; k3 < C; ++k3) {
       const int kz = k1 + 8 * (k2 + 8 * k3);
-      const C2 v = b[dft_at<C>(k3)];
+      const C2 v = b[bitrev<C>(k3)];
       const float sz = s2[kz];
       const float syz0 = sy0 + sz, syz1 = sy1 + sz;
       const float sum0 = syz0 + sx0, sum1 = syz1 + sx1;
@@ -506,9 +433,9 @@ __global__ void __launch_bounds__(ZShape<N>::THREADS, ZShape<N>::MINB) k_z_green
       wsum = fma2(mul2(w2, g), fma2(v.re, v.re, mul2(v.im, v.im)), wsum);
       d[k3] = {mul2(v.re, g), mul2(v.im, g)};
     }
-    c2_dft<C, true>(d);
+    c2_dft_pow2<C, true>(d);
 #pragma unroll
-    for (int i = 0; i < C; ++i) c2_st(s + i * ZC_PAIRS, c2_mul<true>(d[dft_at<C>(i)], W[8 * i * k2]));
+    for (int i = 0; i < C; ++i) c2_st(s + i * ZC_PAIRS, c2_mul<true>(d[bitrev<C>(i)], W[8 * i * k2]));
   }
   zc_inverse<N>(a, T, W, c, j);
   float4* dst = reinterpret_cast<float4*>(spec + col);
@@ -554,13 +481,12 @@ cudaError_t pass_potential(const float* rho, float* phi, float2* spec, const flo
 
 }  // namespace
 
-bool pass_fft_supported(int n) { return n == 384 || n == 512; }
+bool pass_fft_supported(int n) { return n == 512; }
 int pass_fft_tiles(int n) { return n * (n / 2 + 1) / ZC_COLS; }
 
 cudaError_t launch_pass_fft(int stage, const float* rho, float* phi, void* spec, const float2* tw, const float* s2, int n,
                             double coef, double* part, cudaStream_t s) {
   switch (n) {
-    case 384: return pass_potential<384>(rho, phi, static_cast<float2*>(spec), tw, s2, float(coef), part, s, stage);
     case 512: return pass_potential<512>(rho, phi, static_cast<float2*>(spec), tw, s2, float(coef), part, s, stage);
     default: return cudaErrorInvalidValue;
   }

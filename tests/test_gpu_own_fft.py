@@ -1,6 +1,5 @@
-"""The transforms of 64^3 and 128^3 meshes (a CTA per plane) and of 384^3 and 512^3 meshes
-(pass by pass): a particle density's potential
-against the same Poisson solve in float64, plane waves on the packed columns and at the edges of
+"""The transforms of 64^3 and 128^3 meshes (a CTA per plane) and of 512^3 meshes (pass by pass):
+a particle density's potential against the same Poisson solve in float64, plane waves on the packed columns and at the edges of
 the column tiles in closed form, the gravitational energy (one partial per tile), and
 packed batch members against single runs."""
 import numpy as np
@@ -27,7 +26,7 @@ def _sim(pm, n_mesh, box=2.0, **kw):
     return sim
 
 
-@pytest.mark.parametrize("n_mesh", [64, 128, 384, 512])
+@pytest.mark.parametrize("n_mesh", [64, 128, 512])
 def test_potential_of_particles_against_float64(pm, n_mesh):
     """Every mode at once: the density of random particles, as the other transforms are tested on."""
     import torch
@@ -45,7 +44,7 @@ def test_potential_of_particles_against_float64(pm, n_mesh):
     sim.close()
 
 
-@pytest.mark.parametrize("n_mesh", [64, 128, 384, 512])
+@pytest.mark.parametrize("n_mesh", [64, 128, 512])
 def test_plane_waves(pm, n_mesh):
     N, box, dx = n_mesh, 2.0, 2.0 / n_mesh
     h = N // 2
@@ -63,7 +62,7 @@ def test_plane_waves(pm, n_mesh):
     sim.close()
 
 
-@pytest.mark.parametrize("n_mesh", [64, 128, 384])
+@pytest.mark.parametrize("n_mesh", [64, 128])
 def test_energy_of_the_tiles(pm, n_mesh):
     """W_g from the z pass's partials against the sum over the mesh."""
     rng = np.random.default_rng(2)
@@ -78,7 +77,7 @@ def test_energy_of_the_tiles(pm, n_mesh):
     sim.close()
 
 
-@pytest.mark.parametrize("n_mesh", [64, 128, 384])
+@pytest.mark.parametrize("n_mesh", [64, 128])
 def test_batch_members_equal_single_runs(pm, n_mesh):
     rng = np.random.default_rng(4)
     n, N = 70000, n_mesh
