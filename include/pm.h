@@ -261,6 +261,14 @@ enum {
  * usable.  Needs more than 2048 particles.  Sync. */
 pm_status pm_debug_sort_timeout(pm_sim* sim, int32_t spin_limit);
 
+/* Test aid for the recovery from a failed launch: the simulation's next incremental
+ * re-sort returns PM_ERR_CUDA before its kernel group `part` (0 the partition, 1 the
+ * rows, 2 the placement; -1 takes the request back), once, as if that launch
+ * had failed.  Nothing else changes: the drift's particles and keys stay, and
+ * the next call that needs them in order sorts them in full.  Not for batch runs'
+ * packed classes.  Async. */
+pm_status pm_debug_fail_resort(pm_sim* sim, int32_t part);
+
 /* Incremental re-sorts since pm_create (one per drift of the particles) and
  * the particles they moved to another cell, summed on the device.  Sync. */
 pm_status pm_sort_stats(pm_sim* sim, int64_t* resorts, int64_t* movers);

@@ -262,6 +262,8 @@ struct pm_sim {
   uint32_t* keys;  // sorted (current) keys
   uint32_t* keys_tmp[2];
   bool keys_marked = false;  // a drift has flagged the movers in `keys` since the last sort
+  bool resort_open = false;  // and a re-sort of them has begun (an error stopped it)
+  int fail_resort = -1;      // test aid: the re-sort kernel group whose launch "fails" next
   Tuning tune;                // launch shapes
   // spline kernel smoothed in real space (fp32, support within three cells):
   // the smoothed density lives in the spec2 region, and `rho` holds the
@@ -366,6 +368,11 @@ struct ProfScope {
     cudaError_t e_ = (expr);                                                                     \
     if (e_ != cudaSuccess) return fail(sim, PM_ERR_CUDA, "%s: %s", #expr, cudaGetErrorString(e_)); \
   } while (0)
+#define PMST(expr)                  \
+  do {                              \
+    pm_status st_ = (expr);         \
+    if (st_ != PM_OK) return st_;   \
+  } while (0)
 #define CF(sim, expr)                                                                      \
   do {                                                                                     \
     cufftResult r_ = (expr);                                                               \
@@ -389,6 +396,25 @@ int kr_blocks(const pm_sim* s) {
   return tiled ? stencil_launch_blocks(s->cfg.n_mesh, s->tune.st_ty, s->tune.st_zlen) : MESH_GRID;
 }
 
+// the counts of a drift whose re-sort did not run, or not to its end (an error between them)
+pm_status drop_mover_counts(pm_sim* s) {
+  const size_t N = size_t(s->cfg.n_mesh);
+  CU(s, cudaMemsetAsync(s->at<uint32_t>(s->L.tcount), 0, size_t(mover_count_words(s->n())) * 4, s->stream));
+  CU(s, cudaMemsetAsync(s->at<uint32_t>(s->L.rcnt), 0, size_t(3) * N * N * 4, s->stream));
+  return PM_OK;
+}
+
+// A drift's marks without counts to re-sort by (loaded from a checkpoint, or a re-sort stopped half way: the
+// partition would place its tiles by counts that are not this drift's, or count rows twice): the keys lose their marks
+// and the full sort takes them.  It is stable too, so the order is the re-sort's.  The records and keys are
+// still the drift's: only the re-sort's last kernel writes them.
+pm_status unmark_movers(pm_sim* s) {
+  PMST(drop_mover_counts(s));
+  CU(s, launch_unmark_keys(s->keys, s->n(), s->stream));
+  s->keys_marked = s->resort_open = false;
+  return PM_OK;
+}
+
 // Incremental re-sort after a drift: the stayers are still in order, so every
 // particle's place follows from the stayers and movers of its mesh row (stable
 // partition with per-row counts, a scan of the rows, the movers in per-row
@@ -402,6 +428,11 @@ pm_status resort_movers(pm_sim* s, uint32_t* step) {
   const int nxt = s->cur ^ 1;
   const int stages[3] = {PM_STAGE_SORT_PARTITION, PM_STAGE_SORT_PASS, PM_STAGE_SORT_MERGE};
   for (int part = 0; part < 3; ++part) {
+    if (part == s->fail_resort) {  // (pm_debug_fail_resort)
+      s->fail_resort = -1;
+      return fail(s, PM_ERR_CUDA, "re-sort: injected launch failure");
+    }
+    s->resort_open = true;
     PROF(s, stages[part]);
     CU(s, launch_resort<R>(part, s->keys, s->n(), s->at<uint32_t>(L.tcount), s->keys_tmp[0],
                            s->at<uint32_t>(L.vals[0]), s->keys_tmp[1], s->at<uint32_t>(L.vals[1]),
@@ -411,14 +442,17 @@ pm_status resort_movers(pm_sim* s, uint32_t* step) {
                            s->keys, s->pos(), s->mom(), s->arena + L.pos[nxt], s->arena + L.mom[nxt], s->sms, s->stream));
   }
   s->cur = nxt;
-  s->keys_marked = false;
+  s->keys_marked = s->resort_open = false;
   s->sorted = true;
   return PM_OK;
 }
 
 template <typename R>
 pm_status sort_particles(pm_sim* s, uint32_t* step = nullptr, const double* p_in = nullptr) {
-  if (s->keys_marked) return resort_movers<R>(s, step);
+  if (s->keys_marked) {
+    if (!s->resort_open) return resort_movers<R>(s, step);
+    PMST(unmark_movers(s));
+  }
   const Layout& L = s->L;
   const int64_t n = s->n();
   if (n <= SORT_SMALL_MAX) {  // one kernel, the keys in place
@@ -536,12 +570,6 @@ pm_status fft_c2r(pm_sim* s, void* in, void* out) {
   return PM_OK;
 }
 
-#define PMST(expr)                  \
-  do {                              \
-    pm_status st_ = (expr);         \
-    if (st_ != PM_OK) return st_;   \
-  } while (0)
-
 bool spline(const pm_sim* s) { return s->cfg.kernel == PM_KERNEL_SPLINE; }
 
 // the normalised node weights of the spline at squared distance i^2 + s (in
@@ -626,14 +654,6 @@ bool plane_fft(const pm_sim* s) {
 
 // the Green multiplication inside the z transform, between batched 2D transforms
 bool green_fused(const pm_sim* s) { return s->tune.green_fused && s->spec_ready; }
-
-// the counts of a drift whose re-sort did not run, or not to its end (an error between them)
-pm_status drop_mover_counts(pm_sim* s) {
-  const size_t N = size_t(s->cfg.n_mesh);
-  CU(s, cudaMemsetAsync(s->at<uint32_t>(s->L.tcount), 0, size_t(mover_count_words(s->n())) * 4, s->stream));
-  CU(s, cudaMemsetAsync(s->at<uint32_t>(s->L.rcnt), 0, size_t(3) * N * N * 4, s->stream));
-  return PM_OK;
-}
 
 // The batched 2D transforms of the N z planes (forward: the real density to
 // the (ky, kx) half planes; inverse: back to the real potential), sharing the
@@ -1335,7 +1355,7 @@ static pm_status load_particles(pm_sim* s, const double* x, const double* p) {
   }
   s->have_particles = true;
   if (s->keys_marked) PMST(drop_mover_counts(s));
-  s->sorted = s->fields_valid = s->keys_marked = false;
+  s->sorted = s->fields_valid = s->keys_marked = s->resort_open = false;
   return DISPATCH(s, sort_particles, s, nullptr, split ? dp : nullptr);
 }
 
@@ -1536,7 +1556,7 @@ pm_status pm_run(pm_sim* s, int32_t nsteps, double a_start, double a_end) {
       if (slot.exec) cudaGraphExecDestroy(slot.exec);
       slot = pm_sim::RunGraph();
       s->cur = want;
-      const bool sorted0 = s->sorted, fields0 = s->fields_valid, marked0 = s->keys_marked;
+      const bool sorted0 = s->sorted, fields0 = s->fields_valid, marked0 = s->keys_marked, open0 = s->resort_open;
       cudaGraph_t graph = nullptr;
       ec = cudaStreamBeginCapture(s->cap, cudaStreamCaptureModeThreadLocal);
       if (ec == cudaSuccess) {
@@ -1554,6 +1574,7 @@ pm_status pm_run(pm_sim* s, int32_t nsteps, double a_start, double a_end) {
       s->sorted = sorted0;
       s->fields_valid = fields0;
       s->keys_marked = marked0;
+      s->resort_open = open0;
     }
     cudaGraphExec_t exec = nullptr;
     for (auto& g : s->run_graph)
@@ -1787,6 +1808,13 @@ pm_status pm_debug_sort_timeout(pm_sim* s, int32_t spin_limit) {
   return device_errors(s);
 }
 
+pm_status pm_debug_fail_resort(pm_sim* s, int32_t part) {
+  if (!s) return PM_ERR_INVALID_ARG;
+  if (part < -1 || part > 2) return fail(s, PM_ERR_INVALID_ARG, "part must be in [-1, 2]");
+  s->fail_resort = part;
+  return PM_OK;
+}
+
 pm_status pm_sort_stats(pm_sim* s, int64_t* resorts, int64_t* movers) {
   if (!s || !resorts || !movers) return PM_ERR_INVALID_ARG;
   unsigned long long h[2];
@@ -1868,7 +1896,8 @@ pm_status pm_load(pm_sim* s, const void* host, size_t bytes) {
   CU(s, cudaMemcpyAsync(s->mom(), in + CKPT_HEADER + rb, rb, cudaMemcpyHostToDevice, s->stream));
   CU(s, cudaMemcpyAsync(s->keys, in + CKPT_HEADER + 2 * rb, size_t(s->n()) * 4, cudaMemcpyHostToDevice, s->stream));
   CU(s, cudaMemcpyAsync(s->sort_stats(), stats, sizeof stats, cudaMemcpyHostToDevice, s->stream));
-  PMST(drop_mover_counts(s));
+  // a checkpoint does not hold the counts of a drift whose re-sort is still to come
+  PMST(h.flags & 2 ? unmark_movers(s) : drop_mover_counts(s));
   // sorted records: the deposit reads the row starts of the keys (integer, so the same as the re-sort's)
   if (h.flags & 1) {
     CU(s, cudaMemsetAsync(s->at<uint32_t>(s->L.row_start) + s->mesh.n2 + 1, 0, 4, s->stream));
@@ -1876,8 +1905,8 @@ pm_status pm_load(pm_sim* s, const void* host, size_t bytes) {
   }
   CU(s, cudaStreamSynchronize(s->stream));
   s->have_particles = true;
-  s->sorted = (h.flags & 1) != 0;
-  s->keys_marked = (h.flags & 2) != 0;
+  s->sorted = (h.flags & 3) == 1;
+  s->keys_marked = s->resort_open = false;
   s->fields_valid = false;
   s->krho_valid = false;
   return PM_OK;

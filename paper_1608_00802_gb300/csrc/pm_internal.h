@@ -173,6 +173,8 @@ cudaError_t launch_resort(int part, const uint32_t* keys, int64_t n, uint32_t* t
                           unsigned long long* stats, uint32_t* step, uint32_t* keys_out, const void* pos_in,
                           const void* mom_in, void* pos_out, void* mom_out, int sms, cudaStream_t s, int nm = 1,
                           size_t ms = 0);
+// clears the drift's marks of n keys
+cudaError_t launch_unmark_keys(uint32_t* keys, int64_t n, cudaStream_t s);
 inline size_t row_scan_tiles(int n_mesh) { return (size_t(n_mesh) * n_mesh + 1023) / 1024; }  // tiles of 1024 rows
 // the x-y transforms of the z-planes of 64^3 and 128^3 fp32 meshes, one CTA per plane (unnormalised, the layouts of
 // the batched 2D R2C / C2R)

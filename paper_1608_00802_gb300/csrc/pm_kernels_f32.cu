@@ -5,6 +5,15 @@
 
 namespace pm {
 
+static __global__ void k_unmark_keys(uint32_t* keys, int64_t n) {
+  const int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+  if (i < n) keys[i] &= ~KEY_MOVER;
+}
+cudaError_t launch_unmark_keys(uint32_t* keys, int64_t n, cudaStream_t s) {
+  k_unmark_keys<<<unsigned((n + 255) / 256), 256, 0, s>>>(keys, n);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_sort_histogram(const uint32_t* keys, int64_t n, int passes, int digit_bits, int key_bits,
                                   uint32_t* hist, uint32_t* epoch, cudaStream_t s, const uint32_t* n_dev,
                                   uint32_t* crowd) {

@@ -30,7 +30,8 @@ EXPORTS = ["pm_config_default", "pm_hbar_over_m", "pm_arena_bytes", "pm_create",
            "pm_profile_begin", "pm_profile_end", "pm_deposit_noalloc", "pm_last_error",
            "pm_batch_arena_bytes", "pm_batch_create", "pm_batch_destroy", "pm_batch_member", "pm_batch_run",
            "pm_batch_last_error", "pm_get_tuning", "pm_set_tuning", "pm_autotune", "pm_run_adaptive",
-           "pm_sort_stats", "pm_batch_info", "pm_debug_sort_timeout", "pm_checkpoint_bytes", "pm_save", "pm_load"]
+           "pm_sort_stats", "pm_batch_info", "pm_debug_sort_timeout", "pm_debug_fail_resort",
+           "pm_checkpoint_bytes", "pm_save", "pm_load"]
 NOALLOC_MAX_PARTICLES = 65536
 NOALLOC_MAX_MESH = 128
 STAGES = ["sort_histogram", "sort_pass", "row_start", "deposit", "fft_r2c", "green", "fft_c2r", "stencil",
@@ -340,6 +341,10 @@ class Sim:
         """Status of a radix pass whose look-back waits on a tile that never
         publishes (a test of the bounded device waits; PM_ERR_TIMEOUT)."""
         return int(lib().pm_debug_sort_timeout(self.handle, int(spin_limit)))
+
+    def debug_fail_resort(self, part):
+        """The next incremental re-sort fails before its kernel group `part` (0..2; -1: none), once."""
+        self._check(lib().pm_debug_fail_resort(self.handle, int(part)))
 
     def sort_stats(self):
         """(incremental re-sorts, particles they moved) since creation."""
