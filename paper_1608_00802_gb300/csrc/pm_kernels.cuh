@@ -17,6 +17,7 @@
 
 #include "pm_internal.h"
 #include "pm_bulk.cuh"
+#include "pm_mode.h"
 
 namespace pm {
 
@@ -2064,8 +2065,8 @@ __global__ void __launch_bounds__(KICK_THREADS, (FM == KICK_FM_HYBRID_Q && !PACK
 // ---------------------------------------------------------------- power spectrum
 // P(k) shells.  Bound by the fp64 pipe (a warp's fp64 operation takes 16 cycles of an SM), so a mode costs
 // as few as it can: the modes (+-m_y, +-m_z) share |k| and the window and are added before they are
-// weighted, the window comes from a table, and |k| is an fp32 square root with one exact-residual
-// correction.  A warp takes one quadrant row (|m_y|, |m_z|): along x the shell index does not fall, so
+// weighted, the window comes from a table, and |k| is an fp32 square root with its correction to fp64
+// (mode_norm).  A warp takes one quadrant row (|m_y|, |m_z|): along x the shell index does not fall, so
 // equal shells are runs of lanes, summed by a segmented scan, and the run's last lane adds to the warp's
 // own bins (no atomics; the sums are reproducible).  150^3: 365 us with a square root, three sinpi and three
 // shared fp64 atomics (compare-and-swap loops) per mode, 38 us so.
@@ -2126,9 +2127,7 @@ __global__ void __launch_bounds__(MESH_THREADS) k_power(const typename VT<R>::cp
       }
       const uint32_t wx = jx == 0 || jx == h ? 1u : 2u;
       uint32_t cnt[1] = {wx * uint32_t(ny * nz)};
-      const float res = fmaf(-s, s, float(m2));  // m2 - s^2, exact
-      const double kk = double(s) + double(0.5f * res / s);
-      double v[2] = {double(cnt[0]) * kk, p2 * (double(wx) * fyz * iw[jx <= h ? jx : 0])};
+      double v[2] = {double(cnt[0]) * mode_norm(m2, s), p2 * (double(wx) * fyz * iw[jx <= h ? jx : 0])};
       const uint32_t key = in ? shell : 0x80000000u + uint32_t(lane);
       const uint32_t kp = __shfl_up_sync(0xffffffffu, key, 1);
       const uint32_t runs = __ballot_sync(0xffffffffu, lane == 0 || kp != key);
