@@ -5,7 +5,44 @@
 #include <cufft.h>
 #include <stdint.h>
 
+#include <atomic>
+
 namespace pm {
+
+// Host preparation of a kernel on the current device (shared-memory opt-ins and the like; no stream
+// operation, so it may fall inside a capture), once per device, by whichever thread launches there first: a
+// server admits simulations from several threads.  Threads that meet all prepare, which stores the same
+// attributes; none goes on before its device is prepared.
+class DeviceOnce {
+  std::atomic<int> value_[64] = {};  // 0: not prepared
+
+ public:
+  // prepare(int& value) sets a value > 0 (1 unless it says otherwise), handed to every caller through `value`
+  template <typename F>
+  cudaError_t operator()(F prepare, int* value = nullptr) {
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    const bool kept = dev >= 0 && dev < 64;
+    int v = kept ? value_[dev].load(std::memory_order_acquire) : 0;
+    if (v == 0) {
+      v = 1;
+      e = prepare(v);
+      if (e != cudaSuccess) return e;
+      if (kept) value_[dev].store(v, std::memory_order_release);
+    }
+    if (value) *value = v;
+    return cudaSuccess;
+  }
+};
+// the dynamic shared-memory limit of kernels
+template <size_t N>
+cudaError_t raise_smem(const void* const (&fns)[N], size_t bytes) {
+  cudaError_t e = cudaSuccess;
+  for (const void* f : fns)
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, int(bytes));
+  return e;
+}
 
 // 32-byte record for the fp64 path (CUDA 13 deprecates the plain double4).
 struct __align__(32) D4 {

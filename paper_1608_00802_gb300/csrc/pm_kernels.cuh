@@ -2295,22 +2295,16 @@ cudaError_t launch_deposit(const void* pos, const uint32_t* row_start, int64_t n
   const int shape = deposit_shape<R>(m.n, ty, tz);
   if (size_t(warps) * ty * tz * deposit_stride_of<R>(m.n) * sizeof(R) > 40 * 1024) {
     // once per device, for every tile shape, so that no attribute call falls inside a stream capture
-    static bool done[64];
-    int dev = 0;
-    cudaGetDevice(&dev);
-    if (dev < 0 || dev >= 64 || !done[dev]) {
-      const int most = int(DEP_WARPS * PM_DEPOSIT_WARP_BYTES * sizeof(R) / 4);
-      cudaError_t e = cudaSuccess;
-      void* fns[10] = {(void*)k_deposit<R, 2, 1, false>, (void*)k_deposit<R, 2, 1, true>,
-                       (void*)k_deposit<R, 2, 4, false>, (void*)k_deposit<R, 2, 4, true>,
-                      (void*)k_deposit<R, 2, 2, false>, (void*)k_deposit<R, 2, 2, true>,
-                      (void*)k_deposit<R, 1, 2, false>, (void*)k_deposit<R, 1, 2, true>,
-                      (void*)k_deposit<R, 1, 1, false>, (void*)k_deposit<R, 1, 1, true>};
-      for (void* f : fns)
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
-      if (e != cudaSuccess) return e;
-      if (dev >= 0 && dev < 64) done[dev] = true;
-    }
+    static DeviceOnce once;
+    const cudaError_t e = once([](int&) {
+      const void* const fns[] = {(const void*)k_deposit<R, 2, 1, false>, (const void*)k_deposit<R, 2, 1, true>,
+                                 (const void*)k_deposit<R, 2, 4, false>, (const void*)k_deposit<R, 2, 4, true>,
+                                 (const void*)k_deposit<R, 2, 2, false>, (const void*)k_deposit<R, 2, 2, true>,
+                                 (const void*)k_deposit<R, 1, 2, false>, (const void*)k_deposit<R, 1, 2, true>,
+                                 (const void*)k_deposit<R, 1, 1, false>, (const void*)k_deposit<R, 1, 1, true>};
+      return raise_smem(fns, DEP_WARPS * PM_DEPOSIT_WARP_BYTES * sizeof(R) / 4);
+    });
+    if (e != cudaSuccess) return e;
   }
   switch (shape) {
     case 0: return launch_deposit_tile<R, 2, 4>(pos, row_start, n, m, norm, rho, s, warps, nm, ms);
@@ -2437,18 +2431,12 @@ cudaError_t launch_stencil(const R* rho, Mesh m, StencilParams sp, R* q, double*
     // fp32 compact path: shared-memory tiles, ill-conditioned near-empty nodes redone in float-float
     const float slim = sp.rho_fp64 > 0 ? float(sqrt(sp.rho_fp64)) : 0.0f;
     if (stencil_tile_path(m.n, sp, true)) {
-      static bool done[64];
-      int dev = 0;
-      cudaGetDevice(&dev);
-      if (dev < 0 || dev >= 64 || !done[dev]) {
-        cudaError_t e = cudaFuncSetAttribute(k_stencil_tile<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             int(SB_SMEM_MAX));
-        if (e == cudaSuccess)
-          e = cudaFuncSetAttribute(k_stencil_tile<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   int(SB_SMEM_MAX));
-        if (e != cudaSuccess) return e;
-        if (dev >= 0 && dev < 64) done[dev] = true;
-      }
+      static DeviceOnce once;
+      const cudaError_t e = once([](int&) {
+        const void* const fns[] = {(const void*)k_stencil_tile<false>, (const void*)k_stencil_tile<true>};
+        return raise_smem(fns, SB_SMEM_MAX);
+      });
+      if (e != cudaSuccess) return e;
       const dim3 g(unsigned(m.n / sp.ty), unsigned((m.n + sp.zlen - 1) / sp.zlen), unsigned(nm));
       if (nm > 1)
         k_stencil_tile<true><<<g, SB_THREADS, stencil_tile_smem(m.n, sp.ty, sp.zlen), s>>>(
@@ -2461,15 +2449,12 @@ cudaError_t launch_stencil(const R* rho, Mesh m, StencilParams sp, R* q, double*
       return cudaGetLastError();
     }
     if (sp.ty > 0 && stencil_bulk_shape_ok(m.n, sp.ty, sp.zlen, sp.stages)) {
-      static bool done[64];  // the shared-memory opt-in, once per device (never inside a capture)
-      int dev = 0;
-      cudaGetDevice(&dev);
-      if (dev < 0 || dev >= 64 || !done[dev]) {
-        cudaError_t e = cudaFuncSetAttribute(k_stencil_bulk, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             int(SB_SMEM_MAX));
-        if (e != cudaSuccess) return e;
-        if (dev >= 0 && dev < 64) done[dev] = true;
-      }
+      static DeviceOnce once;
+      const cudaError_t e = once([](int&) {
+        const void* const fns[] = {(const void*)k_stencil_bulk};
+        return raise_smem(fns, SB_SMEM_MAX);
+      });
+      if (e != cudaSuccess) return e;
       const dim3 g(unsigned(m.n / sp.ty), unsigned((m.n + sp.zlen - 1) / sp.zlen));
       k_stencil_bulk<<<g, SB_THREADS, stencil_bulk_smem(m.n, sp.ty, sp.stages), s>>>(
           (const float*)rho, m, float(sp.rho_floor), float(sp.qcoef), slim, sp.ty, sp.zlen, sp.stages, (float*)q,
@@ -2494,19 +2479,22 @@ cudaError_t launch_stencil(const R* rho, Mesh m, StencilParams sp, R* q, double*
 // if the query fails, one particle per thread
 template <typename R>
 int kick_stream_resident(int threads, int fm = KICK_FM_ANY) {
-  static int cache[64][2][2];
-  int dev = 0;
-  cudaGetDevice(&dev);
+  static DeviceOnce once[2][2];
   const int t = threads == 128 ? 0 : 1, f = fm == KICK_FM_HYBRID_Q ? 1 : 0;
-  if (dev >= 0 && dev < 64 && cache[dev][t][f] > 0) return cache[dev][t][f];
-  int per_sm = 0, sms = 0, r = 1 << 30;
-  const void* fn = f ? (const void*)k_kick_stream<R, false, KICK_FM_HYBRID_Q> : (const void*)k_kick_stream<R, false, KICK_FM_ANY>;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, threads, 0) == cudaSuccess &&
-      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && per_sm > 0 && sms > 0)
-    r = per_sm * sms;
-  else
-    cudaGetLastError();
-  if (dev >= 0 && dev < 64) cache[dev][t][f] = r;
+  int r = 1 << 30;
+  once[t][f]([&](int& blocks) {
+    int dev = 0, per_sm = 0, sms = 0;
+    const void* fn = f ? (const void*)k_kick_stream<R, false, KICK_FM_HYBRID_Q> : (const void*)k_kick_stream<R, false, KICK_FM_ANY>;
+    if (cudaGetDevice(&dev) == cudaSuccess &&
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, threads, 0) == cudaSuccess &&
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && per_sm > 0 && sms > 0) {
+      blocks = per_sm * sms;
+    } else {
+      blocks = 1 << 30;
+      cudaGetLastError();
+    }
+    return cudaSuccess;
+  }, &r);
   return r;
 }
 // the compile-time force form of a kick's parameters (the common HYBRID run with the quantum force)

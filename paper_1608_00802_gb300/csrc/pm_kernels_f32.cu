@@ -134,16 +134,12 @@ static size_t spec_z_symbol_smem(int n) {
   return size_t(n) * (SPZ_COLS * (sizeof(float2) + sizeof(float)) + sizeof(float2) + sizeof(float));
 }
 static cudaError_t spec_z_symbol_prepare() {
-  static bool done[64];
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess || (dev >= 0 && dev < 64 && done[dev])) return e;
-  const int most = int(spec_z_symbol_smem(256));
-  e = cudaFuncSetAttribute(k_spec_z<16, 16, false, SPZ_SPLINE>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_spec_z<16, 16, false, SPZ_SMOOTH>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
-  if (e == cudaSuccess && dev >= 0 && dev < 64) done[dev] = true;
-  return e;
+  static DeviceOnce once;
+  return once([](int&) {
+    const void* const fns[] = {(const void*)k_spec_z<16, 16, false, SPZ_SPLINE>,
+                               (const void*)k_spec_z<16, 16, false, SPZ_SMOOTH>};
+    return raise_smem(fns, spec_z_symbol_smem(256));
+  });
 }
 
 cudaError_t launch_spec_z_spline(void* spec, const void* what, const float2* tw, const float* s2, Mesh m, double coef,

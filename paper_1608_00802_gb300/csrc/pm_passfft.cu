@@ -21,8 +21,6 @@
 // registers a thread.  Slots of the exchange tile are padded by one in C, so that the third step's stride of
 // C slots does not meet one bank group (the z kernel's slots are whole bank rows).  Inverses run the same steps
 // backwards with conjugate twiddles.
-#include <atomic>
-
 #include "pm_kernels.cuh"
 
 namespace pm {
@@ -446,16 +444,13 @@ __global__ void __launch_bounds__(ZShape<N>::THREADS, ZShape<N>::MINB) k_z_green
   block_sum_store<1>(acc, part, gridDim.x);
 }
 
-// the z kernel's shared memory needs the opt-in, once per device
 template <int N>
 cudaError_t z_prepare() {
-  static std::atomic<bool> done[64];
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess || (dev >= 0 && dev < 64 && done[dev])) return e;
-  e = cudaFuncSetAttribute(k_z_green<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(ZShape<N>::smem()));
-  if (e == cudaSuccess && dev >= 0 && dev < 64) done[dev] = true;
-  return e;
+  static DeviceOnce once;
+  return once([](int&) {
+    const void* const fns[] = {(const void*)k_z_green<N>};
+    return raise_smem(fns, ZShape<N>::smem());
+  });
 }
 
 template <int N>

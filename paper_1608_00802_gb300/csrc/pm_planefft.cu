@@ -171,16 +171,12 @@ __global__ void __launch_bounds__(Plane<N>::THREADS, 1) k_plane_c2r(const float2
 
 template <int N>
 cudaError_t plane_prepare() {
-  static bool done[64];  // the shared-memory opt-in, once per device (outside any capture)
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess || (dev >= 0 && dev < 64 && done[dev])) return e;
-  const void* fns[4] = {(const void*)k_plane_r2c<N, false>, (const void*)k_plane_r2c<N, true>,
-                        (const void*)k_plane_c2r<N, false>, (const void*)k_plane_c2r<N, true>};
-  for (const void* f : fns)
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, int(Plane<N>::smem()));
-  if (e == cudaSuccess && dev >= 0 && dev < 64) done[dev] = true;
-  return e;
+  static DeviceOnce once;
+  return once([](int&) {
+    const void* const fns[] = {(const void*)k_plane_r2c<N, false>, (const void*)k_plane_r2c<N, true>,
+                               (const void*)k_plane_c2r<N, false>, (const void*)k_plane_c2r<N, true>};
+    return raise_smem(fns, Plane<N>::smem());
+  });
 }
 
 template <int N>

@@ -1050,19 +1050,17 @@ cudaError_t launch_sort_small(const uint32_t* keys_in, int64_t n, int key_bits, 
   using I2 = std::integral_constant<int, 2>;
   using I4 = std::integral_constant<int, 4>;
   using I8 = std::integral_constant<int, 8>;
-  static int most[64];  // CTAs of a cluster on each device (0: not prepared)
-  int dev = 0, ctas = 16;
-  cudaGetDevice(&dev);
-  if (dev < 0 || dev >= 64 || most[dev] == 0) {
-    cudaError_t e = run(I1(), &ctas);
-    if (e == cudaSuccess) e = run(I2(), &ctas);
-    if (e == cudaSuccess) e = run(I4(), &ctas);
-    if (e == cudaSuccess) e = run(I8(), &ctas);
-    if (e != cudaSuccess) return e;
-    if (dev >= 0 && dev < 64) most[dev] = ctas;
-  } else {
-    ctas = most[dev];
-  }
+  static DeviceOnce once;
+  int ctas = 16;  // of a cluster on this device
+  const cudaError_t e = once([&](int& most) {
+    most = 16;
+    cudaError_t p = run(I1(), &most);
+    if (p == cudaSuccess) p = run(I2(), &most);
+    if (p == cudaSuccess) p = run(I4(), &most);
+    if (p == cudaSuccess) p = run(I8(), &most);
+    return p;
+  }, &ctas);
+  if (e != cudaSuccess) return e;
   // the smallest chunks whose cluster holds all particles
   if (n <= int64_t(ctas) * SS_THREADS) return run(I1(), nullptr);
   if (n <= int64_t(ctas) * SS_THREADS * 2) return run(I2(), nullptr);
@@ -1147,17 +1145,12 @@ cudaError_t launch_sort_pass(bool last, const uint32_t* keys_in, const uint32_t*
   const dim3 grid = dim3(unsigned(ntiles < per ? ntiles : per), unsigned(nm), 1u);
   const size_t smem = radix_smem_bytes(bits);
   // shared-memory limits are raised once per device (for the largest digit), outside any capture
-  static bool done[64];
-  int dev = 0;
-  cudaGetDevice(&dev);
-  if (dev < 0 || dev >= 64 || !done[dev]) {
-    const int most = int(radix_smem_bytes(RS_MAX_BITS));
-    cudaError_t e = cudaFuncSetAttribute(k_sort_pass<true, V4>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(k_sort_pass<false, V4>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
-    if (e != cudaSuccess) return e;
-    if (dev >= 0 && dev < 64) done[dev] = true;
-  }
+  static DeviceOnce once;
+  const cudaError_t e = once([](int&) {
+    const void* const fns[] = {(const void*)k_sort_pass<true, V4>, (const void*)k_sort_pass<false, V4>};
+    return raise_smem(fns, radix_smem_bytes(RS_MAX_BITS));
+  });
+  if (e != cudaSuccess) return e;
   if (last) {
     k_sort_pass<true, V4><<<grid, RS_THREADS, smem, s>>>(keys_in, vals_in, n, shift, bits, digit_total, status,
                                                          tile_counter, epoch, pass, keys_out, vals_out,

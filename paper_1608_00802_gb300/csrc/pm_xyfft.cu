@@ -286,17 +286,12 @@ __global__ void __cluster_dims__(XY_CL, 1, 1) __launch_bounds__(XY_THREADS, XY_M
 // the shared-memory attribute of all four kernels, once per device (so that no attribute call falls
 // inside a stream capture)
 cudaError_t xy_prepare() {
-  static bool done[64];
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  if (dev >= 0 && dev < 64 && done[dev]) return cudaSuccess;
-  const void* fns[4] = {(const void*)k_xy_r2c<false>, (const void*)k_xy_r2c<true>, (const void*)k_xy_c2r<false>,
-                        (const void*)k_xy_c2r<true>};
-  for (const void* f : fns)
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, int(XY_SMEM));
-  if (e == cudaSuccess && dev >= 0 && dev < 64) done[dev] = true;
-  return e;
+  static DeviceOnce once;
+  return once([](int&) {
+    const void* const fns[] = {(const void*)k_xy_r2c<false>, (const void*)k_xy_r2c<true>, (const void*)k_xy_c2r<false>,
+                               (const void*)k_xy_c2r<true>};
+    return raise_smem(fns, XY_SMEM);
+  });
 }
 
 }  // namespace
