@@ -390,6 +390,11 @@ const char* pm_batch_last_error(const pm_batch* b);
 pm_status pm_deposit_noalloc(const double* x_dev, int64_t n_part, int32_t n_mesh, double box, float* rho_dev,
                              uint32_t* err_dev, void* stream);
 
+/* Test aid for the recovery from a failed launch: the calling thread's next
+ * pm_deposit_noalloc returns PM_ERR_CUDA after `launches` (0..2; -1 takes the
+ * request back) of its launches, once, as if the next one had failed. */
+pm_status pm_debug_fail_noalloc(int32_t launches);
+
 /* Message of the last failure on this handle (or of the last pm_create
  * failure when sim is NULL). */
 const char* pm_last_error(const pm_sim* sim);

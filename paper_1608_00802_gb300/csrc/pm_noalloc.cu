@@ -12,6 +12,7 @@
 #include <stdio.h>
 #include <string.h>
 
+#include <atomic>
 #include <mutex>
 
 #include "../../include/pm.h"
@@ -43,8 +44,12 @@ static __device__ __align__(256) unsigned char g_scratch[PM_NOALLOC_SCRATCH_BYTE
 std::mutex g_mu;
 void* g_addr[64];
 bool g_ready[64];
+// A call is on its way, or stopped at an error between its launches: the error word may hold bits of positions that
+// it placed.  The next call clears them.
+std::atomic<bool> g_unfinished[64];
 
 thread_local char g_msg[256];
+thread_local int g_fail_after = -1;  // test aid: launches after which this thread's next call "fails"
 
 // hands the call's error bits to the caller's word (device or mapped host
 // memory) and clears them for the next call
@@ -59,7 +64,7 @@ pm_status nfail(pm_status st, const char* msg) {
   return st;
 }
 
-pm_status scratch_address(unsigned char** out) {
+pm_status scratch_address(unsigned char** out, int* device) {
   int dev = -1;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return nfail(PM_ERR_CUDA, "no current device");
   std::lock_guard<std::mutex> lock(g_mu);  // also serialises the message buffer
@@ -74,6 +79,7 @@ pm_status scratch_address(unsigned char** out) {
     g_ready[dev] = true;
   }
   *out = static_cast<unsigned char*>(g_addr[dev]);
+  *device = dev;
   return PM_OK;
 }
 
@@ -95,7 +101,8 @@ pm_status pm_deposit_noalloc(const double* x_dev, int64_t n_part, int32_t n_mesh
   }
   if (!x_dev || !rho_dev || !(box > 0)) return nfail(PM_ERR_INVALID_ARG, "x, rho must be device pointers, box > 0");
   unsigned char* base = nullptr;
-  pm_status st = scratch_address(&base);
+  int dev = 0;
+  pm_status st = scratch_address(&base, &dev);
   if (st != PM_OK) return st;
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   const int64_t n = n_part;
@@ -111,17 +118,25 @@ pm_status pm_deposit_noalloc(const double* x_dev, int64_t n_part, int32_t n_mesh
   uint32_t* rows = reinterpret_cast<uint32_t*>(base + kRows);
   void* pos[2] = {base + kPos0, base + kPos1};
 
+  int fail_after = g_fail_after;
+  g_fail_after = -1;
 #define NA_CU(expr)                                                                             \
   do {                                                                                          \
-    cudaError_t e_ = (expr);                                                                    \
+    cudaError_t e_ = fail_after-- == 0 ? cudaErrorLaunchFailure : (expr);                       \
     if (e_ != cudaSuccess) {                                                                    \
       snprintf(g_msg, sizeof g_msg, "%s: %s", #expr, cudaGetErrorString(e_));                   \
       return nfail(PM_ERR_CUDA, g_msg);                                                         \
     }                                                                                           \
   } while (0)
   // the array keeps the previous call's contents; every buffer is written before it is read, except the error
-  // word, which starts at zero and is zero again after each call: cleared as it is handed over, or, with
-  // nobody to hand it to, by the sort
+  // word, which starts at zero and is zero again after each call that came to its end: cleared as it is handed
+  // over, or, with nobody to hand it to, by the sort
+  const bool stale = g_unfinished[dev].exchange(true);
+  cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+  if (stale) {
+    NA_CU(cudaMemsetAsync(err, 0, 4, s));
+    NA_CU(cudaStreamIsCapturing(s, &capture));
+  }
   // positions to cell + offset as pm_set_particles converts them (1/dx with dx = box/N)
   NA_CU(launch_init_particles<float>(x_dev, nullptr, n, m, 1.0 / (box / n_mesh), pos[0], nullptr, keys, err, s));
   NA_CU(launch_sort_small<float>(keys, n, bits, keys, pos[0], nullptr, pos[1], nullptr, rows, m,
@@ -133,6 +148,13 @@ pm_status pm_deposit_noalloc(const double* x_dev, int64_t n_part, int32_t n_mesh
     NA_CU(cudaGetLastError());
   }
 #undef NA_CU
+  g_unfinished[dev] = stale && capture != cudaStreamCaptureStatusNone;  // (a captured clear has not run yet)
+  return PM_OK;
+}
+
+pm_status pm_debug_fail_noalloc(int32_t launches) {
+  if (launches < -1 || launches > 2) return nfail(PM_ERR_INVALID_ARG, "launches must be in [-1, 2]");
+  g_fail_after = launches;
   return PM_OK;
 }
 

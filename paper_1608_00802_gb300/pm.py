@@ -30,7 +30,7 @@ EXPORTS = ["pm_config_default", "pm_hbar_over_m", "pm_arena_bytes", "pm_create",
            "pm_profile_begin", "pm_profile_end", "pm_deposit_noalloc", "pm_last_error",
            "pm_batch_arena_bytes", "pm_batch_create", "pm_batch_destroy", "pm_batch_member", "pm_batch_run",
            "pm_batch_last_error", "pm_get_tuning", "pm_set_tuning", "pm_autotune", "pm_run_adaptive",
-           "pm_sort_stats", "pm_batch_info", "pm_debug_sort_timeout", "pm_debug_fail_resort",
+           "pm_sort_stats", "pm_batch_info", "pm_debug_sort_timeout", "pm_debug_fail_resort", "pm_debug_fail_noalloc",
            "pm_checkpoint_bytes", "pm_save", "pm_load"]
 NOALLOC_MAX_PARTICLES = 65536
 NOALLOC_MAX_MESH = 128
@@ -98,6 +98,8 @@ def load_library(path: str = LIB_PATH) -> C.CDLL:
         "pm_get_order": (C.c_int, [vp, C.POINTER(C.c_uint32), C.POINTER(C.c_uint32)]),
         "pm_sort_stats": (C.c_int, [vp, C.POINTER(C.c_int64), C.POINTER(C.c_int64)]),
         "pm_debug_sort_timeout": (C.c_int, [vp, C.c_int32]),
+        "pm_debug_fail_resort": (C.c_int, [vp, C.c_int32]),
+        "pm_debug_fail_noalloc": (C.c_int, [C.c_int32]),
         "pm_checkpoint_bytes": (C.c_size_t, [vp]),
         "pm_save": (C.c_int, [vp, vp, C.c_size_t]),
         "pm_load": (C.c_int, [vp, vp, C.c_size_t]),
@@ -391,6 +393,13 @@ def deposit_noalloc(x_dev, n_mesh, box, rho_dev, stream=None, err_dev=None):
     st_obj = stream if stream is not None else torch.cuda.current_stream(x_dev.device)
     st = lib().pm_deposit_noalloc(C.c_void_p(x_dev.data_ptr()), int(x_dev.shape[0]), int(n_mesh), float(box),
                                   C.c_void_p(rho_dev.data_ptr()), err_ptr, C.c_void_p(st_obj.cuda_stream))
+    if st != PM_OK:
+        raise PMError(st, lib().pm_last_error(None).decode())
+
+
+def debug_fail_noalloc(launches):
+    """This thread's next deposit_noalloc fails after that many of its launches (0..2; -1: none), once."""
+    st = lib().pm_debug_fail_noalloc(int(launches))
     if st != PM_OK:
         raise PMError(st, lib().pm_last_error(None).decode())
 
