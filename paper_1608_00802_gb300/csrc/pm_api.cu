@@ -1243,12 +1243,13 @@ pm_status pm_create(const pm_config* c, void* dev_arena, size_t bytes, void* str
       return fail(nullptr, PM_ERR_CUDA, "coefficient upload failed");
     }
   }
-  if (DISPATCH(s, launch_sin2_table, s->arena + L.sin2, N, s->stream) != cudaSuccess ||
+  if ((s->fp64() ? deposit_prepare<double>() : deposit_prepare<float>()) != cudaSuccess ||
+      DISPATCH(s, launch_sin2_table, s->arena + L.sin2, N, s->stream) != cudaSuccess ||
       cudaStreamSynchronize(s->stream) != cudaSuccess) {
     cufftDestroy(s->plan_fwd);
     cufftDestroy(s->plan_inv);
     delete s;
-    return fail(nullptr, PM_ERR_CUDA, "sin^2 table failed");
+    return fail(nullptr, PM_ERR_CUDA, "deposit preparation or sin^2 table failed");
   }
   if (c->precision == PM_FP32) kick_stream_prepare();
   // fp32 cloud-in-cell on power-of-two meshes from 128^3: the Green multiplication inside the z

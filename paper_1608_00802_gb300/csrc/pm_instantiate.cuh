@@ -11,6 +11,7 @@
                                            void*, uint32_t*, cudaStream_t, const uint32_t*, int, size_t, int);           \
   template cudaError_t launch_sort_small<R>(const uint32_t*, int64_t, int, uint32_t*, const void*, const void*,   \
                                             void*, void*, uint32_t*, Mesh, uint32_t*, cudaStream_t);              \
+  template cudaError_t deposit_prepare<R>();                                                                      \
   template cudaError_t launch_deposit<R>(const void*, const uint32_t*, int64_t, Mesh, double, R*, cudaStream_t,    \
                                          int, int, size_t);                                                       \
   template cudaError_t launch_resort<R>(int, const uint32_t*, int64_t, uint32_t*, uint32_t*, uint32_t*, uint32_t*, \

@@ -7,6 +7,8 @@
 
 #include <atomic>
 
+#include "pm_deposit_shape.h"
+
 namespace pm {
 
 // Host preparation of a kernel on the current device (shared-memory opt-ins and the like; no stream
@@ -149,17 +151,6 @@ constexpr int RS_MAX_BITS = 10;
 // set in a sort key by the drift when the particle's cell changed (keys use at most 30 bits)
 constexpr uint32_t KEY_MOVER = 0x80000000u;
 
-// Mesh rows with more records than this are "crowded": the deposit computes the rows they add to by whole
-// blocks instead of one warp each.  A warp takes 0.4 us per batch of 32 records when few warps are busy,
-// so a tile of nine rows of 256 records is ~30 us, about the length of the whole kernel at 256^3.
-// The word after the row starts, row_start[N^2 + 1], says whether any row is (CROWD_WORDS entries follow
-// the N^2 row starts: the closing one and the flag).
-#ifndef PM_DEP_CROWD
-#define PM_DEP_CROWD 256
-#endif
-constexpr uint32_t DEP_CROWD = PM_DEP_CROWD;
-constexpr size_t CROWD_WORDS = 2;
-
 constexpr int KICK_THREADS = 256;
 constexpr int MESH_THREADS = 256;
 constexpr int RED_GRID = 608;    // 4 blocks per SM on 152 SMs, fixed for deterministic reductions
@@ -281,6 +272,9 @@ int stencil_launch_blocks(int n, int ty, int zlen);
 int stencil_max_blocks(int n);
 bool stencil_shape_ok(int n, int ty, int zlen, int stages);
 Tuning default_tuning(int n, int64_t n_part, bool fp64);
+// shared-memory limits of the deposit (call outside any stream capture)
+template <typename R>
+cudaError_t deposit_prepare();
 // sizes the fp32 streaming kick's grid for this device (an occupancy query;
 // call outside any stream capture, before the first kick)
 void kick_stream_prepare();

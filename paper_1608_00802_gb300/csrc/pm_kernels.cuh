@@ -345,16 +345,8 @@ __device__ __forceinline__ uint32_t divu32(uint32_t e, DivU32 dv) {
 //    (to the next row); within a phase no two source rows meet.
 // The warp alone writes its rows, in a fixed order of chains, batches and
 // phases, so the result is reproducible.
-// Tiles with crowded source rows are left to the launch's last `helpers`
-// blocks (deposit_crowded).
-constexpr int DEP_WARPS = 8;
-
-// slots of a deposit row: N + 1 rounded up to 16 bytes
-template <typename R>
-__host__ __device__ inline int deposit_stride_of(int n) {
-  const int q = 16 / int(sizeof(R));
-  return (n + 1 + q - 1) / q * q;
-}
+// Tiles with crowded source rows are left to the launch's last blocks, past
+// the `mains` of the tiles (deposit_crowded).  pm_deposit_shape.h has the launch.
 
 // sums v over each run of lanes with equal keys (a segmented inclusive scan in a fixed tree order; the
 // run's last lane ends with the run's sum); runs: the ballot of the lanes that start a run.  The scan stops
@@ -378,7 +370,7 @@ __device__ __forceinline__ void run_sums(R (&v)[NV], uint32_t runs, int lane) {
   }
 }
 
-// ---- crowded tiles.  A tile one of whose source rows holds more than DEP_CROWD records (clustered
+// ---- crowded tiles.  A tile one of whose source rows holds more than `crowd` records (deposit_crowd; clustered
 // states: a core of 10^6 particles puts thousands into each of a few hundred rows) is left to helper
 // blocks of the same launch, one destination row at a time, because its warp's chain would be the whole
 // kernel's length: 1496 us for that core on a 128^3 mesh, 87 us with the helpers.  The helpers add the
@@ -386,15 +378,6 @@ __device__ __forceinline__ void run_sums(R (&v)[NV], uint32_t runs, int lane) {
 // is serial about a sum is only each node's own chain of additions, one per batch its two cells are in, so
 // the block computes the sums of all batches first (a warp per batch, any order) and then every node adds
 // up its own (a thread per node, in the batches' order).
-
-// records per window (the batch sums of a window are kept in shared memory)
-template <typename R>
-constexpr int DEP_WINDOW = sizeof(R) == 4 ? 2048 : 1024;
-// shared memory of a helper block: the window's sums, each cell's first and last record of the window, the row
-template <typename R>
-__host__ __device__ inline size_t deposit_crowd_smem(int n) {
-  return size_t(2 * DEP_WINDOW<R> + deposit_stride_of<R>(n)) * sizeof(R) + size_t(2 * n) * sizeof(uint32_t);
-}
 
 struct DepRow {
   uint32_t b, e;  // records of a source row
@@ -511,7 +494,8 @@ __device__ __forceinline__ void deposit_crowded_row(const typename VT<R>::v4* __
 template <typename R, int TY, int TZ>
 __device__ __noinline__ void deposit_crowded(const typename VT<R>::v4* __restrict__ pos,
                                              const uint32_t* __restrict__ row_start, uint32_t np, const Mesh m, R norm,
-                                             R* __restrict__ rho, unsigned char* smem, uint32_t hb, uint32_t H) {
+                                             R* __restrict__ rho, unsigned char* smem, uint32_t crowd, uint32_t hb,
+                                             uint32_t H) {
   __shared__ uint32_t list[DEP_WARPS * 32];
   __shared__ uint32_t found;
   const int n = m.n;
@@ -529,7 +513,7 @@ __device__ __noinline__ void deposit_crowded(const typename VT<R>::v4* __restric
           const DepRow r = deposit_row_of(row_start, src, np);
           most = max(most, r.e - r.b);
         }
-      if (most > DEP_CROWD) list[atomicAdd(&found, 1u)] = row;
+      if (most > crowd) list[atomicAdd(&found, 1u)] = row;
     }
     __syncthreads();
     const uint32_t c = found;
@@ -542,7 +526,7 @@ template <typename R, int TY, int TZ, bool PACKED>
 __global__ void __launch_bounds__(DEP_WARPS * 32) k_deposit(const typename VT<R>::v4* __restrict__ pos,
                                                             const uint32_t* __restrict__ row_start, uint32_t np,
                                                             Mesh m, DivU32 dvn, R norm, R* __restrict__ rho,
-                                                            uint32_t helpers, size_t ms) {
+                                                            uint32_t mains, uint32_t crowd, size_t ms) {
   using V4 = typename VT<R>::v4;
   static_assert((TY + 1) * (TZ + 1) <= 32, "one source row per lane");
   if constexpr (PACKED) {  // member blockIdx.y of a packed group
@@ -550,9 +534,10 @@ __global__ void __launch_bounds__(DEP_WARPS * 32) k_deposit(const typename VT<R>
     pos = moff(pos, o), row_start = moff(row_start, o), rho = moff(rho, o);
   }
   extern __shared__ __align__(16) unsigned char dep_smem[];
-  if (blockIdx.x >= gridDim.x - helpers) {
+  if (blockIdx.x >= mains) {
     if (__ldg(row_start + m.n2 + 1))  // some row is crowded
-      deposit_crowded<R, TY, TZ>(pos, row_start, np, m, norm, rho, dep_smem, blockIdx.x - (gridDim.x - helpers), helpers);
+      deposit_crowded<R, TY, TZ>(pos, row_start, np, m, norm, rho, dep_smem, crowd, blockIdx.x - mains,
+                                 gridDim.x - mains);
     return;
   }
   const int n = m.n, stride = deposit_stride_of<R>(n);
@@ -580,7 +565,7 @@ __global__ void __launch_bounds__(DEP_WARPS * 32) k_deposit(const typename VT<R>
     head = ly_l == 0 || yr != wrap(y0 - 2 + ly_l, n) + 1;
     base = srow * uint32_t(n);
   }
-  if (helpers && __any_sync(0xffffffffu, e > b && e - b > DEP_CROWD)) return;  // a crowded tile: the helpers'
+  if (__any_sync(0xffffffffu, e > b && e - b > crowd)) return;  // a crowded tile: the helpers'
   const uint32_t heads = __ballot_sync(0xffffffffu, head);
   const uint32_t later = heads & ~((2u << lane) - 1u);
   const int last = (later ? __ffs(later) - 1 : nr) - 1;                  // the chain's last row (head lanes)
@@ -2228,62 +2213,32 @@ cudaError_t launch_init_particles(const double* x, const double* p, int64_t n, M
   return cudaGetLastError();
 }
 
-// deposit tile of TY x TZ rows per warp: by size the largest of 2 x 4, 2 x 2, 1 x 2, 1 x 1 whose rows fit
-// PM_DEPOSIT_WARP_BYTES of shared memory per 4-byte accumulator (4.25 KB: 2 x 2 rows of a 256^3
-// fp32 mesh; measured there: 43 us against 53 us for 2 x 4 rows, whose 8.3 KB per warp leave
-// too few resident warps)
-#ifndef PM_DEP_HELPERS
-#define PM_DEP_HELPERS 608
-#endif
-#ifndef PM_DEPOSIT_WARP_BYTES
-#define PM_DEPOSIT_WARP_BYTES 4352
-#endif
-// Small meshes take fewer planes per tile while the tiles are fewer than PM_DEPOSIT_MIN_TILES warps (16 per SM):
-// a warp's time is its chain of batches, one or two per plane, so 64^3 goes from 512 tiles of five source
-// planes (6.9 us) to 2048 of two (4.2 us; 4096 particles on 32^3 7.2 -> 3.9 us).  Not in fp64, whose pipe pays
-// for every record read again (14.1 -> 14.7 us).  The planes of a tile do not enter its result: a row's batches
-// are cut by its chain, which only the rows in y decide, and added plane by plane.
-#ifndef PM_DEPOSIT_MIN_TILES
-#define PM_DEPOSIT_MIN_TILES 2432
-#endif
+// the shared-memory opt-in of every tile shape, once per device (pm_create asks first, outside any capture)
 template <typename R>
-inline int deposit_shape(int n, int& ty, int& tz) {
-  static const int shapes[5][2] = {{2, 4}, {2, 2}, {2, 1}, {1, 2}, {1, 1}};
-  const size_t row = size_t(deposit_stride_of<R>(n)) * sizeof(R);
-  const size_t most = size_t(PM_DEPOSIT_WARP_BYTES) * sizeof(R) / 4;
-  int s = 0;
-  while (s < 4 && (size_t(shapes[s][0] * shapes[s][1]) * row > most || s == 2)) ++s;
-  while (sizeof(R) == 4 && s < 2 && ((n + 1) / 2) * ((n + shapes[s][1] - 1) / shapes[s][1]) < PM_DEPOSIT_MIN_TILES) ++s;
-  ty = shapes[s][0], tz = shapes[s][1];
-  return s;
+cudaError_t deposit_prepare() {
+  static DeviceOnce once;
+  return once([](int&) {
+    const void* const fns[] = {(const void*)k_deposit<R, 2, 1, false>, (const void*)k_deposit<R, 2, 1, true>,
+                               (const void*)k_deposit<R, 2, 4, false>, (const void*)k_deposit<R, 2, 4, true>,
+                               (const void*)k_deposit<R, 2, 2, false>, (const void*)k_deposit<R, 2, 2, true>,
+                               (const void*)k_deposit<R, 1, 2, false>, (const void*)k_deposit<R, 1, 2, true>,
+                               (const void*)k_deposit<R, 1, 1, false>, (const void*)k_deposit<R, 1, 1, true>};
+    return raise_smem(fns, DEP_WARPS * PM_DEPOSIT_WARP_BYTES * sizeof(R) / 4);
+  });
 }
 
 template <typename R, int TY, int TZ>
-cudaError_t launch_deposit_tile(const void* pos, const uint32_t* row_start, int64_t n, Mesh m, double norm, R* rho,
-                                cudaStream_t s, int warps, int nm, size_t ms) {
+cudaError_t launch_deposit_tile(const DepositLaunch& d, const void* pos, const uint32_t* row_start, int64_t n, Mesh m,
+                                double norm, R* rho, cudaStream_t s, int nm, size_t ms) {
   using V4 = typename VT<R>::v4;
-  // helper blocks for crowded tiles (none with so few particles): at most PM_DEP_HELPERS of 8 warps in all,
-  // and no fewer than 16 rows each.  A helper takes every helpers-th row, and rows crowd together, so their
-  // number is q N + 0.382 N: a block's rows then lie far apart in y from plane to plane (a core of 10^6
-  // particles on 128^3: the longest share is one row's, 1.0 .. 1.1 of it over meshes of 64 .. 160; with
-  // 2 N + 1 blocks it is 7 of them, 800 us instead of 87)
-  unsigned helpers = 0;
-  size_t smem = size_t(warps) * TY * TZ * deposit_stride_of<R>(m.n) * sizeof(R);
-  if (n > int64_t(DEP_CROWD)) {
-    const unsigned most = std::max(8u, std::min(unsigned(PM_DEP_HELPERS * DEP_WARPS / (warps * nm)), m.n2 / 16 + 1));
-    const unsigned N = unsigned(m.n), part = unsigned(0.382 * m.n);
-    helpers = most >= N + part ? (most - part) / N * N + part : most;
-    smem = std::max(smem, deposit_crowd_smem<R>(m.n));
-  }
-  const unsigned tiles_y = unsigned((m.n + warps * TY - 1) / (warps * TY));
-  const unsigned blocks = tiles_y * unsigned((m.n + TZ - 1) / TZ);
   const DivU32 dv = divu32_make(uint32_t(m.n));
+  const unsigned grid = d.blocks + d.helpers, threads = unsigned(d.warps) * 32;
   if (nm > 1)
-    k_deposit<R, TY, TZ, true><<<dim3(blocks + helpers, unsigned(nm)), warps * 32, smem, s>>>(
-        (const V4*)pos, row_start, uint32_t(n), m, dv, R(norm), rho, helpers, ms);
+    k_deposit<R, TY, TZ, true><<<dim3(grid, unsigned(nm)), threads, d.smem, s>>>(
+        (const V4*)pos, row_start, uint32_t(n), m, dv, R(norm), rho, d.blocks, d.crowd, ms);
   else
-    k_deposit<R, TY, TZ, false><<<blocks + helpers, warps * 32, smem, s>>>((const V4*)pos, row_start, uint32_t(n), m, dv,
-                                                                           R(norm), rho, helpers, 0);
+    k_deposit<R, TY, TZ, false><<<grid, threads, d.smem, s>>>((const V4*)pos, row_start, uint32_t(n), m, dv, R(norm), rho,
+                                                              d.blocks, d.crowd, 0);
   return cudaGetLastError();
 }
 
@@ -2291,27 +2246,17 @@ template <typename R>
 cudaError_t launch_deposit(const void* pos, const uint32_t* row_start, int64_t n, Mesh m, double norm, R* rho,
                            cudaStream_t s, int warps, int nm, size_t ms) {
   if (warps < 1 || warps > DEP_WARPS) warps = DEP_WARPS;
-  int ty = 1, tz = 1;
-  const int shape = deposit_shape<R>(m.n, ty, tz);
-  if (size_t(warps) * ty * tz * deposit_stride_of<R>(m.n) * sizeof(R) > 40 * 1024) {
-    // once per device, for every tile shape, so that no attribute call falls inside a stream capture
-    static DeviceOnce once;
-    const cudaError_t e = once([](int&) {
-      const void* const fns[] = {(const void*)k_deposit<R, 2, 1, false>, (const void*)k_deposit<R, 2, 1, true>,
-                                 (const void*)k_deposit<R, 2, 4, false>, (const void*)k_deposit<R, 2, 4, true>,
-                                 (const void*)k_deposit<R, 2, 2, false>, (const void*)k_deposit<R, 2, 2, true>,
-                                 (const void*)k_deposit<R, 1, 2, false>, (const void*)k_deposit<R, 1, 2, true>,
-                                 (const void*)k_deposit<R, 1, 1, false>, (const void*)k_deposit<R, 1, 1, true>};
-      return raise_smem(fns, DEP_WARPS * PM_DEPOSIT_WARP_BYTES * sizeof(R) / 4);
-    });
+  const DepositLaunch d = deposit_launch<R>(n, m.n, warps, nm);
+  if (d.smem > 40 * 1024) {
+    const cudaError_t e = deposit_prepare<R>();
     if (e != cudaSuccess) return e;
   }
-  switch (shape) {
-    case 0: return launch_deposit_tile<R, 2, 4>(pos, row_start, n, m, norm, rho, s, warps, nm, ms);
-    case 1: return launch_deposit_tile<R, 2, 2>(pos, row_start, n, m, norm, rho, s, warps, nm, ms);
-    case 2: return launch_deposit_tile<R, 2, 1>(pos, row_start, n, m, norm, rho, s, warps, nm, ms);
-    case 3: return launch_deposit_tile<R, 1, 2>(pos, row_start, n, m, norm, rho, s, warps, nm, ms);
-    default: return launch_deposit_tile<R, 1, 1>(pos, row_start, n, m, norm, rho, s, warps, nm, ms);
+  switch (d.shape) {
+    case 0: return launch_deposit_tile<R, 2, 4>(d, pos, row_start, n, m, norm, rho, s, nm, ms);
+    case 1: return launch_deposit_tile<R, 2, 2>(d, pos, row_start, n, m, norm, rho, s, nm, ms);
+    case 2: return launch_deposit_tile<R, 2, 1>(d, pos, row_start, n, m, norm, rho, s, nm, ms);
+    case 3: return launch_deposit_tile<R, 1, 2>(d, pos, row_start, n, m, norm, rho, s, nm, ms);
+    default: return launch_deposit_tile<R, 1, 1>(d, pos, row_start, n, m, norm, rho, s, nm, ms);
   }
 }
 

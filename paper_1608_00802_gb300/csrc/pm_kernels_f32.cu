@@ -26,7 +26,8 @@ cudaError_t launch_sort_histogram(const uint32_t* keys, int64_t n, int passes, i
 }
 
 cudaError_t launch_row_start(const uint32_t* keys, int64_t n, uint32_t n_mesh, uint32_t* row_start, cudaStream_t s) {
-  k_row_start<<<unsigned((n + 1 + 255) / 256), 256, 0, s>>>(keys, n, n_mesh, n_mesh * n_mesh, row_start);
+  k_row_start<<<unsigned((n + 1 + 255) / 256), 256, 0, s>>>(keys, n, n_mesh, n_mesh * n_mesh, row_start,
+                                                             deposit_crowd(n, int(n_mesh)));
   return cudaGetLastError();
 }
 

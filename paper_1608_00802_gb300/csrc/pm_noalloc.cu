@@ -71,8 +71,9 @@ pm_status scratch_address(unsigned char** out, int* device) {
   if (!g_ready[dev]) {
     void* p = nullptr;
     cudaError_t e = cudaGetSymbolAddress(&p, g_scratch);
+    if (e == cudaSuccess) e = deposit_prepare<float>();
     if (e != cudaSuccess || !p) {
-      snprintf(g_msg, sizeof g_msg, "cudaGetSymbolAddress of the static scratch failed: %s", cudaGetErrorString(e));
+      snprintf(g_msg, sizeof g_msg, "static scratch address or deposit preparation: %s", cudaGetErrorString(e));
       return nfail(PM_ERR_CUDA, g_msg);
     }
     g_addr[dev] = p;

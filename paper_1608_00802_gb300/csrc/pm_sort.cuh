@@ -337,14 +337,14 @@ __global__ void __launch_bounds__(RS_THREADS) k_sort_pass(
 // at all).  Rows are clamped to N^2: a key outside the mesh (a slot left
 // unwritten by a sort whose look-back timed out) writes nothing past the table.
 static __global__ void k_row_start(const uint32_t* __restrict__ keys, int64_t n, uint32_t n_mesh, uint32_t nrows,
-                                   uint32_t* row_start) {
+                                   uint32_t* row_start, uint32_t crowd) {
   const int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
   if (i > n) return;
   const int64_t prev = i == 0 ? -1 : min(int64_t(__ldg(keys + i - 1) / n_mesh), int64_t(nrows));
   const int64_t cur = i == n ? int64_t(nrows) : min(int64_t(__ldg(keys + i) / n_mesh), int64_t(nrows));
   for (int64_t r = prev + 1; r <= cur; ++r) row_start[r] = uint32_t(i);
-  // row of slot i holds slot i - DEP_CROWD too: more than DEP_CROWD records (every such slot stores the same)
-  if (i < n && i >= int64_t(DEP_CROWD) && cur < int64_t(nrows) && int64_t(__ldg(keys + i - DEP_CROWD) / n_mesh) == cur)
+  // row of slot i holds slot i - crowd too: more than `crowd` records (every such slot stores the same)
+  if (i < n && i >= int64_t(crowd) && cur < int64_t(nrows) && int64_t(__ldg(keys + i - crowd) / n_mesh) == cur)
     row_start[nrows + 1] = 1u;
 }
 
@@ -594,7 +594,7 @@ static __global__ void __launch_bounds__(RT_THREADS) k_row_scan(const uint32_t* 
                                                                 const uint32_t* __restrict__ btot,
                                                                 uint32_t* __restrict__ srow, uint32_t* __restrict__ mrow,
                                                                 uint32_t* __restrict__ row_start,
-                                                                uint32_t* __restrict__ step, size_t ms) {
+                                                                uint32_t* __restrict__ step, uint32_t crowd, size_t ms) {
   __shared__ uint32_t sh[2][32];
   __shared__ uint32_t base[2];
   if (ms) {
@@ -676,7 +676,7 @@ static __global__ void __launch_bounds__(RT_THREADS) k_row_scan(const uint32_t* 
       srow[r] = xa;
       mrow[r] = xb;
       row_start[r] = xa + xb;
-      if (ca[k] + cb[k] > DEP_CROWD) row_start[nrows + 1] = 1u;  // (every such row stores the same)
+      if (ca[k] + cb[k] > crowd) row_start[nrows + 1] = 1u;  // (every such row stores the same)
     }
     xa += ca[k];
     xb += cb[k];
@@ -865,7 +865,7 @@ __global__ void __launch_bounds__(SS_THREADS, 1) k_sort_small(const uint32_t* ke
                                                               const V4* __restrict__ pos_in, const V4* __restrict__ mom_in,
                                                               V4* __restrict__ pos_out, V4* __restrict__ mom_out,
                                                               uint32_t* __restrict__ row_start, uint32_t n_mesh,
-                                                              int log2n, uint32_t* clear) {
+                                                              int log2n, uint32_t crowd, uint32_t* clear) {
   constexpr uint32_t chunk = ITEMS * SS_THREADS;
   namespace cg = cooperative_groups;
   extern __shared__ __align__(16) unsigned char ss_smem[];
@@ -991,7 +991,7 @@ __global__ void __launch_bounds__(SS_THREADS, 1) k_sort_small(const uint32_t* ke
       if (i > 0) a = int(min(key_row(key_at(i - 1), n_mesh, log2n), nrows - 1)) + 1;
       b = row;
       if (i == n - 1) a2 = row + 1, b2 = int(nrows);
-      if (i >= DEP_CROWD && key_row(key_at(i - DEP_CROWD), n_mesh, log2n) == uint32_t(row)) row_start[nrows + 1] = 1u;
+      if (i >= crowd && key_row(key_at(i - crowd), n_mesh, log2n) == uint32_t(row)) row_start[nrows + 1] = 1u;
     }
     fill_rows(row_start, a, b, i);
     fill_rows(row_start, a2, b2, n);
@@ -1032,7 +1032,7 @@ cudaError_t launch_sort_small_items(const uint32_t* keys_in, uint32_t n, int key
   cfg.gridDim = dim3(ctas);
   at[0].val.clusterDim.x = ctas;
   return cudaLaunchKernelEx(&cfg, k_sort_small<V4, ITEMS>, keys_in, n, passes, digit_bits, key_bits, keys_out, pos_in,
-                            mom_in, pos_out, mom_out, row_start, uint32_t(m.n), m.log2n, clear);
+                            mom_in, pos_out, mom_out, row_start, uint32_t(m.n), m.log2n, deposit_crowd(n, m.n), clear);
 }
 
 template <typename R>
@@ -1091,7 +1091,7 @@ inline cudaError_t launch_resort_place(int part, const uint32_t* keys, int64_t n
     const bool direct = nb <= RT_DIRECT_TILES;
     if (!direct) k_row_totals<<<dim3(nb, unsigned(nm)), RT_THREADS, 0, s>>>(rcnt, nrows, btot, o);
     k_row_scan<<<dim3(nb, unsigned(nm)), RT_THREADS, 0, s>>>(rcnt, nrows, direct ? nullptr : btot, srow, mrow, row_start,
-                                                            step, o);
+                                                            step, deposit_crowd(n, m.n), o);
     // the bucket scatter runs over the device's mover count: a grid of resident blocks shared by the members
     int64_t cap = int64_t(16) * sms / nm;
     if (cap < 1) cap = 1;
