@@ -74,13 +74,29 @@ inline int deposit_shape(int n, int& ty, int& tz) {
   return s;
 }
 
-// records per window of a helper block (the batch sums of a window are kept in shared memory)
+// most records per window of a helper block (the batch sums of a window are kept in shared memory)
 template <typename R>
 constexpr int DEP_WINDOW = sizeof(R) == 4 ? 2048 : 1024;
-// shared memory of a helper block: the window's sums, each cell's first and last record of the window, the row
+// shared memory of a helper block with a window of w records: the window's sums, the row, each cell's first and last
+// record of the window
 template <typename R>
-inline size_t deposit_crowd_smem(int n) {
-  return size_t(2 * DEP_WINDOW<R> + deposit_stride_of<R>(n)) * sizeof(R) + size_t(2 * n) * sizeof(uint32_t);
+inline size_t deposit_crowd_smem(int n, int w) {
+  return size_t(2 * w + deposit_stride_of<R>(n)) * sizeof(R) + size_t(2 * n) * sizeof(uint16_t);
+}
+// Shared memory of a deposit block of `warps` warps whose tiles take `tiles` bytes, and its helpers' window.  The
+// window does not enter the result (it is whole batches), so a block of few warps takes a small one, a full window with
+// 8 warps: with a full one for any block, blocks of 1 and 2 warps on 256^3 took 88 and 55 us for 43 and 41, and a batch
+// of mixed sizes with 4 warps 2796 us a step for 2552.
+#ifndef PM_DEP_CROWD_WARP
+#define PM_DEP_CROWD_WARP 2304
+#endif
+template <typename R>
+inline size_t deposit_smem(int n, int warps, size_t tiles, int* window) {
+  size_t smem = std::max(tiles, std::min(deposit_crowd_smem<R>(n, DEP_WINDOW<R>), size_t(warps) * PM_DEP_CROWD_WARP));
+  smem = std::max(smem, deposit_crowd_smem<R>(n, 64));
+  const int w = int((smem - deposit_crowd_smem<R>(n, 0)) / (2 * sizeof(R))) & ~31;
+  *window = std::min(w, DEP_WINDOW<R>);
+  return smem;
 }
 
 struct DepositLaunch {
@@ -88,6 +104,7 @@ struct DepositLaunch {
   int warps;                 // per block
   unsigned blocks, helpers;  // of the tiles, and after them for the crowded rows
   uint32_t crowd;            // deposit_crowd
+  int window;                // records of a helper's window
   size_t smem;               // dynamic shared memory of a block
 };
 
@@ -110,7 +127,7 @@ inline DepositLaunch deposit_launch(int64_t n_part, int n_mesh, int warps, int n
   const unsigned most = std::max(8u, std::min(unsigned(PM_DEP_HELPERS * DEP_WARPS / (warps * nm)), n2 / 16 + 1));
   const unsigned part = unsigned(0.382 * n_mesh);
   d.helpers = most >= N + part ? (most - part) / N * N + part : most;
-  d.smem = std::max(d.smem, deposit_crowd_smem<R>(n_mesh));
+  d.smem = deposit_smem<R>(n_mesh, warps, d.smem, &d.window);
   return d;
 }
 

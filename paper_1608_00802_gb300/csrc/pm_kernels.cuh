@@ -395,11 +395,10 @@ __device__ __forceinline__ DepRow deposit_row_of(const uint32_t* __restrict__ ro
 template <typename R>
 __device__ __forceinline__ void deposit_add_segment(const typename VT<R>::v4* __restrict__ pos, uint32_t s0, uint32_t s1,
                                                     uint32_t cs, uint32_t base, bool dy, bool dz, int n, R* acc,
-                                                    R* sums, uint32_t* cell_range) {
-  constexpr uint32_t W = DEP_WINDOW<R>;
+                                                    R* sums, uint16_t* cell_range, uint32_t W) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-  uint32_t* first = cell_range;    // first[c], last[c]: the window's records of cell c (last < first: none)
-  uint32_t* last = cell_range + n;
+  uint16_t* first = cell_range;    // first[c], last[c]: the window's records of cell c (last < first: none)
+  uint16_t* last = cell_range + n;
   // windows of whole batches
   for (uint32_t w0 = s0; w0 < s1;) {
     const uint32_t w1 = min(s1, cs + ((w0 - cs) / 32 + W / 32) * 32);
@@ -420,11 +419,11 @@ __device__ __forceinline__ void deposit_add_segment(const typename VT<R>::v4* __
       if (runs != 0xffffffffu) run_sums<R, 2>(v, runs, lane);
       if (valid) {
         // a run's first lane opens the cell unless the cell's previous run is in this window too
-        if (((runs >> lane) & 1u) && !(p > w0 && lane == 0 && rec_cell(ldg(pos + p - 1)) == rec_cell(rec))) first[x] = p;
+        if (((runs >> lane) & 1u) && !(p > w0 && lane == 0 && rec_cell(ldg(pos + p - 1)) == rec_cell(rec))) first[x] = uint16_t(p - w0);
         if (lane == 31 || ((runs >> (lane + 1)) & 1u)) {
           sums[2 * (p - w0)] = v[0];
           sums[2 * (p - w0) + 1] = v[1];
-          if (!(p + 1 < w1 && lane == 31 && rec_cell(ldg(pos + p + 1)) == rec_cell(rec))) last[x] = p;
+          if (!(p + 1 < w1 && lane == 31 && rec_cell(ldg(pos + p + 1)) == rec_cell(rec))) last[x] = uint16_t(p - w0);
         }
       }
     }
@@ -436,10 +435,10 @@ __device__ __forceinline__ void deposit_add_segment(const typename VT<R>::v4* __
       for (int h = 1; h >= 0; --h) {
         const int c = X - h;
         if (c < 0 || c >= n) continue;
-        const uint32_t l = last[c];
+        const uint32_t l = last[c], o = w0 - cs;
         for (uint32_t p = first[c]; p <= l;) {
-          const uint32_t at = min(l, cs + ((p - cs) | 31u));  // the run's last record: the cell's, or the batch's
-          a += sums[2 * (at - w0) + h];
+          const uint32_t at = min(l, ((o + p) | 31u) - o);  // the run's last record: the cell's, or the batch's
+          a += sums[2 * at + h];
           p = at + 1;
         }
       }
@@ -456,11 +455,12 @@ __device__ __forceinline__ void deposit_add_segment(const typename VT<R>::v4* __
 template <typename R, int TY>
 __device__ __forceinline__ void deposit_crowded_row(const typename VT<R>::v4* __restrict__ pos,
                                                     const uint32_t* __restrict__ row_start, uint32_t np, const Mesh& m,
-                                                    R norm, R* __restrict__ rho, unsigned char* smem, uint32_t row) {
+                                                    R norm, R* __restrict__ rho, unsigned char* smem, uint32_t W,
+                                                    uint32_t row) {
   const int n = m.n;
   R* sums = reinterpret_cast<R*>(smem);
-  R* acc = sums + 2 * DEP_WINDOW<R>;
-  uint32_t* cell_range = reinterpret_cast<uint32_t*>(acc + deposit_stride_of<R>(n));
+  R* acc = sums + 2 * W;
+  uint16_t* cell_range = reinterpret_cast<uint16_t*>(acc + deposit_stride_of<R>(n));
   const int z = int(row / uint32_t(n)), y = int(row - uint32_t(z) * uint32_t(n)), y0 = y - y % TY;
   for (int i = threadIdx.x; i <= n; i += blockDim.x) acc[i] = R(0);
   __syncthreads();
@@ -477,12 +477,12 @@ __device__ __forceinline__ void deposit_crowded_row(const typename VT<R>::v4* __
       const uint32_t k0 = cb + (B.b - cb) / 32 * 32;
       ae = max(A.b, k0), bs = min(B.e, k0 + 32);
     }
-    deposit_add_segment<R>(pos, A.b, ae, ca, ra * uint32_t(n), true, dz, n, acc, sums, cell_range);
+    deposit_add_segment<R>(pos, A.b, ae, ca, ra * uint32_t(n), true, dz, n, acc, sums, cell_range, W);
     if (bs > B.b) {
-      deposit_add_segment<R>(pos, B.b, bs, cb, rb * uint32_t(n), false, dz, n, acc, sums, cell_range);
-      deposit_add_segment<R>(pos, ae, A.e, ca, ra * uint32_t(n), true, dz, n, acc, sums, cell_range);
+      deposit_add_segment<R>(pos, B.b, bs, cb, rb * uint32_t(n), false, dz, n, acc, sums, cell_range, W);
+      deposit_add_segment<R>(pos, ae, A.e, ca, ra * uint32_t(n), true, dz, n, acc, sums, cell_range, W);
     }
-    deposit_add_segment<R>(pos, bs, B.e, cb, rb * uint32_t(n), false, dz, n, acc, sums, cell_range);
+    deposit_add_segment<R>(pos, bs, B.e, cb, rb * uint32_t(n), false, dz, n, acc, sums, cell_range, W);
   }
   R* out = rho + size_t(row) * n;
   for (int i = threadIdx.x; i < n; i += blockDim.x) out[i] = (i == 0 ? acc[0] + acc[n] : acc[i]) * norm;
@@ -494,8 +494,8 @@ __device__ __forceinline__ void deposit_crowded_row(const typename VT<R>::v4* __
 template <typename R, int TY, int TZ>
 __device__ __noinline__ void deposit_crowded(const typename VT<R>::v4* __restrict__ pos,
                                              const uint32_t* __restrict__ row_start, uint32_t np, const Mesh m, R norm,
-                                             R* __restrict__ rho, unsigned char* smem, uint32_t crowd, uint32_t hb,
-                                             uint32_t H) {
+                                             R* __restrict__ rho, unsigned char* smem, uint32_t crowd, uint32_t W,
+                                             uint32_t hb, uint32_t H) {
   __shared__ uint32_t list[DEP_WARPS * 32];
   __shared__ uint32_t found;
   const int n = m.n;
@@ -517,7 +517,7 @@ __device__ __noinline__ void deposit_crowded(const typename VT<R>::v4* __restric
     }
     __syncthreads();
     const uint32_t c = found;
-    for (uint32_t i = 0; i < c; ++i) deposit_crowded_row<R, TY>(pos, row_start, np, m, norm, rho, smem, list[i]);
+    for (uint32_t i = 0; i < c; ++i) deposit_crowded_row<R, TY>(pos, row_start, np, m, norm, rho, smem, W, list[i]);
     __syncthreads();
   }
 }
@@ -526,7 +526,7 @@ template <typename R, int TY, int TZ, bool PACKED>
 __global__ void __launch_bounds__(DEP_WARPS * 32) k_deposit(const typename VT<R>::v4* __restrict__ pos,
                                                             const uint32_t* __restrict__ row_start, uint32_t np,
                                                             Mesh m, DivU32 dvn, R norm, R* __restrict__ rho,
-                                                            uint32_t mains, uint32_t crowd, size_t ms) {
+                                                            uint32_t mains, uint32_t crowd, uint32_t window, size_t ms) {
   using V4 = typename VT<R>::v4;
   static_assert((TY + 1) * (TZ + 1) <= 32, "one source row per lane");
   if constexpr (PACKED) {  // member blockIdx.y of a packed group
@@ -536,7 +536,7 @@ __global__ void __launch_bounds__(DEP_WARPS * 32) k_deposit(const typename VT<R>
   extern __shared__ __align__(16) unsigned char dep_smem[];
   if (blockIdx.x >= mains) {
     if (__ldg(row_start + m.n2 + 1))  // some row is crowded
-      deposit_crowded<R, TY, TZ>(pos, row_start, np, m, norm, rho, dep_smem, crowd, blockIdx.x - mains,
+      deposit_crowded<R, TY, TZ>(pos, row_start, np, m, norm, rho, dep_smem, crowd, window, blockIdx.x - mains,
                                  gridDim.x - mains);
     return;
   }
@@ -2235,10 +2235,10 @@ cudaError_t launch_deposit_tile(const DepositLaunch& d, const void* pos, const u
   const unsigned grid = d.blocks + d.helpers, threads = unsigned(d.warps) * 32;
   if (nm > 1)
     k_deposit<R, TY, TZ, true><<<dim3(grid, unsigned(nm)), threads, d.smem, s>>>(
-        (const V4*)pos, row_start, uint32_t(n), m, dv, R(norm), rho, d.blocks, d.crowd, ms);
+        (const V4*)pos, row_start, uint32_t(n), m, dv, R(norm), rho, d.blocks, d.crowd, uint32_t(d.window), ms);
   else
     k_deposit<R, TY, TZ, false><<<grid, threads, d.smem, s>>>((const V4*)pos, row_start, uint32_t(n), m, dv, R(norm), rho,
-                                                              d.blocks, d.crowd, 0);
+                                                              d.blocks, d.crowd, uint32_t(d.window), 0);
   return cudaGetLastError();
 }
 

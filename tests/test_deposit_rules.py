@@ -1,7 +1,7 @@
 """The deposit's launch rules.  No GPU: the host functions, compiled by themselves.
 
 A mesh row counts as crowded, so that whole blocks compute the rows it adds to, where it stands out in a clustered
-state, and never in a uniform one, however dense."""
+state, and never in a uniform one, however dense.  Blocks of few warps take little shared memory."""
 import ctypes
 import os
 import subprocess
@@ -12,6 +12,13 @@ CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))),
 SRC = """
 #include "pm_deposit_shape.h"
 extern "C" uint32_t crowd(int64_t n, int mesh) { return pm::deposit_crowd(n, mesh); }
+static void put(const pm::DepositLaunch& d, int64_t* out) {
+  const int64_t v[] = {d.ty, d.tz, d.warps, d.blocks, d.helpers, int64_t(d.smem), d.window};
+  for (int i = 0; i < 7; ++i) out[i] = v[i];
+}
+extern "C" void launch(int fp64, int64_t n, int mesh, int warps, int nm, int64_t* out) {
+  fp64 ? put(pm::deposit_launch<double>(n, mesh, warps, nm), out) : put(pm::deposit_launch<float>(n, mesh, warps, nm), out);
+}
 """
 
 
@@ -46,3 +53,34 @@ def test_the_rows_of_a_core_are_crowded(lib):
     for n_mesh in (8, 64, 1024):
         for n in (1, 10 ** 5, 2 ** 31 - 1):
             assert 256 <= lib.crowd(n, n_mesh) <= max(256, n // 3000, 2 * n // n_mesh ** 2)
+
+
+FIELDS = ("ty", "tz", "warps", "blocks", "helpers", "smem", "window")
+
+
+def _launch(lib, fp64, n, n_mesh, warps, nm=1):
+    out = (ctypes.c_int64 * len(FIELDS))()
+    lib.launch(int(fp64), ctypes.c_int64(n), n_mesh, warps, nm, out)
+    return dict(zip(FIELDS, out))
+
+
+def _tiles(fp64, n_mesh, d):
+    size = 8 if fp64 else 4
+    return d["warps"] * d["ty"] * d["tz"] * (-(-(n_mesh + 1) * size // 16) * 16)
+
+
+@pytest.mark.parametrize("fp64", [False, True])
+@pytest.mark.parametrize("n_mesh", [8, 30, 64, 128, 250, 256, 512, 1024])
+@pytest.mark.parametrize("warps", [1, 2, 4, 8])
+def test_helpers_add_little_shared_memory(lib, fp64, n_mesh, warps):
+    """The helpers' window fits the block's shared memory, and asks for more than the tiles' only up to 2304 bytes
+    a warp (or the least window of 64 records)."""
+    size = 8 if fp64 else 4
+    for n, nm in ((257, 1), (n_mesh ** 3 // 8 + 300, 2), (100000, 16)):
+        d = _launch(lib, fp64, n, n_mesh, warps, nm)
+        row = -(-(n_mesh + 1) * size // 16) * 16
+        assert 64 <= d["window"] <= (1024 if fp64 else 2048) and d["window"] % 32 == 0
+        least = 2 * 64 * size + row + 4 * n_mesh
+        assert 2 * d["window"] * size + row + 4 * n_mesh <= d["smem"]
+        assert d["smem"] <= max(_tiles(fp64, n_mesh, d), 2304 * d["warps"], least)
+    assert _launch(lib, fp64, 256, n_mesh, warps)["helpers"] == 0
