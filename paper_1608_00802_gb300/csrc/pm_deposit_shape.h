@@ -36,6 +36,10 @@ inline uint32_t deposit_crowd(int64_t n_part, int n_mesh) {
 constexpr size_t CROWD_WORDS = 2;
 
 constexpr int DEP_WARPS = 8;  // most warps of a block
+// what fits an SM: blocks of 40 warps together with the kernel's 48 registers; its shared memory, of which a block takes
+// 1040 bytes of its own and 1 KB of the system's besides the dynamic
+constexpr unsigned DEP_SMS = 152, DEP_SM_WARPS = 40;
+constexpr size_t DEP_SM_SMEM = 228 * 1024, DEP_BLOCK_SMEM = 2064;
 
 // slots of a deposit row: N + 1 rounded up to 16 bytes
 template <typename R>
@@ -128,6 +132,19 @@ inline DepositLaunch deposit_launch(int64_t n_part, int n_mesh, int warps, int n
   const unsigned part = unsigned(0.382 * n_mesh);
   d.helpers = most >= N + part ? (most - part) / N * N + part : most;
   d.smem = deposit_smem<R>(n_mesh, warps, d.smem, &d.window);
+  // The helpers come at the end of the tiles' grid.  Where the tiles alone leave room on the SMs, the longer grid is
+  // no longer spread evenly over them and some SMs get more than their share of the tiles (128^3 with a particle
+  // per cell: fp64 359 -> 527 us, fp32 43 -> 51; 64^3 particles in fp64 57 -> 78), so shared memory keeps an SM
+  // to its even share: 357, 43 and 57 us again.  In fp32 only when not all blocks are resident at once and from 2^21
+  // particles: the other kernels' share of the SM changes with the deposit's, which costs ~4 us a call, as
+  // much as the even spread saves there (10^6 particles in a core: 3147 -> 3180 us a run).  Not in packed groups: they
+  // run beside others, which lose more by the shared memory (8 members each of 64^3, 128^3, 256^3: 2552 -> 2728 us).
+  if (nm == 1 && (sizeof(R) == 8 || n_part >= int64_t(1) << 21)) {
+    const unsigned share = (d.blocks + DEP_SMS - 1) / DEP_SMS;
+    const unsigned per_sm = std::min(DEP_SM_WARPS / unsigned(warps), unsigned(DEP_SM_SMEM / (d.smem + DEP_BLOCK_SMEM)));
+    if (share < per_sm && d.blocks + d.helpers > DEP_SMS * (sizeof(R) == 8 ? share : per_sm))
+      d.smem = std::max(d.smem, (DEP_SM_SMEM / (share + 1) - DEP_BLOCK_SMEM) / 256 * 256 + 256);
+  }
   return d;
 }
 

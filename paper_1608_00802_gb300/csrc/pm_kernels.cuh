@@ -2223,7 +2223,7 @@ cudaError_t deposit_prepare() {
                                (const void*)k_deposit<R, 2, 2, false>, (const void*)k_deposit<R, 2, 2, true>,
                                (const void*)k_deposit<R, 1, 2, false>, (const void*)k_deposit<R, 1, 2, true>,
                                (const void*)k_deposit<R, 1, 1, false>, (const void*)k_deposit<R, 1, 1, true>};
-    return raise_smem(fns, DEP_WARPS * PM_DEPOSIT_WARP_BYTES * sizeof(R) / 4);
+    return raise_smem(fns, DEP_SM_SMEM / 2);
   });
 }
 

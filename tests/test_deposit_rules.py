@@ -1,7 +1,8 @@
 """The deposit's launch rules.  No GPU: the host functions, compiled by themselves.
 
 A mesh row counts as crowded, so that whole blocks compute the rows it adds to, where it stands out in a clustered
-state, and never in a uniform one, however dense.  Blocks of few warps take little shared memory."""
+state, and never in a uniform one, however dense.  Blocks of few warps take little shared
+memory, and no SM gets more than its share of the tiles."""
 import ctypes
 import os
 import subprocess
@@ -82,5 +83,21 @@ def test_helpers_add_little_shared_memory(lib, fp64, n_mesh, warps):
         assert 64 <= d["window"] <= (1024 if fp64 else 2048) and d["window"] % 32 == 0
         least = 2 * 64 * size + row + 4 * n_mesh
         assert 2 * d["window"] * size + row + 4 * n_mesh <= d["smem"]
-        assert d["smem"] <= max(_tiles(fp64, n_mesh, d), 2304 * d["warps"], least)
+        assert d["smem"] <= max(_tiles(fp64, n_mesh, d), 2304 * d["warps"], least) or (fp64 and nm == 1)
     assert _launch(lib, fp64, 256, n_mesh, warps)["helpers"] == 0
+
+
+def test_no_sm_gets_more_than_its_share_of_the_tiles(lib):
+    """Tiles that leave room on the SMs, with helper blocks behind them: shared memory keeps an SM to ceil(tiles / 152)
+    blocks (228 KB, of which a block takes 2064 bytes besides) in fp64, and in fp32 from 2^21 particles."""
+    def fit(d):
+        return 228 * 1024 // (d["smem"] + 2064)
+    for n, n_mesh, warps in ((48 ** 3, 96, 4), (64 ** 3, 128, 8), (128 ** 3, 128, 8), (128 ** 3, 128, 4), (32 ** 3, 64, 2)):
+        d = _launch(lib, True, n, n_mesh, warps)
+        assert fit(d) == -(-d["blocks"] // 152), (n, n_mesh, warps, d)
+        assert d["smem"] <= 228 * 1024 // 2
+    d = _launch(lib, False, 128 ** 3, 128, 8)
+    assert fit(d) == -(-d["blocks"] // 152)
+    for nm, n, n_mesh in ((1, 1_000_000, 128), (1, 64 ** 3, 128), (8, 64 ** 3, 128), (1, 32 ** 3, 64), (1, 128 ** 3, 256)):
+        d = _launch(lib, False, n, n_mesh, 8, nm)
+        assert d["smem"] <= max(_tiles(False, n_mesh, d), 2304 * d["warps"])
