@@ -58,22 +58,24 @@ PM_DEP_HD inline int deposit_stride_of(int n) {
 #ifndef PM_DEPOSIT_WARP_BYTES
 #define PM_DEPOSIT_WARP_BYTES 4352
 #endif
-// Small meshes take fewer planes per tile while the tiles are fewer than PM_DEPOSIT_MIN_TILES warps (16 per SM):
-// a warp's time is its chain of batches, one or two per plane, so 64^3 goes from 512 tiles of five source
-// planes (6.9 us) to 2048 of two (4.2 us; 4096 particles on 32^3 7.2 -> 3.9 us).  Not in fp64, whose pipe pays
+// Small meshes take fewer planes per tile while the launch's tiles (of all nm members of a packed group) are fewer
+// than PM_DEPOSIT_MIN_TILES warps (16 per SM): a warp's time is its chain of batches, one or two per plane, so 64^3
+// goes from 512 tiles of five source planes (6.9 us) to 2048 of two (4.2 us; 4096 particles on 32^3 7.2 -> 3.9 us).  A
+// packed group that has the warps anyway keeps the thick tiles, which read each record less often (16 members: 64^3
+// 124 -> 119 us a step, 128^3 645 -> 637).  Not in fp64, whose pipe pays
 // for every record read again (14.1 -> 14.7 us).  The planes of a tile do not enter its result: a row's batches
 // are cut by its chain, which only the rows in y decide, and added plane by plane.
 #ifndef PM_DEPOSIT_MIN_TILES
 #define PM_DEPOSIT_MIN_TILES 2432
 #endif
 template <typename R>
-inline int deposit_shape(int n, int& ty, int& tz) {
+inline int deposit_shape(int n, int nm, int& ty, int& tz) {
   static const int shapes[5][2] = {{2, 4}, {2, 2}, {2, 1}, {1, 2}, {1, 1}};
   const size_t row = size_t(deposit_stride_of<R>(n)) * sizeof(R);
   const size_t most = size_t(PM_DEPOSIT_WARP_BYTES) * sizeof(R) / 4;
   int s = 0;
   while (s < 4 && (size_t(shapes[s][0] * shapes[s][1]) * row > most || s == 2)) ++s;
-  while (sizeof(R) == 4 && s < 2 && ((n + 1) / 2) * ((n + shapes[s][1] - 1) / shapes[s][1]) < PM_DEPOSIT_MIN_TILES) ++s;
+  while (sizeof(R) == 4 && s < 2 && nm * ((n + 1) / 2) * ((n + shapes[s][1] - 1) / shapes[s][1]) < PM_DEPOSIT_MIN_TILES) ++s;
   ty = shapes[s][0], tz = shapes[s][1];
   return s;
 }
@@ -116,7 +118,10 @@ struct DepositLaunch {
 template <typename R>
 inline DepositLaunch deposit_launch(int64_t n_part, int n_mesh, int warps, int nm) {
   DepositLaunch d = {};
-  d.shape = deposit_shape<R>(n_mesh, d.ty, d.tz);
+  // A packed group fills the chip with any block size, and beside other groups small blocks get in the way of kernels
+  // that need much of an SM (8 members each of 64^3, 128^3 and 256^3: 2761 us a step with 2 warps, 2552 with 4)
+  if (nm > 1 && warps < 4) warps = 4;
+  d.shape = deposit_shape<R>(n_mesh, nm, d.ty, d.tz);
   d.warps = warps;
   const unsigned N = unsigned(n_mesh), n2 = N * N;
   d.blocks = unsigned((n_mesh + warps * d.ty - 1) / (warps * d.ty)) * unsigned((n_mesh + d.tz - 1) / d.tz);

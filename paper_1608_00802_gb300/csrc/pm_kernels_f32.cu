@@ -63,7 +63,7 @@ Tuning default_tuning(int n, int64_t n_part, bool fp64) {
   // small meshes: fewer warps per deposit block while the tiles would leave SMs idle (the 512 tiles of 2 x 4 rows
   // of a 64^3 fp64 mesh: 17.9 us in 64 blocks of 8 warps, 14.1 in 256 of 2)
   int ty = 1, tz = 1;
-  fp64 ? deposit_shape<double>(n, ty, tz) : deposit_shape<float>(n, ty, tz);
+  fp64 ? deposit_shape<double>(n, 1, ty, tz) : deposit_shape<float>(n, 1, ty, tz);
   const int tiles = ((n + ty - 1) / ty) * ((n + tz - 1) / tz);
   t.dep_warps = 8;
   while (t.dep_warps > 2 && tiles / t.dep_warps < 152) t.dep_warps /= 2;

@@ -2,7 +2,7 @@
 
 A mesh row counts as crowded, so that whole blocks compute the rows it adds to, where it stands out in a clustered
 state, and never in a uniform one, however dense.  Blocks of few warps take little shared
-memory, and no SM gets more than its share of the tiles."""
+memory, no SM gets more than its share of the tiles, and a packed group's tiles are those of its whole launch."""
 import ctypes
 import os
 import subprocess
@@ -101,3 +101,13 @@ def test_no_sm_gets_more_than_its_share_of_the_tiles(lib):
     for nm, n, n_mesh in ((1, 1_000_000, 128), (1, 64 ** 3, 128), (8, 64 ** 3, 128), (1, 32 ** 3, 64), (1, 128 ** 3, 256)):
         d = _launch(lib, False, n, n_mesh, 8, nm)
         assert d["smem"] <= max(_tiles(False, n_mesh, d), 2304 * d["warps"])
+
+
+def test_packed_groups_take_the_tiles_of_their_whole_launch(lib):
+    """Thin tiles only while the launch's warps leave SMs idle; blocks of at least four warps."""
+    for n_mesh, alone, packed in ((64, (2, 1), (2, 4)), (128, (2, 2), (2, 4)), (256, (2, 2), (2, 2))):
+        n = (n_mesh // 2) ** 3
+        for warps in (1, 2, 4, 8):
+            d, g = _launch(lib, False, n, n_mesh, warps), _launch(lib, False, n, n_mesh, warps, 16)
+            assert (d["ty"], d["tz"], d["warps"]) == (*alone, warps)
+            assert (g["ty"], g["tz"], g["warps"]) == (*packed, max(warps, 4))
