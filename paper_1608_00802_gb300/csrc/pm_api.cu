@@ -396,6 +396,16 @@ int kr_blocks(const pm_sim* s) {
   return tiled ? stencil_launch_blocks(s->cfg.n_mesh, s->tune.st_ty, s->tune.st_zlen) : MESH_GRID;
 }
 
+// an internal stream or event, made when first needed
+pm_status make_stream(pm_sim* s, cudaStream_t* q) {
+  if (!*q) CU(s, cudaStreamCreateWithFlags(q, cudaStreamNonBlocking));
+  return PM_OK;
+}
+pm_status make_event(pm_sim* s, cudaEvent_t* e) {
+  if (!*e) CU(s, cudaEventCreateWithFlags(e, cudaEventDisableTiming));
+  return PM_OK;
+}
+
 // the counts of a drift whose re-sort did not run, or not to its end (an error between them)
 pm_status drop_mover_counts(pm_sim* s) {
   const size_t N = size_t(s->cfg.n_mesh);
@@ -1294,24 +1304,14 @@ pm_status pm_create(const pm_config* c, void* dev_arena, size_t bytes, void* str
 pm_status pm_destroy(pm_sim* s) {
   if (!s) return PM_ERR_INVALID_ARG;
   cudaStreamSynchronize(s->stream);
-  if (s->cap) {
-    cudaStreamSynchronize(s->cap);
-    cudaStreamDestroy(s->cap);
-    cudaEventDestroy(s->ev_in);
-    cudaEventDestroy(s->ev_out);
-    cudaEventDestroy(s->ev_tab);
-    cudaFreeHost(s->tab_host);
-    cudaStreamSynchronize(s->branch);
-    cudaStreamDestroy(s->branch);
-    cudaEventDestroy(s->ev_rho);
-    cudaEventDestroy(s->ev_q);
-  }
-  if (s->side) {
-    cudaStreamSynchronize(s->side);
-    cudaStreamDestroy(s->side);
-    cudaEventDestroy(s->ev_x);
-    cudaEventDestroy(s->ev_p);
-  }
+  for (cudaStream_t q : {s->cap, s->branch, s->side})
+    if (q) {
+      cudaStreamSynchronize(q);
+      cudaStreamDestroy(q);
+    }
+  for (cudaEvent_t e : {s->ev_in, s->ev_out, s->ev_tab, s->ev_rho, s->ev_q, s->ev_x, s->ev_p})
+    if (e) cudaEventDestroy(e);
+  if (s->tab_host) cudaFreeHost(s->tab_host);
   for (auto& g : s->run_graph)
     if (g.exec) cudaGraphExecDestroy(g.exec);
   for (cudaEvent_t e : s->prof_ev) cudaEventDestroy(e);
@@ -1337,11 +1337,8 @@ static pm_status load_particles(pm_sim* s, const double* x, const double* p) {
   const bool split = s->n() > SORT_SMALL_MAX;
   CU(s, cudaMemcpyAsync(dx, x, bytes, cudaMemcpyHostToDevice, s->stream));
   if (split) {
-    if (!s->side) {
-      CU(s, cudaEventCreateWithFlags(&s->ev_x, cudaEventDisableTiming));
-      CU(s, cudaEventCreateWithFlags(&s->ev_p, cudaEventDisableTiming));
-      CU(s, cudaStreamCreateWithFlags(&s->side, cudaStreamNonBlocking));
-    }
+    PMST(make_stream(s, &s->side));
+    for (cudaEvent_t* e : {&s->ev_x, &s->ev_p}) PMST(make_event(s, e));
     CU(s, cudaEventRecord(s->ev_x, s->stream));  // (also behind everything that still reads the staging area)
     CU(s, cudaStreamWaitEvent(s->side, s->ev_x, 0));
   } else {
@@ -1513,16 +1510,10 @@ pm_status pm_run(pm_sim* s, int32_t nsteps, double a_start, double a_end) {
   if (nsteps >= 2 && nsteps <= PM_RUN_GRAPH_MAX_STEPS && !s->prof_on) {
     // two steps captured as a CUDA graph and replayed: the weights of every
     // step come from a device table indexed by a device step counter
-    if (!s->cap) {
-      CU(s, cudaStreamCreateWithFlags(&s->cap, cudaStreamNonBlocking));
-      CU(s, cudaEventCreateWithFlags(&s->ev_in, cudaEventDisableTiming));
-      CU(s, cudaEventCreateWithFlags(&s->ev_out, cudaEventDisableTiming));
-      CU(s, cudaEventCreateWithFlags(&s->ev_tab, cudaEventDisableTiming));
-      CU(s, cudaStreamCreateWithFlags(&s->branch, cudaStreamNonBlocking));
-      CU(s, cudaEventCreateWithFlags(&s->ev_rho, cudaEventDisableTiming));
-      CU(s, cudaEventCreateWithFlags(&s->ev_q, cudaEventDisableTiming));
-      CU(s, cudaMallocHost(&s->tab_host, size_t(PM_RUN_GRAPH_MAX_STEPS) * sizeof(KickParams)));
-    }
+    // (each by itself: a call after one that could not create them all makes the rest)
+    for (cudaStream_t* q : {&s->cap, &s->branch}) PMST(make_stream(s, q));
+    for (cudaEvent_t* e : {&s->ev_in, &s->ev_out, &s->ev_tab, &s->ev_rho, &s->ev_q}) PMST(make_event(s, e));
+    if (!s->tab_host) CU(s, cudaMallocHost(&s->tab_host, size_t(PM_RUN_GRAPH_MAX_STEPS) * sizeof(KickParams)));
     if (s->tab_pending) CU(s, cudaEventSynchronize(s->ev_tab));  // the previous upload has left the buffer
     for (int i = 0; i < nsteps; ++i) s->tab_host[i] = step_params(s, i, nsteps, a_start, a_end, &pending);
     KickParams* tab_dev = s->at<KickParams>(s->L.ktab);
