@@ -201,6 +201,12 @@ cudaError_t launch_resort(int part, const uint32_t* keys, int64_t n, uint32_t* t
                           unsigned long long* stats, uint32_t* step, uint32_t* keys_out, const void* pos_in,
                           const void* mom_in, void* pos_out, void* mom_out, int sms, cudaStream_t s, int nm = 1,
                           size_t ms = 0);
+// blocks of the placement: a thread per record, and no more than eight of the 3 N^2 per-row counts that it clears on
+// the way per thread (by the records alone, 4096 particles on 512^3 would leave them to 16 blocks)
+inline int64_t place_blocks(int64_t n, int n_mesh, int threads) {
+  const int64_t records = (n + threads - 1) / threads, rows = 3 * int64_t(n_mesh) * n_mesh / (8 * threads) + 1;
+  return records > rows ? records : rows;
+}
 // clears the drift's marks of n keys
 cudaError_t launch_unmark_keys(uint32_t* keys, int64_t n, cudaStream_t s);
 inline size_t row_scan_tiles(int n_mesh) { return (size_t(n_mesh) * n_mesh + 1023) / 1024; }  // tiles of 1024 rows

@@ -1103,7 +1103,7 @@ inline cudaError_t launch_resort_place(int part, const uint32_t* keys, int64_t n
     // a grid of resident blocks shared by the members, striding over the records
     int64_t cap = int64_t(8) * sms / nm;
     if (cap < 1) cap = 1;
-    const int64_t need = (n + PF_THREADS - 1) / PF_THREADS;
+    const int64_t need = place_blocks(n, m.n, PF_THREADS);
     const dim3 grid(unsigned(need < cap ? need : cap), unsigned(nm));
     if (nm > 1)
       k_place<V4, true><<<grid, PF_THREADS, 0, s>>>(sk, sv, bk, bv, srow, mrow, row_start, counts, uint32_t(n), N,
