@@ -339,9 +339,8 @@ def measure(pm, sim, w, K, W, stream, rsz=4, spline=False, tuning=None, peak=Non
         avg = ms / cnt
         per_stage[name] = {"ms_per_step": ms / K, "launches": cnt, "avg_launch_ms": avg,
                            "bytes_per_launch": b, "GBps": (b / (avg / 1e3) / 1e9) if b else None}
-    # the transform stages are cuFFT's, except with the fused x-y kernels of 256^3 meshes (green_fused = 2, and
-    # the fp32 spline runs on such meshes)
-    # and, pass by pass, of (green_fused = 1) 512^3 meshes
+    # the transform stages are cuFFT's, except on 256^3 meshes (the x-y kernels: green_fused = 2, or an fp32 spline
+    # run) and on 512^3 meshes (the pass-by-pass kernels: fp32 cloud-in-cell with green_fused = 1)
     own_xy = sim.get_tuning().get("green_fused") == 2 or (spline and rsz == 4 and nm == 256)
     own_passes = rsz == 4 and not spline and nm == 512 and sim.get_tuning().get("green_fused") == 1
     lib_stages = () if own_xy or own_passes else pm.CUFFT_STAGES

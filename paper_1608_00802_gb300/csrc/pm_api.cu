@@ -601,7 +601,7 @@ void spline_taps(double hc, double* g) {
 // fp32 spline simulations on meshes that the x-y kernels transform (256^3): the transforms of a field are the
 // x-y kernel, one pass along z with the symbol between the two transforms, and the x-y kernel back, instead
 // of cuFFT's 3D plans and separate spectral passes.  Per step (five transforms, green, smoothing) 448 us with
-// those, SPL_FIG so.
+// those, 403 so.
 bool spline_own_fft(const pm_sim* s) { return !s->fp64() && spline(s) && xy_fft_supported(s->cfg.n_mesh); }
 const float2* fft_twiddles(const pm_sim* s) { return s->at<float2>(s->L.green); }
 const float* fft_sin2(const pm_sim* s) { return s->at<float>(s->L.green + size_t(s->cfg.n_mesh) * 8); }

@@ -10,8 +10,10 @@
 // the four-step z kernel at one block of 128 registers per SM (a pass over memory takes 160 us).  So each pass here
 // does as little as it can per value and leaves room for many threads: the five passes take 1193 us.  The
 // potential's error against float64 (particle density, of the largest |phi|): 4.7e-7 -> 4.0e-7.  (384^3 by the
-// same passes: 535 us against 987 by cuFFT's 3D pair and the Green pass, but in one run of a hundred the
-// other rounding moved particles next to nearly empty nodes by more than 1e-3: it keeps cuFFT.)
+// same passes: 535 us against 987 by cuFFT's 3D pair and the Green pass, but in one of 80 jobs the
+// displacements ended 2e-2 of the largest away from cuFFT's, in 7 of 80 more than 1e-4: the quantum force amplifies any
+// other rounding next to nearly empty nodes.  Which of the two is nearer to float64 over such jobs has not been
+// measured; 384^3 keeps cuFFT.)
 //
 // Rows: 16 threads a row (two rows a warp: the exchanges need no block barrier), H = N/2 = 16 Q points in two
 // steps, n = j + 16 m and k = k1 + Q k2: thread j a Q-point DFT over m (Q = 16) and the twiddle, thread
