@@ -2054,7 +2054,7 @@ __global__ void __launch_bounds__(KICK_THREADS, (FM == KICK_FM_HYBRID_Q && !PACK
 // (mode_norm).  A warp takes one quadrant row (|m_y|, |m_z|): along x the shell index does not fall, so
 // equal shells are runs of lanes, summed by a segmented scan, and the run's last lane adds to the warp's
 // own bins (no atomics; the sums are reproducible).  150^3: 365 us with a square root, three sinpi and three
-// shared fp64 atomics (compare-and-swap loops) per mode, 41 us so (39 with |k| to 3.6e-15 only).
+// shared fp64 atomics (compare-and-swap loops) per mode, 37 us so.
 
 // 1 / sinc^4(m / N), m = 0 .. N/2: the inverse cloud-in-cell window of |delta_k|^2 along one axis
 static __global__ void k_power_window(double* iw, int n) {
